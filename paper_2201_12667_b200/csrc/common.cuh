@@ -130,7 +130,7 @@ cudaError_t launch_update(Ctx* c, int batch, const int32_t* row_ptr, const int32
                           float* loss_out, HostResult* host_res, unsigned int host_seq);
 cudaError_t launch_predict(Ctx* c, int batch, const int32_t* row_ptr, const int32_t* col_idx,
                            const float* vals, int k, int dense, int32_t* out_ids, float* out_scores);
-bool dense_tc_usable(const Ctx* c, int k);           // inference over all neurons on the tensor pipe: shapes it covers
+// inference over all neurons, the hidden activations being in c->h
 cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* out_scores);
 cudaError_t setup_forward(Ctx* c);   // chooses the dedup path and the shared-memory layout
 
@@ -215,7 +215,7 @@ struct Ctx {
   int64_t t_host, r_host, next_rebuild;
   int64_t launches;
   int profiling;
-  void* pd_part;       // dense inference: the slices' best-k lists (ids, then scores), grown on demand
+  void* pd_part;       // inference over all neurons: thresholds, candidates and the subset's scores, grown on demand
   size_t pd_cap;
   void* prof;          // std::vector of event pairs while profiling
 };

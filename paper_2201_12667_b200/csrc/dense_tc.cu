@@ -1,4 +1,4 @@
-// Inference over all N neurons on the tensor pipe (dslide_predict_topk with dense = 1, k <= TC_K_MAX).
+// Inference over all N neurons on the tensor pipe (dslide_predict_topk with dense = 1).
 //
 // The logits of a batch against every output neuron are one contraction, Z[B][N] = h[B][H] . W2[N][H]^T + b2
 // (Section 3.6: "layer sparsity is 1"), so this path runs it on the fifth-generation tensor cores: tiles of W2
@@ -34,9 +34,12 @@ constexpr int TC_SPLIT = 4;        // read-back warps per quarter of tensor memo
 constexpr int TC_EPI = 128 * TC_SPLIT;                 // read-back threads
 constexpr int TC_THREADS = 96 + TC_EPI;                // warp 0: TMA producer; warp 1: tensor memory + MMA issue; warp 2: row norms; then the read-back warps
 constexpr int TC_EXTRA = 8;        // candidates kept beyond k: TC_EXTRA + k (the wider the margin, the rarer the exact fall-back)
-constexpr int TC_K_MAX = 8;
+constexpr int TC_H_TMEM = 256;     // hidden layers up to this width sit in tensor memory beside two accumulators; wider ones are
+                                   // streamed through shared memory with the tiles (WIDE)
+constexpr int TC_WIDE_STAGES = 6;  // WIDE: pairs of slabs (32 units of the samples, 32 units of the neurons) in flight
+constexpr int TC_RANK_CAP = 24;    // the threshold's rank in the subset grows with k up to this
 constexpr int TC_GBUF_MIN = 64;    // candidate slots per (buffer, sample) at least; a buffer that runs over sends the sample to the exact scan
-constexpr int TC_TARGET = 64;      // candidates aimed at per sample: TC_TARGET x cap
+constexpr int TC_TARGET = 64;      // candidates aimed at per sample: TC_TARGET x min(cap, TC_RANK_CAP)
 constexpr int TC_SUBSET = 64;      // the threshold pass scores every TC_SUBSET-th tile
 constexpr int TC_SUB_BYTES = TC_M * 128;               // one 32-unit slab of 128 rows
 constexpr float TC_ERR = 2.2e-3f;  // |approximate - exact| <= TC_ERR * |h| * |w|: two operands cut to 10 mantissa bits, fp32 sums
@@ -104,6 +107,11 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint32_t a_tmem, uint64_
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
                ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
+// The same with both operands in shared memory (hidden layers too wide for tensor memory)
+__device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+               ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
 __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, "
@@ -132,25 +140,34 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 __device__ __forceinline__ bool tc_better(float za, int ia, float zb, int ib) { return za > zb || (za == zb && ia < ib); }
 
 // Grid: (slices of the neurons, groups of 128 samples).  Dynamic shared memory (1024-byte aligned):
-// TC_STAGES tiles of W2 as [H/32][128 rows][128 B], then
+// TC_STAGES tiles of W2 as [ceil(H/32)][128 rows][128 B], then
 // the tiles' biases, the barriers.  (The samples' candidate buffers are in global memory.)
-template <bool DUMP>      // DUMP: write every score out (threshold pass); else append the scores that reach the sample's threshold
+// Every width and every k takes this kernel; a scan on the ALUs (one bulk copy per row of W2, 8 to 32 samples against a
+// staged row) took 11,700 us where the filter takes 389 us (H 200, N 253,855, 1,024 samples, k 5).
+// A hidden width that is no multiple of 32 ends in a slab whose missing units the tensor copy fills with zeros.
+// WIDE (H > TC_H_TMEM): the activations do not fit tensor memory, so a stage is one slab of the tile and the same 32
+// units of the block's samples, both by tensor copies; the samples' slabs come from L2 once per tile, which doubles
+// the copies of a tile but keeps the multiplications on the tensor pipe.
+template <bool DUMP, bool WIDE>      // DUMP: write every score out (threshold pass); else append the scores that reach the sample's threshold
 __global__ void __launch_bounds__(TC_THREADS, 1)
-k_dense_tc(const __grid_constant__ CUtensorMap tmW, const TcParams p) {
+k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH, const TcParams p) {
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int ksub = p.H / TC_KB;
-  const uint32_t tile_bytes = (uint32_t)ksub * TC_SUB_BYTES;
+  const int ksub = (p.H + TC_KB - 1) / TC_KB;
+  const int kfull = p.H / TC_KB;
+  const int klast = (p.H - (ksub - 1) * TC_KB + 7) >> 3;      // instructions (eight units each) of the last slab
+  const uint32_t tile_bytes = WIDE ? 2u * TC_SUB_BYTES : (uint32_t)ksub * TC_SUB_BYTES;      // of a stage
   unsigned char* smB = sm;
   const int nst = p.stages;
   float* sb = reinterpret_cast<float*>(smB + (size_t)nst * tile_bytes);                         // [accumulator][128] biases of its tile
   uint64_t* bars = reinterpret_cast<uint64_t*>(sb + TC_NACC * TC_N);
   uint64_t* bar_a = bars;                      // activations are in tensor memory
-  uint64_t* bar_full = bars + 1;               // [TC_STAGES] tile of W2 has arrived
-  uint64_t* bar_empty = bars + 1 + TC_STAGES;  // [TC_STAGES] tile of W2 has been consumed
-  uint64_t* bar_accfull = bars + 1 + 2 * TC_STAGES;              // [TC_NACC] accumulator written
-  uint64_t* bar_accempty = bars + 1 + 2 * TC_STAGES + TC_NACC;   // [TC_NACC] accumulator read back
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 1 + 2 * TC_STAGES + 2 * TC_NACC);
+  constexpr int NST = WIDE ? TC_WIDE_STAGES : TC_STAGES;
+  uint64_t* bar_full = bars + 1;               // [NST] the stage has arrived
+  uint64_t* bar_empty = bars + 1 + NST;        // [NST] the stage has been consumed
+  uint64_t* bar_accfull = bars + 1 + 2 * NST;              // [TC_NACC] accumulator written
+  uint64_t* bar_accempty = bars + 1 + 2 * NST + TC_NACC;   // [TC_NACC] accumulator read back
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 1 + 2 * NST + 2 * TC_NACC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -162,12 +179,12 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const TcParams p) {
   // they pass through shared memory; up to four sample groups share a tile's rows (they all see the same tiles).
   const int nshare = gridDim.y >= 4 ? 4 : (gridDim.y >= 2 ? 2 : 1);      // blocks that share a tile's 128 rows
   const bool norms = !DUMP && (int)blockIdx.y < nshare;
-  const int nacc = p.H <= TC_N ? TC_NACC : 2;      // accumulators in use; the activations follow them
+  const int nacc = WIDE || p.H <= TC_N ? TC_NACC : 2;      // accumulators in use; the activations follow them
   const uint32_t acol = (uint32_t)(nacc * TC_N);
 
   if (tid == 0) {
     tc_bar_init(bar_a, 128);
-    for (int i = 0; i < TC_STAGES; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
+    for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
     for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, TC_EPI); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -188,8 +205,19 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const TcParams p) {
     if (lane == 0) {
       int st = 0, stround = 0;
       for (int i = 0; i < my_tiles; ++i) {
-        if (stround > 0) tc_bar_wait(bar_empty + st, (stround - 1) & 1, abort_flag);
         const int row0 = (slice + i * p.nslices) * p.tile_stride * TC_N;
+        if (WIDE) {
+          for (int ks = 0; ks < ksub; ++ks) {
+            if (stround > 0) tc_bar_wait(bar_empty + st, (stround - 1) & 1, abort_flag);
+            unsigned char* to = smB + (size_t)st * tile_bytes;
+            tc_bar_expect(bar_full + st, tile_bytes);
+            tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
+            tc_tma_2d(to + TC_SUB_BYTES, &tmH, ks * TC_KB, s0, bar_full + st);
+            if (++st == nst) { st = 0; ++stround; }
+          }
+          continue;
+        }
+        if (stround > 0) tc_bar_wait(bar_empty + st, (stround - 1) & 1, abort_flag);
         tc_bar_expect(bar_full + st, tile_bytes);
         for (int ks = 0; ks < ksub; ++ks)
           tc_tma_2d(smB + (size_t)st * tile_bytes + (size_t)ks * TC_SUB_BYTES, &tmW, ks * TC_KB, row0, bar_full + st);
@@ -200,22 +228,42 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const TcParams p) {
     // ---------------- MMA issue: one thread ----------------
     if (lane == 0) {
       const uint32_t idesc = tc_idesc(TC_M, TC_N);
-      tc_bar_wait(bar_a, 0, abort_flag);
+      if (!WIDE) tc_bar_wait(bar_a, 0, abort_flag);
       const uint64_t b_base = tc_desc(tc_smem(smB));      // a descriptor's address field counts 16-byte units
       int st = 0, stround = 0, acc = 0, accround = 0;
       for (int i = 0; i < my_tiles; ++i) {
-        tc_bar_wait(bar_full + st, stround & 1, abort_flag);
+        if (!WIDE) tc_bar_wait(bar_full + st, stround & 1, abort_flag);
         if (accround > 0) tc_bar_wait(bar_accempty + acc, (accround - 1) & 1, abort_flag);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem_base + (uint32_t)(acc * TC_N);
+        if (WIDE) {
+          for (int ks = 0; ks < ksub; ++ks) {
+            tc_bar_wait(bar_full + st, stround & 1, abort_flag);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t b = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
+            const uint64_t a = b + (uint64_t)(TC_SUB_BYTES >> 4);
+            const int kn = ks == ksub - 1 ? klast : TC_KB / 8;
+            for (int kk = 0; kk < kn; ++kk)
+              tc_mma_ss(d, a + (uint64_t)(kk * 2), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
+            tc_commit(bar_empty + st);
+            if (++st == nst) { st = 0; ++stround; }
+          }
+          tc_commit(bar_accfull + acc);
+          if (++acc == nacc) { acc = 0; ++accround; }
+          continue;
+        }
         const uint64_t b_tile = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
-        for (int ks = 0; ks < ksub; ++ks) {
+        for (int ks = 0; ks < kfull; ++ks) {
           const uint32_t a = tmem_base + acol + (uint32_t)(ks * TC_KB);      // lanes = samples, columns = hidden units
           const uint64_t b = b_tile + (uint64_t)((ks * TC_SUB_BYTES) >> 4);
 #pragma unroll
           for (int kk = 0; kk < TC_KB / 8; ++kk)              // eight tf32 = 32 bytes per instruction
             tc_mma(d, a + (uint32_t)(kk * 8), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
         }
+        if (kfull < ksub)                                     // a last slab of fewer units
+          for (int kk = 0; kk < klast; ++kk)
+            tc_mma(d, tmem_base + acol + (uint32_t)(kfull * TC_KB + kk * 8), b_tile + (uint64_t)((kfull * TC_SUB_BYTES) >> 4) + (uint64_t)(kk * 2),
+                   idesc, (kfull | kk) != 0 ? 1u : 0u);
         tc_commit(bar_empty + st);          // the tile's shared memory is free once these instructions have read it
         tc_commit(bar_accfull + acc);       // and the accumulator is complete
         if (++st == nst) { st = 0; ++stround; }
@@ -228,10 +276,33 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const TcParams p) {
     if (norms) {
       float best = 0.f;
       int st = 0, stround = 0;
+      const int nrr = 4 / nshare;                      // rows of this block: nrr per lane
       for (int i = 0; i < my_tiles; ++i) {
+        if (WIDE) {
+          float part[4] = {0.f, 0.f, 0.f, 0.f};        // the sums of the lane's rows over the slabs
+          for (int ks = 0; ks < ksub; ++ks) {
+            tc_bar_wait(bar_full + st, stround & 1, abort_flag);
+            const unsigned char* tile = smB + (size_t)st * tile_bytes;
+#pragma unroll
+            for (int rr = 0; rr < 4; ++rr)
+              if (rr < nrr) {
+                const unsigned char* rowp = tile + (size_t)(32 * (nrr * (int)blockIdx.y + rr) + lane) * 128;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                  const float4 w = *reinterpret_cast<const float4*>(rowp + (size_t)((c ^ (lane & 7)) * 16));
+                  part[rr] = fmaf(w.x, w.x, fmaf(w.y, w.y, fmaf(w.z, w.z, fmaf(w.w, w.w, part[rr]))));
+                }
+              }
+            __syncwarp();
+            if (lane == 0) tc_bar_arrive(bar_empty + st);
+            if (++st == nst) { st = 0; ++stround; }
+          }
+#pragma unroll
+          for (int rr = 0; rr < 4; ++rr) best = fmaxf(best, part[rr]);
+          continue;
+        }
         tc_bar_wait(bar_full + st, stround & 1, abort_flag);
         const unsigned char* tile = smB + (size_t)st * tile_bytes;
-        const int nrr = 4 / nshare;                    // rows of this block: nrr per lane
         for (int rr = 0; rr < nrr; ++rr) {
           const unsigned char* rowp = tile + (size_t)(32 * (nrr * (int)blockIdx.y + rr) + lane) * 128;
           unsigned long long s0 = 0ull, s1 = 0ull;    // two pairs of partial sums (packed fp32 fused multiply-adds)
@@ -264,13 +335,13 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const TcParams p) {
     const int et = tid - 96;                // the first 128 read-back threads fetch the tile's biases
     const int vslice = slice * TC_SPLIT + half;    // buffers are kept per (slice, share of the columns)
     int2* mybuf = p.cand + ((size_t)vslice * p.Bpad + s0 + row) * p.gbuf;
-    const float tau = DUMP ? 0.f : p.tau[s0 + row];
+    const float tau = DUMP ? 0.f : (s0 + row < p.B ? p.tau[s0 + row] : INFINITY);      // rows past the batch keep nothing
     int cnt = 0;
     if (DUMP && slice == 0 && half == 0) {      // the threshold pass also clears what the filter pass accumulates into
       if (s0 + row < p.B) p.need_fix[s0 + row] = 0;
       if (tid == 96 && blockIdx.y == 0) *p.norm2max = 0u;
     }
-    if (half == 0) {
+    if (!WIDE && half == 0) {
       // the block's activations -> tensor memory: lane = sample, column = hidden unit (samples past the batch: zeros)
       const float4* hrow = reinterpret_cast<const float4*>(p.h + (size_t)(s0 + row) * p.H);
       const bool live = s0 + row < p.B;
@@ -278,7 +349,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const TcParams p) {
         uint32_t r[32];
 #pragma unroll
         for (int c4 = 0; c4 < 8; ++c4) {
-          const float4 v = live ? __ldg(hrow + (c0 >> 2) + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 v = live && c0 + 4 * c4 < p.H ? __ldg(hrow + (c0 >> 2) + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
           r[4 * c4] = __float_as_uint(v.x); r[4 * c4 + 1] = __float_as_uint(v.y);
           r[4 * c4 + 2] = __float_as_uint(v.z); r[4 * c4 + 3] = __float_as_uint(v.w);
         }
@@ -413,6 +484,7 @@ __global__ void __launch_bounds__(TAU_THREADS) k_tc_tau(const float* dump, int c
 // A flagged sample: every neuron scored exactly in fp32 by the sample's block (rare; the block walks all of W2).
 // fx_smem: [H] activation, then [warps][k] lists of scores and of ids, then the lists' lengths.
 constexpr int FX_THREADS = 256;
+constexpr int FX_FLOATS = 2112;      // H <= 1024 activations, 8 lists of k <= 64 scores and ids, their lengths
 __device__ void tc_exact_scan(float* fx_smem, int s, const float* W2, const RowHdr* hdr2, const float* h, int H, int N, int k,
                               int32_t* out_ids, float* out_scores) {
   float* hs = fx_smem;
@@ -469,12 +541,12 @@ __device__ void tc_exact_scan(float* fx_smem, int s, const float* W2, const RowH
 // ascending).  need_fix[s] = 1 when the filter cannot be shown to be exact.
 constexpr int RF_THREADS = FX_THREADS;
 constexpr int RF_MAXV = 512;       // buffers per sample at most
-constexpr int RF_SLOTS = 64;       // candidates scored exactly at most
+constexpr int RF_SLOTS = 384;      // candidates scored exactly at most (k = 64: about 190 reach the cut)
 __global__ void __launch_bounds__(RF_THREADS)
 k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* cand, const int* cand_cnt, int gbuf, const float* tau, int Bpad,
             const unsigned int* norm2max, int B, int H, int N, int cap, int nvs, int k, int32_t* out_ids, float* out_scores,
             const int* need_fix) {
-  __shared__ float fx_space[1024];               // the exact scan's work space (H <= 256 activations + 2 x 8 x 8 list entries + 8)
+  __shared__ float fx_space[FX_FLOATS];
   __shared__ int offs[RF_MAXV + 1];
   __shared__ float ez[RF_SLOTS], sz[RF_SLOTS];
   __shared__ int ei[RF_SLOTS], si[RF_SLOTS];
@@ -570,8 +642,8 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
   if (lane == 0) red[warp] = hs;
   __syncthreads();
   // order the exact scores: an entry's place is the number of better ones ((score, id) pairs are all different)
-  if (tid < nc) {
-    const float z = ez[tid]; const int j = ei[tid];
+  for (int e = tid; e < nc; e += RF_THREADS) {
+    const float z = ez[e]; const int j = ei[e];
     int rank = 0;
     for (int u = 0; u < nc; ++u) rank += tc_better(ez[u], ei[u], z, j) ? 1 : 0;
     sz[rank] = z; si[rank] = j;
@@ -588,6 +660,7 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
     // were dropped here, else the sample's threshold (a neuron below it was never a candidate).  Its exact score is
     // at most T plus the error bound; the k best are certain when the k-th exact score lies above.
     const float T = total > cap ? tc_unkey(K) : tau[s];
+    if (nc < k && nc < N) sh_fix = 1;            // scores that are not numbers never become candidates
     if (T > -INFINITY) {
       const float bound = T + TC_ERR * sqrtf(hn) * sqrtf(__uint_as_float(*norm2max)) + 1e-30f;
       const int kth = (k < nc ? k : nc) - 1;
@@ -597,6 +670,13 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
   }
   __syncthreads();
   if (fix || sh_fix) tc_exact_scan(fx_space, s, W2, hdr2, h, H, N, k, out_ids, out_scores);
+}
+
+// The exact scan by itself, one block per sample: fewer neurons than a tile, or no room for the filter's work space.
+__global__ void __launch_bounds__(FX_THREADS)
+k_exact_scan(const float* W2, const RowHdr* hdr2, const float* h, int H, int N, int k, int32_t* out_ids, float* out_scores) {
+  __shared__ float fx_space[FX_FLOATS];
+  tc_exact_scan(fx_space, blockIdx.x, W2, hdr2, h, H, N, k, out_ids, out_scores);
 }
 
 // ---------------------------------------------------------------------------
@@ -629,12 +709,15 @@ static bool make_map(CUtensorMap* m, const float* base, int rows, int H) {
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool dense_tc_usable(const Ctx* c, int k) {
-  return k >= 1 && k <= TC_K_MAX && c->H % TC_KB == 0 && c->H >= TC_KB && c->H <= 256 && c->N >= TC_N && encode_fn() != nullptr;
+static cudaError_t launch_exact_scan(Ctx* c, int batch, int k, int32_t* out_ids, float* out_scores) {
+  LaunchScope ls(c, KID_PREDICT);
+  k_exact_scan<<<batch, FX_THREADS, 0, c->stream>>>(c->W2, c->hdr2, c->h, c->H, c->N, k, out_ids, out_scores);
+  return cudaGetLastError();
 }
 
 // The hidden activations of the batch are in c->h (left there by the forward kernel in predict mode).
 cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* out_scores) {
+  if (c->N < TC_N || encode_fn() == nullptr) return launch_exact_scan(c, batch, k, out_ids, out_scores);
   const int cap = 2 * k + TC_EXTRA;
   const int groups = (batch + TC_M - 1) / TC_M;
   const int ntiles = (c->N + TC_N - 1) / TC_N;
@@ -658,8 +741,9 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   const size_t off_cand = off_cnt + up((size_t)nvs * Bpad * 4);
   // The threshold is the rank-th best of the subset's maxima, the rank chosen so that about TC_TARGET x cap neurons
   // reach it over all N whatever the subset's share; a buffer has room for four times its expected fill.
-  int rank = (cap * TC_TARGET + stride - 1) / stride;
-  if (rank > cap) rank = cap;
+  const int want = cap < TC_RANK_CAP ? cap : TC_RANK_CAP;
+  int rank = (want * TC_TARGET + stride - 1) / stride;
+  if (rank > want) rank = want;
   if (rank < 4) rank = 4;
   int gbuf = TC_GBUF_MIN;
   while (gbuf * nvs < 4 * rank * stride) gbuf <<= 1;
@@ -670,7 +754,12 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return e;
     if (c->pd_part) cudaFree(c->pd_part);
     c->pd_part = nullptr; c->pd_cap = 0;
-    if ((e = cudaMalloc(&c->pd_part, need)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&c->pd_part, need)) != cudaSuccess) {
+      c->pd_part = nullptr;
+      if (e != cudaErrorMemoryAllocation) return e;
+      cudaGetLastError();                 // no room for the filter: scored without it (slower, same results)
+      return launch_exact_scan(c, batch, k, out_ids, out_scores);
+    }
     c->pd_cap = need;
   }
   unsigned char* ws = reinterpret_cast<unsigned char*>(c->pd_part);
@@ -681,30 +770,32 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   int2* cand = reinterpret_cast<int2*>(ws + off_cand);
   float* dump = reinterpret_cast<float*>(ws + off_dump);
 
-  CUtensorMap tmW;
-  if (!make_map(&tmW, c->W2, c->N, c->H)) return cudaErrorInvalidValue;
-
+  const bool wide = c->H > TC_H_TMEM;
+  CUtensorMap tmW, tmH;
+  if (!make_map(&tmW, c->W2, c->N, c->H) || !make_map(&tmH, c->h, batch, c->H)) return cudaErrorInvalidValue;
 
   TcParams p;
   p.hdr2 = c->hdr2; p.h = c->h; p.cand = cand; p.cand_cnt = cand_cnt; p.dump = dump; p.tau = tau; p.need_fix = need_fix; p.norm2max = norm2; p.st = c->dstate;
   p.B = batch; p.Bpad = Bpad; p.H = c->H; p.N = c->N; p.dump_cols = dump_cols; p.gbuf = gbuf;
-  const size_t tile_bytes = (size_t)(c->H / TC_KB) * TC_SUB_BYTES;
+  const size_t tile_bytes = wide ? (size_t)2 * TC_SUB_BYTES : (size_t)((c->H + TC_KB - 1) / TC_KB) * TC_SUB_BYTES;
   int stages = (int)(((size_t)200 << 10) / tile_bytes);
-  if (stages > TC_STAGES) stages = TC_STAGES;
+  if (stages > (wide ? TC_WIDE_STAGES : TC_STAGES)) stages = wide ? TC_WIDE_STAGES : TC_STAGES;
   p.stages = stages;
   const size_t smem = 1024 + tile_bytes * stages + TC_NACC * TC_N * 4 + 24 * 8 + 64;
-  if ((e = cudaFuncSetAttribute(k_dense_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_dense_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  auto k_sub = wide ? k_dense_tc<true, true> : k_dense_tc<true, false>;
+  auto k_all = wide ? k_dense_tc<false, true> : k_dense_tc<false, false>;
+  if ((e = cudaFuncSetAttribute(k_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   {
     LaunchScope ls(c, KID_PREDICT);
     p.nslices = nslices_sub; p.ntiles = nsub; p.tile_stride = stride;
     // each kernel of the call may be placed while the kernel before it drains (they wait for it before they read or
     // write anything); the first follows the hidden-layer kernel in the same way
-    if ((e = launch_dependent(k_dense_tc<true>, dim3(nslices_sub, groups), dim3(TC_THREADS), smem, c->stream, tmW, p)) != cudaSuccess) return e;
+    if ((e = launch_dependent(k_sub, dim3(nslices_sub, groups), dim3(TC_THREADS), smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_tau, dim3(Bpad), dim3(TAU_THREADS), 0, c->stream, (const float*)dump, dump_cols, rank, tau)) != cudaSuccess)
       return e;
     p.nslices = nslices; p.ntiles = ntiles; p.tile_stride = 1;
-    if ((e = launch_dependent(k_dense_tc<false>, dim3(nslices, groups), dim3(TC_THREADS), smem, c->stream, tmW, p)) != cudaSuccess) return e;
+    if ((e = launch_dependent(k_all, dim3(nslices, groups), dim3(TC_THREADS), smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_refine, dim3(batch), dim3(RF_THREADS), 0, c->stream, (const float*)c->W2, (const RowHdr*)c->hdr2,
                               (const float*)c->h, (const int2*)cand, (const int*)cand_cnt, gbuf, (const float*)tau, Bpad,
                               (const unsigned int*)norm2, batch, c->H, c->N, cap, nvs, k, out_ids, out_scores, (const int*)need_fix)) !=
