@@ -64,7 +64,7 @@ void free_all(Ctx* c) {
                   c->hash_idx, c->hash_sign, c->bucket_off, c->bucket_ids, c->h, c->dh, c->loss, c->codes,
                   c->act_cnt, c->act_ids, c->act_z, c->act_p, c->act_g, c->mask1, c->ovf1, c->ovf2, c->hotmap1, c->hotcoef1,
                   c->mask2, c->proj1, c->bucket1_off, c->bucket1_ids, c->codes1n, c->codes1, c->hmask, c->cmask1, c->own1, c->own2, c->hot_rows, c->med_rows, c->hot_part, c->hot_done, c->dstate, c->keysA, c->keysB, c->valsA, c->valsB, c->tile_hist, c->bucket_part, c->ord_mid, c->ord_big, c->ord_cnt,
-                  c->st_dev[0], c->st_dev[1], c->st_dev[2], c->pd_part};
+                  c->st_dev[0], c->st_dev[1], c->st_dev[2], c->pd_part, c->touch2, c->wpre, c->trows, c->tstart, c->tinfo, c->act_loc, c->seg, c->tpart, c->rinfo, c->tlist, c->tlab, c->hash_pk};
   for (void* p : ptrs) if (p) cudaFree(p);
   for (int b = 0; b < ST_SETS; ++b) {
     if (c->st_host[b]) cudaFreeHost(c->st_host[b]);
@@ -228,7 +228,7 @@ dslide_status dslide_init(const dslide_config* cfg, dslide_ctx** out) {
   A(b1, H, true); A(mb1, H, true); A(vb1, H, true);
   A(W2, N * H, false); A(mW2, N * H, true); A(vW2, N * H, true);
   A(hdr2, N, true);
-  A(hash_idx, (size_t)c->KL * fn_len, true); A(hash_sign, (size_t)c->KL * fn_len, true);
+  A(hash_idx, (size_t)c->KL * fn_len, true); A(hash_sign, (size_t)c->KL * fn_len, true); A(hash_pk, (size_t)c->KL * fn_len, true);
   A(h, B * H, true); A(dh, B * H, true); A(loss, B, true); A(codes, B * c->L, true);
   A(act_cnt, B, true); A(act_z, B * S, true); A(act_p, B * S, true); A(act_g, B * S, true);
   A(hdr1, D, true); A(mask1, D * c->Wd, true); A(own1, D, true); A(ovf1, D * PAIR_T, false);
@@ -275,6 +275,7 @@ dslide_status dslide_init(const dslide_config* cfg, dslide_ctx** out) {
   }
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->st_copy_in, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = setup_forward(c);
+  if (e == cudaSuccess) e = setup_tiles(c);
   if (e == cudaSuccess) e = launch_init_gauss(c, c->W1, (int64_t)(D * H), RNG_W1);
   if (e == cudaSuccess) e = launch_init_gauss(c, c->W2, (int64_t)(N * H), RNG_W2);
   if (e == cudaSuccess && !c->dense) e = launch_draw_hash(c, 0);
@@ -581,6 +582,7 @@ dslide_status dslide_set_tensor(dslide_ctx* ctx, int32_t which, const void* host
   if (tr.pitch) CU(cudaMemcpy2DAsync(tr.ptr, (size_t)tr.pitch, host_src, sizeof(float), sizeof(float), (size_t)want / sizeof(float),
                                      cudaMemcpyHostToDevice, c->stream));
   else CU(cudaMemcpyAsync(tr.ptr, host_src, (size_t)want, cudaMemcpyHostToDevice, c->stream));
+  if (which == DSLIDE_T_HASH_IDX || which == DSLIDE_T_HASH_SIGN) CU(launch_pack_hash(c));
   return drain(c);
 }
 

@@ -120,6 +120,7 @@ struct LaunchScope {
 // launches (implemented in the .cu files)
 cudaError_t launch_init_gauss(Ctx* c, float* w, int64_t n, uint64_t stream_id);
 cudaError_t launch_draw_hash(Ctx* c, int64_t r);
+cudaError_t launch_pack_hash(Ctx* c);                // after hash_idx / hash_sign have changed
 cudaError_t launch_build_tables(Ctx* c);
 cudaError_t launch_draw_proj1(Ctx* c, int64_t r);   // the hidden layer's projections of rebuild count r
 cudaError_t launch_build_tables1(Ctx* c);           // codes of the hidden neurons and their tables
@@ -132,6 +133,10 @@ cudaError_t launch_predict(Ctx* c, int batch, const int32_t* row_ptr, const int3
                            const float* vals, int k, int dense, int32_t* out_ids, float* out_scores);
 // inference over all neurons, the hidden activations being in c->h
 cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* out_scores);
+// Active sets of many neurons, worked on by tiles of rows of W2 (tiles.cu; the weight update's part is in update.cu)
+cudaError_t setup_tiles(Ctx* c);                     // geometry and work space
+bool use_tiles(const Ctx* c, int batch);
+cudaError_t launch_tiles_forward(Ctx* c, int batch, const int32_t* label_ptr, const int32_t* labels);
 cudaError_t setup_forward(Ctx* c);   // chooses the dedup path and the shared-memory layout
 
 struct Ctx {
@@ -151,6 +156,7 @@ struct Ctx {
   float *mW1, *vW1, *mb1, *vb1, *mW2, *vW2;
   RowHdr *hdr1, *hdr2;             // per row of W1 / W2: touch count, slots and (W2) the bias b2 with its moments
   int32_t *hash_idx, *hash_sign;
+  uint16_t* hash_pk;               // SimHash: [fn_len][KL] coordinate and sign (top bit), made from the two above
   int32_t *bucket_off, *bucket_ids;
   // LSH-sampled hidden layer (hidden_L > 0): projections over the input coordinates, tables over the hidden neurons,
   // per-step codes and active masks, per row of W1 the hidden units some sample of the step touches it for
@@ -176,6 +182,23 @@ struct Ctx {
   float* hot_part;                 // [HOT_CAP][HOT_SLICES][H + 4] slice sums of those rows
   int* hot_done;                   // [HOT_CAP] finished slices per listed row (returns to 0)
   DevState* dstate;
+
+  // tiles of touched rows of W2 (tile_rows > 0: the context has the work space for them)
+  int tile_rows;                   // rows of a tile at most
+  int tile_step;                   // a tile starts at the first 32-id word whose touched rows begin at or past a multiple of this
+  int tile_max;                    // tiles at most
+  double tile_got, tile_pool;      // expected size of an active set, and how many rows the tables hand out at all
+  uint32_t* touch2;                // [ceil(N/32)] the touched rows; cleared again within the step
+  int* wpre;                       // [ceil(N/32) + 1] touched rows before each word
+  int* trows;                      // [N] touched rows, ascending
+  int* tstart;                     // [tile_max + 1] first of trows of every tile
+  int* tinfo;                      // number of tiles; 1 when a tile's rows did not come in time; entries of tlist handed out
+  uint16_t* act_loc;               // [B][act_stride] place of the neuron's row in its tile
+  int* seg;                        // [tile_max + 1][max_batch] where a sample's entries of every tile start
+  float* tpart;                    // [row chunks][B][H + 4] sums of exp(z - M) W2, M and the sum of exp(z - M)
+  int2* rinfo;                     // [N] per touched row: where its touches start in tlist, and how many they are
+  int2* tlist;                     // [B * act_stride] (sample, error bits) row by row, ascending samples in a row
+  int* tlab;                       // [B][max_labels] where the sample's labels are in its active set, -1 for a repeat
 
   // rebuild work space
   uint32_t *keysA, *keysB;

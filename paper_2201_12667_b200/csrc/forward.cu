@@ -31,6 +31,7 @@ constexpr unsigned FULLM = 0xffffffffu;
 struct FwdParams {
   const float *W1, *b1, *W2;
   const int32_t *hash_idx, *hash_sign, *bucket_off, *bucket_ids;
+  const uint16_t* hash_pk;     // SimHash: [fn_len][KL] coordinate, top bit = minus
   const int32_t *row_ptr, *col_idx;
   const float* vals;
   const int32_t *label_ptr, *labels;
@@ -39,6 +40,7 @@ struct FwdParams {
   int32_t *act_cnt, *act_ids;
   float *act_z, *act_p, *act_g;
   uint32_t *mask1, *mask2;
+  uint32_t* touch2;         // MODE 2: a bit per row of W2 that some sample touches
   int2 *ovf1, *ovf2;
   const int32_t* hotmap1;   // rows of W1 with a line of the coefficient table
   float* hotcoef1;
@@ -164,6 +166,21 @@ __device__ __forceinline__ void finish_touch(const FwdParams& p, bool live, RowH
   const bool first = live && nth == 0u;
   const unsigned base = own_reserve(first, n_own);
   own_store(first, base, own, row, s);
+}
+
+// The whole hand-off of one nonzero (entry e of the batch's columns) of sample s, by a whole warp.
+__device__ __forceinline__ void touch_w1(const FwdParams& p, bool live, int e, int s) {
+  int c = 0;
+  unsigned nth = 0u;
+  float x = 0.f;
+  if (live) {
+    c = __ldg(p.col_idx + e);
+    x = __ldg(p.vals + e);
+    nth = atomicAdd(&p.hdr1[c].cnt, 1u) & CNT_MASK;
+    const int line = __ldg(p.hotmap1 + c);
+    if (line >= 0) p.hotcoef1[(size_t)line * p.bstride + s] = x;
+  }
+  finish_touch(p, live, p.hdr1 + c, p.mask1 + (size_t)c * p.Wd, p.ovf1 + (size_t)c * PAIR_T, p.own1, &p.st->n_own[p.parity][1], c, ~c, nth, s, x);
 }
 
 // Maximum / sum over the lanes of a warp in a fixed order (same value in every lane).
@@ -440,7 +457,7 @@ __device__ __noinline__ int budget_select(int budget, int fill, int N, uint64_t 
 template <int MODE>
 __device__ __forceinline__ void skip_sample(const FwdParams& p, int s, int code) {
   const int tid = threadIdx.x;
-  if (MODE == 0) {
+  if (MODE != 1) {
     for (int k = tid; k < p.H; k += FWD_THREADS) { p.h[(size_t)s * p.H + k] = 0.f; p.dh[(size_t)s * p.H + k] = 0.f; }
     if (tid == 0) { p.act_cnt[s] = 0; p.loss[s] = 0.f; }
   } else {
@@ -452,7 +469,8 @@ __device__ __forceinline__ void skip_sample(const FwdParams& p, int s, int code)
   if (tid == 0) set_status(p.st, code);
 }
 
-// MODE 0 = training step, 1 = predict top-k; KPT = hidden units per thread (H <= KPT * FWD_THREADS); BULK: active sets of
+// MODE 0 = training step, 1 = predict top-k, 2 = the part of a training step up to the active sets (tiles.cu goes on from
+// there: sets of many neurons that the batch's samples share); KPT = hidden units per thread (H <= KPT * FWD_THREADS); BULK: active sets of
 // many chunks are expected (the host's estimate from the tables' shape) and their rows come by bulk copies
 template <int MODE, int KPT, bool BULK = false>
 __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
@@ -492,7 +510,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   const int rbeg = p.row_ptr[s], rend = p.row_ptr[s + 1];
   const int nnz = rend - rbeg;
   int lbeg = 0, nlab = 0;
-  if (MODE == 0) { lbeg = p.label_ptr[s]; nlab = p.label_ptr[s + 1] - lbeg; }
+  if (MODE != 1) { lbeg = p.label_ptr[s]; nlab = p.label_ptr[s + 1] - lbeg; }
 
   griddep_launch_dependents();       // the update kernel may be placed as blocks of this one leave
   if (tid == 0) {
@@ -513,13 +531,13 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   // ---- label checks: ids in range, list within the maximum (merged with the column checks by the first barrier) ----
   int bad = 0;
   if (nnz < 0 || nlab < 0) bad = DSLIDE_ERR_BAD_INDEX;
-  else if (MODE == 0) {
+  else if (MODE != 1) {
     for (int i = tid; i < nlab; i += FWD_THREADS) {
       int y = p.labels[lbeg + i];
       if (y < 0 || y >= N) bad = DSLIDE_ERR_BAD_INDEX;
     }
   }
-  const bool too_many_labels = MODE == 0 && nnz >= 0 && nlab > p.max_labels;
+  const bool too_many_labels = MODE != 1 && nnz >= 0 && nlab > p.max_labels;
 
   // ---- hidden layer: bias, then one fused multiply-add per nonzero in stored order, ReLU.  The rows of W1 of a
   //      chunk of nonzeros are copied into shared memory together, 16 bytes per thread and copy (cp.async: all of
@@ -618,7 +636,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     if (tid < p.L1) {
       uint32_t code = 0;
       for (int k = 0; k < p.K1; ++k) code |= (uint32_t)sh_b1[tid * p.K1 + k] << k;
-      if (MODE == 0) p.codes1[(size_t)s * p.L1 + tid] = code;
+      if (MODE != 1) p.codes1[(size_t)s * p.L1 + tid] = code;
       const int32_t* off = p.bucket1_off + (size_t)tid * ((1 << p.K1) + 1) + code;
       const int beg = __ldg(off);
       int cnt = __ldg(off + 1) - beg;
@@ -632,7 +650,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
         atomicOr(&sh_hmask[k >> 5], 1u << (k & 31));
       }
     __syncthreads();
-    if (MODE == 0 && tid < p.Hw) p.hmask[(size_t)s * p.Hw + tid] = sh_hmask[tid];
+    if (MODE != 1 && tid < p.Hw) p.hmask[(size_t)s * p.Hw + tid] = sh_hmask[tid];
   }
 #pragma unroll
   for (int u = 0; u < KPT; ++u) {
@@ -641,7 +659,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       const bool on = p.L1 == 0 || ((sh_hmask[k >> 5] >> (k & 31)) & 1u);
       const float hv = (on && acc[u] > 0.f) ? acc[u] : 0.f;
       sh_h[k] = hv;
-      if (MODE == 0 || p.dense) p.h[(size_t)s * H + k] = hv;
+      if (MODE != 1 || p.dense) p.h[(size_t)s * H + k] = hv;
     }
   }
   if (MODE == 1 && p.dense) return;        // inference over all neurons: the logits are taken by the kernels of dense_tc.cu
@@ -668,7 +686,23 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     }
     for (int f = tid; f < p.KL; f += FWD_THREADS) {
       const int32_t* ix = hidx + (size_t)f * p.fn_len;
-      if (p.family == DSLIDE_SIMHASH) {
+      if (p.family == DSLIDE_SIMHASH && p.hash_sm_off < 0) {
+        // the packed table: a warp reads 32 functions' i-th coordinates (sign in the top bit) side by side, sixteen rounds
+        // of them in flight; sums in stored order as ever
+        float sum = 0.f;
+        for (int i0 = 0; i0 < p.fn_len; i0 += 16) {
+          unsigned e[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) e[i] = i0 + i < p.fn_len ? (unsigned)__ldg(p.hash_pk + (size_t)(i0 + i) * p.KL + f) : 0u;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (i0 + i < p.fn_len) {
+              const float x = sh_h[e[i] & 0x7fffu];
+              sum = __fadd_rn(sum, (e[i] & 0x8000u) ? -x : x);
+            }
+        }
+        sh_part[f] = sum >= 0.f ? 1 : 0;
+      } else if (p.family == DSLIDE_SIMHASH) {
         const int32_t* sg = hsgn + (size_t)f * p.fn_len;
         float sum = 0.f;
         for (int i = 0; i < p.fn_len; ++i) {
@@ -736,7 +770,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
           if (t < p.L) {
             const uint32_t code = table_code(t);
             sh_code[t] = code;
-            if (MODE == 0) p.codes[(size_t)s * p.L + t] = code;
+            if (MODE != 1) p.codes[(size_t)s * p.L + t] = code;
             const int32_t* off = p.bucket_off + (size_t)t * (size_t)(p.nb + 1) + code;
             beg[u] = __ldg(off);
             cnt[u] = __ldg(off + 1);
@@ -764,7 +798,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       for (int t = tid; t < p.L; t += FWD_THREADS) {
         const uint32_t code = table_code(t);
         sh_code[t] = code;
-        if (MODE == 0) p.codes[(size_t)s * p.L + t] = code;
+        if (MODE != 1) p.codes[(size_t)s * p.L + t] = code;
         const int32_t* off = p.bucket_off + (size_t)t * (size_t)(p.nb + 1) + code;
         const int beg = __ldg(off);
         int cnt = __ldg(off + 1) - beg;
@@ -807,14 +841,29 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       for (int w = tid; w < n4; w += FWD_THREADS) dd4[w] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
     }
-    for (int c = tid; c < ncand; c += FWD_THREADS) {
-      int lo = 0, hi = p.L - 1;          // last table whose candidates start at or before c
-      while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (sh_tbase[mid] <= c) lo = mid; else hi = mid - 1; }
-      const int j = __ldg(p.bucket_ids + (size_t)lo * N + sh_tbeg[lo] + (c - sh_tbase[lo]));
-      if (bitmap) atomicOr(&sh_dd[j >> 5], 1u << (j & 31));
-      else sh_dd[c] = packed ? ((uint32_t)j << RANK_BITS) | (uint32_t)c : (uint32_t)j;
+    constexpr int CU = MODE == 2 ? 4 : 1;      // thousands of candidates: several per thread and round, their loads in flight together
+    for (int c0 = tid; c0 < ncand; c0 += CU * FWD_THREADS) {
+      int j[CU];
+#pragma unroll
+      for (int u = 0; u < CU; ++u) {
+        const int c = c0 + u * FWD_THREADS;
+        j[u] = 0;
+        if (c < ncand) {
+          int lo = 0, hi = p.L - 1;        // last table whose candidates start at or before c
+          while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (sh_tbase[mid] <= c) lo = mid; else hi = mid - 1; }
+          j[u] = __ldg(p.bucket_ids + (size_t)lo * N + sh_tbeg[lo] + (c - sh_tbase[lo]));
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < CU; ++u) {
+        const int c = c0 + u * FWD_THREADS;
+        if (c < ncand) {
+          if (bitmap) atomicOr(&sh_dd[j[u] >> 5], 1u << (j[u] & 31));
+          else sh_dd[c] = packed ? ((uint32_t)j[u] << RANK_BITS) | (uint32_t)c : (uint32_t)j[u];
+        }
+      }
     }
-    if (MODE == 0)
+    if (MODE != 1)
       for (int i = tid; i < nlab; i += FWD_THREADS) {
         const int y = p.labels[lbeg + i];
         if (bitmap) atomicOr(&sh_dd[y >> 5], 1u << (y & 31));
@@ -822,32 +871,49 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       }
     if (bitmap) {
       __syncthreads();
+      // every warp takes a contiguous share of the words, 32 at a time; a lane writes out the ids of its word
       const int nwords = (N + 31) >> 5;
-      const int chunk = (nwords + FWD_THREADS - 1) / FWD_THREADS;
-      const int wbeg = tid * chunk, wend = min(nwords, wbeg + chunk);
+      const int share = ((nwords + FWD_WARPS - 1) / FWD_WARPS + 31) & ~31;
+      const int wbeg = min(nwords, warp * share), wend = min(nwords, wbeg + share);
       int cnt = 0;
-      for (int w = wbeg; w < wend; ++w) cnt += __popc(sh_dd[w]);
-      int pos = block_excl_scan(cnt, sh_misc, &total);
-      if (total <= p.act_stride && cnt > 0) {
-        for (int w = wbeg; w < wend; ++w) {
-          uint32_t bits = sh_dd[w];
+      for (int w = wbeg + lane; w < wend; w += 32) cnt += __popc(sh_dd[w]);
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) cnt += __shfl_xor_sync(FULLM, cnt, d);
+      if (lane == 0) sh_misc[warp] = cnt;
+      __syncthreads();
+      int pos = 0;
+      for (int q = 0; q < FWD_WARPS; ++q) {
+        const int cq = sh_misc[q];
+        if (q < warp) pos += cq;
+        total += cq;
+      }
+      if (total <= p.act_stride && cnt > 0)
+        for (int w0 = wbeg; w0 < wend; w0 += 32) {
+          uint32_t bits = w0 + lane < wend ? sh_dd[w0 + lane] : 0u;
+          const int mine = __popc(bits);
+          int incl = mine;
+#pragma unroll
+          for (int d = 1; d < 32; d <<= 1) {
+            const int n = __shfl_up_sync(FULLM, incl, d);
+            if (lane >= d) incl += n;
+          }
+          int at = pos + incl - mine;
           while (bits) {
-            const int b = __ffs(bits) - 1;
-            const int j = (w << 5) + b;
-            ids[pos] = j;
-            if (pos < ACT_SM) sh_ids[pos] = j;
-            ++pos;
+            const int j = ((w0 + lane) << 5) + __ffs(bits) - 1;
+            ids[at] = j;
+            if (at < ACT_SM) sh_ids[at] = j;
+            ++at;
             bits &= bits - 1;
           }
+          pos += __shfl_sync(FULLM, incl, 31);
         }
-      }
     } else if (ncand + nlab <= RANK_MAX) {
       const int n = ncand + nlab;
       if (packed && tid < 4 && n + tid < ((n + 3) & ~3)) sh_dd[n + tid] = 0xffffffffu;
       __syncthreads();
       uint32_t* srt = sh_dd + RANK_MAX;
       const int per = (n + FWD_THREADS - 1) / FWD_THREADS;
-      if (packed && n <= FWD_THREADS - 64) {
+      if (MODE != 2 && packed && n <= FWD_THREADS - 64) {
         // the warps the counting below leaves idle ask L2 for the candidates' rows of W2 meanwhile (the staging after
         // the dedup then finds most of them there); a hint only: duplicates are asked twice, nothing waits for it
         const int idle0 = (n + 31) & ~31;                          // first thread without a value to rank
@@ -954,10 +1020,39 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     na = total;
     __syncthreads();                 // ids visible to the block; the dedup work space is free from here on
     if (p.budget > 0)
-      na = budget_select(p.budget, p.budget_fill, N, p.seed, p.tcount, s, ids, sh_ids, na, MODE == 0 ? p.labels + lbeg : nullptr,
+      na = budget_select(p.budget, p.budget_fill, N, p.seed, p.tcount, s, ids, sh_ids, na, MODE != 1 ? p.labels + lbeg : nullptr,
                          nlab, smem + p.off_dedup, p.stage_bytes, sh_misc, p.st);
   }
-  if (MODE == 0 && tid == 0) p.act_cnt[s] = na;
+  if (MODE != 1 && tid == 0) p.act_cnt[s] = na;
+  if (MODE == 2) {
+    // ---- the rows of W2 that the batch touches, as a bit per row (most are marked already: a read is enough), and the
+    //      hand-off of the sample's rows of W1 ----
+    constexpr int TU = 4;
+    for (int a0 = tid; a0 < na; a0 += TU * FWD_THREADS) {
+      int j[TU];
+      uint32_t have[TU];
+#pragma unroll
+      for (int u = 0; u < TU; ++u) j[u] = a0 + u * FWD_THREADS < na ? ids[a0 + u * FWD_THREADS] : -1;
+#pragma unroll
+      for (int u = 0; u < TU; ++u) have[u] = j[u] >= 0 ? __ldcg(p.touch2 + (j[u] >> 5)) : 0xffffffffu;
+#pragma unroll
+      for (int u = 0; u < TU; ++u)
+        if (j[u] >= 0 && !((have[u] >> (j[u] & 31)) & 1u)) atomicOr(p.touch2 + (j[u] >> 5), 1u << (j[u] & 31));
+    }
+    if (p.L1 > 0)
+      for (int i = tid; i < nnz; i += FWD_THREADS) {
+        const int c = __ldg(p.col_idx + rbeg + i);
+        for (int w = 0; w < p.Hw; ++w)
+          if (sh_hmask[w]) atomicOr(&p.cmask1[(size_t)c * p.Hw + w], sh_hmask[w]);
+      }
+    for (int i0 = 0; i0 < nnz; i0 += FWD_THREADS) touch_w1(p, i0 + tid < nnz, rbeg + i0 + tid, s);
+    if (tid == 0) {
+      atomicAdd(&p.st->acc[p.parity][0], (unsigned long long)na);
+      atomicAdd(&p.st->acc[p.parity][1], (unsigned long long)nnz);
+      atomicAdd(&p.st->acc[p.parity][2], (unsigned long long)sh_misc[24]);
+    }
+    return;
+  }
   const bool small = !dense && na <= ACT_SM;      // ids and logits mirrored in shared memory
   // one pointer per array, to shared or to global memory (a conditional expression over two loads would issue both)
   const int* idp = small ? sh_ids : ids;
@@ -1310,21 +1405,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       for (int w = 0; w < p.Hw; ++w)
         if (sh_hmask[w]) atomicOr(&p.cmask1[(size_t)c * p.Hw + w], sh_hmask[w]);
     }
-  for (int i0 = FWD_THREADS; i0 < nnz; i0 += FWD_THREADS) {
-    const int i = i0 + tid;
-    const bool live = i < nnz;
-    int c = 0;
-    unsigned nth = 0u;
-    float x = 0.f;
-    if (live) {
-      c = __ldg(p.col_idx + rbeg + i);
-      x = __ldg(p.vals + rbeg + i);
-      nth = atomicAdd(&p.hdr1[c].cnt, 1u) & CNT_MASK;
-      const int line = __ldg(p.hotmap1 + c);
-      if (line >= 0) p.hotcoef1[(size_t)line * p.bstride + s] = x;
-    }
-    finish_touch(p, live, p.hdr1 + c, p.mask1 + (size_t)c * p.Wd, p.ovf1 + (size_t)c * PAIR_T, p.own1, &p.st->n_own[p.parity][1], c, ~c, nth, s, x);
-  }
+  for (int i0 = FWD_THREADS; i0 < nnz; i0 += FWD_THREADS) touch_w1(p, i0 + tid < nnz, rbeg + i0 + tid, s);
   if (!dense) {
 #pragma unroll
     for (int u = 0; u < HO_PER; ++u)
@@ -1457,6 +1538,8 @@ cudaError_t setup_forward(Ctx* c) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<0, MAX_KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<0, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<0, MAX_KPT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<2, MAX_KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<1, MAX_KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   return e;
@@ -1466,11 +1549,11 @@ static FwdParams make_params(Ctx* c, int batch, const int32_t* row_ptr, const in
                              const int32_t* label_ptr, const int32_t* labels) {
   FwdParams p;
   p.W1 = c->W1; p.b1 = c->b1; p.W2 = c->W2;
-  p.hash_idx = c->hash_idx; p.hash_sign = c->hash_sign; p.bucket_off = c->bucket_off; p.bucket_ids = c->bucket_ids;
+  p.hash_idx = c->hash_idx; p.hash_sign = c->hash_sign; p.hash_pk = c->hash_pk; p.bucket_off = c->bucket_off; p.bucket_ids = c->bucket_ids;
   p.row_ptr = row_ptr; p.col_idx = col_idx; p.vals = vals; p.label_ptr = label_ptr; p.labels = labels;
   p.h = c->h; p.dh = c->dh; p.loss = c->loss; p.codes = c->codes;
   p.act_cnt = c->act_cnt; p.act_ids = c->act_ids; p.act_z = c->act_z; p.act_p = c->act_p; p.act_g = c->act_g;
-  p.mask1 = c->mask1; p.mask2 = c->mask2; p.ovf1 = c->ovf1; p.ovf2 = c->ovf2;
+  p.mask1 = c->mask1; p.mask2 = c->mask2; p.touch2 = c->touch2; p.ovf1 = c->ovf1; p.ovf2 = c->ovf2;
   p.hotmap1 = c->hotmap1; p.hotcoef1 = c->hotcoef1; p.bstride = c->cfg.max_batch; p.hdr1 = c->hdr1; p.hdr2 = c->hdr2;
   p.own1 = c->own1; p.own2 = c->own2; p.hot_rows = c->hot_rows; p.med_rows = c->med_rows; p.parity = (int)(c->t_host & 1);
   p.st = c->dstate; p.out_ids = nullptr; p.out_scores = nullptr;
@@ -1498,6 +1581,13 @@ cudaError_t launch_forward_train(Ctx* c, int batch, const int32_t* row_ptr, cons
                                  const int32_t* label_ptr, const int32_t* labels, int inputs_ready) {
   FwdParams p = make_params(c, batch, row_ptr, col_idx, vals, label_ptr, labels);
   p.inputs_ready = inputs_ready;
+  if (use_tiles(c, batch)) {
+    LaunchScope ls(c, KID_FORWARD);
+    cudaError_t e = c->H <= FWD_THREADS
+                        ? launch_dependent(k_forward<2, 1>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p)
+                        : launch_dependent(k_forward<2, MAX_KPT>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
+    return e != cudaSuccess ? e : launch_tiles_forward(c, batch, label_ptr, labels);
+  }
   {
     LaunchScope ls(c, KID_FORWARD);
     // hidden layers of up to FWD_THREADS units take the variant with one unit per thread (less code, fewer registers)

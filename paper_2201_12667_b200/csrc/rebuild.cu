@@ -89,17 +89,37 @@ __global__ void __launch_bounds__(DRAW_THREADS) k_draw_dwta(int32_t* idx, long l
   }
 }
 
-cudaError_t launch_draw_hash(Ctx* c, int64_t r) {
+// SimHash functions as the forward kernel reads them: [coordinate of the function][function], 16 bits each, top bit =
+// minus, so that the threads of a warp (one function each) read side by side.
+__global__ void k_pack_simhash(const int32_t* idx, const int32_t* sign, uint16_t* pk, int KL, int m) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= KL * m) return;
+  const int i = e / KL, f = e - i * KL;
+  pk[e] = (uint16_t)((idx[(size_t)f * m + i] & 0x7fff) | (sign[(size_t)f * m + i] > 0 ? 0 : 0x8000));
+}
+
+cudaError_t launch_pack_hash(Ctx* c) {
+  if (c->cfg.hash_family != DSLIDE_SIMHASH || c->dense) return cudaSuccess;
   LaunchScope ls(c, KID_DRAW_HASH);
-  if (c->cfg.hash_family == DSLIDE_SIMHASH) {
-    k_draw_simhash<<<(c->KL + 63) / 64, 64, 0, c->stream>>>(c->hash_idx, c->hash_sign, c->KL, c->H, c->fn_len,
-                                                           c->cfg.seed, (uint64_t)r);
-  } else {
-    long long total = (long long)c->KL * c->fn_len;
-    int nperm = (int)((total + c->H - 1) / c->H);
-    k_draw_dwta<<<nperm, DRAW_THREADS, 2 * c->H * sizeof(int), c->stream>>>(c->hash_idx, total, c->H, c->cfg.seed, (uint64_t)r);
-  }
+  const int n = c->KL * c->fn_len;
+  k_pack_simhash<<<(n + 255) / 256, 256, 0, c->stream>>>(c->hash_idx, c->hash_sign, c->hash_pk, c->KL, c->fn_len);
   return cudaGetLastError();
+}
+
+cudaError_t launch_draw_hash(Ctx* c, int64_t r) {
+  {
+    LaunchScope ls(c, KID_DRAW_HASH);
+    if (c->cfg.hash_family == DSLIDE_SIMHASH) {
+      k_draw_simhash<<<(c->KL + 63) / 64, 64, 0, c->stream>>>(c->hash_idx, c->hash_sign, c->KL, c->H, c->fn_len,
+                                                             c->cfg.seed, (uint64_t)r);
+    } else {
+      long long total = (long long)c->KL * c->fn_len;
+      int nperm = (int)((total + c->H - 1) / c->H);
+      k_draw_dwta<<<nperm, DRAW_THREADS, 2 * c->H * sizeof(int), c->stream>>>(c->hash_idx, total, c->H, c->cfg.seed, (uint64_t)r);
+    }
+  }
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_pack_hash(c);
 }
 
 // ------------------------------------------------------------------ LSH-sampled hidden layer

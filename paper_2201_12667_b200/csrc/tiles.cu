@@ -1,0 +1,734 @@
+// Training steps whose active sets hold thousands of neurons that the batch's samples share: logits and the
+// back-propagated error by tiles of rows of W2 instead of sample by sample.
+//
+// A block per sample fetches every active row once per sample that has it active (14 to 60 times over a batch: 5 GB
+// per step where the rows are 82 MB), and counts every touch with an atomic.  Here the rows that the batch touches
+// are numbered in id order and cut into tiles that fit shared memory; a tile's rows are fetched once and serve all
+// samples.  A sample's active ids are ascending, so its entries of a tile are one run of its list.
+//
+//   k_forward<2>    : hidden layer, codes, active sets; marks the touched rows in a bitmap (forward.cu)
+//   k_tile_scan     : touched rows before every word of the bitmap, and where the tiles start
+//   k_tile_index    : the list of touched rows; per active neuron its place in its tile; per (tile, sample) the run
+//   k_tile_forward  : a block holds a tile; a warp takes a sample's run: four rows at a time are read into registers,
+//                     their logits taken, and the sums S = sum_a exp(z_a - M) W2[a], E = sum_a exp(z_a - M) carried
+//                     along with a running maximum M (so a row is read from shared memory once for both).
+//   k_tile_combine  : per sample: the row chunks' S, E, M put together, loss, errors, error at the hidden layer
+//   k_tile_lists    : per touched row the list of (sample, error), ascending samples
+//   k_rows_update   : gradients and Adam of the touched rows of W2 (update.cu)
+// The order of every sum follows from the touched rows alone: results are the same from run to run.
+#include <math.h>
+
+#include "common.cuh"
+
+namespace dslide {
+
+constexpr unsigned TFULL = 0xffffffffu;
+// x / step for 0 <= x <= TILE_N_MAX and step <= TILE_ROWS_MAX, by a multiplication with ceil(2^32 / step)
+__host__ __device__ __forceinline__ unsigned tile_magic(int step) { return (unsigned)(((1ull << 32) + (unsigned)step - 1) / (unsigned)step); }
+__device__ __forceinline__ int tile_of(int x, unsigned magic, int step) { return step == 1 ? x : (int)__umulhi((unsigned)x, magic); }
+// two fused multiply-adds in one instruction: a += b * c on pairs of floats
+__device__ __forceinline__ void fma2(unsigned long long& a, unsigned long long b, unsigned long long c) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(b), "l"(c));
+}
+__device__ __forceinline__ unsigned long long pair2(float lo, float hi) {
+  return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
+constexpr int TS_THREADS = 1024;
+constexpr int TI_THREADS = 512;
+constexpr int TF_THREADS = 512;
+constexpr int TF_WARPS = TF_THREADS / 32;
+constexpr int TC3_THREADS = 512;
+constexpr int TL_THREADS = 512;
+constexpr int TL_WARPS = TL_THREADS / 32;
+constexpr int TL_CHUNK = 1024;                         // samples listed at a time
+constexpr int TILE_BYTES = 196 * 1024;                 // shared memory for a tile's rows
+constexpr int TILE_N_MAX = 8 << 20;
+constexpr int TILE_ROWS_MAX = 512;                     // a thread of k_tile_lists each
+constexpr size_t TILE_PART_BYTES = (size_t)32 << 20;   // the row chunks' sums stay in L2
+constexpr size_t TILE_SEG_BYTES = (size_t)512 << 20, TILE_LIST_BYTES = (size_t)2 << 30;      // beyond these the work space is not worth it
+// Which steps go by tiles: from TILE_MIN_SET neurons per sample on, when a sample has at least TILE_MIN_RUN of them in a
+// tile on average (below that, walking the (tile, sample) pairs costs more than the shared rows save).
+constexpr double TILE_MIN_SET = 512.0, TILE_MIN_RUN = 1.5;
+
+// Expected size of an active set and of the pool of rows the tables hand out, from the tables' shape: L buckets of
+// about N / 2^bits ids; where the cap cuts them, the lowest ids of every bucket are what all samples share.
+static void expect_sets(Ctx* c) {
+  const double mean = (double)c->N / (double)c->nb;
+  const double per = mean < c->cap ? mean : (double)c->cap;
+  double pool = (double)c->N;
+  if (mean > c->cap && 1.6 * c->cap * (double)c->nb < pool) pool = 1.6 * c->cap * (double)c->nb;
+  double got = pool * -expm1(-(double)c->L * per / pool);
+  if (c->cfg.sample_budget > 0 && got > c->cfg.sample_budget) got = c->cfg.sample_budget;
+  c->tile_got = got;
+  c->tile_pool = pool;
+}
+
+bool use_tiles(const Ctx* c, int batch) {
+  if (c->tile_rows == 0) return false;
+  const double touched = c->tile_pool * -expm1(-(double)batch * c->tile_got / c->tile_pool);
+  return c->tile_got * (double)c->tile_step >= TILE_MIN_RUN * touched;
+}
+
+// Row chunks (blocks that walk the tiles side by side) and groups of samples of k_tile_forward.
+static void tile_grid(const Ctx* c, int batch, int* chunks, int* groups) {
+  const size_t one = (size_t)batch * (c->H + 4) * sizeof(float);
+  int most = (int)(TILE_PART_BYTES / one);
+  if (most < 1) most = 1;
+  int q = (c->num_sms + most - 1) / most;
+  const int qmax = (batch + TF_WARPS - 1) / TF_WARPS;
+  if (q > qmax) q = qmax;
+  if (q < 1) q = 1;
+  int p = c->num_sms / q;
+  if (p < 1) p = 1;
+  if (p > c->tile_max) p = c->tile_max;
+  *chunks = p;
+  *groups = q;
+}
+
+cudaError_t setup_tiles(Ctx* c) {
+  c->tile_rows = 0;
+  if (c->dense) return cudaSuccess;
+  expect_sets(c);
+  if (c->tile_got < TILE_MIN_SET) return cudaSuccess;
+  int rows = TILE_BYTES / ((c->H + 4) * 4);
+  if (rows > TILE_ROWS_MAX) rows = TILE_ROWS_MAX;
+  const int step = rows - 31;                // a tile takes whole words of the bitmap
+  if (step < 1 || c->N > TILE_N_MAX) return cudaSuccess;
+  const int64_t tmax = (int64_t)c->N / step + 2;
+  const size_t B = c->cfg.max_batch;
+  if ((size_t)(tmax + 1) * B * 4 > TILE_SEG_BYTES || B * (size_t)c->act_stride * 8 > TILE_LIST_BYTES) return cudaSuccess;
+  c->tile_step = step;
+  c->tile_max = (int)tmax;
+  size_t most = 0;
+  for (int b = 1; b <= c->cfg.max_batch; ++b) {
+    int p, q;
+    tile_grid(c, b, &p, &q);
+    const size_t n = (size_t)p * b * (c->H + 4);
+    if (n > most) most = n;
+  }
+  const size_t nw = ((size_t)c->N + 31) / 32;
+  cudaError_t e = cudaSuccess;
+  auto get = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
+  get((void**)&c->touch2, nw * 4);
+  get((void**)&c->wpre, (nw + 1) * 4);
+  get((void**)&c->trows, (size_t)c->N * 4);
+  get((void**)&c->tstart, (size_t)(tmax + 1) * 4);
+  get((void**)&c->tinfo, 16);
+  get((void**)&c->act_loc, B * (size_t)c->act_stride * 2);
+  get((void**)&c->seg, (size_t)(tmax + 1) * B * 4);
+  get((void**)&c->tpart, most * 4);
+  get((void**)&c->rinfo, (size_t)c->N * 8);
+  get((void**)&c->tlist, B * (size_t)c->act_stride * 8);
+  get((void**)&c->tlab, B * (size_t)c->cfg.max_labels * 4);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->touch2, 0, nw * 4, c->stream);
+  if (e == cudaSuccess) c->tile_rows = rows;
+  return e;
+}
+
+// One block: touched rows before every word (exclusive running sum of the words' bit counts), and the first row of
+// every tile: word w belongs to tile wpre[w] / step.
+__global__ void __launch_bounds__(TS_THREADS)
+k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int* tinfo, unsigned int* n_touched) {
+  __shared__ int sh[TS_THREADS / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  griddep_launch_dependents();
+  griddep_wait();
+  const int per = ((nw + TS_THREADS - 1) / TS_THREADS + 3) & ~3;
+  const int w0 = min(nw, tid * per), w1 = min(nw, w0 + per);
+  int mine = 0;
+  int w = w0;
+  for (; w + 4 <= w1; w += 4) {
+    const uint4 x = __ldcg(reinterpret_cast<const uint4*>(touch + w));
+    mine += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+  }
+  for (; w < w1; ++w) mine += __popc(__ldcg(touch + w));
+  int incl = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int o = __shfl_up_sync(TFULL, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) sh[warp] = incl;
+  __syncthreads();
+  if (warp == 0) {
+    int v = sh[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int o = __shfl_up_sync(TFULL, v, d);
+      if (lane >= d) v += o;
+    }
+    sh[lane] = v;
+  }
+  __syncthreads();
+  const int total = sh[TS_THREADS / 32 - 1];
+  int run = incl - mine + (warp > 0 ? sh[warp - 1] : 0);
+  // the tile of the word before this thread's first one: its start, or that of a tile further back, covers `run`
+  const unsigned magic = tile_magic(step);
+  int tile = -1;
+  if (w0 > 0 && w0 < w1) {
+    const int before = run - __popc(__ldcg(touch + w0 - 1));
+    tile = tile_of(before, magic, step);
+  }
+  for (w = w0; w < w1; ++w) {
+    wpre[w] = run;
+    const int t = tile_of(run, magic, step);
+    for (; tile < t;) tstart[++tile] = run;
+    run += __popc(__ldcg(touch + w));
+  }
+  if (w0 < w1 && w1 == nw) {                 // the thread with the last word
+    wpre[nw] = total;
+    tstart[tile + 1] = total;
+    tinfo[0] = tile + 1;
+    tinfo[1] = 0;
+    tinfo[2] = 0;
+    *n_touched = (unsigned)total;
+  }
+}
+
+// Blocks [0, B): a sample's entries -- place in the tile, and where the runs of the tiles start (a tile without
+// entries has an empty run).  The blocks after them write the list of touched rows.
+__global__ void __launch_bounds__(TI_THREADS)
+k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const int* tinfo, int nw, int step, int B, int bstride,
+             const int* act_cnt, const int32_t* act_ids, int act_stride, const int32_t* label_ptr, const int32_t* labels,
+             int max_labels, uint16_t* act_loc, int* seg, int* trows, int* tlab) {
+  const int tid = threadIdx.x;
+  griddep_launch_dependents();
+  griddep_wait();
+  if ((int)blockIdx.x >= B) {
+    const int nb = (int)gridDim.x - B;
+    for (int w = ((int)blockIdx.x - B) * TI_THREADS + tid; w < nw; w += nb * TI_THREADS) {
+      uint32_t bits = __ldcg(touch + w);
+      int at = __ldcg(wpre + w);
+      while (bits) {
+        trows[at++] = (w << 5) + __ffs(bits) - 1;
+        bits &= bits - 1;
+      }
+    }
+    return;
+  }
+  const int s = blockIdx.x;
+  const int na = __ldcg(act_cnt + s), nt = __ldcg(tinfo);
+  const int32_t* ids = act_ids + (size_t)s * act_stride;
+  uint16_t* loc = act_loc + (size_t)s * act_stride;
+  if (na == 0) {
+    for (int t = tid; t <= nt; t += TI_THREADS) seg[(size_t)t * bstride + s] = 0;
+    return;
+  }
+  constexpr int U = 4;                       // entries per thread and round: their chains of loads run side by side
+  const unsigned magic = tile_magic(step);
+  for (int a0 = 0; a0 < na; a0 += U * TI_THREADS) {
+    int j[U], pre[U], prev[U], ts[U];
+    uint32_t bits[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int a = a0 + u * TI_THREADS + tid;
+      j[u] = a < na ? __ldcg(ids + a) : 0;
+      prev[u] = a < na && a > 0 && (tid & 31) == 0 ? __ldcg(ids + a - 1) : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      pre[u] = __ldcg(wpre + (j[u] >> 5));
+      bits[u] = __ldcg(touch + (j[u] >> 5));
+      if (prev[u] >= 0) prev[u] = __ldcg(wpre + (prev[u] >> 5));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      bits[u] = (uint32_t)__popc(bits[u] & ((1u << (j[u] & 31)) - 1u));      // touched rows of the word before this one
+      ts[u] = __ldcg(tstart + tile_of(pre[u], magic, step));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int a = a0 + u * TI_THREADS + tid;
+      const int t = tile_of(pre[u], magic, step);
+      const int up = __shfl_up_sync(TFULL, t, 1);
+      const int before = (tid & 31) == 0 ? (prev[u] >= 0 ? tile_of(prev[u], magic, step) : -1) : up;
+      if (a >= na) continue;
+      loc[a] = (uint16_t)(pre[u] + (int)bits[u] - ts[u]);
+      for (int q = before + 1; q <= t; ++q) seg[(size_t)q * bstride + s] = a;
+      if (a == na - 1)
+        for (int q = t + 1; q <= nt; ++q) seg[(size_t)q * bstride + s] = na;
+    }
+  }
+  // the labels' places in the active set (a repeated label counts once)
+  const int lbeg = label_ptr[s], nlab = label_ptr[s + 1] - lbeg;
+  for (int i = TI_THREADS - 1 - tid; i < nlab; i += TI_THREADS) {
+    const int y = labels[lbeg + i];
+    bool first = true;
+    for (int q = 0; q < i; ++q) first = first && labels[lbeg + q] != y;
+    int lo = 0, hi = na;
+    while (lo < hi) { const int mid = (lo + hi) >> 1; if (__ldcg(ids + mid) < y) lo = mid + 1; else hi = mid; }
+    tlab[(size_t)s * max_labels + i] = first ? lo : -1;
+  }
+}
+
+struct TileParams {
+  const float* W2;
+  const RowHdr* hdr2;
+  const float* h;
+  const int *trows, *tstart, *seg;
+  int* tinfo;            // number of tiles; whether a tile's rows did not come in time
+  const uint16_t* act_loc;
+  float *act_z, *part;
+  DevState* st;
+  int B, H, act_stride, bstride, chunks, gs;      // gs: samples of a group
+};
+
+__device__ __forceinline__ uint32_t t_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void t_bulk(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(t_smem(dst)), "l"(src), "r"(bytes), "r"(t_smem(bar)) : "memory");
+}
+__device__ __forceinline__ bool t_wait(uint64_t* bar, uint32_t parity) {      // bounded
+  for (int it = 0; it < (1 << 22); ++it) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(t_smem(bar)), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// Grid (row chunks, groups of samples).  Dynamic shared memory: the tile's rows, each followed by the head of its
+// record (count, bias, bias moments), then the barrier.
+// A lane holds the 16-byte pieces lane, lane + 32, ... of a row.  Four rows at a time: their dot products with the
+// sample's activations are reduced together (six shuffles leave row i's sum in the lanes 8 i .. 8 i + 7).
+template <int NCH>
+__global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams p) {
+  constexpr bool KEEP = NCH <= 2;            // rows of up to 1 KB stay in registers between the two uses; longer ones are read again
+  extern __shared__ __align__(128) unsigned char t_sm[];
+  __shared__ __align__(8) uint64_t bar;
+  float* tile = reinterpret_cast<float*>(t_sm);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int H = p.H, H4 = H >> 2, ld = H + 4;
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(t_smem(&bar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  // the pieces of a row this lane reads; past the row's end a piece that exists (its activations are zero)
+  int off[NCH];
+#pragma unroll
+  for (int u = 0; u < NCH; ++u) off[u] = 4 * min(lane + 32 * u, H4 - 1);
+  griddep_launch_dependents();
+  griddep_wait();
+  const int nt = __ldcg(p.tinfo);
+  const int q0 = (int)blockIdx.y * p.gs, q1 = min(p.B, q0 + p.gs);
+  uint32_t phase = 0u;
+  for (int t = blockIdx.x; t < nt; t += p.chunks) {
+    const int r0 = __ldcg(p.tstart + t), nr = __ldcg(p.tstart + t + 1) - r0;
+    __syncthreads();                           // readers of the tile before are done
+    if (tid == 0)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(t_smem(&bar)), "r"((uint32_t)nr * ((uint32_t)H * 4u + 16u)) : "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    for (int r = tid; r < nr; r += TF_THREADS) {
+      const int j = __ldcg(p.trows + r0 + r);
+      t_bulk(tile + (size_t)r * ld, p.W2 + (size_t)j * H, (uint32_t)H * 4u, &bar);
+      t_bulk(tile + (size_t)r * ld + H, p.hdr2 + j, 16u, &bar);
+    }
+    const bool ok = t_wait(&bar, phase);
+    phase ^= 1u;
+    if (__syncthreads_or(ok ? 0 : 1)) {        // the rows did not come: one more bounded wait for the copies in flight, then out
+      t_wait(&bar, phase ^ 1u);
+      if (tid == 0) { p.tinfo[1] = 1; atomicCAS(&p.st->status, 0, (int)DSLIDE_ERR_TIMEOUT); }
+      return;
+    }
+    const bool fresh = t == (int)blockIdx.x;   // the chunk's first tile: nothing to carry on from
+    // a warp's samples: q0 + warp, + TF_WARPS, ...; lane i holds the run of the i-th of 32 of them
+    for (int sb = q0 + warp; sb < q1; sb += 32 * TF_WARPS) {
+      const int ms = sb + lane * TF_WARPS;
+      int ra = 0, rn = 0;
+      if (ms < q1) {
+        ra = __ldcg(p.seg + (size_t)t * p.bstride + ms);
+        rn = __ldcg(p.seg + (size_t)(t + 1) * p.bstride + ms) - ra;
+      }
+      unsigned todo = __ballot_sync(TFULL, ms < q1 && (rn > 0 || fresh));
+      while (todo) {
+        const int i = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int s = sb + i * TF_WARPS;
+        const int a0 = __shfl_sync(TFULL, ra, i), n = __shfl_sync(TFULL, rn, i);
+        float* part = p.part + ((size_t)blockIdx.x * p.B + s) * ld;
+        if (n == 0) {
+          if (lane == 0) { part[H] = -INFINITY; part[H + 1] = 0.f; }
+          continue;
+        }
+        const uint16_t* locp = p.act_loc + (size_t)s * p.act_stride + a0;
+        float* zp = p.act_z + (size_t)s * p.act_stride + a0;
+        int loc = lane < n ? (int)__ldcg(locp + lane) : 0;
+        ulonglong2 hx[NCH], S[NCH];              // pairs of floats: two multiply-adds per instruction
+        float M = -INFINITY, E = 0.f;            // E: this lane's rows only, until the end of the run
+#pragma unroll
+        for (int u = 0; u < NCH; ++u) {
+          const int c = lane + 32 * u;
+          hx[u] = c < H4 ? __ldg(reinterpret_cast<const ulonglong2*>(p.h + (size_t)s * H) + c) : make_ulonglong2(0ull, 0ull);
+          S[u] = make_ulonglong2(0ull, 0ull);
+        }
+        float E0 = 0.f;
+        if (!fresh) {
+          const float2 me = *reinterpret_cast<const float2*>(part + H);
+          ulonglong2 sv[NCH];
+#pragma unroll
+          for (int u = 0; u < NCH; ++u) {
+            const int c = lane + 32 * u;
+            sv[u] = c < H4 ? reinterpret_cast<const ulonglong2*>(part)[c] : make_ulonglong2(0ull, 0ull);
+          }
+          if (me.y > 0.f || me.y != me.y) {       // something was summed before
+            M = me.x;
+            E0 = me.y;
+#pragma unroll
+            for (int u = 0; u < NCH; ++u) S[u] = sv[u];
+          }
+        }
+        for (int c0 = 0; c0 < n; c0 += 32) {
+          if (c0 > 0) loc = c0 + lane < n ? (int)__ldcg(locp + c0 + lane) : 0;
+          const int m = min(32, n - c0);
+          {
+            const int first = __shfl_sync(TFULL, loc, 0);
+            if (lane >= m) loc = first;
+          }
+          for (int k = 0; k < m; k += 4) {
+            const float* rp[4];
+            ulonglong2 x[4][KEEP ? NCH : 1];
+            float d[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              rp[r] = tile + __shfl_sync(TFULL, loc, k + r) * ld;      // past the run: a row of the run, with weight zero below
+              unsigned long long d0 = 0ull, d1 = 0ull;
+#pragma unroll
+              for (int u = 0; u < NCH; ++u) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(rp[r] + off[u]);
+                if (KEEP) x[r][KEEP ? u : 0] = v;
+                fma2(d0, v.x, hx[u].x);
+                fma2(d1, v.y, hx[u].y);
+              }
+              d[r] = (lo2(d0) + hi2(d0)) + (lo2(d1) + hi2(d1));
+            }
+            const bool hi = (lane & 16) != 0, od = (lane & 8) != 0;
+            const float u0 = (hi ? d[2] : d[0]) + __shfl_xor_sync(TFULL, hi ? d[0] : d[2], 16);
+            const float u1 = (hi ? d[3] : d[1]) + __shfl_xor_sync(TFULL, hi ? d[1] : d[3], 16);
+            float y = (od ? u1 : u0) + __shfl_xor_sync(TFULL, od ? u0 : u1, 8);
+            y += __shfl_xor_sync(TFULL, y, 4);
+            y += __shfl_xor_sync(TFULL, y, 2);
+            y += __shfl_xor_sync(TFULL, y, 1);
+            const float* mr = hi ? (od ? rp[3] : rp[2]) : (od ? rp[1] : rp[0]);      // this lane's row of the four
+            float z = mr[H + 1] + y;                                 // the bias came with the row
+            const int mine = k + (lane >> 3);
+            if (mine >= m) z = -INFINITY;
+            else if ((lane & 7) == 0) zp[c0 + mine] = z;
+            if (__any_sync(TFULL, z > M)) {
+              float zm = fmaxf(z, __shfl_xor_sync(TFULL, z, 8));
+              zm = fmaxf(fmaxf(zm, __shfl_xor_sync(TFULL, zm, 16)), M);
+              const float scale = expf(M - zm);
+              const unsigned long long sc = pair2(scale, scale);
+              M = zm;
+              E *= scale;
+              E0 *= scale;
+#pragma unroll
+              for (int u = 0; u < NCH; ++u) {
+                asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(S[u].x) : "l"(sc));
+                asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(S[u].y) : "l"(sc));
+              }
+            }
+            const float e = mine < m ? expf(z - M) : 0.f;
+            E += e;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              const float g = __shfl_sync(TFULL, e, 8 * r);
+              const unsigned long long gg = pair2(g, g);
+#pragma unroll
+              for (int u = 0; u < NCH; ++u) {
+                const ulonglong2 v = KEEP ? x[r][KEEP ? u : 0] : *reinterpret_cast<const ulonglong2*>(rp[r] + off[u]);
+                fma2(S[u].x, gg, v.x);
+                fma2(S[u].y, gg, v.y);
+              }
+            }
+          }
+        }
+        E += __shfl_xor_sync(TFULL, E, 8);       // the four groups of lanes hold different rows
+        E += __shfl_xor_sync(TFULL, E, 16);
+#pragma unroll
+        for (int u = 0; u < NCH; ++u) {
+          const int c = lane + 32 * u;
+          if (c < H4) reinterpret_cast<ulonglong2*>(part)[c] = S[u];
+        }
+        if (lane == 0) *reinterpret_cast<float2*>(part + H) = make_float2(M, E0 + E);
+      }
+    }
+  }
+}
+
+// One block per sample: softmax, loss and errors over the active set, and the error at the hidden layer,
+// dh = [h > 0] (S / E - T / |Y|) / B with T the sum of the label rows.  Also clears the bitmap for the next step.
+struct CombineParams {
+  const float *W2, *h, *part, *act_z;
+  const int32_t *label_ptr, *act_ids;
+  const int *act_cnt, *tinfo, *tlab;
+  float *act_p, *act_g, *dh, *loss;
+  uint32_t* touch;
+  int B, H, act_stride, chunks, nw, max_labels;
+};
+
+__global__ void __launch_bounds__(TC3_THREADS) k_tile_combine(const CombineParams p) {
+  extern __shared__ __align__(16) unsigned char tc3_sm[];      // [chunks] factors, [parts][H] partial sums, [max_labels] places of the labels
+  __shared__ float sh_M, sh_E;
+  __shared__ int sh_ny;
+  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int H = p.H, ld = H + 4;
+  const int parts = H >= TC3_THREADS ? 1 : TC3_THREADS / H;    // threads that share a hidden unit's sum over the chunks
+  float* fac = reinterpret_cast<float*>(tc3_sm);
+  float* ps = fac + ((p.chunks + 3) & ~3);
+  int* lab = reinterpret_cast<int*>(ps + parts * H);
+  griddep_launch_dependents();
+  griddep_wait();
+  {
+    const int per = (p.nw + p.B - 1) / p.B;
+    for (int w = s * per + tid; w < min(p.nw, (s + 1) * per); w += TC3_THREADS) p.touch[w] = 0u;
+  }
+  const int na = p.act_cnt[s];
+  if (na == 0) return;                         // skipped sample: loss, h and dh are zero already
+  const int np = min(p.chunks, __ldcg(p.tinfo));
+  const int nlab = p.label_ptr[s + 1] - p.label_ptr[s];
+  if (warp == 0) {
+    // maximum and sum over the chunks (lane i takes the chunks i, i + 32, ...; then the lanes, in a fixed order)
+    float M = -INFINITY;
+    for (int b = lane; b < np; b += 32) M = fmaxf(M, __ldcg(p.part + ((size_t)b * p.B + s) * ld + H));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(TFULL, M, d));
+    float E = 0.f;
+    for (int b = lane; b < np; b += 32) {
+      const float2 me = __ldcg(reinterpret_cast<const float2*>(p.part + ((size_t)b * p.B + s) * ld + H));
+      const float f = me.y == 0.f ? 0.f : expf(me.x - M);
+      fac[b] = f;
+      E += me.y * f;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) E += __shfl_xor_sync(TFULL, E, d);
+    if (lane == 0) { sh_M = M; sh_E = E; }
+  } else if (warp == 1) {
+    int ny = 0;
+    for (int i = lane; i < nlab; i += 32) {
+      const int at = __ldcg(p.tlab + (size_t)s * p.max_labels + i);
+      lab[i] = at;
+      ny += at >= 0 ? 1 : 0;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) ny += __shfl_xor_sync(TFULL, ny, d);
+    if (lane == 0) sh_ny = ny;
+  }
+  const int32_t* ids = p.act_ids + (size_t)s * p.act_stride;
+  const float* z = p.act_z + (size_t)s * p.act_stride;
+  float* g = p.act_g + (size_t)s * p.act_stride;
+  float* pr = p.act_p + (size_t)s * p.act_stride;
+  __syncthreads();
+  if (__ldcg(p.tinfo + 1) != 0) {              // rows missing: the step's samples are given up, every coefficient zero
+    if (tid == 0) p.loss[s] = 0.f;
+    for (int a = tid; a < na; a += TC3_THREADS) { pr[a] = 0.f; g[a] = 0.f; }
+    for (int k = tid; k < H; k += TC3_THREADS) p.dh[(size_t)s * H + k] = 0.f;
+    return;
+  }
+  const float M = sh_M, E = sh_E, fB = (float)p.B;
+  const int ny = sh_ny;
+  if (tid == TC3_THREADS - 1) {
+    float sum = 0.f;
+    const float logE = logf(E);
+    for (int i = 0; i < nlab; ++i)
+      if (lab[i] >= 0) sum += z[lab[i]] - M - logE;
+    p.loss[s] = ny > 0 ? -sum / (float)ny : 0.f;
+  }
+  constexpr int U = 4;
+  for (int a0 = tid; a0 < na; a0 += U * TC3_THREADS) {
+    float zv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) zv[u] = a0 + u * TC3_THREADS < na ? __ldcg(z + a0 + u * TC3_THREADS) : 0.f;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int a = a0 + u * TC3_THREADS;
+      if (a < na) {
+        const float pa = expf(zv[u] - M) / E;
+        pr[a] = pa;
+        g[a] = pa / fB;
+      }
+    }
+  }
+  // sums over the chunks: `parts` threads per hidden unit, each a contiguous share of the chunks, added in order below
+  for (int e = tid; e < parts * H; e += TC3_THREADS) {
+    const int part = e / H, k = e - part * H;
+    const int per = (np + parts - 1) / parts;
+    const int b1 = min(np, (part + 1) * per);
+    float S = 0.f;
+#pragma unroll 8
+    for (int b = part * per; b < b1; ++b) {
+      const float f = fac[b];
+      const float v = f != 0.f ? __ldcg(p.part + ((size_t)b * p.B + s) * ld + k) : 0.f;
+      S = fmaf(f, v, S);
+    }
+    ps[e] = S;
+  }
+  __syncthreads();
+  for (int k = tid; k < H; k += TC3_THREADS) {
+    float S = 0.f, T = 0.f;
+    for (int q = 0; q < parts; ++q) S += ps[q * H + k];
+#pragma unroll 4
+    for (int i = 0; i < nlab; ++i)
+      if (lab[i] >= 0) T += __ldg(p.W2 + (size_t)__ldg(ids + lab[i]) * H + k);
+    const float v = (S / E - (ny > 0 ? T / (float)ny : 0.f)) / fB;
+    p.dh[(size_t)s * H + k] = p.h[(size_t)s * H + k] > 0.f ? v : 0.f;
+  }
+  for (int i = tid; i < nlab; i += TC3_THREADS)
+    if (lab[i] >= 0) g[lab[i]] = (pr[lab[i]] - 1.f / (float)ny) / fB;
+}
+
+// The touches of a tile's rows, row by row, in ascending sample order.  Per chunk of TL_CHUNK samples a bit per (row,
+// sample) is set in shared memory; a row's words are then counted up, so that the place of an entry is known from the
+// bits before its own whatever the order the entries are met in.  The tile's share of the list comes from a counter
+// (where a tile's entries lie does not matter).
+struct ListParams {
+  const int *tstart, *seg;
+  int* tinfo;
+  const uint16_t* act_loc;
+  const float* act_g;
+  int2 *rinfo, *list;
+  int B, act_stride, bstride, rows;      // rows: of a tile at most
+};
+
+__global__ void __launch_bounds__(TL_THREADS) k_tile_lists(const ListParams p) {
+  extern __shared__ __align__(16) unsigned char tl_sm[];
+  constexpr int NWD = TL_CHUNK / 32, LD = NWD + 1;
+  uint32_t* mask = reinterpret_cast<uint32_t*>(tl_sm);                             // [rows][LD]
+  int* start = reinterpret_cast<int*>(mask + (size_t)p.rows * LD);                 // [rows] where the row's next entries go
+  int* cnt = start + p.rows;                                                       // [rows]
+  uint16_t* pre = reinterpret_cast<uint16_t*>(cnt + p.rows);                       // [rows][LD]
+  __shared__ int wsum[TL_WARPS];
+  __shared__ int sh_base;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  griddep_launch_dependents();
+  griddep_wait();
+  const int nt = __ldcg(p.tinfo);
+  const int nchunks = (p.B + TL_CHUNK - 1) / TL_CHUNK;
+  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
+    const int r0 = __ldcg(p.tstart + t), nr = __ldcg(p.tstart + t + 1) - r0;
+    // every entry of the samples [s0, s0 + TL_CHUNK) by some thread: f(sample, place, index); four runs side by side
+    auto runs = [&](int s0, auto f) {
+      const int s1 = min(p.B, s0 + TL_CHUNK);
+      for (int sb = s0 + warp; sb < s1; sb += 32 * TL_WARPS) {
+        const int ms = sb + lane * TL_WARPS;
+        int ra = 0, rn = 0;
+        if (ms < s1) {
+          ra = __ldcg(p.seg + (size_t)t * p.bstride + ms);
+          rn = __ldcg(p.seg + (size_t)(t + 1) * p.bstride + ms) - ra;
+        }
+        const int most = min(32, (s1 - sb + TL_WARPS - 1) / TL_WARPS);
+        for (int i0 = 0; i0 < most; i0 += 4) {
+          int loc[4], n[4];
+          size_t at[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            n[u] = __shfl_sync(TFULL, rn, i0 + u);
+            at[u] = (size_t)(sb + (i0 + u) * TL_WARPS) * p.act_stride + __shfl_sync(TFULL, ra, i0 + u);
+            loc[u] = lane < n[u] ? (int)__ldg(p.act_loc + at[u] + lane) : -1;
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (loc[u] >= 0) f(sb + (i0 + u) * TL_WARPS, loc[u], at[u] + lane);
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            for (int c = 32 + lane; c < n[u]; c += 32) f(sb + (i0 + u) * TL_WARPS, (int)__ldg(p.act_loc + at[u] + c), at[u] + c);
+        }
+      }
+    };
+    __syncthreads();                           // readers of the tile before are done
+    for (int r = tid; r < nr; r += TL_THREADS) cnt[r] = 0;
+    __syncthreads();
+    if (nchunks > 1) {
+      for (int ch = 0; ch < nchunks; ++ch) runs(ch * TL_CHUNK, [&](int, int loc, size_t) { atomicAdd(&cnt[loc], 1); });
+      __syncthreads();
+    }
+    for (int ch = 0; ch < nchunks; ++ch) {
+      for (int e = tid; e < nr * LD; e += TL_THREADS) mask[e] = 0u;
+      __syncthreads();
+      runs(ch * TL_CHUNK, [&](int s, int loc, size_t) { const int b = s - ch * TL_CHUNK; atomicOr(&mask[loc * LD + (b >> 5)], 1u << (b & 31)); });
+      __syncthreads();
+      int here = 0;                            // the row's entries in this chunk
+      if (tid < nr) {
+#pragma unroll 8
+        for (int w = 0; w < NWD; ++w) {
+          pre[tid * LD + w] = (uint16_t)here;
+          here += __popc(mask[tid * LD + w]);
+        }
+      }
+      if (ch == 0) {
+        // the rows' places in the list: running sum of their counts from the tile's base
+        const int mine = tid < nr ? (nchunks > 1 ? cnt[tid] : here) : 0;
+        int incl = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int o = __shfl_up_sync(TFULL, incl, d);
+          if (lane >= d) incl += o;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        int before = 0, total = 0;
+        for (int w = 0; w < TL_WARPS; ++w) {
+          if (w < warp) before += wsum[w];
+          total += wsum[w];
+        }
+        if (tid == 0) sh_base = atomicAdd(p.tinfo + 2, total);
+        __syncthreads();
+        if (tid < nr) {
+          start[tid] = sh_base + before + incl - mine;
+          p.rinfo[r0 + tid] = make_int2(start[tid], mine);
+        }
+      }
+      __syncthreads();
+      runs(ch * TL_CHUNK, [&](int s, int loc, size_t at) {
+        const int b = s - ch * TL_CHUNK, w = b >> 5;
+        const int to = start[loc] + pre[loc * LD + w] + __popc(mask[loc * LD + w] & ((1u << (b & 31)) - 1u));
+        p.list[to] = make_int2(s, __float_as_int(__ldg(p.act_g + at)));
+      });
+      __syncthreads();
+      if (tid < nr) start[tid] += here;
+    }
+  }
+}
+
+cudaError_t launch_tiles_forward(Ctx* c, int batch, const int32_t* label_ptr, const int32_t* labels) {
+  const int nw = (c->N + 31) / 32;
+  int chunks, groups;
+  tile_grid(c, batch, &chunks, &groups);
+  c->launches += 5;          // with the kernel before them they make one entry of the profile
+  cudaError_t e = launch_dependent(k_tile_scan, dim3(1), dim3(TS_THREADS), 0, c->stream, (const uint32_t*)c->touch2, nw, c->tile_step,
+                                   c->wpre, c->tstart, c->tinfo, &c->dstate->n_own[c->t_host & 1][0]);
+  if (e != cudaSuccess) return e;
+  const int extra = (nw + 4 * TI_THREADS - 1) / (4 * TI_THREADS);
+  e = launch_dependent(k_tile_index, dim3(batch + extra), dim3(TI_THREADS), 0, c->stream, (const uint32_t*)c->touch2, (const int*)c->wpre,
+                       (const int*)c->tstart, (const int*)c->tinfo, nw, c->tile_step, batch, c->cfg.max_batch, (const int*)c->act_cnt,
+                       (const int32_t*)c->act_ids, c->act_stride, label_ptr, labels, c->cfg.max_labels, c->act_loc, c->seg, c->trows, c->tlab);
+  if (e != cudaSuccess) return e;
+  TileParams p;
+  p.W2 = c->W2; p.hdr2 = c->hdr2; p.h = c->h; p.trows = c->trows; p.tstart = c->tstart; p.tinfo = c->tinfo; p.seg = c->seg;
+  p.act_loc = c->act_loc; p.act_z = c->act_z; p.part = c->tpart; p.st = c->dstate;
+  p.B = batch; p.H = c->H; p.act_stride = c->act_stride; p.bstride = c->cfg.max_batch; p.chunks = chunks; p.gs = (batch + groups - 1) / groups;
+  const int smem = c->tile_rows * (c->H + 4) * 4;
+  const int nch = (c->H / 4 + 31) / 32;
+  auto k = nch <= 1 ? k_tile_forward<1> : nch <= 2 ? k_tile_forward<2> : nch <= 4 ? k_tile_forward<4> : k_tile_forward<8>;
+  if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+  if ((e = launch_dependent(k, dim3(chunks, groups), dim3(TF_THREADS), (size_t)smem, c->stream, p)) != cudaSuccess) return e;
+  CombineParams q;
+  q.W2 = c->W2; q.h = c->h; q.part = c->tpart; q.act_z = c->act_z; q.label_ptr = label_ptr; q.act_ids = c->act_ids;
+  q.act_cnt = c->act_cnt; q.tinfo = c->tinfo; q.tlab = c->tlab; q.act_p = c->act_p; q.act_g = c->act_g; q.dh = c->dh; q.loss = c->loss;
+  q.touch = c->touch2; q.B = batch; q.H = c->H; q.act_stride = c->act_stride; q.chunks = chunks; q.nw = nw; q.max_labels = c->cfg.max_labels;
+  const int parts = c->H >= TC3_THREADS ? 1 : TC3_THREADS / c->H;
+  const size_t csm = (size_t)(((chunks + 3) & ~3) + parts * c->H + c->cfg.max_labels) * 4;
+  if ((e = launch_dependent(k_tile_combine, dim3(batch), dim3(TC3_THREADS), csm, c->stream, q)) != cudaSuccess) return e;
+  ListParams l;
+  l.tstart = c->tstart; l.seg = c->seg; l.tinfo = c->tinfo; l.act_loc = c->act_loc; l.act_g = c->act_g; l.rinfo = c->rinfo; l.list = c->tlist;
+  l.B = batch; l.act_stride = c->act_stride; l.bstride = c->cfg.max_batch; l.rows = c->tile_rows;
+  const size_t lsm = (size_t)c->tile_rows * ((TL_CHUNK / 32 + 1) * 6 + 8);
+  if ((e = cudaFuncSetAttribute(k_tile_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm)) != cudaSuccess) return e;
+  return launch_dependent(k_tile_lists, dim3(2 * c->num_sms), dim3(TL_THREADS), lsm, c->stream, l);
+}
+
+}  // namespace dslide

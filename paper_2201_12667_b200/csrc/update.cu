@@ -58,6 +58,7 @@ struct UpdParams {
   HostResult* host_res;        // mapped host memory that receives {status, loss, sequence number}, or null
   unsigned int host_seq;
   int B, H, N, D, Wd, act_stride, dense, parity;
+  int w2_done;                 // the rows of W2 were updated by another kernel
   float lr, beta1, beta2, eps, rb1, rb2;
   // LSH-sampled hidden layer (L1 > 0): per row of W1 the hidden units some sample touches it for; per sample its active units
   uint32_t* cmask1;
@@ -532,7 +533,7 @@ __global__ void __launch_bounds__(UPD_THREADS, (NCH == 1 ? 2 : (NCH == 2 ? 2 : 1
   if ((int)blockIdx.x < naux) { aux_block(p, (int)blockIdx.x, sm_part, reinterpret_cast<unsigned*>(&scratch[0][0])); return; }
 
 
-  const int n2 = p.dense ? 0 : (int)p.st->n_own[p.parity][0];
+  const int n2 = p.w2_done ? 0 : (int)p.st->n_own[p.parity][0];
   const int n1 = (int)p.st->n_own[p.parity][1];
   const int nrows = n2 + n1;
   const int nwB = (B + 31) >> 5;
@@ -679,6 +680,146 @@ __global__ void __launch_bounds__(UPD_THREADS) k_adam_dense(const UpdParams p) {
   }
 }
 
+// Rows of W2 whose touches tiles.cu has listed row by row (sample, error; ascending samples).  A block holds a share of
+// the hidden units -- all that fits of [B][cw] activations -- in shared memory and its warps take rows: the list's
+// entries come 32 at a time, a row of activations is read by gl = cw / 4 lanes, so 32 / gl entries are added side by
+// side, each group of lanes to its own sum; the groups' sums are added in group order.  So a sum's order follows from
+// the list alone, nothing is searched for, and the activations (5 GB of reads per step at 1,024 samples x 6,100
+// neurons x 200 units) come from shared memory instead of L2.  The next row's list and the one after's place are asked
+// for while a row is added.
+struct RowsUpd {
+  const int* trows;
+  const int2 *rinfo, *list;    // per touched row (start, entries); the entries
+  int cw, shares;              // hidden units of a block, blocks side by side over the hidden units
+};
+constexpr int RU_THREADS = 1024;
+constexpr int RU_WARPS = RU_THREADS / 32;
+constexpr int RU_SMEM = 216 * 1024;
+
+__global__ void __launch_bounds__(RU_THREADS, 1) k_rows_update(const UpdParams p, const RowsUpd q) {
+  extern __shared__ __align__(16) unsigned char upd_smem[];
+  float* hs = reinterpret_cast<float*>(upd_smem);              // [B][cw]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int H = p.H, cw = q.cw, gl = cw >> 2, npar = 32 / gl;
+  const int k0 = (int)blockIdx.y * cw;                         // first hidden unit
+  const int grp = lane / gl, sub = lane - grp * gl;
+  const bool on = grp < npar && k0 + 4 * sub < H;
+  griddep_launch_dependents();
+  griddep_wait();
+  const int nrows = (int)p.st->n_own[p.parity][0];
+  for (int e = tid; e < p.B * gl; e += RU_THREADS) {
+    const int s = e / gl, c = e - s * gl;
+    const float4 v = k0 + 4 * c < H ? __ldg(reinterpret_cast<const float4*>(p.h + (size_t)s * H + k0) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    reinterpret_cast<float4*>(hs)[e] = v;
+  }
+  __syncthreads();
+  const int stride = (int)gridDim.x * RU_WARPS;
+  int u = (int)blockIdx.x * RU_WARPS + warp;
+  if (u >= nrows) return;
+  const int mysub = on ? sub : 0, mygrp = grp < npar ? grp : 0;
+  int2 info = __ldg(q.rinfo + u), info1 = u + stride < nrows ? __ldg(q.rinfo + u + stride) : make_int2(0, 0);
+  int row = __ldg(q.trows + u), row1 = u + stride < nrows ? __ldg(q.trows + u + stride) : 0;
+  int2 en = lane < info.y ? __ldg(q.list + info.x + lane) : make_int2(0, 0);
+  for (; u < nrows; u += stride) {
+    const size_t at = (size_t)row * H + k0 + 4 * sub;
+    float4 w, m, v;
+    const bool mine = on && grp == 0;
+    if (mine) {
+      w = *reinterpret_cast<const float4*>(p.W2 + at);
+      m = *reinterpret_cast<const float4*>(p.mW2 + at);
+      v = *reinterpret_cast<const float4*>(p.vW2 + at);
+    }
+    const bool bias = blockIdx.y == 0;
+    const int2 hv = bias ? load_hdr(p.hdr2 + row, lane) : make_int2(0, 0);
+    const int2 en1 = lane < info1.y ? __ldg(q.list + info1.x + lane) : make_int2(0, 0);
+    const int2 info2 = u + 2 * stride < nrows ? __ldg(q.rinfo + u + 2 * stride) : make_int2(0, 0);
+    const int row2 = u + 2 * stride < nrows ? __ldg(q.trows + u + 2 * stride) : 0;
+    unsigned long long a0 = 0ull, a1 = 0ull;      // this lane's four units, as pairs: two multiply-adds per instruction
+    float csum = 0.f;
+    auto add = [&](int s, float g) {
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(hs + (size_t)s * cw + 4 * mysub);
+      unsigned long long gg;
+      asm("mov.b64 %0, {%1, %1};" : "=l"(gg) : "f"(g));
+      asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a0) : "l"(gg), "l"(x.x));
+      asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a1) : "l"(gg), "l"(x.y));
+    };
+    for (int e0 = 0; e0 < info.y; e0 += 32) {
+      if (e0 > 0) en = e0 + lane < info.y ? __ldg(q.list + info.x + e0 + lane) : make_int2(0, 0);
+      csum += __int_as_float(en.y);
+      const int n = min(32, info.y - e0);
+      int e = mygrp;
+      for (; e - mygrp + 4 * npar <= n; e += 4 * npar) {        // four entries per group of lanes
+        int s[4];
+        float g[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          s[r] = __shfl_sync(FULL, en.x, e + r * npar);
+          g[r] = __int_as_float(__shfl_sync(FULL, en.y, e + r * npar));
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) add(s[r], g[r]);
+      }
+      for (; e - mygrp < n; e += npar) {
+        const int s = __shfl_sync(FULL, en.x, e);               // past the chunk: sample 0 with coefficient 0
+        const float g = __int_as_float(__shfl_sync(FULL, en.y, e));
+        if (e < n) add(s, g);
+      }
+    }
+    float4 acc = make_float4(__uint_as_float((unsigned)a0), __uint_as_float((unsigned)(a0 >> 32)), __uint_as_float((unsigned)a1),
+                             __uint_as_float((unsigned)(a1 >> 32)));
+    for (int o = 1; o < npar; ++o) {            // the other groups' sums, in group order
+      const int from = (sub + o * gl) & 31;
+      const float4 a = make_float4(__shfl_sync(FULL, acc.x, from), __shfl_sync(FULL, acc.y, from), __shfl_sync(FULL, acc.z, from),
+                                   __shfl_sync(FULL, acc.w, from));
+      if (grp == 0) { acc.x += a.x; acc.y += a.y; acc.z += a.z; acc.w += a.w; }
+    }
+    if (mine) {
+      adam1(w.x, m.x, v.x, acc.x, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+      adam1(w.y, m.y, v.y, acc.y, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+      adam1(w.z, m.z, v.z, acc.z, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+      adam1(w.w, m.w, v.w, acc.w, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+      *reinterpret_cast<float4*>(p.W2 + at) = w;
+      __stcs(reinterpret_cast<float4*>(p.mW2 + at), m);
+      __stcs(reinterpret_cast<float4*>(p.vW2 + at), v);
+    }
+    if (bias) {
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) csum += __shfl_xor_sync(FULL, csum, d);
+      finish_hdr(p, p.hdr2 + row, true, hv, csum, lane);
+    }
+    info = info1; info1 = info2; row = row1; row1 = row2; en = en1;
+  }
+}
+
+static cudaError_t launch_rows_update(Ctx* c, const UpdParams& p) {
+  RowsUpd q;
+  q.trows = c->trows; q.rinfo = c->rinfo; q.list = c->tlist;
+  // hidden units of a block: as many as fit for the whole batch, whole 32-byte sectors, at most 128 (a lane each four)
+  int cw = RU_SMEM / (4 * p.B);
+  cw = cw >= 128 ? 128 : cw & ~7;
+  if (cw < 8) cw = 8;
+  // fewer and wider shares, but with lanes to spare for another entry side by side: the least shares per entry in flight
+  int best = cw, hcap = (c->H + 3) & ~3;
+  double cost = 1e30;
+  for (int x = cw; x >= 8; x -= 4) {
+    const int wide = x < hcap ? x : hcap;
+    if (wide % 8 && wide != hcap) continue;
+    const double now = (double)((c->H + wide - 1) / wide) * (1.0 / (32 / (wide >> 2)) + 0.15);      // 0.15: the list is read again by every share
+    if (now < cost) { cost = now; best = wide; }
+  }
+  q.cw = best;
+  q.shares = (c->H + best - 1) / best;
+  const int smem = p.B * best * 4;
+  cudaError_t e = cudaFuncSetAttribute(k_rows_update, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_update, RU_THREADS, smem)) != cudaSuccess) return e;
+  int nb = c->num_sms * (per_sm > 0 ? per_sm : 1) / q.shares;
+  if (nb < 1) nb = 1;
+  LaunchScope ls(c, KID_ADAM);
+  return launch_dependent(k_rows_update, dim3(nb, q.shares), dim3(RU_THREADS), (size_t)smem, c->stream, p, q);
+}
+
 template <int NCH, int G, bool UMASK>
 static cudaError_t launch_k_update(Ctx* c, const UpdParams& p, int smem) {
   cudaError_t e = cudaSuccess;
@@ -723,6 +864,12 @@ cudaError_t launch_update(Ctx* c, int batch, const int32_t* row_ptr, const int32
   p.rb1 = (float)(1.0 / (1.0 - pow((double)c->cfg.beta1, t)));
   p.rb2 = (float)(1.0 / (1.0 - pow((double)c->cfg.beta2, t)));
 
+  p.w2_done = c->dense;
+  if (use_tiles(c, batch)) {
+    cudaError_t e = launch_rows_update(c, p);
+    if (e != cudaSuccess) return e;
+    p.w2_done = 1;
+  }
   if (c->dense) {
     LaunchScope ls(c, KID_ADAM_DENSE);
     k_adam_dense<<<c->num_sms * 4, UPD_THREADS, 0, c->stream>>>(p);

@@ -1,0 +1,55 @@
+"""Training steps whose active sets go by tiles of rows (thousands of neurons per sample that the batch shares): hidden
+widths around the register layouts, batches around a warp, a block of warps and a chunk of listed samples, odd
+vocabularies, options that change the sets."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2201_12667_b200 import binding as ds
+from paper_2201_12667_b200 import workloads
+from paper_2201_12667_b200.workloads import DWTA, SIMHASH
+from tests.gpu_harness import MOMENTS, WEIGHTS, Pair, to_dev
+from tests.test_gpu_shapes import one_and_two_steps
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [            # family, H, N, K, L, cap, batch, budget
+    (SIMHASH, 4, 2011, 2, 8, 256, 5, 0), (SIMHASH, 36, 5003, 3, 16, 256, 33, 0), (SIMHASH, 128, 5003, 3, 16, 256, 1, 0),
+    (SIMHASH, 128, 5003, 3, 16, 200, 130, 0), (SIMHASH, 200, 9001, 4, 20, 128, 47, 0), (DWTA, 264, 4001, 1, 16, 128, 20, 0),
+    (SIMHASH, 516, 3001, 2, 10, 256, 17, 0), (DWTA, 1024, 2500, 1, 12, 128, 19, 0), (SIMHASH, 32, 1500, 1, 6, 300, 1100, 0),
+    (SIMHASH, 64, 5003, 3, 16, 200, 40, 700),
+]
+
+
+@pytest.mark.parametrize("family,H,N,K,L,cap,B,budget", SHAPES)
+def test_steps_by_tiles(family, H, N, K, L, cap, B, budget):
+    pr = Pair(D=3001, H=H, N=N, family=family, K=K, L=L, bucket_cap=cap, max_batch=B, max_labels=16, lr=1e-3, seed=H + B, budget=budget)
+    try:
+        wl = workloads.Workload(workloads.config("mid", D=3001, N=N), seed=12)
+        launches = ds.dslide_kernel_launches(pr.ctx)
+        one_and_two_steps(pr, [wl.batch(i, batch_size=B) for i in range(2)])
+        assert ds.dslide_kernel_launches(pr.ctx) - launches == 2 * 8          # the route by tiles was taken
+    finally:
+        pr.close()
+
+
+def test_two_runs_by_tiles_are_bit_identical_and_skipped_samples_touch_nothing():
+    cfg = dict(D=3001, H=128, N=5003, family=SIMHASH, K=3, L=16, bucket_cap=200, max_batch=64, max_labels=16, lr=1e-3, seed=5)
+    wl = workloads.Workload(workloads.config("mid", D=3001, N=5003), seed=4)
+    batches = [[a.copy() for a in wl.batch(i, batch_size=64)] for i in range(3)]
+    batches[1][4][batches[1][3][7]] = -1                                      # sample 7 of the second batch has a bad label
+    got = []
+    for _ in range(2):
+        pr = Pair(**cfg)
+        try:
+            for i, b in enumerate(batches):
+                ds.dslide_train_step(pr.ctx, 64, *to_dev(b), torch.zeros(1, device="cuda"))
+                assert ds.dslide_sync(pr.ctx, check=False) == (ds.ERR_BAD_INDEX if i == 1 else ds.OK)
+                if i == 1:
+                    assert ds.dslide_get_last(pr.ctx, "act_count", 64)[7] == 0 and ds.dslide_get_last(pr.ctx, "loss", 64)[7] == 0
+                    assert not ds.dslide_get_last(pr.ctx, "dhidden", 64)[7].any()
+            got.append([ds.dslide_get_tensor(pr.ctx, n) for n in WEIGHTS + MOMENTS])
+        finally:
+            pr.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
