@@ -26,6 +26,7 @@ constexpr int ACT_SM = 1024;      // active ids and logits are mirrored in share
 constexpr int HID_MIN_BYTES = 64 * 1024;   // staging space for the hidden layer's rows of W1
 constexpr int RANK_MAX = 1024;    // candidate sets up to this size are put in order by counting, larger ones by a bitonic sort
 constexpr int SORT_SMALL = 1024;  // candidate sets up to this size are sorted rather than run through the bitmap
+constexpr int SORT_FEW = 160, BITMAP_CHEAP = 32768;      // ... and up to this size when all neurons are few
 constexpr unsigned FULLM = 0xffffffffu;
 
 struct FwdParams {
@@ -1444,6 +1445,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
 static int align16(int x) { return (x + 15) & ~15; }
 static int align128(int x) { return (x + 127) & ~127; }
 
+constexpr int TWO_PER_SM = (227 * 1024) / 2 - 1024;      // shared memory of a block of which two are resident
+
 struct FwdLayout {
   int off_dh, off_code, off_part, off_misc, off_lab, off_tbase, off_tbeg, off_topk, off_ids, off_z, off_col, off_val,
       off_h1, off_dedup, fixed_bytes, hid_rows;
@@ -1455,6 +1458,9 @@ static FwdLayout fwd_layout(const Ctx* c) {
   int hid_rows = HID_MIN_BYTES / (c->H * 4);
   if (hid_rows > 128) hid_rows = 128;
   if (hid_rows < 8) hid_rows = 8;
+  // wide hidden layers: two rows less rather than one block per multiprocessor less
+  const int around = align16(c->H * 4) * (1 + FWD_WARPS) + c->L * 12 + 2 * c->KL + c->cfg.max_labels * 4 + FWD_WARPS * 64 * 8 + 2 * ACT_SM * 4 + 2048;
+  while (hid_rows > 8 && around + hid_rows * (c->H * 4 + 8) > TWO_PER_SM) --hid_rows;
   l.hid_rows = hid_rows;
   int o = align16(c->H * 4);
   l.off_dh = o;      o = align16(o + FWD_WARPS * c->H * 4);
@@ -1499,7 +1505,7 @@ cudaError_t setup_forward(Ctx* c) {
   c->dedup_mode = mode;
   int stage = dd_bytes > stage_min ? dd_bytes : stage_min;
   // when the dedup work space leaves room for two blocks per multiprocessor, staging gets the rest of a half
-  const int two_per_sm = (227 * 1024) / 2 - 1024 - l.fixed_bytes;
+  const int two_per_sm = TWO_PER_SM - l.fixed_bytes;
   if (stage < two_per_sm) stage = two_per_sm;
   if (stage > budget) stage = budget;
   if (stage < stage_min || stage < c->H * 4) return cudaErrorInvalidValue;
@@ -1508,7 +1514,9 @@ cudaError_t setup_forward(Ctx* c) {
   c->fwd_sort_small = 0;
   if (mode == 1 && c->cfg.dedup_mode == 0 && !c->dense) {
     int cap_small = c->fwd_stage_bytes / 8;      // the sort pads to a power of two
-    c->fwd_sort_small = cap_small < SORT_SMALL ? cap_small : SORT_SMALL;
+    // a bitmap of a few words per thread is cleared and read out faster than more than a few hundred pairs are ranked
+    const int most = c->N <= BITMAP_CHEAP ? SORT_FEW : SORT_SMALL;
+    c->fwd_sort_small = cap_small < most ? cap_small : most;
   }
   // the hash functions' tables are mirrored above the hidden layer's chunk when they fit there
   {
