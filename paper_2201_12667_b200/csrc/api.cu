@@ -17,6 +17,7 @@ int sort_max_width();
 int bucket_scan_chunk();
 int order_small_max();
 int order_block_max();
+size_t part_ints(int L);
 }
 
 using namespace dslide;
@@ -64,7 +65,7 @@ void free_all(Ctx* c) {
                   c->hash_idx, c->hash_sign, c->bucket_off, c->bucket_ids, c->h, c->dh, c->loss, c->codes,
                   c->act_cnt, c->act_ids, c->act_z, c->act_p, c->act_g, c->mask1, c->ovf1, c->ovf2, c->hotmap1, c->hotcoef1,
                   c->mask2, c->proj1, c->bucket1_off, c->bucket1_ids, c->codes1n, c->codes1, c->hmask, c->cmask1, c->own1, c->own2, c->hot_rows, c->med_rows, c->hot_part, c->hot_done, c->dstate, c->keysA, c->keysB, c->valsA, c->valsB, c->tile_hist, c->bucket_part, c->ord_mid, c->ord_big, c->ord_cnt,
-                  c->st_dev[0], c->st_dev[1], c->st_dev[2], c->pd_part, c->touch2, c->wpre, c->trows, c->tstart, c->tinfo, c->act_loc, c->seg, c->tpart, c->rinfo, c->tlist, c->tlab, c->hash_pk};
+                  c->st_dev[0], c->st_dev[1], c->st_dev[2], c->pd_part, c->touch2, c->wpre, c->trows, c->tstart, c->tinfo, c->act_loc, c->seg, c->tpart, c->rinfo, c->tlist, c->tlab, c->hash_pk, c->part_work};
   for (void* p : ptrs) if (p) cudaFree(p);
   for (int b = 0; b < ST_SETS; ++b) {
     if (c->st_host[b]) cudaFreeHost(c->st_host[b]);
@@ -248,12 +249,12 @@ dslide_status dslide_init(const dslide_config* cfg, dslide_ctx** out) {
     A(ovf2, N * PAIR_T, false);
     A(own2, N, true);
     A(bucket_off, (size_t)c->L * (size_t)(c->nb + 1), true); A(bucket_ids, (size_t)c->L * N, true);
-    A(keysA, (size_t)c->L * N, false);
+    A(keysA, (size_t)c->L * N, false); A(part_work, part_ints(c->L), false);
     // codes wider than one radix digit: every id is placed at its bucket's start plus its rank of arrival there and the
     // large buckets are ordered afterwards, no radix passes
     c->place_path = c->bits > sort_max_width() ? 1 : 0;
     if (c->place_path) {
-      A(keysB, (size_t)c->L * N, false);      // here: the rank of every id inside its bucket
+      A(keysB, (size_t)c->L * N, false);      // here: words of the partition, or the rank of every id inside its bucket
       A(ord_mid, (size_t)c->L * (N / (order_small_max() + 1) + 1), false);
       A(ord_big, (size_t)c->L * (N / (order_block_max() + 1) + 1), false);
       A(ord_cnt, 2, true);

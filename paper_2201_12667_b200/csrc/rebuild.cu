@@ -268,19 +268,16 @@ constexpr int HN_ROWS = 32;
 constexpr int HN_THREADS = 256;
 constexpr int HN_WARPS = HN_THREADS / 32;
 constexpr int HN_FN_SMEM_MAX = 96 * 1024;    // hash-function tables larger than this stay in global memory
-constexpr size_t COUNT_SPLIT_BYTES = (size_t)64 << 20;   // bucket counters beyond this are counted table by table
 
 // A block stages HN_ROWS rows of W2 in shared memory (padded, so that 32 threads reading the same
 // column of 32 different rows hit 32 banks) and evaluates the L codes of each row: lane = row, the
 // warps share out the tables.  The hash functions sit in shared memory too, 16 bits per coordinate
 // (the top bit carries a negative SimHash sign), read as warp-wide broadcasts.
-// keys[t][j] = code of neuron j in table t; counts[t][code + 1] += 1; with `ranks`, ranks[t][j] = the count before
-// (the neuron's place inside its bucket, in order of arrival).
+// keys[t][j] = code of neuron j in table t.
 template <bool FN_SMEM>
 __global__ void __launch_bounds__(HN_THREADS)
 k_hash_neurons(const float* __restrict__ W2, const int32_t* __restrict__ hidx, const int32_t* __restrict__ hsign,
-               uint32_t* keys, uint32_t* ranks, int32_t* counts, int N, int H, int K, int L, int family, int lg_bin,
-               int fn_len, long long nb) {      // counts == nullptr: codes only (k_count_ranks counts afterwards)
+               uint32_t* keys, int N, int H, int K, int L, int family, int lg_bin, int fn_len) {
   extern __shared__ __align__(16) unsigned char hn_smem[];
   float* tile = reinterpret_cast<float*>(hn_smem);                    // [HN_ROWS][H + 1]
   const int ld = H + 1;
@@ -370,128 +367,147 @@ k_hash_neurons(const float* __restrict__ W2, const int32_t* __restrict__ hidx, c
           }
         }
         keys[(size_t)t * N + j0 + lane] = code;
-        if (counts) {
-          int32_t* cnt = counts + (size_t)t * (size_t)(nb + 1) + code + 1;
-          if (ranks) ranks[(size_t)t * N + j0 + lane] = (uint32_t)atomicAdd(cnt, 1);
-          else atomicAdd(cnt, 1);
-        }
       }
     }
   }
 }
 
-// DWTA with bins of eight, hash functions in shared memory: the same tiles, but two rows per lane.  A tile holds
-// 64 rows as 32 pairs (row r and row r + 32 interleaved per coordinate), so that one 8-byte load fetches a
-// coordinate of both rows and the index arithmetic is shared; the two rows' winners are found side by side.
-constexpr int HN2_ROWS = 64;
-
-__device__ __forceinline__ void wta_step(float x, int i, float& bv, int& best) {
-  if (x > bv) { bv = x; best = i; }          // strict: the lowest position wins ties
+// DWTA with bins of eight, hash functions in shared memory: 2 * RP rows per lane (rows lane, lane + 32, ... of a tile of
+// 64 * RP), interleaved per coordinate, so that one 8- or 16-byte load fetches a coordinate of all of them and the
+// address arithmetic is shared; the function table holds byte offsets.
+//
+// The winner of a bin is found without a chain of compare-and-select (three instructions per value on the half-rate
+// pipe, which bounded the kernel): m = the maximum of the eight (three-input maxima); d_i = (x_i - m) 2^40 by one
+// multiply-add, exactly zero where x_i equals m and at most -2^-109 elsewhere; t_i = d_i 2^120 - i, which is -i at the
+// winners and below -2^11 elsewhere; so the maximum of the t_i is minus the lowest winning position.  The multiply-adds
+// take two rows per instruction.  Weights that are not numbers, infinite or beyond 2^87 leave a maximum below -7 (or
+// none): such a row's table is done again by the chain.  Bound now by the loads from shared memory (a value is read
+// K L 8 / H times: 6.4 GB for 670,091 rows of 128 units and 300 functions).
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
 }
+__device__ __forceinline__ float max8_nan(float a, float b, float c, float d, float e, float f, float g, float h) {
+  float r = max3_nan(max3_nan(a, b, c), d, e);
+  r = max3_nan(r, f, g);
+  asm("max.NaN.f32 %0, %0, %1;" : "+f"(r) : "f"(h));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma_pair(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ unsigned long long pair_of(float lo, float hi) {
+  return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ float pair_lo(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float pair_hi(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
 
-template <bool COUNT>      // COUNT = false: codes only, the counting is a pass of its own
-__global__ void __launch_bounds__(HN_THREADS)
-k_hash_neurons_dwta8(const float* __restrict__ W2, const int32_t* __restrict__ hidx, uint32_t* keys, uint32_t* ranks,
-                     int32_t* counts, int N, int H, int K, int L, int lg_bin, long long nb) {
+constexpr int HN8_WARPS_MAX = 16;
+
+template <int RP>
+__global__ void __launch_bounds__(32 * HN8_WARPS_MAX)
+k_hash_neurons_dwta8(const float* __restrict__ W2, const int32_t* __restrict__ hidx, uint32_t* keys, int N, int H, int K, int L) {
+  constexpr int ROWS = 64 * RP, ES = 8 * RP;                          // rows of a tile, bytes of a coordinate of a lane's rows
   extern __shared__ __align__(16) unsigned char hn_smem[];
-  float2* tile = reinterpret_cast<float2*>(hn_smem);                  // [32 pairs][H + 1]
-  const int ld = H + 1;
-  unsigned short* fn = reinterpret_cast<unsigned short*>(hn_smem + (((size_t)32 * ld * 8 + 15) & ~(size_t)15));
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nfn = K * L * 8;
-  // Inside a tile coordinate k sits at place (k / 4) + (H / 4) * (k % 4): the four components of a 16-byte global
-  // load then go to four distant places and a warp's stores spread over the banks.  The function table holds places.
-  const int Hq = H >> 2;
-  for (int e = threadIdx.x; e < nfn; e += HN_THREADS) {
-    const int k = hidx[e];
-    fn[e] = (unsigned short)((k >> 2) + Hq * (k & 3));
-  }
-  const int ntiles = (N + HN2_ROWS - 1) / HN2_ROWS;
+  const int ld = H + 1;                                               // odd: a warp's loads of one coordinate spread over the banks
+  uint32_t* fn = reinterpret_cast<uint32_t*>(hn_smem + (((size_t)32 * ld * ES + 15) & ~(size_t)15));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  for (int e = threadIdx.x; e < K * L * 8; e += blockDim.x) fn[e] = (uint32_t)hidx[e] * ES;
+  const unsigned char* v = hn_smem + (size_t)lane * ld * ES;
+  const unsigned long long S = pair_of(0x1p40f, 0x1p40f), BIG = pair_of(0x1p120f, 0x1p120f);
+  const int ntiles = (N + ROWS - 1) / ROWS;
   for (int tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
-    const int j0 = tl * HN2_ROWS;
-    const int rows = min(HN2_ROWS, N - j0);
+    const int j0 = tl * ROWS;
+    const int rows = min(ROWS, N - j0);
     __syncthreads();
-    {
-      const int H4 = H >> 2, total4 = rows * H4;
-      const float4* src = reinterpret_cast<const float4*>(W2 + (size_t)j0 * H);
-      float* tile1 = reinterpret_cast<float*>(tile);
-      for (int e = threadIdx.x; e < total4; e += HN_THREADS) {
-        const float4 x = __ldg(src + e);
-        const int r = e / H4, c4 = e - r * H4;
-        float* d = tile1 + ((size_t)(r & 31) * ld + c4) * 2 + (r >> 5);
-        d[0] = x.x; d[2 * H4] = x.y; d[4 * H4] = x.z; d[6 * H4] = x.w;
+    // a thread takes one coordinate of one lane's rows: reads run along a row, one vector store places them
+    for (int g = warp; g < 32; g += nwarps)
+      for (int k = lane; k < H; k += 32) {
+        float x[2 * RP];
+#pragma unroll
+        for (int u = 0; u < 2 * RP; ++u) x[u] = g + 32 * u < rows ? __ldg(W2 + (size_t)(j0 + g + 32 * u) * H + k) : 0.f;
+        unsigned char* to = hn_smem + ((size_t)g * ld + k) * ES;
+        if (RP == 2) *reinterpret_cast<float4*>(to) = make_float4(x[0], x[1], x[2 * RP - 2], x[2 * RP - 1]);
+        else *reinterpret_cast<float2*>(to) = make_float2(x[0], x[1]);
       }
-    }
     __syncthreads();
-    const bool live0 = lane < rows, live1 = lane + 32 < rows;
-    if (live0) {
-      const float2* v = tile + (size_t)lane * ld;
-      uint32_t pr0 = 0, pr1 = 0;
-      size_t pidx = 0;
-      bool pend = false, pend1 = false;
-      for (int t = warp; t < L; t += HN_WARPS) {
-        uint32_t code0 = 0, code1 = 0;
-        for (int k = 0; k < K; ++k) {
-          const uint4 q = *reinterpret_cast<const uint4*>(fn + (size_t)(t * K + k) * 8);
-          const float2 x0 = v[q.x & 0xffffu], x1 = v[q.x >> 16], x2 = v[q.y & 0xffffu], x3 = v[q.y >> 16];
-          const float2 x4 = v[q.z & 0xffffu], x5 = v[q.z >> 16], x6 = v[q.w & 0xffffu], x7 = v[q.w >> 16];
-          float a = x0.x, b = x0.y;
-          int ia = 0, ib = 0;
-          wta_step(x1.x, 1, a, ia); wta_step(x1.y, 1, b, ib);
-          wta_step(x2.x, 2, a, ia); wta_step(x2.y, 2, b, ib);
-          wta_step(x3.x, 3, a, ia); wta_step(x3.y, 3, b, ib);
-          wta_step(x4.x, 4, a, ia); wta_step(x4.y, 4, b, ib);
-          wta_step(x5.x, 5, a, ia); wta_step(x5.y, 5, b, ib);
-          wta_step(x6.x, 6, a, ia); wta_step(x6.y, 6, b, ib);
-          wta_step(x7.x, 7, a, ia); wta_step(x7.y, 7, b, ib);
-          code0 |= (uint32_t)ia << (k * lg_bin);
-          code1 |= (uint32_t)ib << (k * lg_bin);
+    for (int t = warp; t < L; t += nwarps) {
+      unsigned long long code[RP];
+      float worst = 0.f;
+      float scale = -1.f;
+#pragma unroll
+      for (int r = 0; r < RP; ++r) code[r] = 0ull;
+      for (int k = 0; k < K; ++k) {
+        const uint4 qa = *reinterpret_cast<const uint4*>(fn + (size_t)(t * K + k) * 8);
+        const uint4 qb = *reinterpret_cast<const uint4*>(fn + (size_t)(t * K + k) * 8 + 4);
+        const uint32_t q[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+        unsigned long long x[8][RP];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (RP == 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(v + q[i]);
+            x[i][0] = w.x; x[i][RP - 1] = w.y;
+          } else {
+            x[i][0] = *reinterpret_cast<const unsigned long long*>(v + q[i]);
+          }
         }
-        // the ranks asked for in the previous round have arrived by now: they are stored a round late so that
-        // no warp waits on its atomics
-        if (pend) {
-          ranks[pidx] = pr0;
-          if (pend1) ranks[pidx + 32] = pr1;
+        const unsigned long long sc = pair_of(scale, scale);
+#pragma unroll
+        for (int r = 0; r < RP; ++r) {
+          const float ma = max8_nan(pair_lo(x[0][r]), pair_lo(x[1][r]), pair_lo(x[2][r]), pair_lo(x[3][r]), pair_lo(x[4][r]),
+                                    pair_lo(x[5][r]), pair_lo(x[6][r]), pair_lo(x[7][r]));
+          const float mb = max8_nan(pair_hi(x[0][r]), pair_hi(x[1][r]), pair_hi(x[2][r]), pair_hi(x[3][r]), pair_hi(x[4][r]),
+                                    pair_hi(x[5][r]), pair_hi(x[6][r]), pair_hi(x[7][r]));
+          const unsigned long long nm = pair_of((0.f - ma) * 0x1p40f, (0.f - mb) * 0x1p40f);      // 0 - m: a zero of either sign gives +0
+          unsigned long long d[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) d[i] = fma_pair(fma_pair(x[i][r], S, nm), BIG, pair_of(-(float)i, -(float)i));
+          const float ta = max8_nan(pair_lo(d[0]), pair_lo(d[1]), pair_lo(d[2]), pair_lo(d[3]), pair_lo(d[4]), pair_lo(d[5]), pair_lo(d[6]), pair_lo(d[7]));
+          const float tb = max8_nan(pair_hi(d[0]), pair_hi(d[1]), pair_hi(d[2]), pair_hi(d[3]), pair_hi(d[4]), pair_hi(d[5]), pair_hi(d[6]), pair_hi(d[7]));
+          asm("min.NaN.f32 %0, %0, %1, %2;" : "+f"(worst) : "f"(ta), "f"(tb));
+          code[r] = fma_pair(pair_of(ta, tb), sc, code[r]);          // minus position times minus 8^k: exact below 2^24
         }
-        keys[(size_t)t * N + j0 + lane] = code0;
-        if (!COUNT) {                        // codes only: k_count_ranks counts afterwards, table by table
-          if (live1) keys[(size_t)t * N + j0 + 32 + lane] = code1;
-          continue;
-        }
-        int32_t* cnt = counts + (size_t)t * (size_t)(nb + 1) + 1;
-        if (ranks) {
-          pr0 = (uint32_t)atomicAdd(cnt + code0, 1);
-          pidx = (size_t)t * N + j0 + lane;
-          pend = true;
-          pend1 = live1;
-        } else {
-          atomicAdd(cnt + code0, 1);
-        }
-        if (live1) {
-          keys[(size_t)t * N + j0 + 32 + lane] = code1;
-          if (ranks) pr1 = (uint32_t)atomicAdd(cnt + code1, 1);
-          else atomicAdd(cnt + code1, 1);
+        scale *= 8.f;
+      }
+      uint32_t c[2 * RP];
+#pragma unroll
+      for (int r = 0; r < RP; ++r) { c[2 * r] = __float2uint_rn(pair_lo(code[r])); c[2 * r + 1] = __float2uint_rn(pair_hi(code[r])); }
+      if (!(worst >= -7.f)) {                                          // rare: see above
+        for (int u = 0; u < 2 * RP; ++u) {
+          uint32_t cc = 0;
+          for (int k = 0; k < K; ++k) {
+            const uint32_t* q = fn + (size_t)(t * K + k) * 8;
+            int best = 0;
+            float bv = reinterpret_cast<const float*>(v + q[0])[u];
+            for (int i = 1; i < 8; ++i) {
+              const float y = reinterpret_cast<const float*>(v + q[i])[u];
+              if (y > bv) { bv = y; best = i; }
+            }
+            cc |= (uint32_t)best << (3 * k);
+          }
+          c[u] = cc;
         }
       }
-      if (pend) {
-        ranks[pidx] = pr0;
-        if (pend1) ranks[pidx + 32] = pr1;
-      }
+#pragma unroll
+      for (int u = 0; u < 2 * RP; ++u)
+        if (lane + 32 * u < rows) keys[(size_t)t * N + j0 + 32 * u + lane] = c[u];
     }
   }
 }
 
-// Counting as a pass of its own, for tables whose counters do not fit the L2 cache together (2^21 buckets x 64 tables
-// are half a gigabyte): the blocks walk table after table, so that the counters being incremented at any moment are
-// those of one or two tables and the atomics stay in L2.  ranks[t][j] = arrivals before j in its bucket.
+// Counting as a pass of its own (the counters of 2^21 buckets x 64 tables are half a gigabyte): the blocks walk table
+// after table, so that the counters being incremented at any moment are those of one or two tables and the atomics stay
+// in L2.  ranks[t][j] = arrivals before j in its bucket.
 __global__ void __launch_bounds__(256) k_count_ranks(const uint32_t* keys, uint32_t* ranks, int32_t* counts, int N, long long nb) {
   const int t = blockIdx.y;
   const uint32_t* k = keys + (size_t)t * N;
-  uint32_t* r = ranks ? ranks + (size_t)t * N : nullptr;
+  uint32_t* r = ranks + (size_t)t * N;
   int32_t* cnt = counts + (size_t)t * (size_t)(nb + 1) + 1;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-    const uint32_t v = (uint32_t)atomicAdd(cnt + k[j], 1);
-    if (r) r[j] = v;
+    r[j] = (uint32_t)atomicAdd(cnt + k[j], 1);
   }
 }
 
@@ -742,10 +758,213 @@ k_sort_scatter(const uint32_t* keys_in, const int32_t* vals_in, uint32_t* keys_o
   }
 }
 
+// ------------------------------------------------------------------ wide codes: partition, then place in shared memory
+// Codes wider than one radix digit: the ids of a table are first partitioned by the upper bits of their codes (about a
+// thousand ids per part; order inside a part does not matter), as words that hold the lower bits of the code and the
+// id.  A block then takes a part: counts its buckets, writes their offsets, places the ids in shared memory and writes
+// them out in one run.  So neither a counter nor an id goes to memory as a scattered 4-byte access (33.5 M of each at
+// 670,091 neurons x 50 tables were what the placement by rank of arrival cost), and the offsets come out with it.
+// Buckets larger than the cap are put in ascending order afterwards (k_order_*), as on the other path.
+constexpr int PT_THREADS = 512;
+constexpr int PT_TILE = 6144;
+constexpr int PT_PER = PT_TILE / PT_THREADS;
+constexpr int PT_HIST = 32768;                      // ids that a block counts
+constexpr int PT_MAX_UP = 10, PT_MAX_LOW = 11;      // upper and lower bits of a code at most
+constexpr int PP_THREADS = 256, PP_CAP = 4096;      // ids of a part that fit shared memory
+
+__global__ void __launch_bounds__(PT_THREADS) k_part_hist(const uint32_t* keys, int* total, int N, int low, int up) {
+  __shared__ int cnt[1 << PT_MAX_UP];
+  const int t = blockIdx.y, P = 1 << up;
+  for (int d = threadIdx.x; d < P; d += PT_THREADS) cnt[d] = 0;
+  __syncthreads();
+  const uint32_t* k = keys + (size_t)t * N;
+  const int beg = blockIdx.x * PT_HIST, end = min(N, beg + PT_HIST);
+  for (int i0 = beg + threadIdx.x; i0 < end; i0 += 8 * PT_THREADS) {
+    uint32_t c[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) c[u] = i0 + u * PT_THREADS < end ? k[i0 + u * PT_THREADS] : 0u;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i0 + u * PT_THREADS < end) atomicAdd(&cnt[c[u] >> low], 1);
+  }
+  __syncthreads();
+  for (int d = threadIdx.x; d < P; d += PT_THREADS)
+    if (cnt[d]) atomicAdd(&total[t * P + d], cnt[d]);
+}
+
+// One block per table: where the parts start (base[t][P + 1]) and the cursors that hand out their space.
+__global__ void __launch_bounds__(1 << PT_MAX_UP) k_part_scan(int* total, int* base, int up) {
+  __shared__ int sh[32];
+  const int P = 1 << up, t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int mine = tid < P ? total[t * P + tid] : 0;
+  int incl = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) sh[warp] = incl;
+  __syncthreads();
+  int before = 0;
+  for (int w = 0; w < warp; ++w) before += sh[w];
+  if (tid < P) {
+    base[t * (P + 1) + tid] = before + incl - mine;
+    total[t * P + tid] = before + incl - mine;
+    if (tid == P - 1) base[t * (P + 1) + P] = before + incl;
+  }
+}
+
+__global__ void __launch_bounds__(PT_THREADS, 4) k_part_scatter(const uint32_t* keys, int* cursor, uint32_t* out, int N, int low, int up, int id_bits) {
+  __shared__ int cnt[1 << PT_MAX_UP], at[1 << PT_MAX_UP];      // of a part: the tile's ids; where they go globally minus where they are in the tile
+  __shared__ uint32_t word[PT_TILE];
+  __shared__ uint16_t part[PT_TILE];
+  __shared__ int sh[PT_THREADS / 32];
+  const int t = blockIdx.y, P = 1 << up, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int d = tid; d < P; d += PT_THREADS) cnt[d] = 0;
+  __syncthreads();
+  const uint32_t* k = keys + (size_t)t * N;
+  const int beg = blockIdx.x * PT_TILE, n = min(PT_TILE, N - beg);
+  uint32_t key[PT_PER];
+#pragma unroll
+  for (int u = 0; u < PT_PER; ++u) {
+    const int i = u * PT_THREADS + tid;
+    key[u] = i < n ? k[beg + i] : 0u;
+  }
+#pragma unroll
+  for (int u = 0; u < PT_PER; ++u)
+    if (u * PT_THREADS + tid < n) atomicAdd(&cnt[key[u] >> low], 1);
+  __syncthreads();
+  // running sum over the parts (two per thread at most), and the tile's space in every part
+  int c0 = 2 * tid < P ? cnt[2 * tid] : 0, c1 = 2 * tid + 1 < P ? cnt[2 * tid + 1] : 0;
+  int incl = c0 + c1;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) sh[warp] = incl;
+  __syncthreads();
+  int run = incl - c0 - c1;
+  for (int w = 0; w < warp; ++w) run += sh[w];
+  if (2 * tid < P) {
+    cnt[2 * tid] = run;
+    at[2 * tid] = (c0 ? atomicAdd(&cursor[t * P + 2 * tid], c0) : 0) - run;
+  }
+  if (2 * tid + 1 < P) {
+    cnt[2 * tid + 1] = run + c0;
+    at[2 * tid + 1] = (c1 ? atomicAdd(&cursor[t * P + 2 * tid + 1], c1) : 0) - (run + c0);
+  }
+  __syncthreads();
+  const uint32_t lmask = (1u << low) - 1u;
+#pragma unroll
+  for (int u = 0; u < PT_PER; ++u) {
+    const int i = u * PT_THREADS + tid;
+    if (i < n) {
+      const int d = (int)(key[u] >> low), to = atomicAdd(&cnt[d], 1);
+      word[to] = ((key[u] & lmask) << id_bits) | (uint32_t)(beg + i);
+      part[to] = (uint16_t)d;
+    }
+  }
+  __syncthreads();
+  uint32_t* o = out + (size_t)t * N;
+#pragma unroll
+  for (int u = 0; u < PT_PER; ++u) {
+    const int i = u * PT_THREADS + tid;
+    if (i < n) o[at[part[i]] + i] = word[i];
+  }
+}
+
+// Grid (parts, tables).  Also enters the buckets of more than min_n ids in the lists of the ordering kernels.  The words
+// are read twice (the second time from the caches) and nothing of them is kept in registers, so that eight blocks are
+// resident: a block is a chain of short phases.
+__global__ void __launch_bounds__(PP_THREADS, 8)
+k_part_place(const uint32_t* __restrict__ words, const int* base, int32_t* off, int32_t* ids, int N, long long nb, int low, int up, int id_bits,
+             int min_n, int2* mid, int2* big, int* ord_cnt) {
+  __shared__ int cnt[1 << PT_MAX_LOW];
+  __shared__ int out[PP_CAP];
+  __shared__ int sh[PP_THREADS / 32];
+  const int t = blockIdx.y, d = blockIdx.x, P = 1 << up, R = 1 << low, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b0 = base[t * (P + 1) + d], n = base[t * (P + 1) + d + 1] - b0;
+  const uint32_t* w = words + (size_t)t * N + b0;
+  int32_t* to = ids + (size_t)t * N + b0;
+  const uint32_t imask = (1u << id_bits) - 1u;
+  for (int c = tid; c < R; c += PP_THREADS) cnt[c] = 0;
+  __syncthreads();
+  for (int i0 = tid; i0 < n; i0 += 4 * PP_THREADS) {
+    uint32_t e[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) e[u] = i0 + u * PP_THREADS < n ? __ldg(w + i0 + u * PP_THREADS) : 0u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * PP_THREADS < n) atomicAdd(&cnt[e[u] >> id_bits], 1);
+  }
+  __syncthreads();
+  // running sum over the part's buckets; a thread owns R / PP_THREADS consecutive ones (at least one)
+  const int per = (R + PP_THREADS - 1) / PP_THREADS;
+  const int c0 = min(R, tid * per), c1 = min(R, c0 + per);
+  int mine = 0;
+  for (int c = c0; c < c1; ++c) mine += cnt[c];
+  int incl = mine;
+#pragma unroll
+  for (int q = 1; q < 32; q <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, incl, q);
+    if (lane >= q) incl += o;
+  }
+  if (lane == 31) sh[warp] = incl;
+  __syncthreads();
+  int run = incl - mine;
+  for (int q = 0; q < warp; ++q) run += sh[q];
+  for (int c = c0; c < c1; ++c) {
+    const int m = cnt[c];
+    cnt[c] = run;
+    if (ord_cnt && m > min_n) {
+      const int2 tc = make_int2(t, (d << low) + c);
+      if (m <= ORD_BLOCK) mid[atomicAdd(ord_cnt, 1)] = tc;
+      else big[atomicAdd(ord_cnt + 1, 1)] = tc;
+    }
+    run += m;
+  }
+  __syncthreads();
+  int32_t* o = off + (size_t)t * (size_t)(nb + 1) + ((size_t)d << low);
+  for (int c = tid; c < R; c += PP_THREADS) o[c] = b0 + cnt[c];
+  if (d == P - 1 && tid == 0) o[R] = N;
+  __syncthreads();                      // the offsets have been read out of cnt
+  const bool fits = n <= PP_CAP;        // a crowded part (codes far from evenly spread) is placed straight in memory
+  for (int i0 = tid; i0 < n; i0 += 4 * PP_THREADS) {
+    uint32_t e[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) e[u] = i0 + u * PP_THREADS < n ? __ldg(w + i0 + u * PP_THREADS) : 0u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * PP_THREADS < n) {
+        const int at = atomicAdd(&cnt[e[u] >> id_bits], 1), id = (int)(e[u] & imask);
+        if (fits) out[at] = id;
+        else to[at] = id;
+      }
+  }
+  if (!fits) return;
+  __syncthreads();
+  for (int i = tid; i < n; i += PP_THREADS) to[i] = out[i];
+}
+
+// Upper and lower bits of the partition, or false when a word cannot hold the lower bits and an id.
+static bool part_shape(const Ctx* c, int* low, int* up, int* id_bits) {
+  int ib = 1;
+  while (((int64_t)1 << ib) < c->N) ++ib;
+  int u = 0;
+  while (u < PT_MAX_UP && (c->N >> u) > 1536) ++u;              // about a thousand ids per part
+  if (u > c->bits - 1) u = c->bits - 1;
+  if (c->bits - u > PT_MAX_LOW) u = c->bits - PT_MAX_LOW;
+  if (c->bits - u + ib > 32) u = c->bits + ib - 32;
+  if (u < 1) u = 1;
+  *up = u; *low = c->bits - u; *id_bits = ib;
+  return c->place_path && u <= PT_MAX_UP && u < c->bits;
+}
+size_t part_ints(int L) { return (size_t)L * (2 * (1 << PT_MAX_UP) + 1); }
+
 // ------------------------------------------------------------------ wide codes: place, then order inside buckets
-// With codes wider than one radix digit the buckets are small (a few ids on average), and sorting the whole table
-// twice is a detour.  Instead the hashing kernel's counting atomics hand every id its rank of arrival inside its
-// bucket, the id goes to the bucket's start plus that rank, and the ids of each bucket are then put in ascending
+// What is left when the lower bits and an id do not fit a word (2^21 buckets x 4 M neurons): a counting pass hands every
+// id its rank of arrival inside its bucket, the id goes to the bucket's start plus that rank, and the ids of each bucket are then put in ascending
 // order where they stand: in registers for
 // buckets of up to ORD_SMALL ids, by a block-wide sort in shared memory up to ORD_BLOCK, and for a larger bucket by
 // one ordered pass over the table's codes that writes the matching ids out again.
@@ -879,35 +1098,45 @@ static cudaError_t order_buckets(Ctx* c, int min_n, bool listed) {
 
 cudaError_t launch_order_buckets(Ctx* c, int min_n) { return order_buckets(c, min_n, false); }
 
+// Warps of a block of the bins-of-eight kernel: the tables go round the warps, so as many as leave the fewest idle.
+static int dwta8_warps(int L) {
+  int best = 8;
+  double eff = 0.0;
+  for (int w = 8; w <= HN8_WARPS_MAX; ++w) {
+    const double now = (double)L / (double)(w * ((L + w - 1) / w));
+    if (now > eff + 1e-9) { eff = now; best = w; }
+  }
+  return best;
+}
+
+template <int RP>
+static cudaError_t launch_dwta8(Ctx* c, int smem) {
+  cudaError_t e = cudaFuncSetAttribute(k_hash_neurons_dwta8<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int threads = 32 * dwta8_warps(c->L);
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hash_neurons_dwta8<RP>, threads, smem);
+  if (e != cudaSuccess) return e;
+  LaunchScope ls(c, KID_HASH_NEURONS);
+  k_hash_neurons_dwta8<RP><<<c->num_sms * (per_sm > 0 ? per_sm : 1), threads, smem, c->stream>>>(c->W2, c->hash_idx, c->keysA, c->N, c->H, c->K, c->L);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_build_tables(Ctx* c) {
   const size_t off_bytes = (size_t)c->L * (size_t)(c->nb + 1) * sizeof(int32_t);
-  cudaError_t e = cudaMemsetAsync(c->bucket_off, 0, off_bytes, c->stream);
-  if (e != cudaSuccess) return e;
-  // the counting atomics ride with the hashing while all the tables' counters fit the L2 cache together; beyond that
-  // every atomic would be a read-modify-write in DRAM, and the counting becomes a pass of its own, table by table
-  const bool split_count = off_bytes > COUNT_SPLIT_BYTES;
-  int32_t* hash_counts = split_count ? nullptr : c->bucket_off;
+  int low = 0, up = 0, id_bits = 0;
+  const bool parts = part_shape(c, &low, &up, &id_bits);
+  cudaError_t e = cudaSuccess;
+  if (c->place_path && !parts && (e = cudaMemsetAsync(c->bucket_off, 0, off_bytes, c->stream)) != cudaSuccess) return e;
   const int tile_bytes = (HN_ROWS * (c->H + 1) * (int)sizeof(float) + 15) & ~15;
   const long long fn_bytes = (long long)c->KL * c->fn_len * 2;
   const bool fn_smem = fn_bytes <= HN_FN_SMEM_MAX && c->H <= 0x7fff;
   const int smem = tile_bytes + (fn_smem ? (int)fn_bytes : 0);
-  const long long smem2_ll = ((32LL * (c->H + 1) * 8 + 15) & ~15LL) + fn_bytes;
-  if (fn_smem && c->cfg.hash_family == DSLIDE_DWTA && c->fn_len == 8 && smem2_ll <= 100 * 1024) {
-    const int smem2 = (int)smem2_ll;
-    if (smem2 > 48 * 1024) {
-      e = cudaFuncSetAttribute(split_count ? k_hash_neurons_dwta8<false> : k_hash_neurons_dwta8<true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
-      if (e != cudaSuccess) return e;
-    }
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, split_count ? k_hash_neurons_dwta8<false> : k_hash_neurons_dwta8<true>,
-                                                      HN_THREADS, smem2);
+  // bins of eight: four rows per lane while two blocks fit a multiprocessor, else two rows
+  const long long smem4 = ((32LL * (c->H + 1) * 16 + 15) & ~15LL) + 2 * fn_bytes, smem2 = ((32LL * (c->H + 1) * 8 + 15) & ~15LL) + 2 * fn_bytes;
+  if (fn_smem && c->cfg.hash_family == DSLIDE_DWTA && c->fn_len == 8 && smem2 <= 200 * 1024) {
+    e = smem4 <= 112 * 1024 ? launch_dwta8<2>(c, (int)smem4) : launch_dwta8<1>(c, (int)smem2);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    LaunchScope ls(c, KID_HASH_NEURONS);
-    auto kern8 = split_count ? k_hash_neurons_dwta8<false> : k_hash_neurons_dwta8<true>;
-    kern8<<<c->num_sms * per_sm, HN_THREADS, smem2, c->stream>>>(c->W2, c->hash_idx, c->keysA, c->place_path ? c->keysB : nullptr,
-                                                               hash_counts, c->N, c->H, c->K, c->L, c->lg_bin, c->nb);
   } else {
     auto kern = fn_smem ? k_hash_neurons<true> : k_hash_neurons<false>;
     if (smem > 48 * 1024) {
@@ -919,24 +1148,61 @@ cudaError_t launch_build_tables(Ctx* c) {
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     LaunchScope ls(c, KID_HASH_NEURONS);
-    kern<<<c->num_sms * per_sm, HN_THREADS, smem, c->stream>>>(c->W2, c->hash_idx, c->hash_sign, c->keysA,
-                                                             c->place_path ? c->keysB : nullptr, hash_counts, c->N, c->H, c->K, c->L,
-                                                             c->cfg.hash_family, c->lg_bin, c->fn_len, c->nb);
+    kern<<<c->num_sms * per_sm, HN_THREADS, smem, c->stream>>>(c->W2, c->hash_idx, c->hash_sign, c->keysA, c->N, c->H, c->K, c->L,
+                                                             c->cfg.hash_family, c->lg_bin, c->fn_len);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (split_count) {
+  const bool list_in_scan = c->place_path && c->cap >= ORD_SMALL;
+  // on the wide-code paths, with a cap of at least ORD_SMALL, the buckets that must be in order for the step (those
+  // above the cap) are listed on the way: no separate pass over all bucket sizes
+  if (list_in_scan && (e = cudaMemsetAsync(c->ord_cnt, 0, 2 * sizeof(int), c->stream)) != cudaSuccess) return e;
+  if (parts) {
+    int* total = c->part_work;
+    int* base = total + (size_t)c->L * ((size_t)1 << up);
+    if ((e = cudaMemsetAsync(total, 0, (size_t)c->L * ((size_t)1 << up) * sizeof(int), c->stream)) != cudaSuccess) return e;
+    const dim3 grid((c->N + PT_TILE - 1) / PT_TILE, c->L);
+    {
+      LaunchScope ls(c, KID_SORT_HIST);
+      k_part_hist<<<dim3((c->N + PT_HIST - 1) / PT_HIST, c->L), PT_THREADS, 0, c->stream>>>(c->keysA, total, c->N, low, up);
+    }
+    {
+      LaunchScope ls(c, KID_SORT_SCAN);
+      k_part_scan<<<c->L, 1 << (up < 5 ? 5 : up), 0, c->stream>>>(total, base, up);
+    }
+    {
+      LaunchScope ls(c, KID_SORT_SCATTER);
+      k_part_scatter<<<grid, PT_THREADS, 0, c->stream>>>(c->keysA, total, c->keysB, c->N, low, up, id_bits);
+    }
+    {
+      LaunchScope ls(c, KID_PLACE_IDS);
+      k_part_place<<<dim3(1 << up, c->L), PP_THREADS, 0, c->stream>>>(c->keysB, base, c->bucket_off, c->bucket_ids, c->N, c->nb, low, up, id_bits,
+                                                                    c->cap, c->ord_mid, c->ord_big, list_in_scan ? c->ord_cnt : nullptr);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // A query reads a whole bucket unless it holds more than `cap` ids, and the union of the buckets is put in
+    // order afterwards anyway: only buckets larger than the cap must be in ascending order for the step.  The
+    // smaller ones are ordered when the table is read back (launch_order_buckets(c, 1)).
+    c->ids_ordered_above = c->cap;
+    return order_buckets(c, c->cap, list_in_scan);
+  }
+  if (!c->place_path) {
+    // codes of at most one radix digit: the buckets are counted tile by tile in shared memory, and the running sum over
+    // a table's counts is its offsets
+    if ((e = cudaMemsetAsync(c->part_work, 0, (size_t)c->L * (size_t)c->nb * sizeof(int), c->stream)) != cudaSuccess) return e;
+    LaunchScope ls(c, KID_BUCKET_SCAN);
+    c->launches += 1;
+    k_part_hist<<<dim3((c->N + PT_HIST - 1) / PT_HIST, c->L), PT_THREADS, 0, c->stream>>>(c->keysA, c->part_work, c->N, 0, c->bits);
+    k_part_scan<<<c->L, 1 << (c->bits < 5 ? 5 : c->bits), 0, c->stream>>>(c->part_work, c->bucket_off, c->bits);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  } else {
     LaunchScope ls(c, KID_HASH_NEURONS);
     dim3 grid((unsigned)min((long long)(c->N + 255) / 256, 2048LL), c->L);
-    k_count_ranks<<<grid, 256, 0, c->stream>>>(c->keysA, c->place_path ? c->keysB : nullptr, c->bucket_off, c->N, c->nb);
+    k_count_ranks<<<grid, 256, 0, c->stream>>>(c->keysA, c->keysB, c->bucket_off, c->N, c->nb);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  const bool list_in_scan = c->place_path && c->cap >= ORD_SMALL;
-  {
+  if (c->place_path) {
     const int nchunks = (int)((c->nb + 1 + BS_CHUNK - 1) / BS_CHUNK);
     dim3 grid(nchunks, c->L);
-    // on the place path, with a cap of at least ORD_SMALL, the buckets that must be in order for the step (those
-    // above the cap) are listed by the scan itself: no separate pass over all bucket sizes
-    if (list_in_scan && (e = cudaMemsetAsync(c->ord_cnt, 0, 2 * sizeof(int), c->stream)) != cudaSuccess) return e;
     LaunchScope ls(c, KID_BUCKET_SCAN);
     k_bucket_sums<<<grid, BS_THREADS, 0, c->stream>>>(c->bucket_off, c->nb, c->bucket_part, nchunks);
     k_bucket_scan<<<grid, BS_THREADS, 0, c->stream>>>(c->bucket_off, c->nb, c->bucket_part, nchunks, c->cap, c->ord_mid,
@@ -951,10 +1217,7 @@ cudaError_t launch_build_tables(Ctx* c) {
       k_place_ids<<<grid, 256, 0, c->stream>>>(c->keysA, c->keysB, c->bucket_off, c->bucket_ids, c->N, c->nb);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // A query reads a whole bucket unless it holds more than `cap` ids, and the union of the buckets is put in
-    // order afterwards anyway: only buckets larger than the cap must be in ascending order for the step.  The
-    // smaller ones are ordered when the table is read back (launch_order_buckets(c, 1)).
-    c->ids_ordered_above = c->cap;
+    c->ids_ordered_above = c->cap;      // as above
     return order_buckets(c, c->cap, list_in_scan);
   }
 
