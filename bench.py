@@ -537,7 +537,7 @@ def measure(args, c, B, world, rank, local, windows, with_e2e, with_cpu, sampler
     achieved = booked / dur / 1e9
     step_gbs = model["total"] / (ms_step * 1e-3) / 1e9
     rebuild_us = 1e3 * rebuild_ms / args.rebuild_period if args.rebuild_period else 0.0
-    roofline = {"bound": "hbm", "kernel": {"adam": "k_update", "adam_dense": "k_adam_dense", "forward": "k_forward"}[dominant], "achieved": achieved, "peak": peak, "unit": "GB/s",
+    roofline = {"bound": "hbm", "kernel": {"adam": "k_update", "adam_dense": "k_adam_dense / k_rows_update", "forward": "k_forward"}[dominant], "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": ncu_traffic(dominant, model_prof),
                 "algorithmic_bytes_per_launch": booked, "us_per_launch": dur * 1e6,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of %s)" % peak_kind,

@@ -185,16 +185,15 @@ struct Ctx {
 
   // tiles of touched rows of W2 (tile_rows > 0: the context has the work space for them)
   int tile_rows;                   // rows of a tile at most
-  int tile_step;                   // a tile starts at the first 32-id word whose touched rows begin at or past a multiple of this
-  int tile_max;                    // tiles at most
+  int tile_step;                   // a tile starts at the first 32-id word whose touched rows begin at or past a multiple of this (or less: small batches)
   double tile_got, tile_pool;      // expected size of an active set, and how many rows the tables hand out at all
   uint32_t* touch2;                // [ceil(N/32)] the touched rows; cleared again within the step
   int* wpre;                       // [ceil(N/32) + 1] touched rows before each word
   int* trows;                      // [N] touched rows, ascending
-  int* tstart;                     // [tile_max + 1] first of trows of every tile
+  int* tstart;                     // [tiles + 1] first of trows of every tile
   int* tinfo;                      // number of tiles; 1 when a tile's rows did not come in time; entries of tlist handed out
   uint16_t* act_loc;               // [B][act_stride] place of the neuron's row in its tile
-  int* seg;                        // [tile_max + 1][max_batch] where a sample's entries of every tile start
+  int* seg;                        // [tiles + 1][batch] where a sample's entries of every tile start
   float* tpart;                    // [row chunks][B][H + 4] sums of exp(z - M) W2, M and the sum of exp(z - M)
   int2* rinfo;                     // [N] per touched row: where its touches start in tlist, and how many they are
   int2* tlist;                     // [B * act_stride] (sample, error bits) row by row, ascending samples in a row

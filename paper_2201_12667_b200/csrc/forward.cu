@@ -454,6 +454,34 @@ __device__ __noinline__ int budget_select(int budget, int fill, int N, uint64_t 
   return total;
 }
 
+// One SimHash bit of the hidden activation: the projection's sum in stored order, its sign.  Out of line: the kernel's
+// straight path (DWTA) stays short.
+__device__ __noinline__ unsigned char simhash_bit(const float* h, const int32_t* ix, const int32_t* sg, int n) {
+  float sum = 0.f;
+  for (int i = 0; i < n; ++i) {
+    const float x = h[ix[i]];
+    sum = __fadd_rn(sum, sg[i] > 0 ? x : -x);
+  }
+  return sum >= 0.f ? 1 : 0;
+}
+// The same from the packed table, where a warp reads 32 functions' i-th coordinates (top bit = minus) side by side,
+// sixteen rounds of them in flight.
+__device__ __noinline__ unsigned char simhash_bit_packed(const float* h, const uint16_t* pk, int KL, int n) {
+  float sum = 0.f;
+  for (int i0 = 0; i0 < n; i0 += 16) {
+    unsigned e[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) e[i] = i0 + i < n ? (unsigned)__ldg(pk + (size_t)(i0 + i) * KL) : 0u;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i0 + i < n) {
+        const float x = h[e[i] & 0x7fffu];
+        sum = __fadd_rn(sum, (e[i] & 0x8000u) ? -x : x);
+      }
+  }
+  return sum >= 0.f ? 1 : 0;
+}
+
 // The sample is skipped: no loss, no gradient, nothing touched (predict: no candidates).
 template <int MODE>
 __device__ __forceinline__ void skip_sample(const FwdParams& p, int s, int code) {
@@ -687,30 +715,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     }
     for (int f = tid; f < p.KL; f += FWD_THREADS) {
       const int32_t* ix = hidx + (size_t)f * p.fn_len;
-      if (p.family == DSLIDE_SIMHASH && p.hash_sm_off < 0) {
-        // the packed table: a warp reads 32 functions' i-th coordinates (sign in the top bit) side by side, sixteen rounds
-        // of them in flight; sums in stored order as ever
-        float sum = 0.f;
-        for (int i0 = 0; i0 < p.fn_len; i0 += 16) {
-          unsigned e[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) e[i] = i0 + i < p.fn_len ? (unsigned)__ldg(p.hash_pk + (size_t)(i0 + i) * p.KL + f) : 0u;
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            if (i0 + i < p.fn_len) {
-              const float x = sh_h[e[i] & 0x7fffu];
-              sum = __fadd_rn(sum, (e[i] & 0x8000u) ? -x : x);
-            }
-        }
-        sh_part[f] = sum >= 0.f ? 1 : 0;
-      } else if (p.family == DSLIDE_SIMHASH) {
-        const int32_t* sg = hsgn + (size_t)f * p.fn_len;
-        float sum = 0.f;
-        for (int i = 0; i < p.fn_len; ++i) {
-          float x = sh_h[ix[i]];
-          sum = __fadd_rn(sum, sg[i] > 0 ? x : -x);
-        }
-        sh_part[f] = sum >= 0.f ? 1 : 0;
+      if (p.family == DSLIDE_SIMHASH) {
+        sh_part[f] = p.hash_sm_off < 0 ? simhash_bit_packed(sh_h, p.hash_pk + f, p.KL, p.fn_len)
+                                       : simhash_bit(sh_h, ix, hsgn + (size_t)f * p.fn_len, p.fn_len);
       } else if (p.fn_len == 8 && (reinterpret_cast<uintptr_t>(hidx) & 15) == 0) {
         // bins of eight: both halves of the index list in one load each, the eight values fetched side by side
         const int4 ia = reinterpret_cast<const int4*>(ix)[0], ib = reinterpret_cast<const int4*>(ix)[1];
@@ -842,7 +849,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       for (int w = tid; w < n4; w += FWD_THREADS) dd4[w] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
     }
-    constexpr int CU = MODE == 2 ? 4 : 1;      // thousands of candidates: several per thread and round, their loads in flight together
+    constexpr int CU = MODE == 0 ? 1 : 4;      // thousands of candidates: several per thread and round, their loads in flight together
     for (int c0 = tid; c0 < ncand; c0 += CU * FWD_THREADS) {
       int j[CU];
 #pragma unroll
@@ -1624,10 +1631,11 @@ cudaError_t launch_predict(Ctx* c, int batch, const int32_t* row_ptr, const int3
   p.out_ids = out_ids;
   p.out_scores = out_scores;
   if (dense) p.dense = 1;
+  p.inputs_ready = 0;            // the batch may come from the kernel before this one in the stream: nothing is read before it has completed
   LaunchScope ls(c, KID_PREDICT);
-  if (c->H <= FWD_THREADS) k_forward<1, 1><<<batch, FWD_THREADS, c->fwd_smem, c->stream>>>(p);
-  else k_forward<1, MAX_KPT><<<batch, FWD_THREADS, c->fwd_smem, c->stream>>>(p);
-  cudaError_t e = cudaGetLastError();
+  // placed while the kernel before it drains (the call before this one, in a serving loop)
+  cudaError_t e = c->H <= FWD_THREADS ? launch_dependent(k_forward<1, 1>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p)
+                                      : launch_dependent(k_forward<1, MAX_KPT>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
   if (e != cudaSuccess || !dense) return e;
   return launch_dense_tc(c, batch, k, out_ids, out_scores);      // over all neurons: the kernel above has left the hidden activations
 }

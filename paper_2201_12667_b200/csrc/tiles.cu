@@ -9,7 +9,7 @@
 //   k_forward<2>    : hidden layer, codes, active sets; marks the touched rows in a bitmap (forward.cu)
 //   k_tile_scan     : touched rows before every word of the bitmap, and where the tiles start
 //   k_tile_index    : the list of touched rows; per active neuron its place in its tile; per (tile, sample) the run
-//   k_tile_forward  : a block holds a tile; a warp takes a sample's run: four rows at a time are read into registers,
+//   k_tile_forward  : a block holds a tile; a warp takes a sample's run: rows are read into registers several at a time,
 //                     their logits taken, and the sums S = sum_a exp(z_a - M) W2[a], E = sum_a exp(z_a - M) carried
 //                     along with a running maximum M (so a row is read from shared memory once for both).
 //   k_tile_combine  : per sample: the row chunks' S, E, M put together, loss, errors, error at the hidden layer
@@ -36,6 +36,7 @@ __device__ __forceinline__ unsigned long long pair2(float lo, float hi) {
 __device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
 constexpr int TS_THREADS = 1024;
+constexpr int TS_WORDS = 16;
 constexpr int TI_THREADS = 512;
 constexpr int TF_THREADS = 512;
 constexpr int TF_WARPS = TF_THREADS / 32;
@@ -45,12 +46,15 @@ constexpr int TL_WARPS = TL_THREADS / 32;
 constexpr int TL_CHUNK = 1024;                         // samples listed at a time
 constexpr int TILE_BYTES = 196 * 1024;                 // shared memory for a tile's rows
 constexpr int TILE_N_MAX = 8 << 20;
+constexpr int TILE_STEP_MIN = 32;
 constexpr int TILE_ROWS_MAX = 512;                     // a thread of k_tile_lists each
 constexpr size_t TILE_PART_BYTES = (size_t)32 << 20;   // the row chunks' sums stay in L2
 constexpr size_t TILE_SEG_BYTES = (size_t)512 << 20, TILE_LIST_BYTES = (size_t)2 << 30;      // beyond these the work space is not worth it
 // Which steps go by tiles: from TILE_MIN_SET neurons per sample on, when a sample has at least TILE_MIN_RUN of them in a
 // tile on average (below that, walking the (tile, sample) pairs costs more than the shared rows save).
-constexpr double TILE_MIN_SET = 512.0, TILE_MIN_RUN = 1.5;
+// A touched row must serve several samples: at three (81,000 pairs over 28,600 rows of 64 units) the eight launches took
+// 138 us against 95 of the block per sample, at twenty (36,000 pairs over 1,741 rows of 252 units) 102 against 186.
+constexpr double TILE_MIN_SET = 512.0, TILE_MIN_RUN = 1.5, TILE_MIN_SHARE = 6.0;
 
 // Expected size of an active set and of the pool of rows the tables hand out, from the tables' shape: L buckets of
 // about N / 2^bits ids; where the cap cuts them, the lowest ids of every bucket are what all samples share.
@@ -68,8 +72,19 @@ static void expect_sets(Ctx* c) {
 bool use_tiles(const Ctx* c, int batch) {
   if (c->tile_rows == 0) return false;
   const double touched = c->tile_pool * -expm1(-(double)batch * c->tile_got / c->tile_pool);
-  return c->tile_got * (double)c->tile_step >= TILE_MIN_RUN * touched;
+  return c->tile_got * (double)c->tile_step >= TILE_MIN_RUN * touched && (double)batch * c->tile_got >= TILE_MIN_SHARE * touched;
 }
+
+// Rows of a tile for this batch (a tile may hold up to 31 more): as many as fit, or so few that every multiprocessor has
+// two tiles -- small batches -- while a sample still has a dozen entries in a tile on average.
+static int call_step(const Ctx* c, int batch) {
+  const double touched = c->tile_pool * -expm1(-(double)batch * c->tile_got / c->tile_pool);
+  double want = touched / (2.0 * c->num_sms);
+  if (want < 12.0 * touched / c->tile_got) want = 12.0 * touched / c->tile_got;
+  if (want < TILE_STEP_MIN) want = TILE_STEP_MIN;
+  return want < c->tile_step ? (int)want : c->tile_step;
+}
+static int call_tiles(const Ctx* c, int batch) { return c->N / call_step(c, batch) + 2; }      // tiles at most
 
 // Row chunks (blocks that walk the tiles side by side) and groups of samples of k_tile_forward.
 static void tile_grid(const Ctx* c, int batch, int* chunks, int* groups) {
@@ -82,7 +97,7 @@ static void tile_grid(const Ctx* c, int batch, int* chunks, int* groups) {
   if (q < 1) q = 1;
   int p = c->num_sms / q;
   if (p < 1) p = 1;
-  if (p > c->tile_max) p = c->tile_max;
+  if (p > call_tiles(c, batch)) p = call_tiles(c, batch);
   *chunks = p;
   *groups = q;
 }
@@ -91,33 +106,34 @@ cudaError_t setup_tiles(Ctx* c) {
   c->tile_rows = 0;
   if (c->dense) return cudaSuccess;
   expect_sets(c);
-  if (c->tile_got < TILE_MIN_SET) return cudaSuccess;
+  const double most_shared = c->cfg.max_batch * c->tile_got / (c->tile_pool * -expm1(-c->cfg.max_batch * c->tile_got / c->tile_pool));
+  if (c->tile_got < TILE_MIN_SET || most_shared < TILE_MIN_SHARE) return cudaSuccess;      // no batch would take them
   int rows = TILE_BYTES / ((c->H + 4) * 4);
   if (rows > TILE_ROWS_MAX) rows = TILE_ROWS_MAX;
   const int step = rows - 31;                // a tile takes whole words of the bitmap
   if (step < 1 || c->N > TILE_N_MAX) return cudaSuccess;
-  const int64_t tmax = (int64_t)c->N / step + 2;
-  const size_t B = c->cfg.max_batch;
-  if ((size_t)(tmax + 1) * B * 4 > TILE_SEG_BYTES || B * (size_t)c->act_stride * 8 > TILE_LIST_BYTES) return cudaSuccess;
   c->tile_step = step;
-  c->tile_max = (int)tmax;
-  size_t most = 0;
+  const size_t B = c->cfg.max_batch;
+  size_t most = 0, runs = 0, tiles = 0;
   for (int b = 1; b <= c->cfg.max_batch; ++b) {
     int p, q;
     tile_grid(c, b, &p, &q);
-    const size_t n = (size_t)p * b * (c->H + 4);
+    const size_t n = (size_t)p * b * (c->H + 4), t = (size_t)call_tiles(c, b) + 1;
     if (n > most) most = n;
+    if (t * b > runs) runs = t * b;
+    if (t > tiles) tiles = t;
   }
+  if (runs * 4 > TILE_SEG_BYTES || B * (size_t)c->act_stride * 8 > TILE_LIST_BYTES) return cudaSuccess;
   const size_t nw = ((size_t)c->N + 31) / 32;
   cudaError_t e = cudaSuccess;
   auto get = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
   get((void**)&c->touch2, nw * 4);
   get((void**)&c->wpre, (nw + 1) * 4);
   get((void**)&c->trows, (size_t)c->N * 4);
-  get((void**)&c->tstart, (size_t)(tmax + 1) * 4);
+  get((void**)&c->tstart, tiles * 4);
   get((void**)&c->tinfo, 16);
   get((void**)&c->act_loc, B * (size_t)c->act_stride * 2);
-  get((void**)&c->seg, (size_t)(tmax + 1) * B * 4);
+  get((void**)&c->seg, runs * 4);
   get((void**)&c->tpart, most * 4);
   get((void**)&c->rinfo, (size_t)c->N * 8);
   get((void**)&c->tlist, B * (size_t)c->act_stride * 8);
@@ -137,13 +153,14 @@ k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int
   griddep_wait();
   const int per = ((nw + TS_THREADS - 1) / TS_THREADS + 3) & ~3;
   const int w0 = min(nw, tid * per), w1 = min(nw, w0 + per);
+  // a thread's words stay in registers between the count and the walk (more of them than that are read again)
+  uint32_t word[TS_WORDS];
+#pragma unroll
+  for (int i = 0; i < TS_WORDS; ++i) word[i] = i < w1 - w0 ? __ldcg(touch + w0 + i) : 0u;
   int mine = 0;
-  int w = w0;
-  for (; w + 4 <= w1; w += 4) {
-    const uint4 x = __ldcg(reinterpret_cast<const uint4*>(touch + w));
-    mine += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
-  }
-  for (; w < w1; ++w) mine += __popc(__ldcg(touch + w));
+#pragma unroll
+  for (int i = 0; i < TS_WORDS; ++i) mine += __popc(word[i]);
+  for (int w = w0 + TS_WORDS; w < w1; ++w) mine += __popc(__ldcg(touch + w));
   int incl = mine;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -171,12 +188,16 @@ k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int
     const int before = run - __popc(__ldcg(touch + w0 - 1));
     tile = tile_of(before, magic, step);
   }
-  for (w = w0; w < w1; ++w) {
+  auto walk = [&](int w, uint32_t bits) {
     wpre[w] = run;
     const int t = tile_of(run, magic, step);
     for (; tile < t;) tstart[++tile] = run;
-    run += __popc(__ldcg(touch + w));
-  }
+    run += __popc(bits);
+  };
+#pragma unroll
+  for (int i = 0; i < TS_WORDS; ++i)
+    if (i < w1 - w0) walk(w0 + i, word[i]);
+  for (int w = w0 + TS_WORDS; w < w1; ++w) walk(w, __ldcg(touch + w));
   if (w0 < w1 && w1 == nw) {                 // the thread with the last word
     wpre[nw] = total;
     tstart[tile + 1] = total;
@@ -189,7 +210,7 @@ k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int
 
 // Blocks [0, B): a sample's entries -- place in the tile, and where the runs of the tiles start (a tile without
 // entries has an empty run).  The blocks after them write the list of touched rows.
-__global__ void __launch_bounds__(TI_THREADS)
+__global__ void __launch_bounds__(TI_THREADS + 32)
 k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const int* tinfo, int nw, int step, int B, int bstride,
              const int* act_cnt, const int32_t* act_ids, int act_stride, const int32_t* label_ptr, const int32_t* labels,
              int max_labels, uint16_t* act_loc, int* seg, int* trows, int* tlab) {
@@ -197,6 +218,7 @@ k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const in
   griddep_launch_dependents();
   griddep_wait();
   if ((int)blockIdx.x >= B) {
+    if (tid >= TI_THREADS) return;
     const int nb = (int)gridDim.x - B;
     for (int w = ((int)blockIdx.x - B) * TI_THREADS + tid; w < nw; w += nb * TI_THREADS) {
       uint32_t bits = __ldcg(touch + w);
@@ -212,6 +234,18 @@ k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const in
   const int na = __ldcg(act_cnt + s), nt = __ldcg(tinfo);
   const int32_t* ids = act_ids + (size_t)s * act_stride;
   uint16_t* loc = act_loc + (size_t)s * act_stride;
+  if (tid >= TI_THREADS) {                    // the last warp: the labels' places in the active set (a repeated label counts once)
+    const int lbeg = label_ptr[s], nlab = na > 0 ? label_ptr[s + 1] - lbeg : 0;
+    for (int i = tid - TI_THREADS; i < nlab; i += 32) {
+      const int y = labels[lbeg + i];
+      bool first = true;
+      for (int q = 0; q < i; ++q) first = first && labels[lbeg + q] != y;
+      int lo = 0, hi = na;
+      while (lo < hi) { const int mid = (lo + hi) >> 1; if (__ldcg(ids + mid) < y) lo = mid + 1; else hi = mid; }
+      tlab[(size_t)s * max_labels + i] = first ? lo : -1;
+    }
+    return;
+  }
   if (na == 0) {
     for (int t = tid; t <= nt; t += TI_THREADS) seg[(size_t)t * bstride + s] = 0;
     return;
@@ -251,16 +285,6 @@ k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const in
         for (int q = t + 1; q <= nt; ++q) seg[(size_t)q * bstride + s] = na;
     }
   }
-  // the labels' places in the active set (a repeated label counts once)
-  const int lbeg = label_ptr[s], nlab = label_ptr[s + 1] - lbeg;
-  for (int i = TI_THREADS - 1 - tid; i < nlab; i += TI_THREADS) {
-    const int y = labels[lbeg + i];
-    bool first = true;
-    for (int q = 0; q < i; ++q) first = first && labels[lbeg + q] != y;
-    int lo = 0, hi = na;
-    while (lo < hi) { const int mid = (lo + hi) >> 1; if (__ldcg(ids + mid) < y) lo = mid + 1; else hi = mid; }
-    tlab[(size_t)s * max_labels + i] = first ? lo : -1;
-  }
 }
 
 struct TileParams {
@@ -290,51 +314,65 @@ __device__ __forceinline__ bool t_wait(uint64_t* bar, uint32_t parity) {      //
   return false;
 }
 
-// Grid (row chunks, groups of samples).  Dynamic shared memory: the tile's rows, each followed by the head of its
-// record (count, bias, bias moments), then the barrier.
-// A lane holds the 16-byte pieces lane, lane + 32, ... of a row.  Four rows at a time: their dot products with the
-// sample's activations are reduced together (six shuffles leave row i's sum in the lanes 8 i .. 8 i + 7).
-template <int NCH>
+// Brings tile t into shared memory, all threads: the rows one after the other, each followed by the head of its record
+// (count, bias, bias moments).  False when they did not come in time (block-uniform; nothing is left in flight).
+__device__ __forceinline__ bool load_tile(const TileParams& p, int t, float* tile, uint64_t* bar, uint32_t phase) {
+  const int H = p.H, ld = H + 4;
+  const int r0 = __ldcg(p.tstart + t), nr = __ldcg(p.tstart + t + 1) - r0;
+  __syncthreads();                             // readers of the tile before are done
+  if (threadIdx.x == 0)
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(t_smem(bar)), "r"((uint32_t)nr * ((uint32_t)H * 4u + 16u)) : "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  for (int r = threadIdx.x; r < nr; r += TF_THREADS) {
+    const int j = __ldcg(p.trows + r0 + r);
+    t_bulk(tile + (size_t)r * ld, p.W2 + (size_t)j * H, (uint32_t)H * 4u, bar);
+    t_bulk(tile + (size_t)r * ld + H, p.hdr2 + j, 16u, bar);
+  }
+  const bool ok = t_wait(bar, phase);
+  if (!__syncthreads_or(ok ? 0 : 1)) return true;
+  t_wait(bar, phase);                          // one more bounded wait for the copies in flight, then out
+  if (threadIdx.x == 0) { p.tinfo[1] = 1; atomicCAS(&p.st->status, 0, (int)DSLIDE_ERR_TIMEOUT); }
+  return false;
+}
+__device__ __forceinline__ void scale2(ulonglong2& v, unsigned long long f) {
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v.x) : "l"(f));
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v.y) : "l"(f));
+}
+
+// Grid (row chunks, groups of samples).  A group of G lanes takes a row: lane g of it holds the 16-byte pieces g, g + G,
+// ... (NP of them).  Four rows per group at a time: their dot products with the sample's activations are reduced
+// together (lanes exchange the values they give up, so that a quarter of the group ends with each row's sum).  Rows of
+// up to 128 units are taken by half warps, eight rows of a run at a time (G = 16); wider ones by whole warps (G = 32: with
+// half warps the eight rows of 200 units do not fit the registers and the one-hot word shape took 1,614 us a step instead
+// of 1,531).  Rows of up to 256 units stay in registers between the logits and the sums, others are read a second time.
+template <int G, int NP>
 __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams p) {
-  constexpr bool KEEP = NCH <= 2;            // rows of up to 1 KB stay in registers between the two uses; longer ones are read again
+  constexpr bool KEEP = G == 16 || NP <= 2;
+  constexpr int Q = G / 4;                     // lanes that end with the same row's sum
+  constexpr int RPI = 128 / G;                 // rows per iteration
   extern __shared__ __align__(128) unsigned char t_sm[];
   __shared__ __align__(8) uint64_t bar;
   float* tile = reinterpret_cast<float*>(t_sm);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int H = p.H, H4 = H >> 2, ld = H + 4;
+  const int gl = lane & (G - 1), first = (lane & ~(G - 1)) * 4 / G;      // place in the group; the group's first row of an iteration
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(t_smem(&bar)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   // the pieces of a row this lane reads; past the row's end a piece that exists (its activations are zero)
-  int off[NCH];
+  int off[NP];
 #pragma unroll
-  for (int u = 0; u < NCH; ++u) off[u] = 4 * min(lane + 32 * u, H4 - 1);
+  for (int u = 0; u < NP; ++u) off[u] = 4 * min(gl + G * u, H4 - 1);
   griddep_launch_dependents();
   griddep_wait();
   const int nt = __ldcg(p.tinfo);
   const int q0 = (int)blockIdx.y * p.gs, q1 = min(p.B, q0 + p.gs);
   uint32_t phase = 0u;
-  for (int t = blockIdx.x; t < nt; t += p.chunks) {
-    const int r0 = __ldcg(p.tstart + t), nr = __ldcg(p.tstart + t + 1) - r0;
-    __syncthreads();                           // readers of the tile before are done
-    if (tid == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(t_smem(&bar)), "r"((uint32_t)nr * ((uint32_t)H * 4u + 16u)) : "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    for (int r = tid; r < nr; r += TF_THREADS) {
-      const int j = __ldcg(p.trows + r0 + r);
-      t_bulk(tile + (size_t)r * ld, p.W2 + (size_t)j * H, (uint32_t)H * 4u, &bar);
-      t_bulk(tile + (size_t)r * ld + H, p.hdr2 + j, 16u, &bar);
-    }
-    const bool ok = t_wait(&bar, phase);
-    phase ^= 1u;
-    if (__syncthreads_or(ok ? 0 : 1)) {        // the rows did not come: one more bounded wait for the copies in flight, then out
-      t_wait(&bar, phase ^ 1u);
-      if (tid == 0) { p.tinfo[1] = 1; atomicCAS(&p.st->status, 0, (int)DSLIDE_ERR_TIMEOUT); }
-      return;
-    }
+  for (int t = blockIdx.x; t < nt; t += p.chunks, phase ^= 1u) {
+    if (!load_tile(p, t, tile, &bar, phase)) return;
     const bool fresh = t == (int)blockIdx.x;   // the chunk's first tile: nothing to carry on from
     // a warp's samples: q0 + warp, + TF_WARPS, ...; lane i holds the run of the i-th of 32 of them
     for (int sb = q0 + warp; sb < q1; sb += 32 * TF_WARPS) {
@@ -358,47 +396,46 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams
         const uint16_t* locp = p.act_loc + (size_t)s * p.act_stride + a0;
         float* zp = p.act_z + (size_t)s * p.act_stride + a0;
         int loc = lane < n ? (int)__ldcg(locp + lane) : 0;
-        ulonglong2 hx[NCH], S[NCH];              // pairs of floats: two multiply-adds per instruction
-        float M = -INFINITY, E = 0.f;            // E: this lane's rows only, until the end of the run
+        ulonglong2 hx[NP], S[NP];                // pairs of floats: two multiply-adds per instruction
+        float M = -INFINITY, E = 0.f, E0 = 0.f;  // E: this lane's rows only, until the end of the run; E0: the tiles before
 #pragma unroll
-        for (int u = 0; u < NCH; ++u) {
-          const int c = lane + 32 * u;
+        for (int u = 0; u < NP; ++u) {
+          const int c = gl + G * u;
           hx[u] = c < H4 ? __ldg(reinterpret_cast<const ulonglong2*>(p.h + (size_t)s * H) + c) : make_ulonglong2(0ull, 0ull);
           S[u] = make_ulonglong2(0ull, 0ull);
         }
-        float E0 = 0.f;
         if (!fresh) {
           const float2 me = *reinterpret_cast<const float2*>(part + H);
-          ulonglong2 sv[NCH];
+          ulonglong2 sv[NP];
 #pragma unroll
-          for (int u = 0; u < NCH; ++u) {
-            const int c = lane + 32 * u;
-            sv[u] = c < H4 ? reinterpret_cast<const ulonglong2*>(part)[c] : make_ulonglong2(0ull, 0ull);
+          for (int u = 0; u < NP; ++u) {
+            const int c = gl + G * u;
+            sv[u] = c < H4 && lane < G ? reinterpret_cast<const ulonglong2*>(part)[c] : make_ulonglong2(0ull, 0ull);
           }
-          if (me.y > 0.f || me.y != me.y) {       // something was summed before
+          if (me.y > 0.f || me.y != me.y) {       // something was summed before: the first group carries it on
             M = me.x;
             E0 = me.y;
 #pragma unroll
-            for (int u = 0; u < NCH; ++u) S[u] = sv[u];
+            for (int u = 0; u < NP; ++u) S[u] = sv[u];
           }
         }
         for (int c0 = 0; c0 < n; c0 += 32) {
           if (c0 > 0) loc = c0 + lane < n ? (int)__ldcg(locp + c0 + lane) : 0;
           const int m = min(32, n - c0);
           {
-            const int first = __shfl_sync(TFULL, loc, 0);
-            if (lane >= m) loc = first;
+            const int some = __shfl_sync(TFULL, loc, 0);      // past the run: a row of the run, with weight zero below
+            if (lane >= m) loc = some;
           }
-          for (int k = 0; k < m; k += 4) {
+          for (int k = 0; k < m; k += RPI) {
             const float* rp[4];
-            ulonglong2 x[4][KEEP ? NCH : 1];
+            ulonglong2 x[4][KEEP ? NP : 1];
             float d[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-              rp[r] = tile + __shfl_sync(TFULL, loc, k + r) * ld;      // past the run: a row of the run, with weight zero below
+              rp[r] = tile + __shfl_sync(TFULL, loc, k + first + r) * ld;
               unsigned long long d0 = 0ull, d1 = 0ull;
 #pragma unroll
-              for (int u = 0; u < NCH; ++u) {
+              for (int u = 0; u < NP; ++u) {
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(rp[r] + off[u]);
                 if (KEEP) x[r][KEEP ? u : 0] = v;
                 fma2(d0, v.x, hx[u].x);
@@ -406,40 +443,37 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams
               }
               d[r] = (lo2(d0) + hi2(d0)) + (lo2(d1) + hi2(d1));
             }
-            const bool hi = (lane & 16) != 0, od = (lane & 8) != 0;
-            const float u0 = (hi ? d[2] : d[0]) + __shfl_xor_sync(TFULL, hi ? d[0] : d[2], 16);
-            const float u1 = (hi ? d[3] : d[1]) + __shfl_xor_sync(TFULL, hi ? d[1] : d[3], 16);
-            float y = (od ? u1 : u0) + __shfl_xor_sync(TFULL, od ? u0 : u1, 8);
-            y += __shfl_xor_sync(TFULL, y, 4);
-            y += __shfl_xor_sync(TFULL, y, 2);
-            y += __shfl_xor_sync(TFULL, y, 1);
-            const float* mr = hi ? (od ? rp[3] : rp[2]) : (od ? rp[1] : rp[0]);      // this lane's row of the four
+            const bool hi = (lane & (2 * Q)) != 0, od = (lane & Q) != 0;
+            const float u0 = (hi ? d[2] : d[0]) + __shfl_xor_sync(TFULL, hi ? d[0] : d[2], 2 * Q);
+            const float u1 = (hi ? d[3] : d[1]) + __shfl_xor_sync(TFULL, hi ? d[1] : d[3], 2 * Q);
+            float y = (od ? u1 : u0) + __shfl_xor_sync(TFULL, od ? u0 : u1, Q);
+#pragma unroll
+            for (int o = Q / 2; o > 0; o >>= 1) y += __shfl_xor_sync(TFULL, y, o);
+            const float* mr = hi ? (od ? rp[3] : rp[2]) : (od ? rp[1] : rp[0]);      // the row whose sum this lane has
             float z = mr[H + 1] + y;                                 // the bias came with the row
-            const int mine = k + (lane >> 3);
+            const int mine = k + lane / Q;
             if (mine >= m) z = -INFINITY;
-            else if ((lane & 7) == 0) zp[c0 + mine] = z;
+            else if ((lane & (Q - 1)) == 0) zp[c0 + mine] = z;
             if (__any_sync(TFULL, z > M)) {
-              float zm = fmaxf(z, __shfl_xor_sync(TFULL, z, 8));
-              zm = fmaxf(fmaxf(zm, __shfl_xor_sync(TFULL, zm, 16)), M);
+              float zm = fmaxf(z, M);
+#pragma unroll
+              for (int o = Q; o < 32; o <<= 1) zm = fmaxf(zm, __shfl_xor_sync(TFULL, zm, o));
               const float scale = expf(M - zm);
               const unsigned long long sc = pair2(scale, scale);
               M = zm;
               E *= scale;
               E0 *= scale;
 #pragma unroll
-              for (int u = 0; u < NCH; ++u) {
-                asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(S[u].x) : "l"(sc));
-                asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(S[u].y) : "l"(sc));
-              }
+              for (int u = 0; u < NP; ++u) scale2(S[u], sc);
             }
             const float e = mine < m ? expf(z - M) : 0.f;
             E += e;
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-              const float g = __shfl_sync(TFULL, e, 8 * r);
+              const float g = __shfl_sync(TFULL, e, (lane & ~(G - 1)) + Q * r);
               const unsigned long long gg = pair2(g, g);
 #pragma unroll
-              for (int u = 0; u < NCH; ++u) {
+              for (int u = 0; u < NP; ++u) {
                 const ulonglong2 v = KEEP ? x[r][KEEP ? u : 0] : *reinterpret_cast<const ulonglong2*>(rp[r] + off[u]);
                 fma2(S[u].x, gg, v.x);
                 fma2(S[u].y, gg, v.y);
@@ -447,12 +481,18 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams
             }
           }
         }
-        E += __shfl_xor_sync(TFULL, E, 8);       // the four groups of lanes hold different rows
-        E += __shfl_xor_sync(TFULL, E, 16);
 #pragma unroll
-        for (int u = 0; u < NCH; ++u) {
-          const int c = lane + 32 * u;
-          if (c < H4) reinterpret_cast<ulonglong2*>(part)[c] = S[u];
+        for (int o = Q; o < 32; o <<= 1) E += __shfl_xor_sync(TFULL, E, o);      // lanes hold different rows
+#pragma unroll
+        for (int u = 0; u < NP; ++u) {
+          const int c = gl + G * u;
+          if (G == 16) {                         // the two halves' sums
+            const unsigned long long ox = __shfl_xor_sync(TFULL, S[u].x, 16), oy = __shfl_xor_sync(TFULL, S[u].y, 16);
+            const unsigned long long one = pair2(1.f, 1.f);
+            fma2(S[u].x, ox, one);
+            fma2(S[u].y, oy, one);
+          }
+          if (c < H4 && lane < G) reinterpret_cast<ulonglong2*>(part)[c] = S[u];
         }
         if (lane == 0) *reinterpret_cast<float2*>(part + H) = make_float2(M, E0 + E);
       }
@@ -698,23 +738,24 @@ cudaError_t launch_tiles_forward(Ctx* c, int batch, const int32_t* label_ptr, co
   const int nw = (c->N + 31) / 32;
   int chunks, groups;
   tile_grid(c, batch, &chunks, &groups);
+  const int step = call_step(c, batch);
   c->launches += 5;          // with the kernel before them they make one entry of the profile
-  cudaError_t e = launch_dependent(k_tile_scan, dim3(1), dim3(TS_THREADS), 0, c->stream, (const uint32_t*)c->touch2, nw, c->tile_step,
+  cudaError_t e = launch_dependent(k_tile_scan, dim3(1), dim3(TS_THREADS), 0, c->stream, (const uint32_t*)c->touch2, nw, step,
                                    c->wpre, c->tstart, c->tinfo, &c->dstate->n_own[c->t_host & 1][0]);
   if (e != cudaSuccess) return e;
   const int extra = (nw + 4 * TI_THREADS - 1) / (4 * TI_THREADS);
-  e = launch_dependent(k_tile_index, dim3(batch + extra), dim3(TI_THREADS), 0, c->stream, (const uint32_t*)c->touch2, (const int*)c->wpre,
-                       (const int*)c->tstart, (const int*)c->tinfo, nw, c->tile_step, batch, c->cfg.max_batch, (const int*)c->act_cnt,
+  e = launch_dependent(k_tile_index, dim3(batch + extra), dim3(TI_THREADS + 32), 0, c->stream, (const uint32_t*)c->touch2, (const int*)c->wpre,
+                       (const int*)c->tstart, (const int*)c->tinfo, nw, step, batch, batch, (const int*)c->act_cnt,
                        (const int32_t*)c->act_ids, c->act_stride, label_ptr, labels, c->cfg.max_labels, c->act_loc, c->seg, c->trows, c->tlab);
   if (e != cudaSuccess) return e;
   TileParams p;
   p.W2 = c->W2; p.hdr2 = c->hdr2; p.h = c->h; p.trows = c->trows; p.tstart = c->tstart; p.tinfo = c->tinfo; p.seg = c->seg;
   p.act_loc = c->act_loc; p.act_z = c->act_z; p.part = c->tpart; p.st = c->dstate;
-  p.B = batch; p.H = c->H; p.act_stride = c->act_stride; p.bstride = c->cfg.max_batch; p.chunks = chunks; p.gs = (batch + groups - 1) / groups;
-  const int smem = c->tile_rows * (c->H + 4) * 4;
-  const int nch = (c->H / 4 + 31) / 32;
-  auto k = nch <= 1 ? k_tile_forward<1> : nch <= 2 ? k_tile_forward<2> : nch <= 4 ? k_tile_forward<4> : k_tile_forward<8>;
-  if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+  p.B = batch; p.H = c->H; p.act_stride = c->act_stride; p.bstride = batch; p.chunks = chunks; p.gs = (batch + groups - 1) / groups;
+  const int smem = (step + 31) * (c->H + 4) * 4;
+  auto k = c->H <= 64 ? k_tile_forward<16, 1> : c->H <= 128 ? k_tile_forward<16, 2> : c->H <= 256 ? k_tile_forward<32, 2>
+           : c->H <= 512 ? k_tile_forward<32, 4> : k_tile_forward<32, 8>;
+  if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024)) != cudaSuccess) return e;
   if ((e = launch_dependent(k, dim3(chunks, groups), dim3(TF_THREADS), (size_t)smem, c->stream, p)) != cudaSuccess) return e;
   CombineParams q;
   q.W2 = c->W2; q.h = c->h; q.part = c->tpart; q.act_z = c->act_z; q.label_ptr = label_ptr; q.act_ids = c->act_ids;
@@ -725,9 +766,9 @@ cudaError_t launch_tiles_forward(Ctx* c, int batch, const int32_t* label_ptr, co
   if ((e = launch_dependent(k_tile_combine, dim3(batch), dim3(TC3_THREADS), csm, c->stream, q)) != cudaSuccess) return e;
   ListParams l;
   l.tstart = c->tstart; l.seg = c->seg; l.tinfo = c->tinfo; l.act_loc = c->act_loc; l.act_g = c->act_g; l.rinfo = c->rinfo; l.list = c->tlist;
-  l.B = batch; l.act_stride = c->act_stride; l.bstride = c->cfg.max_batch; l.rows = c->tile_rows;
-  const size_t lsm = (size_t)c->tile_rows * ((TL_CHUNK / 32 + 1) * 6 + 8);
-  if ((e = cudaFuncSetAttribute(k_tile_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm)) != cudaSuccess) return e;
+  l.B = batch; l.act_stride = c->act_stride; l.bstride = batch; l.rows = step + 31;
+  const size_t lsm = (size_t)(step + 31) * ((TL_CHUNK / 32 + 1) * 6 + 8);
+  if ((e = cudaFuncSetAttribute(k_tile_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024)) != cudaSuccess) return e;
   return launch_dependent(k_tile_lists, dim3(2 * c->num_sms), dim3(TL_THREADS), lsm, c->stream, l);
 }
 

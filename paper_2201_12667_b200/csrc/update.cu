@@ -816,7 +816,7 @@ static cudaError_t launch_rows_update(Ctx* c, const UpdParams& p) {
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_update, RU_THREADS, smem)) != cudaSuccess) return e;
   int nb = c->num_sms * (per_sm > 0 ? per_sm : 1) / q.shares;
   if (nb < 1) nb = 1;
-  LaunchScope ls(c, KID_ADAM);
+  LaunchScope ls(c, KID_ADAM_DENSE);      // the output layer's part, timed by itself
   return launch_dependent(k_rows_update, dim3(nb, q.shares), dim3(RU_THREADS), (size_t)smem, c->stream, p, q);
 }
 
