@@ -205,7 +205,7 @@ struct Ctx {
   int32_t* tile_hist;
   int32_t* bucket_part;   // per table: sums of chunks of bucket counters (bucket offset scan)
   int* part_work;         // wide codes: per table the parts' sizes / cursors, then where they start
-  int place_path;         // 1: codes wider than a radix digit: ids placed by atomics, then ordered inside buckets
+  int place_path;         // 1: codes wider than a radix digit: ids partitioned and placed (or counted and placed by rank), large buckets ordered afterwards
   int2 *ord_mid, *ord_big; // (table, bucket) of the buckets too large to order in registers / in shared memory
   int* ord_cnt;           // lengths of those two lists
   int ids_ordered_above;  // place path: buckets with more ids than this are in ascending order (1 = every bucket)
