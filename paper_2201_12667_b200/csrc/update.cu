@@ -23,7 +23,7 @@
 //              sums in slice order (rows of W1 that have been hot before find their coefficients in a
 //              table line the forward kernel fills, instead of searching).  Warps draw tickets (the first two are fixed by the warp's number,
 //              the others come from a counter): hot slices, then listed rows, then the ordinary rows four
-//              at a time, the last few thousand two at a time.  Adam is applied to the touched rows only; untouched rows are neither read
+//              at a time (of up to 128 units the last few thousand two at a time).  Adam is applied to the touched rows only; untouched rows are neither read
 //              nor written.  The warp that updates a row resets its count and mask for the next step.
 //              The first blocks of the grid update the hidden bias and reduce the batch loss.
 //   k_adam_dense : the output layer when every neuron is active (no lists, no masks).
@@ -99,6 +99,19 @@ struct Side {
   int is_w2;
 };
 
+// Rows of more than 128 units are walked in pieces of LONG_P x 128 (long_row).  PIECES, a template parameter of what follows:
+// 0 rows of up to 128 units, held in registers with their moments, two rows of a warp at a time; 1 rows of one piece; 2 of
+// several.
+constexpr int LONG_P = 2;
+// Asks L2 for a row's weights, moments and record
+__device__ __forceinline__ void fetch_row(const Side& sd, int row, int H) {
+  const uint32_t bytes = (uint32_t)H * 4u;
+  l2_fetch(sd.W + (size_t)row * H, bytes);
+  l2_fetch(sd.M + (size_t)row * H, bytes);
+  l2_fetch(sd.V + (size_t)row * H, bytes);
+  l2_fetch(sd.hdr + row, (uint32_t)sizeof(RowHdr));
+}
+
 __device__ __forceinline__ Side make_side(const UpdParams& p, bool w2) {
   Side sd;
   sd.W = w2 ? p.W2 : p.W1; sd.M = w2 ? p.mW2 : p.mW1; sd.V = w2 ? p.vW2 : p.vW1;
@@ -163,7 +176,7 @@ __device__ __forceinline__ void accumulate_word(float4 (&acc)[NCH], float& csum,
 // Up to four rows are loaded before they are used, in order.
 template <int NCH>
 __device__ __forceinline__ void accumulate_list(float4 (&acc)[NCH], float& csum, int n, int s_mine, float g_mine,
-                                                const float* src, int H, int H4, int lane) {
+                                                const float* src, int H, int H4, int col) {
   for (int k0 = 0; k0 < n; k0 += 4) {
     int sr[4]; float g[4];
 #pragma unroll
@@ -174,7 +187,7 @@ __device__ __forceinline__ void accumulate_list(float4 (&acc)[NCH], float& csum,
     }
 #pragma unroll
     for (int q = 0; q < NCH; ++q) {
-      int c = lane + q * 32;
+      int c = col + q * 32;
       if (c < H4) {
         float4 x[4];
 #pragma unroll
@@ -190,11 +203,9 @@ __device__ __forceinline__ void accumulate_list(float4 (&acc)[NCH], float& csum,
   }
 }
 
-// Gradient of a row touched by 2..ROW_SLOTS samples: the (sample, coefficient) pairs of its slots, put in
-// ascending sample order through the warp's scratch.
-template <int NCH>
-__device__ __forceinline__ void sum_slots(const Side& sd, int2 sl, int total, int* scr, float4 (&acc)[NCH],
-                                          float& csum, int H, int H4, int lane) {
+// The (sample, coefficient) pairs of the slots of a row touched by 2..ROW_SLOTS samples, put in ascending sample order
+// through the warp's scratch.
+__device__ __forceinline__ void sort_slots(int2 sl, int total, int* scr, int& s_mine, float& g_mine, int lane) {
   if (lane >= total) sl.x = 0x7fffffff;
   int rank = 0;
 #pragma unroll
@@ -205,25 +216,24 @@ __device__ __forceinline__ void sum_slots(const Side& sd, int2 sl, int total, in
   __syncwarp();
   if (lane < total) { scr[rank] = sl.x; scr[32 + rank] = sl.y; }
   __syncwarp();
-  const int s_mine = lane < total ? scr[lane] : 0;
-  const float g_mine = lane < total ? __int_as_float(scr[32 + lane]) : 0.f;
-  accumulate_list<NCH>(acc, csum, total, s_mine, g_mine, sd.src, H, H4, lane);
+  s_mine = lane < total ? scr[lane] : 0;
+  g_mine = lane < total ? __int_as_float(scr[32 + lane]) : 0.f;
 }
 
 // Gradient of a row touched by more than ROW_SLOTS samples, restricted to the samples of the mask words
 // [w0, w1): the samples of the slots and of the mask, ascending.  Up to 32 samples at a time are listed
 // in the warp's scratch, their coefficients looked up in parallel, then added in order.  Clears the mask.
-template <int NCH>
+template <int NCH, bool CLEAR>
 __device__ __forceinline__ void sum_masked(const UpdParams& p, const Side& sd, const int* rowptr, int row,
                                            int slot_s, int w0, int w1, int* scr, float4 (&acc)[NCH], float& csum,
-                                           int H, int H4, int lane, const float* line = nullptr) {
+                                           int H, int H4, int lane, int col, const float* line = nullptr) {
   uint32_t* mrow = sd.mask + (size_t)row * p.Wd;
   int fill = 0;
   const unsigned lt = (1u << lane) - 1u;
   for (int wb = w0; wb < w1; wb += 32) {
     const int wi = wb + lane;
     uint32_t word = wi < w1 ? mrow[wi] : 0u;
-    if (word) mrow[wi] = 0u;                     // clean for the next step
+    if (CLEAR && word) mrow[wi] = 0u;            // clean for the next step
 #pragma unroll
     for (int k = 0; k < ROW_SLOTS; ++k) {
       const int sk = __shfl_sync(FULL, slot_s, k);
@@ -239,7 +249,7 @@ __device__ __forceinline__ void sum_masked(const UpdParams& p, const Side& sd, c
         __syncwarp();
         const int s_mine = lane < fill ? scr[lane] : 0;
         const float g_mine = lane < fill ? (line ? line[s_mine] : find_coef(p, sd, rowptr, row, s_mine)) : 0.f;
-        accumulate_list<NCH>(acc, csum, fill, s_mine, g_mine, sd.src, H, H4, lane);
+        accumulate_list<NCH>(acc, csum, fill, s_mine, g_mine, sd.src, H, H4, col);
         fill = 0;
         __syncwarp();
       }
@@ -251,9 +261,15 @@ __device__ __forceinline__ void sum_masked(const UpdParams& p, const Side& sd, c
   if (fill > 0) {
     const int s_mine = lane < fill ? scr[lane] : 0;
     const float g_mine = lane < fill ? (line ? line[s_mine] : find_coef(p, sd, rowptr, row, s_mine)) : 0.f;
-    accumulate_list<NCH>(acc, csum, fill, s_mine, g_mine, sd.src, H, H4, lane);
+    accumulate_list<NCH>(acc, csum, fill, s_mine, g_mine, sd.src, H, H4, col);
   }
   __syncwarp();
+}
+
+__device__ __forceinline__ void clear_mask(const UpdParams& p, const Side& sd, int row, int nwB, int lane) {
+  uint32_t* mrow = sd.mask + (size_t)row * p.Wd;
+  for (int wi = lane; wi < nwB; wi += 32)
+    if (mrow[wi]) mrow[wi] = 0u;
 }
 
 template <int NCH>
@@ -266,6 +282,23 @@ __device__ __forceinline__ void load_row(const float* base, size_t row, int H, i
   }
 }
 
+// Adam on 16 bytes of a row (piece c), and the stores.  UMASK: a row of W1 under a sampled hidden layer; only the units some
+// sample touched the row for are updated (the others keep weight and moments bit for bit); the row's unit mask is cleared
+// by finish_hdr.
+template <bool UMASK>
+__device__ __forceinline__ void adam_piece(const UpdParams& p, const Side& sd, size_t row, int c, float4& w, float4& m, float4& v, const float4& g,
+                                           float4* w4, float4* m4, float4* v4) {
+  unsigned on = 0xfu;
+  if (UMASK && !sd.is_w2) on = (p.cmask1[row * (size_t)p.Hw + ((4 * c) >> 5)] >> ((4 * c) & 31)) & 0xfu;
+  if (!UMASK || (on & 1u)) adam1(w.x, m.x, v.x, g.x, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+  if (!UMASK || (on & 2u)) adam1(w.y, m.y, v.y, g.y, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+  if (!UMASK || (on & 4u)) adam1(w.z, m.z, v.z, g.z, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+  if (!UMASK || (on & 8u)) adam1(w.w, m.w, v.w, g.w, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+  w4[c] = w;
+  __stcs(m4 + c, m);           // the moments are not read again before the next update of this row
+  __stcs(v4 + c, v);
+}
+
 template <int NCH, bool UMASK = false>      // UMASK: rows of W1 carry a mask of the hidden units to update (sampled hidden layer)
 __device__ __forceinline__ void adam_store(const UpdParams& p, const Side& sd, size_t row, float4 (&w)[NCH],
                                            float4 (&m)[NCH], float4 (&v)[NCH], const float4 (&g)[NCH], int H, int H4,
@@ -273,31 +306,64 @@ __device__ __forceinline__ void adam_store(const UpdParams& p, const Side& sd, s
   float4* w4 = reinterpret_cast<float4*>(sd.W + row * H);
   float4* m4 = reinterpret_cast<float4*>(sd.M + row * H);
   float4* v4 = reinterpret_cast<float4*>(sd.V + row * H);
-  // a row of W1 under a sampled hidden layer: only the units some sample touched the row for are updated (the
-  // others keep weight and moments bit for bit); the row's unit mask is cleared by finish_hdr
-  const uint32_t* um = (UMASK && !sd.is_w2) ? p.cmask1 + row * (size_t)p.Hw : nullptr;
 #pragma unroll
   for (int q = 0; q < NCH; ++q) {
-    int c = lane + q * 32;
-    if (c < H4) {
-      if (UMASK) {
-        unsigned on = 0xfu;
-        if (um) on = (um[(4 * c) >> 5] >> ((4 * c) & 31)) & 0xfu;
-        if (on & 1u) adam1(w[q].x, m[q].x, v[q].x, g[q].x, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
-        if (on & 2u) adam1(w[q].y, m[q].y, v[q].y, g[q].y, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
-        if (on & 4u) adam1(w[q].z, m[q].z, v[q].z, g[q].z, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
-        if (on & 8u) adam1(w[q].w, m[q].w, v[q].w, g[q].w, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
-      } else {
-        adam1(w[q].x, m[q].x, v[q].x, g[q].x, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
-        adam1(w[q].y, m[q].y, v[q].y, g[q].y, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
-        adam1(w[q].z, m[q].z, v[q].z, g[q].z, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
-        adam1(w[q].w, m[q].w, v[q].w, g[q].w, p.beta1, p.beta2, p.lr, p.eps, p.rb1, p.rb2);
+    const int c = lane + q * 32;
+    if (c < H4) adam_piece<UMASK>(p, sd, row, c, w[q], m[q], v[q], g[q], w4, m4, v4);
+  }
+}
+
+// Gradient and Adam of a row of more than 256 units whose n <= 32 touches lane k holds as (s_mine, g_mine), in order: the row
+// is walked in pieces of LONG_P x 128 units, so that neither its weights and moments nor its gradient are held whole and
+// sixteen warps fit a multiprocessor.  (Held whole, rows of 1,024 units left eight warps and 492 bytes of spills: a step of
+// 1,024 samples over 50,021 neurons took 759 us, now 613; 512 units 373 and 300; 256 units, two rows held at a time, 181
+// and 175.)  Bound by what L2 hands the multiprocessors: 2.3 GB at 1,024 units, of which 0.8 GB are the samples' rows, in
+// 270 us.  With eight rows of samples in flight instead of four it is slower (638 us), with a row's pieces taken by eight
+// warps at once much slower (980 us).  Returns the sum of the coefficients.
+template <int PIECES, bool UMASK>
+__device__ __forceinline__ float long_row(const UpdParams& p, const Side& sd, size_t row, int n, int s_mine, float g_mine, int H, int H4, int lane) {
+  float4 *w4 = reinterpret_cast<float4*>(sd.W + row * H), *m4 = reinterpret_cast<float4*>(sd.M + row * H), *v4 = reinterpret_cast<float4*>(sd.V + row * H);
+  float csum = 0.f;
+#pragma unroll 1
+  for (int q0 = 0; q0 == 0 || (PIECES > 1 && q0 < H4); q0 += 32 * LONG_P) {
+    float4 w[LONG_P], m[LONG_P], v[LONG_P], acc[LONG_P];
+#pragma unroll
+    for (int u = 0; u < LONG_P; ++u) {
+      const int c = q0 + u * 32 + lane;
+      acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < H4) { w[u] = w4[c]; m[u] = m4[c]; v[u] = v4[c]; }
+    }
+    csum = 0.f;
+#pragma unroll 1
+    for (int k0 = 0; k0 < n; k0 += 4) {
+      float g[4];
+      float4 x[4][LONG_P];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int k = k0 + r < n ? k0 + r : 0;
+        const float4* x4 = reinterpret_cast<const float4*>(sd.src + (size_t)__shfl_sync(FULL, s_mine, k) * H);
+        g[r] = __shfl_sync(FULL, g_mine, k);
+#pragma unroll
+        for (int u = 0; u < LONG_P; ++u) {
+          const int c = q0 + u * 32 + lane;
+          x[r][u] = k0 + r < n && c < H4 ? x4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       }
-      w4[c] = w[q];
-      __stcs(m4 + c, m[q]);      // the moments are not read again before the next update of this row
-      __stcs(v4 + c, v[q]);
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (k0 + r < n) {
+#pragma unroll
+          for (int u = 0; u < LONG_P; ++u) axpy4(acc[u], g[r], x[r][u]);
+          csum += g[r];
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < LONG_P; ++u) {
+      const int c = q0 + u * 32 + lane;
+      if (c < H4) adam_piece<UMASK>(p, sd, row, c, w[u], m[u], v[u], acc[u], w4, m4, v4);
     }
   }
+  return csum;
 }
 
 // A row record as a warp holds it: lane l < 8 has the l-th 8-byte piece -- lane 0 (count, bias), lane 1 (the
@@ -395,65 +461,112 @@ __device__ void aux_block(const UpdParams& p, int a, float* sm_part, unsigned* s
   }
 }
 
-// One slice of a row touched by many samples: the samples of HOT_SLICES-th of the row's mask words.  The slice
-// sum goes to scratch memory; the warp that completes the row's last slice adds the slices in slice
-// order (so the result does not depend on which warp that is), applies Adam and resets the row's state.
-template <int NCH, bool UMASK>
+// A long row whose touches are in its mask but on no list (the hot list was full): the mask is walked once per piece.
+template <int PIECES, bool UMASK>
+__device__ __forceinline__ float long_masked(const UpdParams& p, const Side& sd, int row, int slot_s, int nwB, int* scr, int H, int H4, int lane) {
+  float4 *w4 = reinterpret_cast<float4*>(sd.W + (size_t)row * H), *m4 = reinterpret_cast<float4*>(sd.M + (size_t)row * H),
+         *v4 = reinterpret_cast<float4*>(sd.V + (size_t)row * H);
+  float csum = 0.f;
+#pragma unroll 1
+  for (int q0 = 0; q0 == 0 || (PIECES > 1 && q0 < H4); q0 += 32 * LONG_P) {
+    float4 acc[LONG_P];
+#pragma unroll
+    for (int u = 0; u < LONG_P; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    csum = 0.f;
+    sum_masked<LONG_P, PIECES == 1>(p, sd, p.row_ptr, row, slot_s, 0, nwB, scr, acc, csum, H, H4, lane, q0 + lane);
+#pragma unroll
+    for (int u = 0; u < LONG_P; ++u) {
+      const int c = q0 + u * 32 + lane;
+      if (c < H4) {
+        float4 w = w4[c], m = m4[c], v = v4[c];
+        adam_piece<UMASK>(p, sd, (size_t)row, c, w, m, v, acc[u], w4, m4, v4);
+      }
+    }
+  }
+  if (PIECES > 1) clear_mask(p, sd, row, nwB, lane);
+  return csum;
+}
+
+// One slice of a row touched by many samples: the samples of HOT_SLICES-th of the row's mask words, and of a long row one
+// piece of its units.  The slice sum goes to scratch memory; the warp that completes the row's last one adds the slices in
+// slice order (so the result does not depend on which warp that is), applies Adam and resets the row's state.
+template <int PIECES>
+__device__ __forceinline__ int hot_pieces(int H4) { return PIECES < 2 ? 1 : (H4 + 32 * LONG_P - 1) / (32 * LONG_P); }
+template <int PIECES, bool UMASK>
 __device__ __forceinline__ void hot_item(const UpdParams& p, const int* rowptr, int item, int nwB, int* scr, int H,
                                          int H4, int lane) {
-  const int hrow = item / HOT_SLICES, slice = item - hrow * HOT_SLICES;
+  constexpr int NA = PIECES ? LONG_P : 1;
+  const int per_row = HOT_SLICES * hot_pieces<PIECES>(H4);
+  const int hrow = item / per_row, slice = (item - hrow * per_row) % HOT_SLICES, piece = (item - hrow * per_row) / HOT_SLICES;
   const int code = p.hot_rows[hrow];
   const bool w2 = code >= 0;
   const int row = w2 ? code : ~code;
   const Side sd = make_side(p, w2);
   const int per_w = (nwB + HOT_SLICES - 1) / HOT_SLICES;
   const int w0 = min(nwB, slice * per_w), w1 = min(nwB, w0 + per_w);
-  float4 acc[NCH];
+  const int col = lane + piece * 32 * LONG_P;
+  float4 acc[NA];
 #pragma unroll
-  for (int u = 0; u < NCH; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int u = 0; u < NA; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
   float csum = 0.f;
   const int2 hv = load_hdr(sd.hdr + row, lane);
   // a row of W1 that has been hot before has its coefficients in its line of the table (left there by the forward
   // kernel of this step), indexed by sample: no search
   const int hline = w2 ? -1 : p.hotmap1[row];
-  sum_masked<NCH>(p, sd, rowptr, row, hdr_slots(hv).x, w0, w1, scr, acc, csum, H, H4, lane,
-                  hline >= 0 ? p.hotcoef1 + (size_t)hline * p.bstride : nullptr);
+  sum_masked<NA, PIECES < 2>(p, sd, rowptr, row, hdr_slots(hv).x, w0, w1, scr, acc, csum, H, H4, lane, col,
+                       hline >= 0 ? p.hotcoef1 + (size_t)hline * p.bstride : nullptr);
   const int ld = H + 4;
   float* part = p.hot_part + (size_t)hrow * HOT_SLICES * ld;
   float4* mine = reinterpret_cast<float4*>(part + (size_t)slice * ld);
 #pragma unroll
-  for (int u = 0; u < NCH; ++u) {
-    const int c = lane + u * 32;
+  for (int u = 0; u < NA; ++u) {
+    const int c = col + u * 32;
     if (c < H4) __stcg(mine + c, acc[u]);
   }
-  if (lane == 0) __stcg(part + (size_t)slice * ld + H, csum);
+  if (lane == 0 && piece == 0) __stcg(part + (size_t)slice * ld + H, csum);
   __threadfence();
   __syncwarp();
   int done = 0;
   if (lane == 0) done = atomicAdd(p.hot_done + hrow, 1);
   done = __shfl_sync(FULL, done, 0);
-  if (done != HOT_SLICES - 1) return;
+  if (done != per_row - 1) return;
   __threadfence();
-  float4 w[NCH], m[NCH], v[NCH];
-  load_row<NCH>(sd.W, (size_t)row, H, H4, lane, w);
-  load_row<NCH>(sd.M, (size_t)row, H, H4, lane, m);
-  load_row<NCH>(sd.V, (size_t)row, H, H4, lane, v);
+  float4 *w4 = reinterpret_cast<float4*>(sd.W + (size_t)row * H), *m4 = reinterpret_cast<float4*>(sd.M + (size_t)row * H),
+         *v4 = reinterpret_cast<float4*>(sd.V + (size_t)row * H);
+#pragma unroll 1
+  for (int q0 = lane; q0 == lane || (PIECES > 1 && q0 < H4 + lane); q0 += 32 * NA) {
+    float4 w[NA], m[NA], v[NA];
+    auto load = [&]() {
 #pragma unroll
-  for (int u = 0; u < NCH; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-  csum = 0.f;
-  for (int sl = 0; sl < HOT_SLICES; ++sl) {
-    const float4* src4 = reinterpret_cast<const float4*>(part + (size_t)sl * ld);
+      for (int u = 0; u < NA; ++u) {
+        const int c = q0 + u * 32;
+        if (c < H4) { w[u] = w4[c]; m[u] = m4[c]; v[u] = v4[c]; }
+      }
+    };
+    if (PIECES == 0) load();
 #pragma unroll
-    for (int u = 0; u < NCH; ++u) {
-      const int c = lane + u * 32;
-      if (c < H4) {
-        const float4 x = __ldcg(src4 + c);
-        acc[u].x += x.x; acc[u].y += x.y; acc[u].z += x.z; acc[u].w += x.w;
+    for (int u = 0; u < NA; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int sl = 0; sl < HOT_SLICES; ++sl) {
+      const float4* src4 = reinterpret_cast<const float4*>(part + (size_t)sl * ld);
+#pragma unroll
+      for (int u = 0; u < NA; ++u) {
+        const int c = q0 + u * 32;
+        if (c < H4) {
+          const float4 x = __ldcg(src4 + c);
+          acc[u].x += x.x; acc[u].y += x.y; acc[u].z += x.z; acc[u].w += x.w;
+        }
       }
     }
-    csum += __ldcg(part + (size_t)sl * ld + H);
+    if (PIECES > 0) load();
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int c = q0 + u * 32;
+      if (c < H4) adam_piece<UMASK>(p, sd, (size_t)row, c, w[u], m[u], v[u], acc[u], w4, m4, v4);
+    }
   }
-  adam_store<NCH, UMASK>(p, sd, (size_t)row, w, m, v, acc, H, H4, lane);
+  csum = 0.f;
+  for (int sl = 0; sl < HOT_SLICES; ++sl) csum += __ldcg(part + (size_t)sl * ld + H);
+  if (PIECES > 1) clear_mask(p, sd, row, nwB, lane);      // the pieces' warps have all read it
   finish_hdr(p, sd.hdr + row, w2, hv, csum, lane);
   if (lane == 0) {
     p.hot_done[hrow] = 0;
@@ -467,7 +580,7 @@ __device__ __forceinline__ void hot_item(const UpdParams& p, const int* rowptr, 
 // A row touched by more than ROW_SLOTS samples that the forward kernel listed: one warp sums it from slots and
 // mask (ascending samples), applies Adam and resets the row's state.  Rows that went on to the hot list are
 // summed in slices instead and skipped here.
-template <int NCH, bool UMASK>
+template <int PIECES, bool UMASK>
 __device__ __forceinline__ void medium_item(const UpdParams& p, const int* rowptr, int idx, int nwB, int* scr, int H,
                                             int H4, int lane) {
   const int code = p.med_rows[idx];
@@ -482,12 +595,15 @@ __device__ __forceinline__ void medium_item(const UpdParams& p, const int* rowpt
   // the pairs of touches ROW_SLOTS .. PAIR_T - 1, asked for together with the rows
   int2 pair = sl;
   if (total <= PAIR_T && lane >= ROW_SLOTS && lane < total) pair = sd.ovf[(size_t)row * PAIR_T + lane];
-  float4 w[NCH], m[NCH], v[NCH], acc[NCH];
-  load_row<NCH>(sd.W, (size_t)row, H, H4, lane, w);
-  load_row<NCH>(sd.M, (size_t)row, H, H4, lane, m);
-  load_row<NCH>(sd.V, (size_t)row, H, H4, lane, v);
-#pragma unroll
-  for (int u = 0; u < NCH; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 w[1], m[1], v[1], acc[1];
+  if (PIECES == 0) {
+    load_row<1>(sd.W, (size_t)row, H, H4, lane, w);
+    load_row<1>(sd.M, (size_t)row, H, H4, lane, m);
+    load_row<1>(sd.V, (size_t)row, H, H4, lane, v);
+  } else if (lane == 0) {
+    fetch_row(sd, row, H);
+  }
+  acc[0] = make_float4(0.f, 0.f, 0.f, 0.f);
   float csum = 0.f;
   if (total <= PAIR_T) {
     // every touch has its pair: lane k holds touch k; put them in ascending sample order (each sample touches a
@@ -500,15 +616,15 @@ __device__ __forceinline__ void medium_item(const UpdParams& p, const int* rowpt
     __syncwarp();
     const int s_mine = lane < total ? scr[lane] : 0;
     const float g_mine = lane < total ? __int_as_float(scr[32 + lane]) : 0.f;
-    accumulate_list<NCH>(acc, csum, total, s_mine, g_mine, sd.src, H, H4, lane);
+    if constexpr (PIECES == 0) accumulate_list<1>(acc, csum, total, s_mine, g_mine, sd.src, H, H4, lane);
+    else csum = long_row<PIECES, UMASK>(p, sd, (size_t)row, total, s_mine, g_mine, H, H4, lane);
     __syncwarp();
-    uint32_t* mrow = sd.mask + (size_t)row * p.Wd;
-    for (int wi = lane; wi < nwB; wi += 32)
-      if (mrow[wi]) mrow[wi] = 0u;
+    clear_mask(p, sd, row, nwB, lane);
   } else {
-    sum_masked<NCH>(p, sd, rowptr, row, sl.x, 0, nwB, scr, acc, csum, H, H4, lane);
+    if constexpr (PIECES == 0) sum_masked<1, true>(p, sd, rowptr, row, sl.x, 0, nwB, scr, acc, csum, H, H4, lane, lane);
+    else csum = long_masked<PIECES, UMASK>(p, sd, row, sl.x, nwB, scr, H, H4, lane);
   }
-  adam_store<NCH, UMASK>(p, sd, (size_t)row, w, m, v, acc, H, H4, lane);
+  if constexpr (PIECES == 0) adam_store<1, UMASK>(p, sd, (size_t)row, w, m, v, acc, H, H4, lane);
   finish_hdr(p, sd.hdr + row, w2, hv, csum, lane);
 }
 
@@ -516,8 +632,8 @@ __device__ __forceinline__ void medium_item(const UpdParams& p, const int* rowpt
 // the listed rows with more than ROW_SLOTS touches, then the ordinary rows, UPD_TROWS per ticket (small tickets keep the tail of the kernel short).
 constexpr int UPD_TROWS = 4;
 
-template <int NCH, int G, bool UMASK>
-__global__ void __launch_bounds__(UPD_THREADS, (NCH == 1 ? 2 : (NCH == 2 ? 2 : 1))) k_update(const UpdParams p) {
+template <int PIECES, int G, bool UMASK>
+__global__ void __launch_bounds__(UPD_THREADS, 2) k_update(const UpdParams p) {
   extern __shared__ __align__(16) unsigned char upd_smem[];
   const int* rowptr = p.row_ptr;      // the batch's row offsets (read through the read-only path where needed)
   float* sm_part = reinterpret_cast<float*>(upd_smem);   // [UPD_WARPS * 32]
@@ -538,7 +654,7 @@ __global__ void __launch_bounds__(UPD_THREADS, (NCH == 1 ? 2 : (NCH == 2 ? 2 : 1
   const int nrows = n2 + n1;
   const int nwB = (B + 31) >> 5;
   const unsigned nh_raw = p.st->n_hot[p.parity], nm_raw = p.st->n_med[p.parity];
-  const int n_hot_items = (int)(nh_raw < (unsigned)HOT_CAP ? nh_raw : (unsigned)HOT_CAP) * HOT_SLICES;
+  const int n_hot_items = (int)(nh_raw < (unsigned)HOT_CAP ? nh_raw : (unsigned)HOT_CAP) * HOT_SLICES * hot_pieces<PIECES>(H4);
   const int n_med = (int)(nm_raw < (unsigned)MED_CAP ? nm_raw : (unsigned)MED_CAP);
   // ordinary rows go out UPD_TROWS per ticket, except the last few thousand, which go out G per ticket so that the
   // warps finish close together
@@ -576,23 +692,50 @@ __global__ void __launch_bounds__(UPD_THREADS, (NCH == 1 ? 2 : (NCH == 2 ? 2 : 1
   for (;; cur = nxt, nxt = __shfl_sync(FULL, fut, 0), fut = (lane == 0 && nxt < n_tickets) ? 2 * nwarps + (int)atomicAdd(ticket, 1u) : fut) {
     const int t = cur;
     if (t >= n_tickets) break;
-    if (t < n_hot_items) { hot_item<NCH, UMASK>(p, rowptr, t, nwB, scratch[warp], H, H4, lane); continue; }
-    if (t < n_hot_items + n_med) { medium_item<NCH, UMASK>(p, rowptr, t - n_hot_items, nwB, scratch[warp], H, H4, lane); continue; }
+    if (t < n_hot_items) { hot_item<PIECES, UMASK>(p, rowptr, t, nwB, scratch[warp], H, H4, lane); continue; }
+    if (t < n_hot_items + n_med) { medium_item<PIECES, UMASK>(p, rowptr, t - n_hot_items, nwB, scratch[warp], H, H4, lane); continue; }
 
     // ---- ordinary rows: consecutive entries of the concatenated lists (rows of W2, then rows of W1) ----
     const int trows = t - n_hot_items - n_med < n_big ? UPD_TROWS : G;
     int2 myrow = nrow;                   // (row, the sample that touched it first = the sample of slot 0)
     int myidx = nidx;
-    if (NCH > 1 || nfor != t) entries_of(t, myrow, myidx);
-    if (NCH == 1) {                      // rows of up to 512 bytes; with longer rows the kernel is near the copy bandwidth
-      entries_of(nxt, nrow, nidx);       // and looking ahead only adds load.  Used after this ticket's own loads are issued
-      nfor = nxt;
+    if (nfor != t) entries_of(t, myrow, myidx);
+    entries_of(nxt, nrow, nidx);         // used after this ticket's own loads are issued
+    nfor = nxt;
+    if (PIECES) {                         // one row after the other, the next one asked into L2 meanwhile
+      for (int b = 0; b < trows; ++b) {
+        const int idx = __shfl_sync(FULL, myidx, b), row = __shfl_sync(FULL, myrow.x, b);
+        if (idx >= nrows) break;
+        const Side sd = make_side(p, idx < n2);
+        const int2 hv = load_hdr(sd.hdr + row, lane);
+        if (b + 1 < trows) {
+          if (lane == b + 1 && myidx < nrows) fetch_row(make_side(p, myidx < n2), myrow.x, H);
+        } else if (lane == 0 && nidx < nrows) {
+          fetch_row(make_side(p, nidx < n2), nrow.x, H);
+        }
+        const unsigned cv = (unsigned)__shfl_sync(FULL, hv.x, 0);
+        const int2 sl = hdr_slots(hv);
+        const int n = (int)(cv & CNT_MASK);
+        if ((cv & (CNT_HOT | CNT_MED)) != 0u || n == 0) continue;      // a listed row is summed by its own ticket
+        float csum = 0.f;
+        if (n <= ROW_SLOTS) {
+          int s_mine = sl.x;
+          float g_mine = __int_as_float(sl.y);
+          if (n > 1) sort_slots(sl, n, scratch[warp], s_mine, g_mine, lane);
+          csum = long_row<PIECES, UMASK>(p, sd, (size_t)row, n, s_mine, g_mine, H, H4, lane);
+        } else {                         // more touches than slots, yet not listed (the list was full)
+          csum = long_masked<PIECES, UMASK>(p, sd, row, sl.x, nwB, scratch[warp], H, H4, lane);
+        }
+        finish_hdr(p, sd.hdr + row, idx < n2, hv, csum, lane);
+      }
+      continue;
     }
+    if constexpr (PIECES == 0)
     for (int b0 = 0; b0 < trows; b0 += G) {
       int rr[G], tt[G];
       bool live[G], w2[G], skip[G];
       int2 hv[G], sl[G];
-      float4 w[G][NCH], m[G][NCH], v[G][NCH], x[G][NCH];
+      float4 w[G][1], m[G][1], v[G][1], x[G][1];
 #pragma unroll
       for (int q = 0; q < G; ++q) {
         const int idx = __shfl_sync(FULL, myidx, b0 + q);
@@ -605,20 +748,13 @@ __global__ void __launch_bounds__(UPD_THREADS, (NCH == 1 ? 2 : (NCH == 2 ? 2 : 1
         if (live[q]) {
           const Side sd = make_side(p, w2[q]);
           hv[q] = load_hdr(sd.hdr + rr[q], lane);
-          load_row<NCH>(sd.src, (size_t)s0, H, H4, lane, x[q]);      // the row of slot 0's sample: all a once-touched row needs
-          load_row<NCH>(sd.W, (size_t)rr[q], H, H4, lane, w[q]);
-          load_row<NCH>(sd.M, (size_t)rr[q], H, H4, lane, m[q]);
-          load_row<NCH>(sd.V, (size_t)rr[q], H, H4, lane, v[q]);
+          load_row<1>(sd.src, (size_t)s0, H, H4, lane, x[q]);      // the row of slot 0's sample: all a once-touched row needs
+          load_row<1>(sd.W, (size_t)rr[q], H, H4, lane, w[q]);
+          load_row<1>(sd.M, (size_t)rr[q], H, H4, lane, m[q]);
+          load_row<1>(sd.V, (size_t)rr[q], H, H4, lane, v[q]);
         }
       }
-      if (NCH == 1 && b0 == 0 && nidx < nrows) {
-        const Side sn = make_side(p, nidx < n2);
-        const uint32_t bytes = (uint32_t)H * 4u;
-        l2_fetch(sn.W + (size_t)nrow.x * H, bytes);
-        l2_fetch(sn.M + (size_t)nrow.x * H, bytes);
-        l2_fetch(sn.V + (size_t)nrow.x * H, bytes);
-        l2_fetch(sn.hdr + nrow.x, (uint32_t)sizeof(RowHdr));
-      }
+      if (b0 == 0 && nidx < nrows) fetch_row(make_side(p, nidx < n2), nrow.x, H);
 #pragma unroll
       for (int q = 0; q < G; ++q)
         if (live[q]) {
@@ -632,21 +768,22 @@ __global__ void __launch_bounds__(UPD_THREADS, (NCH == 1 ? 2 : (NCH == 2 ? 2 : 1
       for (int q = 0; q < G; ++q)
         if (live[q] && !skip[q]) {
           const Side sd = make_side(p, w2[q]);
-          float4 acc[NCH];
-#pragma unroll
-          for (int u = 0; u < NCH; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+          float4 acc[1];
+          acc[0] = make_float4(0.f, 0.f, 0.f, 0.f);
           float csum = 0.f;
           if (tt[q] == 1) {
             const float g0 = __int_as_float(__shfl_sync(FULL, sl[q].y, 0));
-#pragma unroll
-            for (int u = 0; u < NCH; ++u) axpy4(acc[u], g0, x[q][u]);
+            axpy4(acc[0], g0, x[q][0]);
             csum = g0;
           } else if (tt[q] <= ROW_SLOTS) {
-            sum_slots<NCH>(sd, sl[q], tt[q], scratch[warp], acc, csum, H, H4, lane);
+            int s_mine;
+            float g_mine;
+            sort_slots(sl[q], tt[q], scratch[warp], s_mine, g_mine, lane);
+            accumulate_list<1>(acc, csum, tt[q], s_mine, g_mine, sd.src, H, H4, lane);
           } else {      // more touches than slots, yet not listed (the list was full)
-            sum_masked<NCH>(p, sd, rowptr, rr[q], sl[q].x, 0, nwB, scratch[warp], acc, csum, H, H4, lane);
+            sum_masked<1, true>(p, sd, rowptr, rr[q], sl[q].x, 0, nwB, scratch[warp], acc, csum, H, H4, lane, lane);
           }
-          adam_store<NCH, UMASK>(p, sd, (size_t)rr[q], w[q], m[q], v[q], acc, H, H4, lane);
+          adam_store<1, UMASK>(p, sd, (size_t)rr[q], w[q], m[q], v[q], acc, H, H4, lane);
           finish_hdr(p, sd.hdr + rr[q], w2[q], hv[q], csum, lane);
         }
     }
@@ -820,25 +957,25 @@ static cudaError_t launch_rows_update(Ctx* c, const UpdParams& p) {
   return launch_dependent(k_rows_update, dim3(nb, q.shares), dim3(RU_THREADS), (size_t)smem, c->stream, p, q);
 }
 
-template <int NCH, int G, bool UMASK>
+template <int PIECES, int G, bool UMASK>
 static cudaError_t launch_k_update(Ctx* c, const UpdParams& p, int smem) {
   cudaError_t e = cudaSuccess;
   if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_update<NCH, G, UMASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = cudaFuncSetAttribute(k_update<PIECES, G, UMASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
   // the kernel needs little shared memory: the rest of the unified store serves as cache for the h / dh rows
-  e = cudaFuncSetAttribute(k_update<NCH, G, UMASK>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
+  e = cudaFuncSetAttribute(k_update<PIECES, G, UMASK>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
   if (e != cudaSuccess) return e;
   // one wave: the blocks for the hidden bias come first, the rest fill the remaining block slots of the device
   const int naux = (c->H + 31) / 32;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update<NCH, G, UMASK>, UPD_THREADS, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update<PIECES, G, UMASK>, UPD_THREADS, smem);
   if (e != cudaSuccess) return e;
   int nblocks = c->num_sms * (per_sm > 0 ? per_sm : 1);
-  if (nblocks < naux + 1) nblocks = naux + 1;
+  nblocks += naux;           // they soon make room for as many more
   LaunchScope ls(c, KID_ADAM);
-  e = launch_dependent(k_update<NCH, G, UMASK>, dim3(nblocks), dim3(UPD_THREADS), (size_t)smem, c->stream, p);
+  e = launch_dependent(k_update<PIECES, G, UMASK>, dim3(nblocks), dim3(UPD_THREADS), (size_t)smem, c->stream, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -877,17 +1014,13 @@ cudaError_t launch_update(Ctx* c, int batch, const int32_t* row_ptr, const int32
     if (e != cudaSuccess) return e;
   }
   const int smem = UPD_WARPS * 32 * 4;
-  const int nch = (c->H / 4 + 31) / 32;
+  const int width = c->H <= 128 ? 0 : c->H <= 128 * LONG_P ? 1 : 2;
   if (c->L1 > 0) {        // sampled hidden layer: rows of W1 are updated under their unit masks
-    if (nch <= 1) return launch_k_update<1, 2, true>(c, p, smem);
-    if (nch <= 2) return launch_k_update<2, 2, true>(c, p, smem);
-    if (nch <= 4) return launch_k_update<4, 1, true>(c, p, smem);
-    return launch_k_update<8, 1, true>(c, p, smem);
+    if (width == 0) return launch_k_update<0, 2, true>(c, p, smem);
+    return width == 1 ? launch_k_update<1, UPD_TROWS, true>(c, p, smem) : launch_k_update<2, UPD_TROWS, true>(c, p, smem);
   }
-  if (nch <= 1) return launch_k_update<1, 2, false>(c, p, smem);
-  if (nch <= 2) return launch_k_update<2, 2, false>(c, p, smem);
-  if (nch <= 4) return launch_k_update<4, 1, false>(c, p, smem);
-  return launch_k_update<8, 1, false>(c, p, smem);
+  if (width == 0) return launch_k_update<0, 2, false>(c, p, smem);
+  return width == 1 ? launch_k_update<1, UPD_TROWS, false>(c, p, smem) : launch_k_update<2, UPD_TROWS, false>(c, p, smem);
 }
 
 }  // namespace dslide

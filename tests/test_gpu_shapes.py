@@ -119,6 +119,29 @@ def test_more_hot_rows_than_the_hot_list_holds():
         pr.close()
 
 
+@pytest.mark.parametrize("H,D", [
+    (132, 300),      # one piece of 256 units, three quarters of its lanes idle; rows touched by about 30 of the batch's samples
+    (256, 90),       # one whole piece; every row touched by most samples: slices of hot rows
+    (260, 300),      # a second piece of one lane
+    (516, 1400),     # three pieces, 1,400 hot rows against a list of 1,024: the rest walk their masks piece by piece
+    (1024, 90),      # four pieces, hot
+    (1024, 2500),    # four pieces, rows of a few touches and listed ones
+])
+def test_long_rows_by_touches(H, D):
+    """Rows of more than 128 units are updated piece by piece: once touched, from slots, listed, hot and unlisted."""
+    pr = Pair(D=D, H=H, N=2003, family=SIMHASH, K=6, L=6, bucket_cap=12, max_batch=150, max_labels=16, lr=1e-3, seed=6)
+    rng = np.random.default_rng(H + D)
+    try:
+        for i in range(2):
+            batch = dense_features_batch(rng, 150, D, 2003, {90: 75, 300: 60, 1400: 420, 2500: 120}[D], 3)
+            lo = pr.o.train_step(*batch)
+            lg = pr.gpu_step(batch)
+            assert abs(lo - lg) <= (ACT_TOL if i == 0 else W_TOL) * abs(lo)
+            compare_weights(pr)
+    finally:
+        pr.close()
+
+
 def test_more_listed_rows_than_the_list_holds():
     """One table with two buckets and no cap: every sample retrieves about half of 140,000 neurons, so with 16
     samples some 70,000 rows of W2 are touched by more samples than a row has slots -- more than the list of such
