@@ -270,14 +270,13 @@ constexpr int HN_WARPS = HN_THREADS / 32;
 constexpr int HN_FN_SMEM_MAX = 96 * 1024;    // hash-function tables larger than this stay in global memory
 
 // A block stages HN_ROWS rows of W2 in shared memory (padded, so that 32 threads reading the same
-// column of 32 different rows hit 32 banks) and evaluates the L codes of each row: lane = row, the
-// warps share out the tables.  The hash functions sit in shared memory too, 16 bits per coordinate
-// (the top bit carries a negative SimHash sign), read as warp-wide broadcasts.
+// column of 32 different rows hit 32 banks) and evaluates the L DWTA codes of each row: lane = row, the
+// warps share out the tables.  The hash functions sit in shared memory too, 16 bits per coordinate,
+// read as warp-wide broadcasts.
 // keys[t][j] = code of neuron j in table t.
 template <bool FN_SMEM>
 __global__ void __launch_bounds__(HN_THREADS)
-k_hash_neurons(const float* __restrict__ W2, const int32_t* __restrict__ hidx, const int32_t* __restrict__ hsign,
-               uint32_t* keys, int N, int H, int K, int L, int family, int lg_bin, int fn_len) {
+k_hash_neurons(const float* __restrict__ W2, const int32_t* __restrict__ hidx, uint32_t* keys, int N, int H, int K, int L, int lg_bin, int fn_len) {
   extern __shared__ __align__(16) unsigned char hn_smem[];
   float* tile = reinterpret_cast<float*>(hn_smem);                    // [HN_ROWS][H + 1]
   const int ld = H + 1;
@@ -285,11 +284,7 @@ k_hash_neurons(const float* __restrict__ W2, const int32_t* __restrict__ hidx, c
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nfn = K * L * fn_len;
   if (FN_SMEM) {
-    for (int e = threadIdx.x; e < nfn; e += HN_THREADS) {
-      unsigned v = (unsigned)hidx[e];
-      if (family == DSLIDE_SIMHASH && hsign[e] < 0) v |= 0x8000u;
-      fn[e] = (unsigned short)v;
-    }
+    for (int e = threadIdx.x; e < nfn; e += HN_THREADS) fn[e] = (unsigned short)hidx[e];
   }
   const int ntiles = (N + HN_ROWS - 1) / HN_ROWS;
   for (int tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
@@ -314,60 +309,127 @@ k_hash_neurons(const float* __restrict__ W2, const int32_t* __restrict__ hidx, c
 #pragma unroll 2
         for (int k = 0; k < K; ++k) {
           const int f = t * K + k;
-          if (family == DSLIDE_SIMHASH) {
-            float sum = 0.f;
-            if (FN_SMEM) {
-              const unsigned short* ix = fn + (size_t)f * fn_len;
-              for (int i = 0; i < fn_len; ++i) {
-                const unsigned e = ix[i];
-                const float x = v[e & 0x7fffu];
-                sum = __fadd_rn(sum, (e & 0x8000u) ? -x : x);
-              }
-            } else {
-              const int32_t* ix = hidx + (size_t)f * fn_len;
-              const int32_t* sg = hsign + (size_t)f * fn_len;
-              for (int i = 0; i < fn_len; ++i) {
-                const float x = v[__ldg(ix + i)];
-                sum = __fadd_rn(sum, __ldg(sg + i) > 0 ? x : -x);
-              }
+          int best = 0;
+          float bv;
+          if (FN_SMEM && fn_len == 8) {
+            // bin of eight: the eight coordinates come in one 16-byte broadcast load
+            const uint4 q = *reinterpret_cast<const uint4*>(fn + (size_t)f * 8);
+            const float x0 = v[q.x & 0xffffu], x1 = v[q.x >> 16], x2 = v[q.y & 0xffffu], x3 = v[q.y >> 16];
+            const float x4 = v[q.z & 0xffffu], x5 = v[q.z >> 16], x6 = v[q.w & 0xffffu], x7 = v[q.w >> 16];
+            bv = x0;
+            if (x1 > bv) { bv = x1; best = 1; }
+            if (x2 > bv) { bv = x2; best = 2; }
+            if (x3 > bv) { bv = x3; best = 3; }
+            if (x4 > bv) { bv = x4; best = 4; }
+            if (x5 > bv) { bv = x5; best = 5; }
+            if (x6 > bv) { bv = x6; best = 6; }
+            if (x7 > bv) { bv = x7; best = 7; }
+          } else if (FN_SMEM) {
+            const unsigned short* ix = fn + (size_t)f * fn_len;
+            bv = v[ix[0]];
+            for (int i = 1; i < fn_len; ++i) {
+              const float x = v[ix[i]];
+              if (x > bv) { bv = x; best = i; }
             }
-            code |= (sum >= 0.f ? 1u : 0u) << k;
           } else {
-            int best = 0;
-            float bv;
-            if (FN_SMEM && fn_len == 8) {
-              // bin of eight: the eight coordinates come in one 16-byte broadcast load
-              const uint4 q = *reinterpret_cast<const uint4*>(fn + (size_t)f * 8);
-              const float x0 = v[q.x & 0xffffu], x1 = v[q.x >> 16], x2 = v[q.y & 0xffffu], x3 = v[q.y >> 16];
-              const float x4 = v[q.z & 0xffffu], x5 = v[q.z >> 16], x6 = v[q.w & 0xffffu], x7 = v[q.w >> 16];
-              bv = x0;
-              if (x1 > bv) { bv = x1; best = 1; }
-              if (x2 > bv) { bv = x2; best = 2; }
-              if (x3 > bv) { bv = x3; best = 3; }
-              if (x4 > bv) { bv = x4; best = 4; }
-              if (x5 > bv) { bv = x5; best = 5; }
-              if (x6 > bv) { bv = x6; best = 6; }
-              if (x7 > bv) { bv = x7; best = 7; }
-            } else if (FN_SMEM) {
-              const unsigned short* ix = fn + (size_t)f * fn_len;
-              bv = v[ix[0]];
-              for (int i = 1; i < fn_len; ++i) {
-                const float x = v[ix[i]];
-                if (x > bv) { bv = x; best = i; }
-              }
-            } else {
-              const int32_t* ix = hidx + (size_t)f * fn_len;
-              bv = v[__ldg(ix)];
-              for (int i = 1; i < fn_len; ++i) {
-                const float x = v[__ldg(ix + i)];
-                if (x > bv) { bv = x; best = i; }
-              }
+            const int32_t* ix = hidx + (size_t)f * fn_len;
+            bv = v[__ldg(ix)];
+            for (int i = 1; i < fn_len; ++i) {
+              const float x = v[__ldg(ix + i)];
+              if (x > bv) { bv = x; best = i; }
             }
-            code |= (uint32_t)best << (k * lg_bin);
           }
+          code |= (uint32_t)best << (k * lg_bin);
         }
         keys[(size_t)t * N + j0 + lane] = code;
       }
+    }
+  }
+}
+
+// SimHash: R rows per lane (rows lane, lane + 32, ... of a tile of 32 R), interleaved per coordinate, so that one load of
+// 4 R bytes fetches a coordinate of all of them, and its address and sign are worked out once for them.  A projection's sum
+// is the sequential one of the definition: a fused multiply-add by plus or minus one per coordinate, two rows per
+// instruction.  The tables' functions sit in shared memory, 16 bits per coordinate (top bit: minus), filled up to whole
+// 16-byte words with a coordinate that is zero; blocks of another y take other tables, as many at a time as find room.
+// Bound by the loads from shared memory (4 bytes per row, function and coordinate: 30 GB at 253,855 rows of 200 units and 450
+// functions).  With one row per lane, as before, the instructions around the loads bound it: a rebuild of those rows took
+// 2,814 us and now takes 1,506; 128 units 1,818 and 968; 20,011 rows of 1,024 units 6,757 and 3,839 (one row per lane
+// here too, but 32 warps for one tile instead of eight).
+constexpr int HNS_SMEM = 224 * 1024;
+constexpr int HNS_MIN_TABLES = 8;          // more rows per lane only while the functions of so many tables fit beside the tile
+template <int R>
+__global__ void __launch_bounds__(1024)
+k_hash_neurons_sim(const float* __restrict__ W2, const int32_t* __restrict__ hidx, const int32_t* __restrict__ hsign, uint32_t* keys, int N, int H, int K,
+                   int L, int m, int per) {
+  constexpr int ROWS = 32 * R, ES = 4 * R;
+  extern __shared__ __align__(16) unsigned char hn_smem[];
+  const int ld = H + 1;                                               // odd: a warp's loads of one coordinate spread over the banks
+  const int mp = (m + 7) & ~7;
+  unsigned short* fn = reinterpret_cast<unsigned short*>(hn_smem + (((size_t)32 * ld * ES + 15) & ~(size_t)15));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int t0 = blockIdx.y * per, nt = min(L - t0, per);
+  for (int e = threadIdx.x; e < nt * K * mp; e += blockDim.x) {
+    const int f = e / mp, i = e - f * mp;
+    const size_t at = (size_t)(t0 * K + f) * m + i;
+    fn[e] = i < m ? (unsigned short)(hidx[at] | (hsign[at] > 0 ? 0 : 0x8000)) : (unsigned short)H;
+  }
+  if (threadIdx.x < 32)
+    for (int u = 0; u < R; ++u) reinterpret_cast<float*>(hn_smem)[(threadIdx.x * ld + H) * R + u] = 0.f;
+  const unsigned char* v = hn_smem + (size_t)lane * ld * ES;
+  const int ntiles = (N + ROWS - 1) / ROWS;
+  for (int tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
+    const int j0 = tl * ROWS;
+    const int rows = min(ROWS, N - j0);
+    __syncthreads();
+    // a thread takes one coordinate of one lane's rows: reads run along a row, one vector store places them
+    for (int g = warp; g < 32; g += nwarps)
+      for (int k = lane; k < H; k += 32) {
+        float x[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) x[u] = g + 32 * u < rows ? __ldg(W2 + (size_t)(j0 + g + 32 * u) * H + k) : 0.f;
+        float* to = reinterpret_cast<float*>(hn_smem) + ((size_t)g * ld + k) * R;
+        if (R == 4) *reinterpret_cast<float4*>(to) = make_float4(x[0], x[1 % R], x[2 % R], x[3 % R]);
+        else if (R == 2) *reinterpret_cast<float2*>(to) = make_float2(x[0], x[1 % R]);
+        else *to = x[0];
+      }
+    __syncthreads();
+    for (int t = warp; t < nt; t += nwarps) {
+      uint32_t code[R];
+#pragma unroll
+      for (int u = 0; u < R; ++u) code[u] = 0u;
+      for (int k = 0; k < K; ++k) {
+        const uint4* q4 = reinterpret_cast<const uint4*>(fn + (size_t)(t * K + k) * mp);
+        unsigned long long s0 = 0ull, s1 = 0ull;
+        float s = 0.f;
+        for (int i0 = 0; i0 < mp / 8; ++i0) {
+          const uint4 q = q4[i0];
+          const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const uint32_t e = i & 1 ? w[i >> 1] >> 16 : w[i >> 1];
+            const uint32_t sg = ((i & 1 ? w[i >> 1] : w[i >> 1] << 16) & 0x80000000u) | 0x3f800000u;
+            const unsigned char* at = v + (e & 0x7fffu) * ES;
+            const unsigned long long pm = ((unsigned long long)sg << 32) | sg;
+            if (R == 4) {
+              const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(at);
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s0) : "l"(x.x), "l"(pm));
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s1) : "l"(x.y), "l"(pm));
+            } else if (R == 2) {
+              asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s0) : "l"(*reinterpret_cast<const unsigned long long*>(at)), "l"(pm));
+            } else {
+              s = fmaf(*reinterpret_cast<const float*>(at), __uint_as_float(sg), s);
+            }
+          }
+        }
+        const float sum[4] = {R == 1 ? s : __uint_as_float((unsigned)s0), __uint_as_float((unsigned)(s0 >> 32)), __uint_as_float((unsigned)s1),
+                              __uint_as_float((unsigned)(s1 >> 32))};
+#pragma unroll
+        for (int u = 0; u < R; ++u) code[u] |= (sum[u] >= 0.f ? 1u : 0u) << k;
+      }
+#pragma unroll
+      for (int u = 0; u < R; ++u)
+        if (lane + 32 * u < rows) keys[(size_t)(t0 + t) * N + j0 + 32 * u + lane] = code[u];
     }
   }
 }
@@ -1137,6 +1199,34 @@ static cudaError_t launch_dwta8(Ctx* c, int smem) {
   return cudaGetLastError();
 }
 
+template <int R>
+static cudaError_t launch_sim(Ctx* c, int tile_bytes, int table_bytes) {
+  // as many tables at a time as find room; more shares than that where there are few tiles
+  const int ntiles = (c->N + 32 * R - 1) / (32 * R);
+  int per = (HNS_SMEM - tile_bytes) / table_bytes;
+  if (per > c->L) per = c->L;
+  int shares = (c->L + per - 1) / per;
+  if (ntiles * shares < 2 * c->num_sms) shares = (2 * c->num_sms + ntiles - 1) / ntiles;
+  if (shares > c->L) shares = c->L;
+  per = (c->L + shares - 1) / shares;
+  shares = (c->L + per - 1) / per;
+  int warps = 8;                              // the rounds that the tables take decide, then the warps' number
+  for (int w = 9; w <= 32; ++w)
+    if ((per + w - 1) / w * w <= (per + warps - 1) / warps * warps) warps = w;
+  const int smem = tile_bytes + per * table_bytes;
+  cudaError_t e = cudaFuncSetAttribute(k_hash_neurons_sim<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hash_neurons_sim<R>, 32 * warps, smem);
+  if (e != cudaSuccess) return e;
+  int nb = c->num_sms * (per_sm > 0 ? per_sm : 1) / shares;
+  if (nb < 1) nb = 1;
+  if (nb > ntiles) nb = ntiles;
+  LaunchScope ls(c, KID_HASH_NEURONS);
+  k_hash_neurons_sim<R><<<dim3(nb, shares), 32 * warps, smem, c->stream>>>(c->W2, c->hash_idx, c->hash_sign, c->keysA, c->N, c->H, c->K, c->L, c->fn_len, per);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_build_tables(Ctx* c) {
   const size_t off_bytes = (size_t)c->L * (size_t)(c->nb + 1) * sizeof(int32_t);
   int low = 0, up = 0, id_bits = 0;
@@ -1161,7 +1251,14 @@ cudaError_t launch_build_tables(Ctx* c) {
   // 760 units 211 / 135, 223 / 149, 316 / 233; at 392 units (two blocks) 99, 111, 193 against 117, 132, 230 by the kernel
   // before, which the general one equals.
   const long long smem4 = ((32LL * (c->H + 1) * 16 + 15) & ~15LL) + 2 * fn_bytes, smem2 = ((32LL * (c->H + 1) * 8 + 15) & ~15LL) + 2 * fn_bytes;
-  if (fn_smem && c->cfg.hash_family == DSLIDE_DWTA && c->fn_len == 8 && smem2 <= 112 * 1024) {
+  if (c->cfg.hash_family == DSLIDE_SIMHASH) {
+    const int table = c->K * ((c->fn_len + 7) & ~7) * 2;
+    auto tile = [&](int r) { return (32 * (c->H + 1) * 4 * r + 15) & ~15; };
+    if (tile(4) + HNS_MIN_TABLES * table <= HNS_SMEM) e = launch_sim<4>(c, tile(4), table);
+    else if (tile(2) + HNS_MIN_TABLES * table <= HNS_SMEM) e = launch_sim<2>(c, tile(2), table);
+    else e = launch_sim<1>(c, tile(1), table);
+    if (e != cudaSuccess) return e;
+  } else if (fn_smem && c->fn_len == 8 && smem2 <= 112 * 1024) {
     e = smem4 <= 112 * 1024 ? launch_dwta8<2>(c, (int)smem4) : launch_dwta8<1>(c, (int)smem2);
     if (e != cudaSuccess) return e;
   } else {
@@ -1175,8 +1272,7 @@ cudaError_t launch_build_tables(Ctx* c) {
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     LaunchScope ls(c, KID_HASH_NEURONS);
-    kern<<<c->num_sms * per_sm, HN_THREADS, smem, c->stream>>>(c->W2, c->hash_idx, c->hash_sign, c->keysA, c->N, c->H, c->K, c->L,
-                                                             c->cfg.hash_family, c->lg_bin, c->fn_len);
+    kern<<<c->num_sms * per_sm, HN_THREADS, smem, c->stream>>>(c->W2, c->hash_idx, c->keysA, c->N, c->H, c->K, c->L, c->lg_bin, c->fn_len);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (parts) {

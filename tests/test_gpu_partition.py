@@ -32,6 +32,26 @@ def test_tables(family, K, L, N, H, cap):
         pr.close()
 
 
+@pytest.mark.parametrize("K,L,N,H", [
+    (7, 70, 20011, 128),     # four rows per lane, all tables at a time
+    (12, 60, 1601, 400),     # four rows per lane, the functions of some tables beside them
+    (6, 33, 129, 440),       # two rows per lane, a last tile of one row
+    (9, 40, 801, 856),       # one or two rows per lane, few tables at a time
+    (5, 30, 333, 1024),      # one row per lane
+    (8, 1, 31, 100),         # one table, less than a tile
+])
+def test_simhash_tables_at_every_width(K, L, N, H):
+    pr = Pair(D=40, H=H, N=N, family=SIMHASH, K=K, L=L, bucket_cap=16, max_batch=4, seed=K + N)
+    try:
+        same_tables(pr)
+        ds.dslide_rebuild_tables(pr.ctx)
+        ds.dslide_sync(pr.ctx)
+        pr.o.rebuild_tables()
+        same_tables(pr)
+    finally:
+        pr.close()
+
+
 @pytest.mark.parametrize("K,N", [(4, 9001), (6, 30011)])
 def test_crowded_parts_and_bins_that_tie(K, N):
     """Rows with few distinct values, zeros of both signs, infinities, values beyond 2^87 and smaller than any normal
