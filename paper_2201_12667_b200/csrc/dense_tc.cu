@@ -3,7 +3,7 @@
 // The logits of a batch against every output neuron are one contraction, Z[B][N] = h[B][H] . W2[N][H]^T + b2
 // (Section 3.6: "layer sparsity is 1"), so this path runs it on the fifth-generation tensor cores: tiles of W2
 // arrive in shared memory by TMA (cp.async.bulk.tensor, 128-byte swizzle), the 128 samples' hidden activations of a
-// block sit in tensor memory beside the accumulators, a single thread issues tcgen05.mma (kind::tf32), and the
+// block sit in tensor memory beside the accumulators, a single thread of one or two blocks issues tcgen05.mma (kind::tf32), and the
 // read-back warps fetch the accumulators (tcgen05.ld) and keep, per sample, the candidates of the block's slice of
 // neurons; one more warp takes the largest row norm of W2 from the tiles while they are in shared memory.  W2 is
 // streamed once per 128 samples (the groups of samples walk the same tiles together, so HBM sees it once per call).
@@ -27,7 +27,7 @@ namespace dslide {
 constexpr int TC_M = 128;          // samples per block = lanes of the accumulator
 constexpr int TC_N = 128;          // neurons per tile = columns of the accumulator
 constexpr int TC_KB = 32;          // hidden units per 128-byte swizzled row
-constexpr int TC_STAGES = 3;       // tiles of W2 in flight at most (as many as fit in shared memory)
+constexpr int TC_STAGES = 6;       // tiles of W2 in flight at most (as many as fit in shared memory)
 constexpr int TC_NACC = 3;         // tensor memory: up to three accumulators of TC_N columns (two when H > TC_N), then the activations (H columns)
 constexpr int TC_TMEM_COLS = 512;
 constexpr int TC_SPLIT = 4;        // read-back warps per quarter of tensor memory (each takes 1 / TC_SPLIT of a tile's columns)
@@ -36,7 +36,8 @@ constexpr int TC_THREADS = 96 + TC_EPI;                // warp 0: TMA producer; 
 constexpr int TC_EXTRA = 8;        // candidates kept beyond k: TC_EXTRA + k (the wider the margin, the rarer the exact fall-back)
 constexpr int TC_H_TMEM = 256;     // hidden layers up to this width sit in tensor memory beside two accumulators; wider ones are
                                    // streamed through shared memory with the tiles (WIDE)
-constexpr int TC_WIDE_STAGES = 6;  // WIDE: pairs of slabs (32 units of the samples, 32 units of the neurons) in flight
+constexpr int TC_H_SINGLE = 192;   // up to this width two tiles fit a block's shared memory
+constexpr int TC_WIDE_STAGES = TC_STAGES;      // WIDE: pairs of slabs (32 units of the samples, 32 units of the neurons) in flight
 constexpr int TC_RANK_CAP = 24;    // the threshold's rank in the subset grows with k up to this
 constexpr int TC_GBUF_MIN = 64;    // candidate slots per (buffer, sample) at least, many times the expected fill: a buffer takes the 32 neighbouring
                                    // neurons of its tiles, which a trained model may favour together; one that runs over sends the sample to the exact scan
@@ -44,6 +45,11 @@ constexpr int TC_TARGET = 64;      // candidates aimed at per sample: TC_TARGET 
 constexpr int TC_SUBSET = 64;      // the threshold pass scores every TC_SUBSET-th tile
 constexpr int TC_SUB_BYTES = TC_M * 128;               // one 32-unit slab of 128 rows
 constexpr float TC_ERR = 2.2e-3f;  // |approximate - exact| <= TC_ERR * |h| * |w|: two operands cut to 10 mantissa bits, fp32 sums
+
+constexpr int TC_BT = 8;           // tiles whose biases are in shared memory or on their way there
+constexpr int TC_BAHEAD = 6;       // tiles ahead that they are asked for: a tile takes less than a read from HBM under load
+// Neurons of a tile: 256 where the activations do not stand beside the accumulators in tensor memory and two blocks share a tile
+__host__ __device__ constexpr int tc_cols(bool wide, bool pair) { return wide && pair ? 2 * TC_N : TC_N; }
 
 struct TcParams {
   const RowHdr* hdr2;
@@ -79,12 +85,32 @@ __device__ __forceinline__ void tc_bar_wait(uint64_t* bar, uint32_t parity, vola
   const uint32_t a = tc_smem(bar);
   for (int it = 0; it < (1 << 20); ++it) {
     uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(a), "r"(parity), "r"(2000u) : "memory");      // may sleep up to 2 us per try: a waiting warp issues little
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(a), "r"(parity) : "memory");
     if (ok) return;
     if ((it & 1023) == 1023 && *abort) return;
   }
   *abort = 1;
+}
+// The address, in the cluster's shared memory, of a barrier of the block of rank `rank`; an arrival there.  Arrivals and waits
+// order what the block itself needs (default scope): the operands and accumulators are ordered by the copies' and the tensor
+// unit's own completion and by tcgen05.fence.  With release and acquire at cluster scope every one of them cost about 1,000 cycles.
+__device__ __forceinline__ uint32_t tc_at_rank(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(tc_smem(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void tc_bar_arrive_at(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_cluster_sync() {
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// Into this block's shared memory, counted by a barrier of either block of the pair
+__device__ __forceinline__ void tc_tma_2d_pair(void* dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3}], [%4];"
+               ::"r"(tc_smem(dst)), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void tc_tma_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -104,15 +130,22 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
 __host__ __device__ constexpr uint32_t tc_idesc(int M, int N) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// D[tmem] (+)= A[tmem] . B[smem]^T: the first operand is read from tensor memory, so shared memory serves one operand only
+// D[tmem] (+)= A[tmem] . B[smem]^T: the first operand is read from tensor memory, so shared memory serves one operand only.
+// A pair's instruction takes the accumulators and first operands of both blocks and half of the second operand from each.
+template <bool PAIR>
 __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
-               ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+  if (PAIR) asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
+                      ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+  else asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
+                      ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
 // The same with both operands in shared memory (hidden layers too wide for tensor memory)
+template <bool PAIR>
 __device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-               ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+  if (PAIR) asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+                      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+  else asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+                      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
@@ -124,8 +157,14 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32])
         "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
+// Arrives on the barrier -- of both blocks of a pair -- once the instructions issued before have completed
+template <bool PAIR>
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem(bar)) : "memory");
+  if (PAIR)
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(tc_smem(bar)), "h"((uint16_t)3) : "memory");
+  else
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem(bar)) : "memory");
 }
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -149,9 +188,14 @@ __device__ __forceinline__ bool tc_better(float za, int ia, float zb, int ib) { 
 // A hidden width that is no multiple of 32 ends in a slab whose missing units the tensor copy fills with zeros.
 // WIDE (H > TC_H_TMEM): the activations do not fit tensor memory, so a stage is one slab of the tile and the same 32
 // units of the block's samples, both by tensor copies; the samples' slabs come from L2 once per tile, which doubles
-// the copies of a tile but keeps the multiplications on the tensor pipe (1,024 units, 50,021 neurons, 1,024 samples, k 5:
-// 389 us, the scan on the ALUs 43,700; 512 units, 100,003 neurons, 512 samples, k 64: 240 and 31,800).
-template <bool DUMP, bool WIDE>      // DUMP: write every score out (threshold pass); else append the scores that reach the sample's threshold
+// the copies of a tile but keeps the multiplications on the tensor pipe.
+// PAIR: two multiprocessors (a cluster of two blocks) share a tile, half of its rows in the shared memory of each, and take
+// 128 samples each; the first block issues instructions of 256 samples for both (use_pairs says when).  WIDE tiles are
+// then 256 neurons, so that the samples' slabs serve twice as many.
+// What a tile took besides the multiplications, 2,000 cycles at 128 units: its biases asked for only one tile ahead (an HBM
+// latency per tile), and in WIDE the one warp that sums the rows' squares, element by element (26,000 cycles per tile at 512 units,
+// with packed pairs of four rows side by side 16,000; 512 samples x 100,003 neurons x 512 units 206 us before, 138 now with pairs).
+template <bool DUMP, bool WIDE, bool PAIR>      // DUMP: write every score out (threshold pass); else append the scores that reach the sample's threshold
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH, const TcParams p) {
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
@@ -159,45 +203,57 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   const int ksub = (p.H + TC_KB - 1) / TC_KB;
   const int kfull = p.H / TC_KB;
   const int klast = (p.H - (ksub - 1) * TC_KB + 7) >> 3;      // instructions (eight units each) of the last slab
-  const uint32_t tile_bytes = WIDE ? 2u * TC_SUB_BYTES : (uint32_t)ksub * TC_SUB_BYTES;      // of a stage
+  constexpr int NT = tc_cols(WIDE, PAIR);                      // neurons of a tile
+  constexpr int ROWS = PAIR ? NT / 2 : NT;                     // of which this block holds so many rows
+  constexpr uint32_t SLAB = ROWS * 128;                        // 32 units of them
+  const uint32_t tile_bytes = WIDE ? SLAB + TC_SUB_BYTES : (uint32_t)ksub * SLAB;      // of a stage
   unsigned char* smB = sm;
   const int nst = p.stages;
-  float* sb = reinterpret_cast<float*>(smB + (size_t)nst * tile_bytes);                         // [accumulator][128] biases of its tile
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sb + TC_NACC * TC_N);
+  float* sb = reinterpret_cast<float*>(smB + (size_t)nst * tile_bytes);                         // [TC_BT][NT] biases of the tiles
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sb + TC_BT * NT);
   uint64_t* bar_a = bars;                      // activations are in tensor memory
   constexpr int NST = WIDE ? TC_WIDE_STAGES : TC_STAGES;
   uint64_t* bar_full = bars + 1;               // [NST] the stage has arrived
   uint64_t* bar_empty = bars + 1 + NST;        // [NST] the stage has been consumed
   uint64_t* bar_accfull = bars + 1 + 2 * NST;              // [TC_NACC] accumulator written
   uint64_t* bar_accempty = bars + 1 + 2 * NST + TC_NACC;   // [TC_NACC] accumulator read back
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 1 + 2 * NST + 2 * TC_NACC);
+  uint64_t* bar_landed = bars + 1 + 2 * NST + 2 * TC_NACC; // [NST] second block of a pair: the stage has arrived (the pair's bytes are counted in the first)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 1 + 3 * NST + 2 * TC_NACC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int slice = blockIdx.x, s0 = blockIdx.y * TC_M;
+  const uint32_t rank = PAIR ? blockIdx.x & 1u : 0u;       // in the pair: the first block counts arrivals and issues the multiplications
+  const int slice = PAIR ? blockIdx.x >> 1 : blockIdx.x, s0 = PAIR ? (2 * (int)blockIdx.y + (int)rank) * TC_M : (int)blockIdx.y * TC_M;
   // tiles of this slice: slice, slice + nslices, ... (both sample groups walk the same tiles at the same time: the
   // second read of a tile is served by L2)
   const int my_tiles = slice < p.ntiles ? (p.ntiles - slice + p.nslices - 1) / p.nslices : 0;
   // The filter launch also takes the largest squared row norm of W2 (the error bound needs it) from the tiles as
   // they pass through shared memory; up to four sample groups share a tile's rows (they all see the same tiles).
-  const int nshare = gridDim.y >= 4 ? 4 : (gridDim.y >= 2 ? 2 : 1);      // blocks that share a tile's 128 rows
+  constexpr int RL = ROWS / 32;                                    // rows per lane, shared by the blocks that hold the same rows
+  const int nshare = (int)gridDim.y >= 4 && RL >= 4 ? 4 : ((int)gridDim.y >= 2 ? 2 : 1);
   const bool norms = !DUMP && (int)blockIdx.y < nshare;
-  const int nacc = WIDE || p.H <= TC_N ? TC_NACC : 2;      // accumulators in use; the activations follow them
-  const uint32_t acol = (uint32_t)(nacc * TC_N);
+  const int nacc = WIDE ? (PAIR ? 2 : TC_NACC) : (p.H <= TC_N ? TC_NACC : 2);      // accumulators in use; the activations follow them
+  const uint32_t acol = (uint32_t)(nacc * NT);
 
   if (tid == 0) {
-    tc_bar_init(bar_a, 128);
-    for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
-    for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, TC_EPI); }
+    tc_bar_init(bar_a, PAIR ? 8 : 4);            // a warp each
+    for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_landed + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
+    for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, (PAIR ? 2 : 1) * TC_EPI / 32); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {      // tensor memory: all of it (one block per SM)
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(tmem_slot)), "r"(TC_TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(tmem_slot)), "r"(TC_TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(tmem_slot)), "r"(TC_TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
+  if (PAIR) tc_cluster_sync();       // the other block's barriers are ready
+  else __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();       // the next kernel of the call may be placed as blocks of this one leave
@@ -208,29 +264,40 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     if (lane == 0) {
       int st = 0, stround = 0;
       for (int i = 0; i < my_tiles; ++i) {
-        const int row0 = (slice + i * p.nslices) * p.tile_stride * TC_N;
+        const int row0 = (slice + i * p.nslices) * p.tile_stride * NT + (int)rank * ROWS;
         if (WIDE) {
           for (int ks = 0; ks < ksub; ++ks) {
             if (stround > 0) tc_bar_wait(bar_empty + st, (stround - 1) & 1, abort_flag);
             unsigned char* to = smB + (size_t)st * tile_bytes;
-            tc_bar_expect(bar_full + st, tile_bytes);
-            tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
-            tc_tma_2d(to + TC_SUB_BYTES, &tmH, ks * TC_KB, s0, bar_full + st);
+            if (PAIR) {
+              if (rank == 0) tc_bar_expect(bar_full + st, 2u * tile_bytes);
+              const uint32_t full = tc_at_rank(bar_full + st, 0u);
+              tc_tma_2d_pair(to, &tmW, ks * TC_KB, row0, full);
+              tc_tma_2d_pair(to + SLAB, &tmH, ks * TC_KB, s0, full);
+            } else {
+              tc_bar_expect(bar_full + st, tile_bytes);
+              tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
+              tc_tma_2d(to + SLAB, &tmH, ks * TC_KB, s0, bar_full + st);
+            }
             if (++st == nst) { st = 0; ++stround; }
           }
           continue;
         }
         if (stround > 0) tc_bar_wait(bar_empty + st, (stround - 1) & 1, abort_flag);
-        tc_bar_expect(bar_full + st, tile_bytes);
-        for (int ks = 0; ks < ksub; ++ks)
-          tc_tma_2d(smB + (size_t)st * tile_bytes + (size_t)ks * TC_SUB_BYTES, &tmW, ks * TC_KB, row0, bar_full + st);
+        if (rank == 0) tc_bar_expect(bar_full + st, (PAIR ? 2u : 1u) * tile_bytes);
+        const uint32_t full = PAIR ? tc_at_rank(bar_full + st, 0u) : 0u;
+        for (int ks = 0; ks < ksub; ++ks) {
+          unsigned char* to = smB + (size_t)st * tile_bytes + (size_t)ks * SLAB;
+          if (PAIR) tc_tma_2d_pair(to, &tmW, ks * TC_KB, row0, full);
+          else tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
+        }
         if (++st == nst) { st = 0; ++stround; }
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issue: one thread ----------------
-    if (lane == 0) {
-      const uint32_t idesc = tc_idesc(TC_M, TC_N);
+    // ---------------- MMA issue: one thread (of a pair's first block) ----------------
+    if (lane == 0 && rank == 0) {
+      const uint32_t idesc = tc_idesc(PAIR ? 2 * TC_M : TC_M, NT);
       if (!WIDE) tc_bar_wait(bar_a, 0, abort_flag);
       const uint64_t b_base = tc_desc(tc_smem(smB));      // a descriptor's address field counts 16-byte units
       int st = 0, stround = 0, acc = 0, accround = 0;
@@ -238,37 +305,37 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         if (!WIDE) tc_bar_wait(bar_full + st, stround & 1, abort_flag);
         if (accround > 0) tc_bar_wait(bar_accempty + acc, (accround - 1) & 1, abort_flag);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem_base + (uint32_t)(acc * TC_N);
+        const uint32_t d = tmem_base + (uint32_t)(acc * NT);
         if (WIDE) {
           for (int ks = 0; ks < ksub; ++ks) {
             tc_bar_wait(bar_full + st, stround & 1, abort_flag);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t b = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
-            const uint64_t a = b + (uint64_t)(TC_SUB_BYTES >> 4);
+            const uint64_t a = b + (uint64_t)(SLAB >> 4);
             const int kn = ks == ksub - 1 ? klast : TC_KB / 8;
             for (int kk = 0; kk < kn; ++kk)
-              tc_mma_ss(d, a + (uint64_t)(kk * 2), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
-            tc_commit(bar_empty + st);
+              tc_mma_ss<PAIR>(d, a + (uint64_t)(kk * 2), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
+            tc_commit<PAIR>(bar_empty + st);
             if (++st == nst) { st = 0; ++stround; }
           }
-          tc_commit(bar_accfull + acc);
+          tc_commit<PAIR>(bar_accfull + acc);
           if (++acc == nacc) { acc = 0; ++accround; }
           continue;
         }
         const uint64_t b_tile = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
         for (int ks = 0; ks < kfull; ++ks) {
           const uint32_t a = tmem_base + acol + (uint32_t)(ks * TC_KB);      // lanes = samples, columns = hidden units
-          const uint64_t b = b_tile + (uint64_t)((ks * TC_SUB_BYTES) >> 4);
+          const uint64_t b = b_tile + (uint64_t)((ks * SLAB) >> 4);
 #pragma unroll
           for (int kk = 0; kk < TC_KB / 8; ++kk)              // eight tf32 = 32 bytes per instruction
-            tc_mma(d, a + (uint32_t)(kk * 8), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
+            tc_mma<PAIR>(d, a + (uint32_t)(kk * 8), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
         }
         if (kfull < ksub)                                     // a last slab of fewer units
           for (int kk = 0; kk < klast; ++kk)
-            tc_mma(d, tmem_base + acol + (uint32_t)(kfull * TC_KB + kk * 8), b_tile + (uint64_t)((kfull * TC_SUB_BYTES) >> 4) + (uint64_t)(kk * 2),
+            tc_mma<PAIR>(d, tmem_base + acol + (uint32_t)(kfull * TC_KB + kk * 8), b_tile + (uint64_t)((kfull * SLAB) >> 4) + (uint64_t)(kk * 2),
                    idesc, (kfull | kk) != 0 ? 1u : 0u);
-        tc_commit(bar_empty + st);          // the tile's shared memory is free once these instructions have read it
-        tc_commit(bar_accfull + acc);       // and the accumulator is complete
+        tc_commit<PAIR>(bar_empty + st);          // the tile's shared memory is free once these instructions have read it
+        tc_commit<PAIR>(bar_accfull + acc);       // and the accumulator is complete
         if (++st == nst) { st = 0; ++stround; }
         if (++acc == nacc) { acc = 0; ++accround; }
       }
@@ -279,21 +346,31 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     if (norms) {
       float best = 0.f;
       int st = 0, stround = 0;
-      const int nrr = 4 / nshare;                      // rows of this block: nrr per lane
+      const int nrr = RL / nshare;                     // rows of this block: nrr per lane
+      // the bytes of a pair are counted in its first block, which tells the second
+      auto arrived = [&](int st, int stround) {
+        tc_bar_wait(PAIR && rank == 1 ? bar_landed + st : bar_full + st, stround & 1, abort_flag);
+        if (PAIR && rank == 0 && lane == 0) tc_bar_arrive_at(tc_at_rank(bar_landed + st, 1u));
+      };
       for (int i = 0; i < my_tiles; ++i) {
         if (WIDE) {
-          float part[4] = {0.f, 0.f, 0.f, 0.f};        // the sums of the lane's rows over the slabs
+          unsigned long long part[RL][2];              // the sums of the lane's rows over the slabs, in pairs
+#pragma unroll
+          for (int rr = 0; rr < RL; ++rr) part[rr][0] = part[rr][1] = 0ull;
           for (int ks = 0; ks < ksub; ++ks) {
-            tc_bar_wait(bar_full + st, stround & 1, abort_flag);
+            arrived(st, stround);
             const unsigned char* tile = smB + (size_t)st * tile_bytes;
 #pragma unroll
-            for (int rr = 0; rr < 4; ++rr)
+            for (int rr = 0; rr < RL; ++rr)
               if (rr < nrr) {
                 const unsigned char* rowp = tile + (size_t)(32 * (nrr * (int)blockIdx.y + rr) + lane) * 128;
+                ulonglong2 w[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) w[c] = *reinterpret_cast<const ulonglong2*>(rowp + (size_t)((c ^ (lane & 7)) * 16));
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                  const float4 w = *reinterpret_cast<const float4*>(rowp + (size_t)((c ^ (lane & 7)) * 16));
-                  part[rr] = fmaf(w.x, w.x, fmaf(w.y, w.y, fmaf(w.z, w.z, fmaf(w.w, w.w, part[rr]))));
+                  asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(part[rr][0]) : "l"(w[c].x));
+                  asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(part[rr][1]) : "l"(w[c].y));
                 }
               }
             __syncwarp();
@@ -301,10 +378,12 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
             if (++st == nst) { st = 0; ++stround; }
           }
 #pragma unroll
-          for (int rr = 0; rr < 4; ++rr) best = fmaxf(best, part[rr]);
+          for (int rr = 0; rr < RL; ++rr)
+            best = fmaxf(best, (__uint_as_float((unsigned)part[rr][0]) + __uint_as_float((unsigned)(part[rr][0] >> 32))) +
+                                   (__uint_as_float((unsigned)part[rr][1]) + __uint_as_float((unsigned)(part[rr][1] >> 32))));
           continue;
         }
-        tc_bar_wait(bar_full + st, stround & 1, abort_flag);
+        arrived(st, stround);
         const unsigned char* tile = smB + (size_t)st * tile_bytes;
         for (int rr = 0; rr < nrr; ++rr) {
           const unsigned char* rowp = tile + (size_t)(32 * (nrr * (int)blockIdx.y + rr) + lane) * 128;
@@ -312,7 +391,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           for (int ks = 0; ks < ksub; ++ks)
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-              const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(rowp + (size_t)ks * TC_SUB_BYTES + (size_t)((c ^ (lane & 7)) * 16));
+              const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(rowp + (size_t)ks * SLAB + (size_t)((c ^ (lane & 7)) * 16));
               asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(s0) : "l"(w.x));
               asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(s1) : "l"(w.y));
             }
@@ -335,7 +414,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     const int q = warp & 3;                 // a warp reaches the 32 lanes of tensor memory of its number modulo four
     const int half = (warp - 3) >> 2;       // which share of a tile's 128 columns
     const int row = 32 * q + lane;          // sample inside the block
-    const int et = tid - 96;                // the first 128 read-back threads fetch the tile's biases
+    const int et = tid - 96;                // the first NT read-back threads (whole warps) fetch the tile's biases
     const int vslice = slice * TC_SPLIT + half;    // buffers are kept per (slice, share of the columns)
     int2* mybuf = p.cand + ((size_t)vslice * p.Bpad + s0 + row) * p.gbuf;
     const float tau = DUMP ? 0.f : (s0 + row < p.B ? p.tau[s0 + row] : INFINITY);      // rows past the batch keep nothing
@@ -360,28 +439,39 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      tc_bar_arrive(bar_a);
+      __syncwarp();
+      if (lane == 0) {
+        if (PAIR) tc_bar_arrive_at(tc_at_rank(bar_a, 0u));
+        else tc_bar_arrive(bar_a);
+      }
     }
-    // a tile's biases are asked for one tile ahead, so that their latency is not part of the tile's read-back
-    auto bias_of = [&](int i) {
-      const int j = (slice + i * p.nslices) * p.tile_stride * TC_N + et;
-      return et < TC_N && i < my_tiles && j < p.N ? __ldg(&p.hdr2[j].b) : 0.f;
+    // a tile's biases are asked for TC_BAHEAD tiles ahead (a group of copies per tile, empty past the last one)
+    auto ask_bias = [&](int i) {
+      const int j = (slice + i * p.nslices) * p.tile_stride * NT + et;
+      if (i < my_tiles)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                     ::"r"(tc_smem(sb + (i & (TC_BT - 1)) * NT + et)), "l"(&p.hdr2[j < p.N ? j : 0].b), "r"(j < p.N ? 4 : 0) : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float bias_next = bias_of(0);
+    if (et < NT)
+      for (int i = 0; i < TC_BAHEAD; ++i) ask_bias(i);
     int acc = 0, accround = 0;
     for (int i = 0; i < my_tiles; ++i) {
       const int tile = slice + i * p.nslices;
-      const int j0 = tile * p.tile_stride * TC_N;
-      if (et < TC_N) sb[acc * TC_N + et] = bias_next;
-      bias_next = bias_of(i + 1);
+      const int j0 = tile * p.tile_stride * NT;
+      if (et < NT) {
+        ask_bias(i + TC_BAHEAD);                   // where the biases of tile i - 2 were: every warp has left that tile
+        asm volatile("cp.async.wait_group %0;" ::"n"(TC_BAHEAD) : "memory");      // tile i's are there
+      }
+      const float* tb = sb + (i & (TC_BT - 1)) * NT;
       if (warp == 3) tc_bar_wait(bar_accfull + acc, accround & 1, abort_flag);      // one warp polls, the others sleep in the barrier
       asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");          // the accumulator is complete, the tile's biases are in place
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int c0 = (TC_N / TC_SPLIT) * half; c0 < (TC_N / TC_SPLIT) * (half + 1); c0 += 32) {
+      for (int c0 = (NT / TC_SPLIT) * half; c0 < (NT / TC_SPLIT) * (half + 1); c0 += 32) {
         uint32_t r[32];
-        tc_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * TC_N + c0), r);
+        tc_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * NT + c0), r);
         const int jb = j0 + c0;
-        const float4* sb4 = reinterpret_cast<const float4*>(sb + acc * TC_N + c0);
+        const float4* sb4 = reinterpret_cast<const float4*>(tb + c0);
         unsigned hm = 0u;
 #pragma unroll
         for (int c4 = 0; c4 < 8; ++c4) {
@@ -399,7 +489,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         }
         if (DUMP) {
           // neurons past the end score -infinity; a thread's 32 scores are 128 contiguous bytes
-          float4* out = reinterpret_cast<float4*>(p.dump + (size_t)(s0 + row) * p.dump_cols + (size_t)tile * TC_N + c0);
+          float4* out = reinterpret_cast<float4*>(p.dump + (size_t)(s0 + row) * p.dump_cols + (size_t)tile * NT + c0);
 #pragma unroll
           for (int c4 = 0; c4 < 8; ++c4) {
             float4 v;
@@ -418,9 +508,9 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
             any &= any - 1;
             uint32_t raw;
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;"
-                         : "=r"(raw) : "r"(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * TC_N + c0 + c)) : "memory");
+                         : "=r"(raw) : "r"(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * NT + c0 + c)) : "memory");
             if ((hm >> c) & 1u) {
-              const float z = __uint_as_float(raw) + sb[acc * TC_N + c0 + c];
+              const float z = __uint_as_float(raw) + tb[c0 + c];
               if (cnt < p.gbuf) __stcg(mybuf + cnt, make_int2(__float_as_int(z), jb + c));
               ++cnt;
             }
@@ -428,7 +518,11 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      tc_bar_arrive(bar_accempty + acc);
+      __syncwarp();
+      if (lane == 0) {
+        if (PAIR) tc_bar_arrive_at(tc_at_rank(bar_accempty + acc, 0u));
+        else tc_bar_arrive(bar_accempty + acc);
+      }
       if (++acc == nacc) { acc = 0; ++accround; }
     }
     if (!DUMP && s0 + row < p.B) {
@@ -437,10 +531,12 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
+  if (PAIR) tc_cluster_sync();       // nothing of the other block's reaches this one's shared memory any more
+  else __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
+    if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
   }
   if (tid == 0 && *abort_flag) atomicCAS(&p.st->status, 0, (int)DSLIDE_ERR_TIMEOUT);
 }
@@ -840,13 +936,13 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// rows x H fp32, row-major; boxes of 128 rows x 32 units, 128-byte swizzle; rows past the end read as zero
-static bool make_map(CUtensorMap* m, const float* base, int rows, int H) {
+// rows x H fp32, row-major; boxes of box_rows rows x 32 units, 128-byte swizzle; rows past the end read as zero
+static bool make_map(CUtensorMap* m, const float* base, int rows, int H, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)H, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)H * 4};
-  const cuuint32_t box[2] = {(cuuint32_t)TC_KB, (cuuint32_t)TC_M};
+  const cuuint32_t box[2] = {(cuuint32_t)TC_KB, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -895,26 +991,61 @@ static cudaError_t launch_exact_scan(Ctx* c, int batch, int k, int32_t* out_ids,
   return launch_scan_all(c, batch, k, nullptr, nullptr, e == cudaSuccess ? WS_HEAD : 0, out_ids, out_scores);
 }
 
+// As launch_dependent; the two blocks of a pair are a cluster.
+static cudaError_t launch_tc(void (*kernel)(const CUtensorMap, const CUtensorMap, const TcParams), bool pair, int slices, int groups, size_t smem,
+                             cudaStream_t stream, const CUtensorMap& tmW, const CUtensorMap& tmH, const TcParams& p) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((pair ? 2 : 1) * slices, groups); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = pair ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, tmW, tmH, p);
+}
+
+// Whether two multiprocessors share a tile of W2 and 256 samples.  The tile then crosses from L2 once instead of twice, and a
+// stage takes half the shared memory, but a pair's instruction takes as long as two blocks' (124 cycles for 256 samples x
+// 128 neurons x 8 units: the tensor pipe, not the loads, is the bound).  So it pays where a block has room for one tile only
+// (more than 192 units), or streams the activations with the tiles (more than 256): us for a call of 1,024 samples x
+// 253,855 neurons x 200 units 371 by single blocks and 258 by pairs, 512 x 4,000,000 x 256 2,467 and 1,897, 512 x 100,003 x
+// 512 206 and 138; not at 160 units (300 x 100,003: 69 and 80) or 128 (147.9 and 148.8 for 670,091).  And where the tiles
+// keep the pairs busy: a round of tiles takes a pair 0.7 of a block's time, at more than 256 units 1.2 for twice the tile.
+static bool use_pairs(const Ctx* c, int batch) {
+  if (batch <= TC_M || c->H <= TC_H_SINGLE) return false;
+  const bool wide = c->H > TC_H_TMEM;
+  auto rounds = [&](bool pair) {
+    const int per = (pair ? 2 : 1) * TC_M, groups = (batch + per - 1) / per;
+    const int slices = max(1, (pair ? c->num_sms / 2 : c->num_sms) / groups), nt = tc_cols(wide, pair);
+    return ((c->N + nt - 1) / nt + slices - 1) / slices;
+  };
+  return wide ? 6 * rounds(true) < 5 * rounds(false) : 7 * rounds(true) < 10 * rounds(false);
+}
+
 // The hidden activations of the batch are in c->h (left there by the forward kernel in predict mode).
 cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* out_scores) {
   if (c->N < TC_N || encode_fn() == nullptr) return launch_exact_scan(c, batch, k, out_ids, out_scores);
   const int cap = 2 * k + TC_EXTRA;
-  const int groups = (batch + TC_M - 1) / TC_M;
-  const int ntiles = (c->N + TC_N - 1) / TC_N;
-  int nslices = c->num_sms / groups;
+  const bool wide = c->H > TC_H_TMEM;
+  const bool pair = use_pairs(c, batch);
+  const int NT = tc_cols(wide, pair);
+  const int groups = pair ? (batch + 2 * TC_M - 1) / (2 * TC_M) : (batch + TC_M - 1) / TC_M;      // of 256 samples, or of 128
+  const int ntiles = (c->N + NT - 1) / NT;
+  int nslices = (pair ? c->num_sms / 2 : c->num_sms) / groups;
   if (nslices < 1) nslices = 1;
   if (nslices > ntiles) nslices = ntiles;
   if (TC_SPLIT * nslices > RF_MAXV) nslices = RF_MAXV / TC_SPLIT;      // k_tc_refine's table of buffer offsets
   // threshold pass: every `stride`-th tile, at most TAU_MAX_TILES of them
-  constexpr int TAU_MAX_TILES = 128;
+  const int TAU_MAX_TILES = 128 * TC_N / NT;
   int stride = TC_SUBSET;
   if ((ntiles + stride - 1) / stride > TAU_MAX_TILES) stride = (ntiles + TAU_MAX_TILES - 1) / TAU_MAX_TILES;
   const int nsub = (ntiles + stride - 1) / stride;
-  const int dump_cols = nsub * TC_N;
+  const int dump_cols = nsub * NT;
   int nslices_sub = nslices < nsub ? nslices : nsub;
   // work space: the norm bound, the flags, the thresholds, the candidate buffers of every slice and their fill, the
   // threshold pass's scores
-  const int Bpad = groups * TC_M;
+  const int Bpad = groups * (pair ? 2 : 1) * TC_M;
   const int nvs = TC_SPLIT * nslices;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t off_part = WS_HEAD, off_fix = off_part + up(scan_part_bytes(c, k)), off_list = off_fix + up((size_t)Bpad * 4);
@@ -943,20 +1074,20 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   int2* cand = reinterpret_cast<int2*>(ws + off_cand);
   float* dump = reinterpret_cast<float*>(ws + off_dump);
 
-  const bool wide = c->H > TC_H_TMEM;
+  const int rows = pair ? NT / 2 : NT;               // of a tile, in a block
   CUtensorMap tmW, tmH;
-  if (!make_map(&tmW, c->W2, c->N, c->H) || !make_map(&tmH, c->h, batch, c->H)) return cudaErrorInvalidValue;
+  if (!make_map(&tmW, c->W2, c->N, c->H, rows) || !make_map(&tmH, c->h, batch, c->H, TC_M)) return cudaErrorInvalidValue;
 
   TcParams p;
   p.hdr2 = c->hdr2; p.h = c->h; p.cand = cand; p.cand_cnt = cand_cnt; p.dump = dump; p.tau = tau; p.need_fix = need_fix; p.norm2max = norm2; p.n_fix = n_fix; p.st = c->dstate;
   p.B = batch; p.Bpad = Bpad; p.H = c->H; p.N = c->N; p.dump_cols = dump_cols; p.gbuf = gbuf;
-  const size_t tile_bytes = wide ? (size_t)2 * TC_SUB_BYTES : (size_t)((c->H + TC_KB - 1) / TC_KB) * TC_SUB_BYTES;
+  const size_t tile_bytes = wide ? (size_t)rows * 128 + TC_SUB_BYTES : (size_t)((c->H + TC_KB - 1) / TC_KB) * rows * 128;
   int stages = (int)(((size_t)200 << 10) / tile_bytes);
   if (stages > (wide ? TC_WIDE_STAGES : TC_STAGES)) stages = wide ? TC_WIDE_STAGES : TC_STAGES;
   p.stages = stages;
-  const size_t smem = 1024 + tile_bytes * stages + TC_NACC * TC_N * 4 + 24 * 8 + 64;
-  auto k_sub = wide ? k_dense_tc<true, true> : k_dense_tc<true, false>;
-  auto k_all = wide ? k_dense_tc<false, true> : k_dense_tc<false, false>;
+  const size_t smem = 1024 + tile_bytes * stages + (size_t)TC_BT * NT * 4 + (1 + 3 * TC_STAGES + 2 * TC_NACC) * 8 + 64;
+  auto k_sub = pair ? (wide ? k_dense_tc<true, true, true> : k_dense_tc<true, false, true>) : (wide ? k_dense_tc<true, true, false> : k_dense_tc<true, false, false>);
+  auto k_all = pair ? (wide ? k_dense_tc<false, true, true> : k_dense_tc<false, false, true>) : (wide ? k_dense_tc<false, true, false> : k_dense_tc<false, false, false>);
   if ((e = cudaFuncSetAttribute(k_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   {
@@ -964,11 +1095,11 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
     p.nslices = nslices_sub; p.ntiles = nsub; p.tile_stride = stride;
     // each kernel of the call may be placed while the kernel before it drains (they wait for it before they read or
     // write anything); the first follows the hidden-layer kernel in the same way
-    if ((e = launch_dependent(k_sub, dim3(nslices_sub, groups), dim3(TC_THREADS), smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
+    if ((e = launch_tc(k_sub, pair, nslices_sub, groups, smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_tau, dim3(Bpad), dim3(TAU_THREADS), 0, c->stream, (const float*)dump, dump_cols, rank, tau)) != cudaSuccess)
       return e;
     p.nslices = nslices; p.ntiles = ntiles; p.tile_stride = 1;
-    if ((e = launch_dependent(k_all, dim3(nslices, groups), dim3(TC_THREADS), smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
+    if ((e = launch_tc(k_all, pair, nslices, groups, smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_refine, dim3(batch), dim3(RF_THREADS), 0, c->stream, (const float*)c->W2, (const RowHdr*)c->hdr2,
                               (const float*)c->h, (const int2*)cand, (const int*)cand_cnt, gbuf, (const float*)tau, Bpad,
                               (const unsigned int*)norm2, batch, c->H, c->N, cap, nvs, k, out_ids, out_scores, (const int*)need_fix, n_fix, fix_list)) !=

@@ -14,9 +14,13 @@ SHAPES = [            # H, N, batch, k
     (4, 3001, 3, 1), (36, 129, 5, 10), (36, 128, 1, 64), (36, 100, 2, 5), (36, 40, 3, 64), (200, 20011, 130, 5),
     (252, 9000, 33, 64), (256, 5000, 129, 9), (260, 5000, 40, 5), (516, 3000, 131, 17), (1024, 2049, 260, 3), (1020, 700, 1, 64),
 ]
+PAIRS = [             # two multiprocessors to a tile: more than 192 units, more than 128 samples, enough tiles
+    (196, 19001, 256, 5), (200, 38017, 257, 9), (256, 18945, 256, 64), (224, 30011, 130, 3), (260, 38145, 140, 5), (292, 19001, 300, 5),
+    (1020, 13001, 300, 5), (132, 9000, 200, 3),
+]
 
 
-@pytest.mark.parametrize("H,N,B,k", SHAPES)
+@pytest.mark.parametrize("H,N,B,k", SHAPES + PAIRS)
 def test_predict_over_all_neurons(H, N, B, k):
     pr = Pair(D=501, H=H, N=N, family=workloads.SIMHASH, K=4, L=4, bucket_cap=16, max_batch=B, seed=H + N)
     try:
@@ -59,7 +63,7 @@ def test_weights_that_are_not_finite():
 
 FLAGGED = [           # H, N, batch, k, samples whose filter cannot decide (of the batch)
     (4, 3001, 3, 1, 3), (36, 129, 5, 10, 1), (128, 2000, 20, 64, 20), (200, 5011, 260, 5, 9), (128, 20011, 1, 5, 1),
-    (264, 700, 33, 17, 32), (1024, 2049, 40, 3, 8), (1020, 333, 9, 64, 9), (64, 4001, 300, 5, 300),
+    (264, 700, 33, 17, 32), (1024, 2049, 40, 3, 8), (1020, 333, 9, 64, 9), (64, 4001, 300, 5, 300), (256, 20011, 200, 5, 70),
 ]
 
 
