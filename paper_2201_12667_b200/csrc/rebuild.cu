@@ -4,7 +4,7 @@
 //
 //   k_init_gauss   : weights ~ N(0, std^2) from the counter-based generator (Box-Muller).
 //   k_draw_simhash / k_draw_dwta : the hash functions of rebuild count r.
-//   k_hash_neurons : the L bucket codes of every row of W2 (same functions as the queries) and
+//   k_hash_neurons* : the L bucket codes of every row of W2 (same functions as the queries) and
 //                    the size of every bucket.
 //   k_bucket_scan  : bucket sizes -> bucket offsets (one block per table).
 //   k_sort_hist / k_sort_scan / k_sort_scatter : a stable least-significant-digit radix sort of the

@@ -363,23 +363,30 @@ __device__ __forceinline__ void scale2(ulonglong2& v, unsigned long long f) {
 }
 
 // Grid (row chunks, groups of samples).  A group of G lanes takes a row: lane g of it holds the 16-byte pieces g, g + G,
-// ... (NP of them).  Four rows per group at a time: their dot products with the sample's activations are reduced
-// together (lanes exchange the values they give up, so that a quarter of the group ends with each row's sum).  Rows of
-// up to 128 units are taken by half warps, eight rows of a run at a time (G = 16); wider ones by whole warps (G = 32: with
-// half warps the eight rows of 200 units do not fit the registers and the one-hot word shape took 1,614 us a step instead
-// of 1,531).  Rows of up to 256 units stay in registers between the logits and the sums, others are read a second time.
-template <int G, int NP>
+// ... (NP of them).  R rows per group at a time: their dot products with the sample's activations are reduced
+// together (lanes exchange the values they give up, so that Q lanes of the group end with each row's sum).  Rows of
+// up to 128 units are taken by half warps, four rows each (G = 16); wider ones by whole warps (G = 32: with half warps the
+// eight rows of 200 units do not fit the registers and the one-hot word shape took 1,614 us a step instead of 1,531), eight
+// rows up to 256 units -- one reduction, one exponential and one look at the maximum for eight rows: 563 us instead of 587 for
+// 1,024 samples x 6,100 neurons x 200 units -- and four beyond.  At more than 512 units the rows' places and weights pass
+// through shared memory, as with eight rows: by shuffles they cost 700 bytes of spills (512 samples x 60,013 neurons x 1,024
+// units, a step 7,180 us, now 4,240); at 257 to 512 shuffles are the faster (463 us against 535 for 400 samples x 332 units).
+// Rows of up to 256 units stay in registers between the logits and the sums, others are read a second time.
+template <int G, int NP, int R>
 __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams p) {
   constexpr bool KEEP = G == 16 || NP <= 2;
-  constexpr int Q = G / 4;                     // lanes that end with the same row's sum
-  constexpr int RPI = 128 / G;                 // rows per iteration
+  constexpr bool STAGED = R == 8 || NP == 8;   // places and weights of rows by way of shared memory: one load for a shuffle per row, fewer registers
+  constexpr int Q = G / R;                     // lanes that end with the same row's sum
+  constexpr int RPI = R * 32 / G;              // rows per iteration
   extern __shared__ __align__(128) unsigned char t_sm[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ __align__(16) float zeros[4];
+  __shared__ __align__(16) uint16_t places[STAGED ? TF_WARPS : 1][32];       // of 32 entries of the run a warp is at
+  __shared__ __align__(16) float weights[STAGED ? TF_WARPS : 1][RPI];        // of the rows of an iteration
   float* tile = reinterpret_cast<float*>(t_sm);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int H = p.H, H4 = H >> 2, ld = H + 4;
-  const int gl = lane & (G - 1), first = (lane & ~(G - 1)) * 4 / G;      // place in the group; the group's first row of an iteration
+  const int gl = lane & (G - 1), first = lane / G * R;      // place in the group; the group's first row of an iteration
   if (tid < 4) zeros[tid] = 0.f;
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(t_smem(&bar)) : "memory");
@@ -459,13 +466,27 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams
             const int some = __shfl_sync(TFULL, loc, 0);      // past the run: a row of the run, with weight zero below
             if (lane >= m) loc = some;
           }
+          if (STAGED) {
+            __syncwarp();
+            places[warp][lane] = (uint16_t)loc;
+            __syncwarp();
+          }
           for (int k = 0; k < m; k += RPI) {
-            int rl[4];                           // places of the four rows
-            ulonglong2 x[4][KEEP ? NP : 1];
-            float d[4];
+            int rl[R];                           // places of the group's rows
+            if (STAGED) {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              rl[r] = __shfl_sync(TFULL, loc, k + first + r);
+              for (int r = 0; r < R; r += 4) {
+                const uint2 w = *reinterpret_cast<const uint2*>(&places[warp][k + r]);
+                rl[r] = (int)(w.x & 0xffffu); rl[r + 1] = (int)(w.x >> 16); rl[r + 2] = (int)(w.y & 0xffffu); rl[r + 3] = (int)(w.y >> 16);
+              }
+            } else {
+#pragma unroll
+              for (int r = 0; r < R; ++r) rl[r] = __shfl_sync(TFULL, loc, k + first + r);
+            }
+            ulonglong2 x[R][KEEP ? NP : 1];
+            float d[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
               unsigned long long d0 = 0ull, d1 = 0ull;
 #pragma unroll
               for (int u = 0; u < NP; ++u) {
@@ -476,13 +497,23 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams
               }
               d[r] = (lo2(d0) + hi2(d0)) + (lo2(d1) + hi2(d1));
             }
-            const bool hi = (lane & (2 * Q)) != 0, od = (lane & Q) != 0;
-            const float u0 = (hi ? d[2] : d[0]) + __shfl_xor_sync(TFULL, hi ? d[0] : d[2], 2 * Q);
-            const float u1 = (hi ? d[3] : d[1]) + __shfl_xor_sync(TFULL, hi ? d[1] : d[3], 2 * Q);
-            float y = (od ? u1 : u0) + __shfl_xor_sync(TFULL, od ? u0 : u1, Q);
+            // every exchange halves the rows a lane has part of
+#pragma unroll
+            for (int n2 = R / 2, o = G / 2; n2 > 0; n2 >>= 1, o >>= 1) {
+              const bool up = (lane & o) != 0;
+#pragma unroll
+              for (int r = 0; r < n2; ++r) d[r] = (up ? d[r + n2] : d[r]) + __shfl_xor_sync(TFULL, up ? d[r] : d[r + n2], o);
+            }
+            float y = d[0];
 #pragma unroll
             for (int o = Q / 2; o > 0; o >>= 1) y += __shfl_xor_sync(TFULL, y, o);
-            const int ml = hi ? (od ? rl[3] : rl[2]) : (od ? rl[1] : rl[0]);         // the row whose sum this lane has
+            int ml;                              // the row whose sum this lane has
+            if (STAGED) {
+              ml = places[warp][k + lane / Q];
+            } else {
+              const bool hi = (lane & (2 * Q)) != 0, od = (lane & Q) != 0;
+              ml = hi ? (od ? rl[3] : rl[2]) : (od ? rl[1] : rl[0]);
+            }
             float z = tile[ml * ld + H + 1] + y;                     // the bias came with the row
             const int mine = k + lane / Q;
             if (mine >= m) z = -INFINITY;
@@ -502,9 +533,18 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams
             // a masked neuron (bias of minus infinity) weighs nothing, also while nothing else has been met and M is minus infinity
             const float e = z != -INFINITY ? expf(z - M) : 0.f;
             E += e;
+            float4 four[STAGED ? R / 4 : 1];
+            if (STAGED) {
+              __syncwarp();                      // the weights before have been read
+              if ((lane & (Q - 1)) == 0) weights[warp][lane / Q] = e;
+              __syncwarp();
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              const float g = __shfl_sync(TFULL, e, (lane & ~(G - 1)) + Q * r);
+              for (int r = 0; r < R; r += 4) four[STAGED ? r / 4 : 0] = *reinterpret_cast<const float4*>(&weights[warp][r]);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const float4& f4 = four[STAGED ? r / 4 : 0];
+              const float g = !STAGED ? __shfl_sync(TFULL, e, (lane & ~(G - 1)) + Q * r) : (r & 3) == 0 ? f4.x : (r & 3) == 1 ? f4.y : (r & 3) == 2 ? f4.z : f4.w;
               const unsigned long long gg = pair2(g, g);
 #pragma unroll
               for (int u = 0; u < NP; ++u) {
@@ -791,8 +831,8 @@ cudaError_t launch_tiles_forward(Ctx* c, int batch, const int32_t* label_ptr, co
   p.act_loc = c->act_loc; p.act_z = c->act_z; p.part = c->tpart; p.st = c->dstate;
   p.B = batch; p.H = c->H; p.act_stride = c->act_stride; p.bstride = batch; p.chunks = chunks; p.gs = (batch + groups - 1) / groups;
   const int smem = (step + 31) * (c->H + 4) * 4;
-  auto k = c->H <= 64 ? k_tile_forward<16, 1> : c->H <= 128 ? k_tile_forward<16, 2> : c->H <= 256 ? k_tile_forward<32, 2>
-           : c->H <= 512 ? k_tile_forward<32, 4> : k_tile_forward<32, 8>;
+  auto k = c->H <= 64 ? k_tile_forward<16, 1, 4> : c->H <= 128 ? k_tile_forward<16, 2, 4> : c->H <= 256 ? k_tile_forward<32, 2, 8>
+           : c->H <= 512 ? k_tile_forward<32, 4, 4> : k_tile_forward<32, 8, 4>;
   if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024)) != cudaSuccess) return e;
   if ((e = launch_dependent(k, dim3(chunks, groups), dim3(TF_THREADS), (size_t)smem, c->stream, p)) != cudaSuccess) return e;
   CombineParams q;

@@ -26,6 +26,7 @@
 //              at a time (of up to 128 units the last few thousand two at a time).  Adam is applied to the touched rows only; untouched rows are neither read
 //              nor written.  The warp that updates a row resets its count and mask for the next step.
 //              The first blocks of the grid update the hidden bias and reduce the batch loss.
+//              Rows of more than 128 units are not held: a warp takes one row at a time, piece by piece (long_row).
 //   k_adam_dense : the output layer when every neuron is active (no lists, no masks).
 #include "common.cuh"
 
