@@ -21,6 +21,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "waits.cuh"
 
 namespace dslide {
 
@@ -69,7 +70,6 @@ struct TcParams {
   int gbuf;                        // slots per candidate buffer
 };
 
-__device__ __forceinline__ uint32_t tc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void tc_bar_init(uint64_t* bar, int count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc_smem(bar)), "r"(count) : "memory");
 }
@@ -78,19 +78,6 @@ __device__ __forceinline__ void tc_bar_expect(uint64_t* bar, uint32_t bytes) {
 }
 __device__ __forceinline__ void tc_bar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc_smem(bar)) : "memory");
-}
-// Bounded wait; once any wait of the block has run out, *abort is set and every later wait returns at once, so that
-// all the roles run through their loops, tensor memory is released and the kernel ends (its results are flagged).
-__device__ __forceinline__ void tc_bar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  const uint32_t a = tc_smem(bar);
-  for (int it = 0; it < (1 << 20); ++it) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(a), "r"(parity) : "memory");
-    if (ok) return;
-    if ((it & 1023) == 1023 && *abort) return;
-  }
-  *abort = 1;
 }
 // The address, in the cluster's shared memory, of a barrier of the block of rank `rank`; an arrival there.  Arrivals and waits
 // order what the block itself needs (default scope): the operands and accumulators are ordered by the copies' and the tensor
