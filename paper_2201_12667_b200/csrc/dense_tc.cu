@@ -144,12 +144,12 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32])
         "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
-// Arrives on the barrier -- of both blocks of a pair -- once the instructions issued before have completed
+// Arrives on the barrier -- of the blocks of a pair that `ranks` names, both by default -- once the instructions issued before have completed
 template <bool PAIR>
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+__device__ __forceinline__ void tc_commit(uint64_t* bar, int ranks = 3) {
   if (PAIR)
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(tc_smem(bar)), "h"((uint16_t)3) : "memory");
+                 ::"r"(tc_smem(bar)), "h"((uint16_t)ranks) : "memory");
   else
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem(bar)) : "memory");
 }
@@ -205,7 +205,8 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   uint64_t* bar_accfull = bars + 1 + 2 * NST;              // [TC_NACC] accumulator written
   uint64_t* bar_accempty = bars + 1 + 2 * NST + TC_NACC;   // [TC_NACC] accumulator read back
   uint64_t* bar_landed = bars + 1 + 2 * NST + 2 * TC_NACC; // [NST] second block of a pair: the stage has arrived (the pair's bytes are counted in the first)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 1 + 3 * NST + 2 * TC_NACC);
+  uint64_t* bar_drain = bars + 1 + 3 * NST + 2 * TC_NACC;  // after a wait has run out: the multiplications issued before have completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -224,6 +225,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
 
   if (tid == 0) {
     tc_bar_init(bar_a, PAIR ? 8 : 4);            // a warp each
+    tc_bar_init(bar_drain, 1);
     for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_landed + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
     for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, (PAIR ? 2 : 1) * TC_EPI / 32); }
     *abort_flag = 0;
@@ -246,15 +248,18 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   griddep_launch_dependents();       // the next kernel of the call may be placed as blocks of this one leave
   griddep_wait();                    // the filter launch reads the thresholds of the kernel before it
 
+  // Copies, multiplications and commits stop where a wait has run out; the other roles run through to their ends.
+  int fills = 0;                     // stages that this block has asked for
   if (warp == 0) {
     // ---------------- producer: one thread feeds the TMA ----------------
     if (lane == 0) {
       int st = 0, stround = 0;
-      for (int i = 0; i < my_tiles; ++i) {
+      bool on = true;
+      for (int i = 0; on && i < my_tiles; ++i) {
         const int row0 = (slice + i * p.nslices) * p.tile_stride * NT + (int)rank * ROWS;
         if (WIDE) {
-          for (int ks = 0; ks < ksub; ++ks) {
-            if (stround > 0) tc_bar_wait(bar_empty + st, (stround - 1) & 1, abort_flag);
+          for (int ks = 0; ks < ksub; ++ks, ++fills) {
+            if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
             unsigned char* to = smB + (size_t)st * tile_bytes;
             if (PAIR) {
               if (rank == 0) tc_bar_expect(bar_full + st, 2u * tile_bytes);
@@ -270,7 +275,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           }
           continue;
         }
-        if (stround > 0) tc_bar_wait(bar_empty + st, (stround - 1) & 1, abort_flag);
+        if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
         if (rank == 0) tc_bar_expect(bar_full + st, (PAIR ? 2u : 1u) * tile_bytes);
         const uint32_t full = PAIR ? tc_at_rank(bar_full + st, 0u) : 0u;
         for (int ks = 0; ks < ksub; ++ks) {
@@ -278,24 +283,27 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           if (PAIR) tc_tma_2d_pair(to, &tmW, ks * TC_KB, row0, full);
           else tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
         }
+        ++fills;
         if (++st == nst) { st = 0; ++stround; }
       }
+      // the last fill of every stage has been consumed: no copy and no arrival at this block's barriers is on its way any more
+      for (int f = max(0, fills - nst); on && f < fills; ++f) on = tc_bar_wait<PAIR>(bar_empty + f % nst, (f / nst) & 1, abort_flag);
     }
   } else if (warp == 1) {
     // ---------------- MMA issue: one thread (of a pair's first block) ----------------
     if (lane == 0 && rank == 0) {
       const uint32_t idesc = tc_idesc(PAIR ? 2 * TC_M : TC_M, NT);
-      if (!WIDE) tc_bar_wait(bar_a, 0, abort_flag);
+      bool on = WIDE || tc_bar_wait<PAIR>(bar_a, 0, abort_flag);
       const uint64_t b_base = tc_desc(tc_smem(smB));      // a descriptor's address field counts 16-byte units
       int st = 0, stround = 0, acc = 0, accround = 0;
-      for (int i = 0; i < my_tiles; ++i) {
-        if (!WIDE) tc_bar_wait(bar_full + st, stround & 1, abort_flag);
-        if (accround > 0) tc_bar_wait(bar_accempty + acc, (accround - 1) & 1, abort_flag);
+      for (int i = 0; on && i < my_tiles; ++i) {
+        if (!WIDE && !tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag)) break;
+        if (accround > 0 && !tc_bar_wait<PAIR>(bar_accempty + acc, (accround - 1) & 1, abort_flag)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem_base + (uint32_t)(acc * NT);
         if (WIDE) {
           for (int ks = 0; ks < ksub; ++ks) {
-            tc_bar_wait(bar_full + st, stround & 1, abort_flag);
+            if (!(on = tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t b = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
             const uint64_t a = b + (uint64_t)(SLAB >> 4);
@@ -305,6 +313,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
             tc_commit<PAIR>(bar_empty + st);
             if (++st == nst) { st = 0; ++stround; }
           }
+          if (!on) break;
           tc_commit<PAIR>(bar_accfull + acc);
           if (++acc == nacc) { acc = 0; ++accround; }
           continue;
@@ -336,7 +345,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       const int nrr = RL / nshare;                     // rows of this block: nrr per lane
       // the bytes of a pair are counted in its first block, which tells the second
       auto arrived = [&](int st, int stround) {
-        tc_bar_wait(PAIR && rank == 1 ? bar_landed + st : bar_full + st, stround & 1, abort_flag);
+        tc_bar_wait<PAIR>(PAIR && rank == 1 ? bar_landed + st : bar_full + st, stround & 1, abort_flag);
         if (PAIR && rank == 0 && lane == 0) tc_bar_arrive_at(tc_at_rank(bar_landed + st, 1u));
       };
       for (int i = 0; i < my_tiles; ++i) {
@@ -451,7 +460,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         asm volatile("cp.async.wait_group %0;" ::"n"(TC_BAHEAD) : "memory");      // tile i's are there
       }
       const float* tb = sb + (i & (TC_BT - 1)) * NT;
-      if (warp == 3) tc_bar_wait(bar_accfull + acc, accround & 1, abort_flag);      // one warp polls, the others sleep in the barrier
+      if (warp == 3) tc_bar_wait<PAIR>(bar_accfull + acc, accround & 1, abort_flag);      // one warp polls, the others sleep in the barrier
       asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");          // the accumulator is complete, the tile's biases are in place
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       for (int c0 = (NT / TC_SPLIT) * half; c0 < (NT / TC_SPLIT) * (half + 1); c0 += 32) {
@@ -520,6 +529,21 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (PAIR) tc_cluster_sync();       // nothing of the other block's reaches this one's shared memory any more
   else __syncthreads();
+  if (*abort_flag) {                 // of both blocks, or of neither: what has been issued still comes to its end, but not for ever
+    const long long until = clock64() + DRAIN_CYCLES;
+    if (tid == 0) {
+      if (rank == 0)
+        for (int f = max(0, fills - nst); f < fills; ++f) tc_bar_drain(bar_full + f % nst, (f / nst) & 1, until);
+      else
+        while (clock64() < until) __nanosleep(1000);      // its copies are counted in the first block, which may not have asked for the same stages
+    }
+    if (tid == 32 && rank == 0) {
+      tc_commit<PAIR>(bar_drain, 1);
+      tc_bar_drain(bar_drain, 0, until);
+    }
+    if (PAIR) tc_cluster_sync();
+    else __syncthreads();
+  }
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
@@ -1072,7 +1096,7 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   int stages = (int)(((size_t)200 << 10) / tile_bytes);
   if (stages > (wide ? TC_WIDE_STAGES : TC_STAGES)) stages = wide ? TC_WIDE_STAGES : TC_STAGES;
   p.stages = stages;
-  const size_t smem = 1024 + tile_bytes * stages + (size_t)TC_BT * NT * 4 + (1 + 3 * TC_STAGES + 2 * TC_NACC) * 8 + 64;
+  const size_t smem = 1024 + tile_bytes * stages + (size_t)TC_BT * NT * 4 + (2 + 3 * TC_STAGES + 2 * TC_NACC) * 8 + 64;
   auto k_sub = pair ? (wide ? k_dense_tc<true, true, true> : k_dense_tc<true, false, true>) : (wide ? k_dense_tc<true, true, false> : k_dense_tc<true, false, false>);
   auto k_all = pair ? (wide ? k_dense_tc<false, true, true> : k_dense_tc<false, false, true>) : (wide ? k_dense_tc<false, true, false> : k_dense_tc<false, false, false>);
   if ((e = cudaFuncSetAttribute(k_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;

@@ -6,6 +6,7 @@ namespace dslide {
 
 // About a second at the highest clock.  A count of tries is no limit: how long a try may sleep is the hardware's choice.
 constexpr long long WAIT_CYCLES = 2000000000LL;
+constexpr long long DRAIN_CYCLES = 20000000LL;       // for what is in flight when a block has given up: copies and multiplications take microseconds
 
 __device__ __forceinline__ uint32_t tc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // A try may sleep up to 2 us, so that a waiting warp issues little (all-neuron calls of 128 samples x 100,003 neurons x 512 units
@@ -16,17 +17,30 @@ __device__ __forceinline__ bool tc_bar_try(uint32_t bar, uint32_t parity) {
                : "=r"(ok) : "r"(bar), "r"(parity), "r"(2000u) : "memory");
   return ok != 0u;
 }
-// True once the phase of that parity has completed.  False when it has not within the limit -- *abort is then set -- or when
-// another wait of the block has given up: all the roles run through to their ends, and the kernel's results are flagged.
+// Sets the flag of this block and, in a pair (PAIR: a cluster of two blocks), of the other one.
+template <bool PAIR>
+__device__ __forceinline__ void tc_give_up(volatile int* abort) {
+  *abort = 1;
+  if (PAIR)
+    asm volatile("{\n\t.reg .b32 r, a;\n\tmov.u32 r, %%cluster_ctarank;\n\txor.b32 r, r, 1;\n\tmapa.shared::cluster.u32 a, %0, r;\n\t"
+                 "st.relaxed.cluster.shared::cluster.b32 [a], %1;\n\t}" ::"r"(tc_smem(const_cast<int*>(abort))), "r"(1) : "memory");
+}
+// True once the phase of that parity has completed.  False when it has not within the limit -- the flag is then set -- or when
+// another wait of the block, or of the pair, has given up: every later wait returns at once.
+template <bool PAIR>
 __device__ __forceinline__ bool tc_bar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
   const uint32_t a = tc_smem(bar);
   if (tc_bar_try(a, parity)) return true;
   const long long t0 = clock64();
   while (!tc_bar_try(a, parity)) {
     if (*abort) return false;
-    if (clock64() - t0 > WAIT_CYCLES) { *abort = 1; return false; }
+    if (clock64() - t0 > WAIT_CYCLES) { tc_give_up<PAIR>(abort); return false; }
   }
   return true;
+}
+// The same, for a block that has given up: it waits until the time `until`, whatever the flag says.
+__device__ __forceinline__ void tc_bar_drain(uint64_t* bar, uint32_t parity, long long until) {
+  while (!tc_bar_try(tc_smem(bar), parity) && clock64() < until) {}
 }
 
 }  // namespace dslide

@@ -22,7 +22,16 @@ def probe(tmp_path_factory):
 def test_a_wait_that_nothing_ends(probe):
     """It gives up within its limit (a second's cycles, and one try of the hardware's own length beyond), later waits at once."""
     out, cycles = (ctypes.c_int * 4)(), (ctypes.c_longlong * 2)()
-    assert probe.run_waits(out, cycles) == 0
+    assert probe.run_waits(0, out, cycles) == 0
     assert list(out) == [0, 0, 1, 1]
     assert 2.0e9 < cycles[0] < 2.5e9, cycles[0]
     assert cycles[1] < 0.5e9, cycles[1]
+
+
+def test_a_pair_gives_up_together(probe):
+    """The block whose wait has run out tells the other block of the pair, whose waits then return at once; what is in flight
+    is waited for by the clock too."""
+    out, cycles = (ctypes.c_int * 4)(), (ctypes.c_longlong * 2)()
+    assert probe.run_waits(1, out, cycles) == 0
+    assert list(out) == [0, 1, 1, 0]
+    assert cycles[0] < 0.5e9 and 2.0e7 <= cycles[1] < 5.0e8, list(cycles)
