@@ -55,6 +55,7 @@ __host__ __device__ constexpr int tc_cols(bool wide, bool pair) { return wide &&
 struct TcParams {
   const RowHdr* hdr2;
   const float* h;                  // [>= B][H] hidden activations of the batch
+  const float* W2;
   int2* cand;                      // [TC_SPLIT * slices][Bpad][gbuf] (score bits, id), cand_cnt of them valid, no order
   int* cand_cnt;                   // [TC_SPLIT * slices][Bpad]
   float* dump;                     // DUMP launch: [Bpad][dump_cols] scores of the subset's tiles
@@ -79,9 +80,11 @@ __device__ __forceinline__ void tc_bar_expect(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void tc_bar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc_smem(bar)) : "memory");
 }
-// The address, in the cluster's shared memory, of a barrier of the block of rank `rank`; an arrival there.  Arrivals and waits
-// order what the block itself needs (default scope): the operands and accumulators are ordered by the copies' and the tensor
+// The address, in the cluster's shared memory, of a barrier of the block of rank `rank`; an arrival there.  Most arrivals and
+// waits order what the block itself needs (default scope): the operands and accumulators are ordered by the copies' and the tensor
 // unit's own completion and by tcgen05.fence.  With release and acquire at cluster scope every one of them cost about 1,000 cycles.
+// The second block's ordinary loads of rows whose copies the first block counts are ordered by none of these: the first block's
+// wait for the copies, the arrival that passes them on (tc_bar_pass_on) and the second block's wait are at cluster scope.
 __device__ __forceinline__ uint32_t tc_at_rank(const void* p, uint32_t rank) {
   uint32_t a;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(tc_smem(p)), "r"(rank));
@@ -89,6 +92,9 @@ __device__ __forceinline__ uint32_t tc_at_rank(const void* p, uint32_t rank) {
 }
 __device__ __forceinline__ void tc_bar_arrive_at(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_bar_pass_on(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void tc_cluster_sync() {
   __syncthreads();
@@ -181,7 +187,11 @@ __device__ __forceinline__ bool tc_better(float za, int ia, float zb, int ib) { 
 // then 256 neurons, so that the samples' slabs serve twice as many.
 // What a tile took besides the multiplications, 2,000 cycles at 128 units: its biases asked for only one tile ahead (an HBM
 // latency per tile), and in WIDE the one warp that sums the rows' squares, element by element (26,000 cycles per tile at 512 units,
-// with packed pairs of four rows side by side 16,000; 512 samples x 100,003 neurons x 512 units 206 us before, 138 now with pairs).
+// with packed pairs of four rows side by side 16,000).
+// The rows' norms in pairs: the second block reads its half of a tile once the first block, which counts the copies, has passed
+// that on; at cluster scope this takes 1,000 cycles, little beside a tile but more than a slab has (512 samples x 100,003
+// neurons x 512 units 229 us).  WIDE pairs take the norms from global memory, where L2 has the rows (135 us): the read-back
+// warps, before they wait for the tile's scores.
 template <bool DUMP, bool WIDE, bool PAIR>      // DUMP: write every score out (threshold pass); else append the scores that reach the sample's threshold
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH, const TcParams p) {
@@ -208,6 +218,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   uint64_t* bar_drain = bars + 1 + 3 * NST + 2 * TC_NACC;  // after a wait has run out: the multiplications issued before have completed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  unsigned* best_slot = tmem_slot + 2;         // OWN_ROWS: the block's largest squared norm, as bits
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = PAIR ? blockIdx.x & 1u : 0u;       // in the pair: the first block counts arrivals and issues the multiplications
@@ -219,7 +230,8 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   // they pass through shared memory; up to four sample groups share a tile's rows (they all see the same tiles).
   constexpr int RL = ROWS / 32;                                    // rows per lane, shared by the blocks that hold the same rows
   const int nshare = (int)gridDim.y >= 4 && RL >= 4 ? 4 : ((int)gridDim.y >= 2 ? 2 : 1);
-  const bool norms = !DUMP && (int)blockIdx.y < nshare;
+  constexpr bool OWN_ROWS = WIDE && PAIR;                          // norms by the read-back warps
+  const bool norms = !DUMP && !OWN_ROWS && (int)blockIdx.y < nshare;
   const int nacc = WIDE ? (PAIR ? 2 : TC_NACC) : (p.H <= TC_N ? TC_NACC : 2);      // accumulators in use; the activations follow them
   const uint32_t acol = (uint32_t)(nacc * NT);
 
@@ -229,6 +241,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_landed + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
     for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, (PAIR ? 2 : 1) * TC_EPI / 32); }
     *abort_flag = 0;
+    *best_slot = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {      // tensor memory: all of it (one block per SM)
@@ -345,8 +358,8 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       const int nrr = RL / nshare;                     // rows of this block: nrr per lane
       // the bytes of a pair are counted in its first block, which tells the second
       auto arrived = [&](int st, int stround) {
-        tc_bar_wait<PAIR>(PAIR && rank == 1 ? bar_landed + st : bar_full + st, stround & 1, abort_flag);
-        if (PAIR && rank == 0 && lane == 0) tc_bar_arrive_at(tc_at_rank(bar_landed + st, 1u));
+        tc_bar_wait<PAIR, PAIR>(PAIR && rank == 1 ? bar_landed + st : bar_full + st, stround & 1, abort_flag);
+        if (PAIR && rank == 0 && lane == 0) tc_bar_pass_on(tc_at_rank(bar_landed + st, 1u));
       };
       for (int i = 0; i < my_tiles; ++i) {
         if (WIDE) {
@@ -451,6 +464,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     };
     if (et < NT)
       for (int i = 0; i < TC_BAHEAD; ++i) ask_bias(i);
+    float best = 0.f;                              // OWN_ROWS: the largest squared norm of the thread's rows
     int acc = 0, accround = 0;
     for (int i = 0; i < my_tiles; ++i) {
       const int tile = slice + i * p.nslices;
@@ -460,6 +474,27 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         asm volatile("cp.async.wait_group %0;" ::"n"(TC_BAHEAD) : "memory");      // tile i's are there
       }
       const float* tb = sb + (i & (TC_BT - 1)) * NT;
+      if (OWN_ROWS && !DUMP) {
+        // up to four groups share the tile's rows, and so do their blocks and a block's warps: 4, 8 or 16 lanes to a row
+        const int shares = (int)gridDim.y >= 4 ? 8 : ((int)gridDim.y >= 2 ? 4 : 2), share = 2 * (int)blockIdx.y + (int)rank;
+        const int lanes = 2 * shares, j = j0 + share * (NT / shares) + (warp - 3) * (32 / lanes) + lane / lanes;
+        if (share < shares) {
+          unsigned long long n0 = 0ull, n1 = 0ull;
+          if (j < p.N) {
+            const ulonglong2* r = reinterpret_cast<const ulonglong2*>(p.W2 + (size_t)j * p.H);
+#pragma unroll 8
+            for (int c = lane & (lanes - 1); c < p.H >> 2; c += lanes) {
+              const ulonglong2 w = r[c];
+              asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(n0) : "l"(w.x));
+              asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(n1) : "l"(w.y));
+            }
+          }
+          float n = (__uint_as_float((unsigned)n0) + __uint_as_float((unsigned)(n0 >> 32))) +
+                    (__uint_as_float((unsigned)n1) + __uint_as_float((unsigned)(n1 >> 32)));
+          for (int o = lanes / 2; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+          best = fmaxf(best, n);
+        }
+      }
       if (warp == 3) tc_bar_wait<PAIR>(bar_accfull + acc, accround & 1, abort_flag);      // one warp polls, the others sleep in the barrier
       asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");          // the accumulator is complete, the tile's biases are in place
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -521,6 +556,11 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       }
       if (++acc == nacc) { acc = 0; ++accround; }
     }
+    if (OWN_ROWS && !DUMP) {
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, d));
+      if (lane == 0) atomicMax(best_slot, __float_as_uint(best));
+    }
     if (!DUMP && s0 + row < p.B) {
       p.cand_cnt[(size_t)vslice * p.Bpad + s0 + row] = cnt < p.gbuf ? cnt : p.gbuf;
       if (cnt > p.gbuf) p.need_fix[s0 + row] = 1;          // candidates were dropped: the sample is scored exactly
@@ -549,6 +589,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
     else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
   }
+  if (OWN_ROWS && !DUMP && tid == 0) atomicMax(p.norm2max, *best_slot);
   if (tid == 0 && *abort_flag) atomicCAS(&p.st->status, 0, (int)DSLIDE_ERR_TIMEOUT);
 }
 
@@ -1090,7 +1131,7 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   if (!make_map(&tmW, c->W2, c->N, c->H, rows) || !make_map(&tmH, c->h, batch, c->H, TC_M)) return cudaErrorInvalidValue;
 
   TcParams p;
-  p.hdr2 = c->hdr2; p.h = c->h; p.cand = cand; p.cand_cnt = cand_cnt; p.dump = dump; p.tau = tau; p.need_fix = need_fix; p.norm2max = norm2; p.n_fix = n_fix; p.st = c->dstate;
+  p.hdr2 = c->hdr2; p.h = c->h; p.W2 = c->W2; p.cand = cand; p.cand_cnt = cand_cnt; p.dump = dump; p.tau = tau; p.need_fix = need_fix; p.norm2max = norm2; p.n_fix = n_fix; p.st = c->dstate;
   p.B = batch; p.Bpad = Bpad; p.H = c->H; p.N = c->N; p.dump_cols = dump_cols; p.gbuf = gbuf;
   const size_t tile_bytes = wide ? (size_t)rows * 128 + TC_SUB_BYTES : (size_t)((c->H + TC_KB - 1) / TC_KB) * rows * 128;
   int stages = (int)(((size_t)200 << 10) / tile_bytes);

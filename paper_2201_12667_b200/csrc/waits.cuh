@@ -11,9 +11,14 @@ constexpr long long DRAIN_CYCLES = 20000000LL;       // for what is in flight wh
 __device__ __forceinline__ uint32_t tc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // A try may sleep up to 2 us, so that a waiting warp issues little (all-neuron calls of 128 samples x 100,003 neurons x 512 units
 // 101.6 us without, 99.8 with; 1,024 x 100,003 x 64 109.3 and 108.3).
+// CLUSTER: what the arrivals' threads of the other blocks of the cluster had done is then visible too.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool tc_bar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+  if (CLUSTER)
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(2000u) : "memory");
+  else asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                : "=r"(ok) : "r"(bar), "r"(parity), "r"(2000u) : "memory");
   return ok != 0u;
 }
@@ -27,12 +32,12 @@ __device__ __forceinline__ void tc_give_up(volatile int* abort) {
 }
 // True once the phase of that parity has completed.  False when it has not within the limit -- the flag is then set -- or when
 // another wait of the block, or of the pair, has given up: every later wait returns at once.
-template <bool PAIR>
+template <bool PAIR, bool CLUSTER = false>
 __device__ __forceinline__ bool tc_bar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
   const uint32_t a = tc_smem(bar);
-  if (tc_bar_try(a, parity)) return true;
+  if (tc_bar_try<CLUSTER>(a, parity)) return true;
   const long long t0 = clock64();
-  while (!tc_bar_try(a, parity)) {
+  while (!tc_bar_try<CLUSTER>(a, parity)) {
     if (*abort) return false;
     if (clock64() - t0 > WAIT_CYCLES) { tc_give_up<PAIR>(abort); return false; }
   }

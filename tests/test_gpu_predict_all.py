@@ -13,10 +13,11 @@ pytestmark = pytest.mark.gpu
 SHAPES = [            # H, N, batch, k
     (4, 3001, 3, 1), (36, 129, 5, 10), (36, 128, 1, 64), (36, 100, 2, 5), (36, 40, 3, 64), (200, 20011, 130, 5),
     (252, 9000, 33, 64), (256, 5000, 129, 9), (260, 5000, 40, 5), (516, 3000, 131, 17), (1024, 2049, 260, 3), (1020, 700, 1, 64),
+    (132, 9000, 200, 3),
 ]
-PAIRS = [             # two multiprocessors to a tile: more than 192 units, more than 128 samples, enough tiles
+PAIRS = [             # two multiprocessors to a tile: more than 192 units, more than 128 samples, tiles that keep them busy
     (196, 19001, 256, 5), (200, 38017, 257, 9), (256, 18945, 256, 64), (224, 30011, 130, 3), (260, 38145, 140, 5), (292, 19001, 300, 5),
-    (1020, 13001, 300, 5), (132, 9000, 200, 3),
+    (1020, 13001, 300, 5),
 ]
 
 
@@ -64,6 +65,7 @@ def test_weights_that_are_not_finite():
 FLAGGED = [           # H, N, batch, k, samples whose filter cannot decide (of the batch)
     (4, 3001, 3, 1, 3), (36, 129, 5, 10, 1), (128, 2000, 20, 64, 20), (200, 5011, 260, 5, 9), (128, 20011, 1, 5, 1),
     (264, 700, 33, 17, 32), (1024, 2049, 40, 3, 8), (1020, 333, 9, 64, 9), (64, 4001, 300, 5, 300), (256, 20011, 200, 5, 70),
+    (300, 20011, 200, 5, 70),
 ]
 
 
@@ -132,5 +134,57 @@ def test_an_undecided_sample_is_everybodys_work():
         z = W2.astype(np.float64) @ h
         assert np.allclose(sc.cpu().numpy(), np.sort(z)[::-1][:5], rtol=1e-5) and set(ids.tolist()) == set(np.argsort(-z)[:5].tolist())
         assert best < 3.0, best
+    finally:
+        ds.dslide_destroy(ctx)
+
+
+NORMS = [             # H, N, batch: single blocks, wide ones, pairs, wide pairs; one to nine groups of samples
+    (64, 3001, 1), (128, 5003, 300), (160, 5003, 700), (300, 3001, 40),
+    (200, 20011, 200), (196, 19001, 300), (256, 20011, 1100), (260, 20011, 200), (516, 20011, 300), (300, 20011, 600), (292, 20011, 1100),
+]
+
+
+@pytest.mark.parametrize("H,N,B", NORMS)
+def test_the_norm_of_every_row_counts(H, N, B):
+    """A row whose two large weights cancel: its score is 1, the best by far, and 0 once weights lose their last bits, as in the
+    filter.  Only the row's norm in the error bound shows that the filter cannot decide, wherever in a tile the row lies (the
+    halves of a tile are in the shared memory of two blocks, its rows are shared out between the groups of samples)."""
+    import torch
+    from paper_2201_12667_b200 import binding as ds
+    from tests.gpu_harness import to_dev
+    k = 4
+    r = np.random.default_rng(H + B)
+    ctx = ds.dslide_init(ds.make_config(input_dim=50, hidden_dim=H, output_dim=N, hash_family=workloads.SIMHASH, K=4, L=2, bucket_cap=16, max_batch=B))
+    try:
+        W1 = r.standard_normal((50, H)).astype(np.float32)
+        W1[:, :2] = 0
+        b1 = np.zeros(H, np.float32)
+        b1[:2] = 1                                              # two units that are 1 for every sample
+        W2 = (r.standard_normal((N, H)) * (0.03 / np.sqrt(H))).astype(np.float32)
+        W2[:, :2] = 0
+        b2 = np.full(N, -0.01, np.float32)
+        for name, x in (("W1", W1), ("b1", b1), ("b2", b2)):
+            ds.dslide_set_tensor(ctx, name, x)
+        batch = to_dev([np.arange(B + 1, dtype=np.int32), r.integers(0, 50, B).astype(np.int32), r.uniform(0.5, 1, B).astype(np.float32)])
+        ids, sc = torch.empty(B, k, dtype=torch.int32, device="cuda"), torch.empty(B, k, device="cuda")
+
+        def best():
+            ds.dslide_set_tensor(ctx, "W2", W2)
+            ds.dslide_predict_topk(ctx, B, *batch, k, 1, ids, sc)
+            ds.dslide_sync(ctx)
+            return ids.cpu().numpy().copy(), sc.cpu().numpy().copy()
+
+        for first in (0, 256 * (N // 512)):
+            for at in (0, 31, 63, 64, 100, 127, 128, 161, 200, 255):
+                row = min(first + at, N - 1)
+                keep = W2[row].copy()
+                W2[row] = 0
+                ids0, sc0 = best()                              # the row scores -0.01, which others beat
+                assert (sc0[:, -1] > 0).all() and (sc0 < 0.9).all()
+                W2[row, :2] = 4097, -4096
+                ids1, sc1 = best()
+                assert (ids1[:, 0] == row).all() and np.allclose(sc1[:, 0], 0.99, rtol=1e-6), row
+                assert np.allclose(sc1[:, 1:], sc0[:, :-1], rtol=1e-4, atol=1e-6) and (ids1[:, 1:] == ids0[:, :-1]).mean() > 0.99
+                W2[row] = keep
     finally:
         ds.dslide_destroy(ctx)
