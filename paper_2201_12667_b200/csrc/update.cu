@@ -390,7 +390,10 @@ __device__ __forceinline__ void finish_hdr(const UpdParams& p, RowHdr* hd, bool 
     if (lane == 1) reinterpret_cast<int2*>(hd)[1] = make_int2(__float_as_int(mb), __float_as_int(vb));
   } else {
     if (lane == 0) hd->cnt = 0u;
-    if (p.L1 > 0 && lane < p.Hw) p.cmask1[(size_t)(hd - p.hdr1) * p.Hw + lane] = 0u;     // the row's unit mask, for the next step
+    if (p.L1 > 0) {
+      __syncwarp();                  // the other lanes have read the words for their units
+      if (lane < p.Hw) p.cmask1[(size_t)(hd - p.hdr1) * p.Hw + lane] = 0u;     // the row's unit mask, for the next step
+    }
   }
 }
 

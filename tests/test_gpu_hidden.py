@@ -16,6 +16,7 @@ if torch.cuda.is_available():
     from paper_2201_12667_b200 import workloads
     from tests.gpu_harness import Pair
     from tests.test_gpu_parity import ACT_TOL, W_TOL, compare_forward, compare_weights
+    from tests.test_gpu_shapes import dense_features_batch
 
 SIMHASH, DWTA = 0, 1
 
@@ -73,6 +74,43 @@ def test_sampled_hidden_layer_step(H, hK, hL, hcap, family):
         # the tables depend on the signs of sums over each side's own weights (equal within the weight bar only)
         go, oo = ds.dslide_get_tensor(pr.ctx, "bucket1_off"), pr.o.get("bucket1_off")
         assert go.shape == oo.shape and go.reshape(hL, -1)[:, -1].tolist() == [H] * hL
+    finally:
+        pr.close()
+
+
+@pytest.mark.parametrize("H,D,nnz", [
+    (260, 90, 60),       # a last piece of one lane; all rows hot: slices, piece by piece
+    (260, 300, 40),      # rows past their slots, some hot
+    (200, 90, 60),       # one piece, hot
+    (516, 90, 60),       # three pieces, hot
+    (516, 1400, 420),    # 1,400 hot rows against a list of 1,024: the others walk their masks piece by piece
+    (1024, 90, 60),      # four pieces, hot
+    (1024, 2500, 100),   # rows of a few touches
+])
+def test_long_rows_under_unit_masks(H, D, nnz):
+    """Rows of W1 of more than 128 units, updated piece by piece in the units that some sample touched them for: every
+    element of a row as often and with the same gradient as in the oracle, the others not at all."""
+    hK, hL, hcap = 4, 6, 16
+    pr = Pair(D=D, H=H, N=2003, family=SIMHASH, K=6, L=6, bucket_cap=12, max_batch=150, max_labels=16, lr=1e-4, seed=7,
+              hidden_K=hK, hidden_L=hL, hidden_cap=hcap)
+    rng = np.random.default_rng(H + D)
+    try:
+        for i in range(2):
+            batch = dense_features_batch(rng, 150, D, 2003, nnz, 3)
+            before = {n: ds.dslide_get_tensor(pr.ctx, n).reshape(D, H) for n in ("W1", "mW1", "vW1")}
+            lo = pr.o.train_step(*batch)
+            lg = pr.gpu_step(batch)
+            assert abs(lo - lg) <= (ACT_TOL if i == 0 else W_TOL) * abs(lo)
+            compare_weights(pr)
+            if i == 0:
+                hact = pr.o.get("hact").reshape(150, H).astype(bool)
+                touched = np.zeros((D, H), dtype=bool)
+                for s in range(150):
+                    touched[batch[1][batch[0][s]:batch[0][s + 1]]] |= hact[s]
+                for n, a in before.items():
+                    b = ds.dslide_get_tensor(pr.ctx, n).reshape(D, H)
+                    assert np.array_equal(a[~touched].view(np.uint32), b[~touched].view(np.uint32)), n
+                assert 0.05 < hact.mean() < 0.95
     finally:
         pr.close()
 
