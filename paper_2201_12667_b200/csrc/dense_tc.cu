@@ -40,8 +40,9 @@ constexpr int TC_H_TMEM = 256;     // hidden layers up to this width sit in tens
 constexpr int TC_H_SINGLE = 192;   // up to this width two tiles fit a block's shared memory
 constexpr int TC_WIDE_STAGES = TC_STAGES;      // WIDE: pairs of slabs (32 units of the samples, 32 units of the neurons) in flight
 constexpr int TC_RANK_CAP = 24;    // the threshold's rank in the subset grows with k up to this
-constexpr int TC_GBUF_MIN = 64;    // candidate slots per (buffer, sample) at least, many times the expected fill: a buffer takes the 32 neighbouring
-                                   // neurons of its tiles, which a trained model may favour together; one that runs over sends the sample to the exact scan
+constexpr int TC_GBUF_MIN = 2;     // candidate slots per (buffer, sample) at least, in neighbouring neurons that the buffer takes of a tile (32, or 64 of
+                                   // a wide pair's): many times the expected fill, but a trained model may favour neighbours together, and a buffer
+                                   // that runs over sends the sample to the exact scan (512 x 100,003 neurons x 512 units all undecided: 3,300 us for 137)
 constexpr int TC_TARGET = 64;      // candidates aimed at per sample: TC_TARGET x min(cap, TC_RANK_CAP)
 constexpr int TC_SUBSET = 64;      // the threshold pass scores every TC_SUBSET-th tile
 constexpr int TC_SUB_BYTES = TC_M * 128;               // one 32-unit slab of 128 rows
@@ -1109,7 +1110,7 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   int rank = (want * TC_TARGET + stride - 1) / stride;
   if (rank > want) rank = want;
   if (rank < 4) rank = 4;
-  int gbuf = TC_GBUF_MIN;
+  int gbuf = TC_GBUF_MIN * NT / TC_SPLIT;
   while (gbuf * nvs < 4 * rank * stride) gbuf <<= 1;
   const size_t off_dump = off_cand + up((size_t)nvs * Bpad * gbuf * sizeof(int2));
   const size_t need = off_dump + (size_t)Bpad * dump_cols * 4;
