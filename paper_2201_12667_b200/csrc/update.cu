@@ -23,7 +23,7 @@
 //              sums in slice order (rows of W1 that have been hot before find their coefficients in a
 //              table line the forward kernel fills, instead of searching).  Warps draw tickets (the first two are fixed by the warp's number,
 //              the others come from a counter): hot slices, then listed rows, then the ordinary rows four
-//              at a time (of up to 128 units the last few thousand two at a time).  Adam is applied to the touched rows only; untouched rows are neither read
+//              at a time (the last few thousand two or one at a time: launch_update).  Adam is applied to the touched rows only; untouched rows are neither read
 //              nor written.  The warp that updates a row resets its count and mask for the next step.
 //              The first blocks of the grid update the hidden bias and reduce the batch loss.
 //              Rows of more than 128 units are not held: a warp takes one row at a time, piece by piece (long_row).
@@ -1019,12 +1019,18 @@ cudaError_t launch_update(Ctx* c, int batch, const int32_t* row_ptr, const int32
   }
   const int smem = UPD_WARPS * 32 * 4;
   const int width = c->H <= 128 ? 0 : c->H <= 128 * LONG_P ? 1 : 2;
+  // The last rows go out one by one, so that small batches keep every warp busy and a warp with one row waits for one chain
+  // of loads (a step of 1 sample 37 -> 33 us at 256 units, 89 -> 78 at 1,024, of 16 samples 108 -> 98 at 1,024); beyond 512
+  // units and 32 samples four at a time, with the next row asked into L2 meanwhile (64 samples, 768 units: 90 us, one by one 98).
+  const bool by_one = c->H <= 512 || batch <= 32;
   if (c->L1 > 0) {        // sampled hidden layer: rows of W1 are updated under their unit masks
     if (width == 0) return launch_k_update<0, 2, true>(c, p, smem);
-    return width == 1 ? launch_k_update<1, UPD_TROWS, true>(c, p, smem) : launch_k_update<2, UPD_TROWS, true>(c, p, smem);
+    if (width == 1) return launch_k_update<1, 1, true>(c, p, smem);
+    return by_one ? launch_k_update<2, 1, true>(c, p, smem) : launch_k_update<2, UPD_TROWS, true>(c, p, smem);
   }
   if (width == 0) return launch_k_update<0, 2, false>(c, p, smem);
-  return width == 1 ? launch_k_update<1, UPD_TROWS, false>(c, p, smem) : launch_k_update<2, UPD_TROWS, false>(c, p, smem);
+  if (width == 1) return launch_k_update<1, 1, false>(c, p, smem);
+  return by_one ? launch_k_update<2, 1, false>(c, p, smem) : launch_k_update<2, UPD_TROWS, false>(c, p, smem);
 }
 
 }  // namespace dslide
