@@ -240,7 +240,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     tc_bar_init(bar_a, PAIR ? 8 : 4);            // a warp each
     tc_bar_init(bar_drain, 1);
     for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_landed + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
-    for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, (PAIR ? 2 : 1) * TC_EPI / 32); }
+    for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, PAIR ? 2 * TC_EPI / 32 : TC_EPI); }
     *abort_flag = 0;
     *best_slot = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -550,11 +550,11 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) {
-        if (PAIR) tc_bar_arrive_at(tc_at_rank(bar_accempty + acc, 0u));
-        else tc_bar_arrive(bar_accempty + acc);
+      if (PAIR) {
+        __syncwarp();
+        if (lane == 0) tc_bar_arrive_at(tc_at_rank(bar_accempty + acc, 0u));
       }
+      else tc_bar_arrive(bar_accempty + acc);      // every thread: up to 1 % faster than a lane for its warp
       if (++acc == nacc) { acc = 0; ++accround; }
     }
     if (OWN_ROWS && !DUMP) {
@@ -1135,24 +1135,29 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   p.hdr2 = c->hdr2; p.h = c->h; p.W2 = c->W2; p.cand = cand; p.cand_cnt = cand_cnt; p.dump = dump; p.tau = tau; p.need_fix = need_fix; p.norm2max = norm2; p.n_fix = n_fix; p.st = c->dstate;
   p.B = batch; p.Bpad = Bpad; p.H = c->H; p.N = c->N; p.dump_cols = dump_cols; p.gbuf = gbuf;
   const size_t tile_bytes = wide ? (size_t)rows * 128 + TC_SUB_BYTES : (size_t)((c->H + TC_KB - 1) / TC_KB) * rows * 128;
-  int stages = (int)(((size_t)200 << 10) / tile_bytes);
-  if (stages > (wide ? TC_WIDE_STAGES : TC_STAGES)) stages = wide ? TC_WIDE_STAGES : TC_STAGES;
-  p.stages = stages;
-  const size_t smem = 1024 + tile_bytes * stages + (size_t)TC_BT * NT * 4 + (2 + 3 * TC_STAGES + 2 * TC_NACC) * 8 + 64;
+  auto smem_of = [&](int st) { return 1024 + tile_bytes * st + (size_t)TC_BT * NT * 4 + (2 + 3 * TC_STAGES + 2 * TC_NACC) * 8 + 64; };
+  // Tiles in flight: six of a narrow model, but beyond three only what 144 KB hold (300 samples x 600,011 neurons x 64 units: 143 us
+  // with three or six, 139 with four), and in the threshold pass no more than a block has tiles, mostly one: its blocks and those of
+  // the kernels that follow then find room side by side (1 x 5,003 x 64: 28.3 us, with six stages 29.6; 1 x 5,003 x 128 29.1 and 30.4).
+  // Pairs keep to one block per multiprocessor: two that wait for tensor memory of the same two could each hold what the other needs.
+  const int fit = (int)(((size_t)200 << 10) / tile_bytes), lean = (int)(((size_t)144 << 10) / tile_bytes);
+  const int stages = wide ? min(TC_WIDE_STAGES, fit) : min(fit, max(3, min(lean, TC_STAGES)));
+  const int sub_tiles = (nsub + nslices_sub - 1) / nslices_sub;
+  const int stages_sub = wide || pair ? stages : min(stages, sub_tiles);
   auto k_sub = pair ? (wide ? k_dense_tc<true, true, true> : k_dense_tc<true, false, true>) : (wide ? k_dense_tc<true, true, false> : k_dense_tc<true, false, false>);
   auto k_all = pair ? (wide ? k_dense_tc<false, true, true> : k_dense_tc<false, false, true>) : (wide ? k_dense_tc<false, true, false> : k_dense_tc<false, false, false>);
-  if ((e = cudaFuncSetAttribute(k_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(stages_sub))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(stages))) != cudaSuccess) return e;
   {
     LaunchScope ls(c, KID_PREDICT);
-    p.nslices = nslices_sub; p.ntiles = nsub; p.tile_stride = stride;
+    p.nslices = nslices_sub; p.ntiles = nsub; p.tile_stride = stride; p.stages = stages_sub;
     // each kernel of the call may be placed while the kernel before it drains (they wait for it before they read or
     // write anything); the first follows the hidden-layer kernel in the same way
-    if ((e = launch_tc(k_sub, pair, nslices_sub, groups, smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
+    if ((e = launch_tc(k_sub, pair, nslices_sub, groups, smem_of(stages_sub), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_tau, dim3(Bpad), dim3(TAU_THREADS), 0, c->stream, (const float*)dump, dump_cols, rank, tau)) != cudaSuccess)
       return e;
-    p.nslices = nslices; p.ntiles = ntiles; p.tile_stride = 1;
-    if ((e = launch_tc(k_all, pair, nslices, groups, smem, c->stream, tmW, tmH, p)) != cudaSuccess) return e;
+    p.nslices = nslices; p.ntiles = ntiles; p.tile_stride = 1; p.stages = stages;
+    if ((e = launch_tc(k_all, pair, nslices, groups, smem_of(stages), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_refine, dim3(batch), dim3(RF_THREADS), 0, c->stream, (const float*)c->W2, (const RowHdr*)c->hdr2,
                               (const float*)c->h, (const int2*)cand, (const int*)cand_cnt, gbuf, (const float*)tau, Bpad,
                               (const unsigned int*)norm2, batch, c->H, c->N, cap, nvs, k, out_ids, out_scores, (const int*)need_fix, n_fix, fix_list)) !=
