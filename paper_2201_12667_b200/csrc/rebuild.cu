@@ -355,13 +355,16 @@ k_hash_neurons(const float* __restrict__ W2, const int32_t* __restrict__ hidx, u
 // Bound by the loads from shared memory (4 bytes per row, function and coordinate: 30 GB at 253,855 rows of 200 units and 450
 // functions).  With one row per lane, as before, the instructions around the loads bound it: a rebuild of those rows took
 // 2,814 us and now takes 1,506; 128 units 1,818 and 968; 20,011 rows of 1,024 units 6,757 and 3,839 (one row per lane
-// here too, but 32 warps for one tile instead of eight).
+// here too, but 13 warps for one tile instead of eight).  Where a block that fills a multiprocessor has fewer tables at a time
+// than it could have warps, the functions of a table are shared out between warps, and the code's bits meet in shared memory:
+// 6 tables of 24 functions, 20,011 rows of 256 units 670 us with one row per lane, 723 with a warp per table, 630 so.
 constexpr int HNS_SMEM = 224 * 1024;
+constexpr int HNS_WARPS = 24;              // of a block that has a multiprocessor to itself
 constexpr int HNS_MIN_TABLES = 8;          // more rows per lane only while the functions of so many tables fit beside the tile
-template <int R>
+template <int R, bool SPLIT>      // SPLIT: `parts` warps share a table's functions
 __global__ void __launch_bounds__(1024)
 k_hash_neurons_sim(const float* __restrict__ W2, const int32_t* __restrict__ hidx, const int32_t* __restrict__ hsign, uint32_t* keys, int N, int H, int K,
-                   int L, int m, int per) {
+                   int L, int m, int per, int parts) {
   constexpr int ROWS = 32 * R, ES = 4 * R;
   extern __shared__ __align__(16) unsigned char hn_smem[];
   const int ld = H + 1;                                               // odd: a warp's loads of one coordinate spread over the banks
@@ -376,6 +379,9 @@ k_hash_neurons_sim(const float* __restrict__ W2, const int32_t* __restrict__ hid
   }
   if (threadIdx.x < 32)
     for (int u = 0; u < R; ++u) reinterpret_cast<float*>(hn_smem)[(threadIdx.x * ld + H) * R + u] = 0.f;
+  uint32_t* codes = reinterpret_cast<uint32_t*>(fn + (size_t)per * K * mp);      // SPLIT: [table][row], put together from the warps' bits
+  if (SPLIT)
+    for (int e = threadIdx.x; e < nt * ROWS; e += blockDim.x) codes[e] = 0u;
   const unsigned char* v = hn_smem + (size_t)lane * ld * ES;
   const int ntiles = (N + ROWS - 1) / ROWS;
   for (int tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
@@ -394,11 +400,12 @@ k_hash_neurons_sim(const float* __restrict__ W2, const int32_t* __restrict__ hid
         else *to = x[0];
       }
     __syncthreads();
-    for (int t = warp; t < nt; t += nwarps) {
+    for (int it = warp; it < (SPLIT ? nt * parts : nt); it += nwarps) {
+      const int t = SPLIT ? it / parts : it, part = it - t * parts, k1 = SPLIT ? (part + 1) * K / parts : K;
       uint32_t code[R];
 #pragma unroll
       for (int u = 0; u < R; ++u) code[u] = 0u;
-      for (int k = 0; k < K; ++k) {
+      for (int k = SPLIT ? part * K / parts : 0; k < k1; ++k) {
         const uint4* q4 = reinterpret_cast<const uint4*>(fn + (size_t)(t * K + k) * mp);
         unsigned long long s0 = 0ull, s1 = 0ull;
         float s = 0.f;
@@ -427,9 +434,22 @@ k_hash_neurons_sim(const float* __restrict__ W2, const int32_t* __restrict__ hid
 #pragma unroll
         for (int u = 0; u < R; ++u) code[u] |= (sum[u] >= 0.f ? 1u : 0u) << k;
       }
+      if (SPLIT) {
+#pragma unroll
+        for (int u = 0; u < R; ++u) atomicOr(codes + t * ROWS + 32 * u + lane, code[u]);
+        continue;
+      }
 #pragma unroll
       for (int u = 0; u < R; ++u)
         if (lane + 32 * u < rows) keys[(size_t)(t0 + t) * N + j0 + 32 * u + lane] = code[u];
+    }
+    if (SPLIT) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < nt * ROWS; e += blockDim.x) {
+        const int t = e / ROWS, r = e - t * ROWS;
+        if (r < rows) keys[(size_t)(t0 + t) * N + j0 + r] = codes[e];
+        codes[e] = 0u;
+      }
     }
   }
 }
@@ -1201,7 +1221,7 @@ static cudaError_t launch_dwta8(Ctx* c, int smem) {
 
 template <int R>
 static cudaError_t launch_sim(Ctx* c, int tile_bytes, int table_bytes) {
-  // as many tables at a time as find room; more shares than that where there are few tiles
+  // as many tables at a time as find room; more shares than that where the tiles leave multiprocessors idle
   const int ntiles = (c->N + 32 * R - 1) / (32 * R);
   int per = (HNS_SMEM - tile_bytes) / table_bytes;
   if (per > c->L) per = c->L;
@@ -1210,20 +1230,28 @@ static cudaError_t launch_sim(Ctx* c, int tile_bytes, int table_bytes) {
   if (shares > c->L) shares = c->L;
   per = (c->L + shares - 1) / shares;
   shares = (c->L + per - 1) / per;
+  // Few tables at a time are few warps: the functions of a table are then shared out too, where the block has a multiprocessor
+  // to itself (smaller blocks fill it by their number)
+  const int code_bytes = per * 32 * R * 4;
+  int parts = 1;
+  if (tile_bytes + per * table_bytes > 113 * 1024 && per < HNS_WARPS && tile_bytes + per * table_bytes + code_bytes <= HNS_SMEM)
+    parts = min(c->K, HNS_WARPS / per);
   int warps = 8;                              // the rounds that the tables take decide, then the warps' number
+  const int items = per * parts;
   for (int w = 9; w <= 32; ++w)
-    if ((per + w - 1) / w * w <= (per + warps - 1) / warps * warps) warps = w;
-  const int smem = tile_bytes + per * table_bytes;
-  cudaError_t e = cudaFuncSetAttribute(k_hash_neurons_sim<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if ((items + w - 1) / w * w <= (items + warps - 1) / warps * warps) warps = w;
+  const int smem = tile_bytes + per * table_bytes + (parts > 1 ? code_bytes : 0);
+  auto kern = parts > 1 ? k_hash_neurons_sim<R, true> : k_hash_neurons_sim<R, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hash_neurons_sim<R>, 32 * warps, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem);
   if (e != cudaSuccess) return e;
   int nb = c->num_sms * (per_sm > 0 ? per_sm : 1) / shares;
   if (nb < 1) nb = 1;
   if (nb > ntiles) nb = ntiles;
   LaunchScope ls(c, KID_HASH_NEURONS);
-  k_hash_neurons_sim<R><<<dim3(nb, shares), 32 * warps, smem, c->stream>>>(c->W2, c->hash_idx, c->hash_sign, c->keysA, c->N, c->H, c->K, c->L, c->fn_len, per);
+  kern<<<dim3(nb, shares), 32 * warps, smem, c->stream>>>(c->W2, c->hash_idx, c->hash_sign, c->keysA, c->N, c->H, c->K, c->L, c->fn_len, per, parts);
   return cudaGetLastError();
 }
 

@@ -32,16 +32,20 @@ def test_tables(family, K, L, N, H, cap):
         pr.close()
 
 
-@pytest.mark.parametrize("K,L,N,H", [
-    (7, 70, 20011, 128),     # four rows per lane, all tables at a time
-    (12, 60, 1601, 400),     # four rows per lane, the functions of some tables beside them
-    (6, 33, 129, 440),       # two rows per lane, a last tile of one row
-    (9, 40, 801, 856),       # one or two rows per lane, few tables at a time
-    (5, 30, 333, 1024),      # one row per lane
-    (8, 1, 31, 100),         # one table, less than a tile
+@pytest.mark.parametrize("K,L,N,H,nnz", [
+    (7, 70, 20011, 128, 0),     # four rows per lane, all tables at a time
+    (12, 60, 1601, 400, 0),     # four rows per lane, the functions of some tables beside them
+    (6, 33, 129, 440, 0),       # two rows per lane, a last tile of one row
+    (9, 40, 801, 856, 0),       # one or two rows per lane, few tables at a time
+    (5, 30, 333, 1024, 0),      # one row per lane
+    (8, 1, 31, 100, 0),         # one table, less than a tile
+    (17, 5, 1601, 256, 0),      # few tables at a time: a table's functions shared out between warps
+    (5, 7, 4001, 400, 0),       # the same, every function by a warp of its own
+    (18, 3, 333, 1024, 0),      # the same with one row per lane
+    (13, 4, 700, 600, 600),     # dense projections
 ])
-def test_simhash_tables_at_every_width(K, L, N, H):
-    pr = Pair(D=40, H=H, N=N, family=SIMHASH, K=K, L=L, bucket_cap=16, max_batch=4, seed=K + N)
+def test_simhash_tables_at_every_width(K, L, N, H, nnz):
+    pr = Pair(D=40, H=H, N=N, family=SIMHASH, K=K, L=L, srp_nnz=nnz, bucket_cap=16, max_batch=4, seed=K + N)
     try:
         same_tables(pr)
         ds.dslide_rebuild_tables(pr.ctx)
