@@ -422,7 +422,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     // Per 32 columns the bias is added; then, threshold pass: the scores are written out; filter pass: which of them
     // reach the sample's threshold (32 independent comparisons, a bit each), then the appends of those that do.
     const int q = warp & 3;                 // a warp reaches the 32 lanes of tensor memory of its number modulo four
-    const int half = (warp - 3) >> 2;       // which share of a tile's 128 columns
+    const int half = (warp - 3) >> 2;       // which share of a tile's columns
     const int row = 32 * q + lane;          // sample inside the block
     const int et = tid - 96;                // the first NT read-back threads (whole warps) fetch the tile's biases
     const int vslice = slice * TC_SPLIT + half;    // buffers are kept per (slice, share of the columns)
@@ -1059,11 +1059,11 @@ static cudaError_t launch_tc(void (*kernel)(const CUtensorMap, const CUtensorMap
 }
 
 // Whether two multiprocessors share a tile of W2 and 256 samples.  The tile then crosses from L2 once instead of twice, and a
-// stage takes half the shared memory, but a pair's instruction takes as long as two blocks' (124 cycles for 256 samples x
-// 128 neurons x 8 units: the tensor pipe, not the loads, is the bound).  So it pays where a block has room for one tile only
+// stage takes half the shared memory; the multiplications take as long as in two blocks (63 to 68 cycles for 256 samples x
+// 128 neurons x 8 units, as for 128 x 128 x 8 in a block; of the 2,840 cycles of a tile of 200 units they are 1,650).  It pays where a block has room for one tile only
 // (more than 192 units), or streams the activations with the tiles (more than 256): us for a call of 1,024 samples x
-// 253,855 neurons x 200 units 371 by single blocks and 258 by pairs, 512 x 4,000,000 x 256 2,467 and 1,897, 512 x 100,003 x
-// 512 206 and 138; not at 160 units (300 x 100,003: 69 and 80) or 128 (147.9 and 148.8 for 670,091).  And where the tiles
+// 253,855 neurons x 200 units 371 by single blocks and 258 by pairs, 512 x 4,000,000 x 256 2,600 and 1,850, 512 x 100,003 x
+// 512 206 and 135; not at 160 units (300 x 100,003: 69 and 80) or 128 (147.9 and 148.8 for 670,091).  And where the tiles
 // keep the pairs busy: a round of tiles takes a pair 0.7 of a block's time, at more than 256 units 1.2 for twice the tile.
 static bool use_pairs(const Ctx* c, int batch) {
   if (batch <= TC_M || c->H <= TC_H_SINGLE) return false;

@@ -8,7 +8,7 @@
 // it); a bit mask of the samples of any further touches, whose pairs up to touch PAIR_T are kept in a
 // side array as well; and two lists of (row, first-touching sample) for the distinct touched rows.
 //
-//   k_update : a warp works on two rows of the row lists at a time; the loads of a row's weights and
+//   k_update : a warp works on two rows of the row lists at a time (of up to 128 units); the loads of a row's weights and
 //              moments, of its record and of the first-touching sample's row (h for W2, dh for W1) are
 //              all issued together.  A row touched by one sample takes its gradient from slot 0; a row
 //              touched by up to ROW_SLOTS samples from its slots, put in ascending sample order; a row
@@ -83,14 +83,14 @@ __device__ __forceinline__ void axpy4(float4& a, float g, const float4 x) {
   a.x = fmaf(g, x.x, a.x); a.y = fmaf(g, x.y, a.y); a.z = fmaf(g, x.z, a.z); a.w = fmaf(g, x.w, a.w);
 }
 
-// The pieces of one layer's update: the weight / moment arrays, the rows that multiply the
-// coefficients (h for W2, dh for W1), the per-row masks and the per-row records (touch count, slots and,
-// for W2, the bias with its moments).
 // Asks L2 for `bytes` (a multiple of 16, from a 16-byte boundary); nothing comes back to the multiprocessor.
 __device__ __forceinline__ void l2_fetch(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// The pieces of one layer's update: the weight / moment arrays, the rows that multiply the
+// coefficients (h for W2, dh for W1), the per-row masks and the per-row records (touch count, slots and,
+// for W2, the bias with its moments).
 struct Side {
   float *W, *M, *V;
   const float* src;
@@ -223,7 +223,8 @@ __device__ __forceinline__ void sort_slots(int2 sl, int total, int* scr, int& s_
 
 // Gradient of a row touched by more than ROW_SLOTS samples, restricted to the samples of the mask words
 // [w0, w1): the samples of the slots and of the mask, ascending.  Up to 32 samples at a time are listed
-// in the warp's scratch, their coefficients looked up in parallel, then added in order.  Clears the mask.
+// in the warp's scratch, their coefficients looked up in parallel, then added in order.  CLEAR: clears the mask on the way
+// (a long row's pieces all read it, and clear_mask follows the last).
 template <int NCH, bool CLEAR>
 __device__ __forceinline__ void sum_masked(const UpdParams& p, const Side& sd, const int* rowptr, int row,
                                            int slot_s, int w0, int w1, int* scr, float4 (&acc)[NCH], float& csum,
@@ -314,7 +315,7 @@ __device__ __forceinline__ void adam_store(const UpdParams& p, const Side& sd, s
   }
 }
 
-// Gradient and Adam of a row of more than 256 units whose n <= 32 touches lane k holds as (s_mine, g_mine), in order: the row
+// Gradient and Adam of a row of more than 128 units whose n <= 32 touches lane k holds as (s_mine, g_mine), in order: the row
 // is walked in pieces of LONG_P x 128 units, so that neither its weights and moments nor its gradient are held whole and
 // sixteen warps fit a multiprocessor.  (Held whole, rows of 1,024 units left eight warps and 492 bytes of spills: a step of
 // 1,024 samples over 50,021 neurons took 759 us, now 613; 512 units 373 and 300; 256 units, two rows held at a time, 181
@@ -633,7 +634,8 @@ __device__ __forceinline__ void medium_item(const UpdParams& p, const int* rowpt
 }
 
 // Work is handed out in tickets from one counter: first the slices of the hot rows (the longest items), then
-// the listed rows with more than ROW_SLOTS touches, then the ordinary rows, UPD_TROWS per ticket (small tickets keep the tail of the kernel short).
+// the listed rows with more than ROW_SLOTS touches, then the ordinary rows, UPD_TROWS per ticket and the last ones G (small
+// tickets keep the tail of the kernel short).
 constexpr int UPD_TROWS = 4;
 
 template <int PIECES, int G, bool UMASK>
@@ -971,13 +973,13 @@ static cudaError_t launch_k_update(Ctx* c, const UpdParams& p, int smem) {
   // the kernel needs little shared memory: the rest of the unified store serves as cache for the h / dh rows
   e = cudaFuncSetAttribute(k_update<PIECES, G, UMASK>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
   if (e != cudaSuccess) return e;
-  // one wave: the blocks for the hidden bias come first, the rest fill the remaining block slots of the device
+  // One wave of blocks for the rows, and the blocks for the hidden bias, which come first and soon leave their places to the
+  // last of the others (those begin a few microseconds late, with their own first tickets).
   const int naux = (c->H + 31) / 32;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update<PIECES, G, UMASK>, UPD_THREADS, smem);
   if (e != cudaSuccess) return e;
-  int nblocks = c->num_sms * (per_sm > 0 ? per_sm : 1);
-  nblocks += naux;           // they soon make room for as many more
+  const int nblocks = c->num_sms * (per_sm > 0 ? per_sm : 1) + naux;
   LaunchScope ls(c, KID_ADAM);
   e = launch_dependent(k_update<PIECES, G, UMASK>, dim3(nblocks), dim3(UPD_THREADS), (size_t)smem, c->stream, p);
   if (e != cudaSuccess) return e;
