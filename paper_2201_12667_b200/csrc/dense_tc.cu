@@ -723,13 +723,13 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
     const float4* r = reinterpret_cast<const float4*>(W2 + (size_t)j * H);
     float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
     for (int c = lane; c < H4; c += 32) {
-      const float4 w = __ldg(r + c), x = h4[c];
+      const float4 w = r[c], x = h4[c];
       d0 = fmaf(w.x, x.x, d0); d1 = fmaf(w.y, x.y, d1); d2 = fmaf(w.z, x.z, d2); d3 = fmaf(w.w, x.w, d3);
     }
     float d = (d0 + d1) + (d2 + d3);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-    if (lane == 0) ez[e] = __ldg(&hdr2[j].b) + d;
+    if (lane == 0) ez[e] = hdr2[j].b + d;
   }
   // |h|^2 of the sample
   float hs = 0.f;
@@ -845,14 +845,14 @@ __global__ void __launch_bounds__(XS_THREADS, 2) k_scan_all(const ScanParams p) 
 #pragma unroll
       for (int r = 0; r < XS_ROWS; ++r) row[r] = reinterpret_cast<const float4*>(p.W2 + (size_t)min(j0 + r, je - 1) * H);
       const int j = j0 + mr;
-      const float bias = j < je ? __ldg(&p.hdr2[j].b) : 0.f;
+      const float bias = j < je ? p.hdr2[j].b : 0.f;
       float v[32];
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = 0.f;
       for (int c = lane; c < H4; c += 32) {
         float4 w[XS_ROWS];
 #pragma unroll
-        for (int r = 0; r < XS_ROWS; ++r) w[r] = __ldg(row[r] + c);
+        for (int r = 0; r < XS_ROWS; ++r) w[r] = row[r][c];
 #pragma unroll
         for (int s = 0; s < XS_SG; ++s) {
           const float4 x = hs4[s * H4 + c];
