@@ -16,6 +16,7 @@
 // one pass when the set is larger than that space).  Optional steps of the selection: densification
 // of all-zero DWTA bins of the query (Section 4.1) and the sampling budget of Section 3.7.
 #include "common.cuh"
+#include "waits.cuh"
 
 namespace dslide {
 
@@ -96,18 +97,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
-// Waits for the phase with the given parity; gives up after a bounded number of polls (false).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  const uint32_t a = smem_u32(bar);
-  for (int it = 0; it < (1 << 22); ++it) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(a), "r"(parity) : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
 // The touch that takes a row past ROW_SLOTS touching samples enters the row in the list of rows that a warp of
 // the update kernel sums from slots and mask; the touch that takes it past HOT_T enters it in the list of rows
 // summed in slices.  The row's count word is marked so that the update kernel knows where the row is listed.
@@ -651,7 +640,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     }
   }
   if (bad || too_many_labels) {
-    if (p.hash_sm_off >= 0 && !p.dense) mbar_wait(sh_bar2, 0u);     // no copy into this block may be left in flight
+    if (p.hash_sm_off >= 0 && !p.dense) bar_wait_limited(sh_bar2, 0u);     // no copy into this block may be left in flight
     skip_sample<MODE>(p, s, (!bad && too_many_labels) ? DSLIDE_ERR_OVERFLOW : DSLIDE_ERR_BAD_INDEX);
     return;
   }
@@ -703,9 +692,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     const int32_t* hidx = p.hash_idx;
     const int32_t* hsgn = p.hash_sign;
     if (p.hash_sm_off >= 0) {
-      const bool ok = mbar_wait(sh_bar2, 0u);
+      const bool ok = bar_wait_limited(sh_bar2, 0u);
       if (__syncthreads_or(ok ? 0 : 1)) {          // the mirror did not arrive in time: the sample is given up
-        mbar_wait(sh_bar2, 0u);
+        bar_wait_limited(sh_bar2, 0u);
         __syncthreads();
         skip_sample<MODE>(p, s, DSLIDE_ERR_TIMEOUT);
         return;
@@ -1172,7 +1161,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       }
     }
     if (bulk) {
-      const bool ok = mbar_wait(sh_bar, w2phase);
+      const bool ok = bar_wait_limited(sh_bar, w2phase);
       w2phase ^= 1u;
       if (__syncthreads_or(ok ? 0 : 1)) { timed_out = true; break; }
     } else {
@@ -1283,7 +1272,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   if (BULK && timed_out) {
     // a copy did not complete in time: the copies in flight get one more bounded wait, then the sample is given up.
     // Its touches are already counted, so the hand-off below still runs, with every coefficient zero.
-    mbar_wait(sh_bar, w2phase ^ 1u);
+    bar_wait_limited(sh_bar, w2phase ^ 1u);
     __syncthreads();
     if (tid == 0) set_status(p.st, DSLIDE_ERR_TIMEOUT);
   }

@@ -19,6 +19,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "waits.cuh"
 
 namespace dslide {
 
@@ -326,16 +327,6 @@ __device__ __forceinline__ void t_bulk(void* dst, const void* src, uint32_t byte
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(t_smem(dst)), "l"(src), "r"(bytes), "r"(t_smem(bar)) : "memory");
 }
-__device__ __forceinline__ bool t_wait(uint64_t* bar, uint32_t parity) {      // bounded
-  for (int it = 0; it < (1 << 22); ++it) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(t_smem(bar)), "r"(parity) : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
 // Brings tile t into shared memory, all threads: the rows one after the other, each followed by the head of its record
 // (count, bias, bias moments).  False when they did not come in time (block-uniform; nothing is left in flight).
 __device__ __forceinline__ bool load_tile(const TileParams& p, int t, float* tile, uint64_t* bar, uint32_t phase) {
@@ -351,9 +342,9 @@ __device__ __forceinline__ bool load_tile(const TileParams& p, int t, float* til
     t_bulk(tile + (size_t)r * ld, p.W2 + (size_t)j * H, (uint32_t)H * 4u, bar);
     t_bulk(tile + (size_t)r * ld + H, p.hdr2 + j, 16u, bar);
   }
-  const bool ok = t_wait(bar, phase);
+  const bool ok = bar_wait_limited(bar, phase);
   if (!__syncthreads_or(ok ? 0 : 1)) return true;
-  t_wait(bar, phase);                          // one more bounded wait for the copies in flight, then out
+  bar_wait_limited(bar, phase);                          // one more bounded wait for the copies in flight, then out
   if (threadIdx.x == 0) { p.tinfo[1] = 1; atomicCAS(&p.st->status, 0, (int)DSLIDE_ERR_TIMEOUT); }
   return false;
 }

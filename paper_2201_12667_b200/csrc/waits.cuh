@@ -22,6 +22,15 @@ __device__ __forceinline__ bool tc_bar_try(uint32_t bar, uint32_t parity) {
                : "=r"(ok) : "r"(bar), "r"(parity), "r"(2000u) : "memory");
   return ok != 0u;
 }
+// True once the phase of that parity has completed, false when it has not within the limit.
+__device__ __forceinline__ bool bar_wait_limited(uint64_t* bar, uint32_t parity) {
+  const uint32_t a = tc_smem(bar);
+  if (tc_bar_try(a, parity)) return true;
+  const long long t0 = clock64();
+  while (!tc_bar_try(a, parity))
+    if (clock64() - t0 > WAIT_CYCLES) return false;
+  return true;
+}
 // Sets the flag of this block and, in a pair (PAIR: a cluster of two blocks), of the other one.
 template <bool PAIR>
 __device__ __forceinline__ void tc_give_up(volatile int* abort) {
