@@ -33,7 +33,7 @@ constexpr int TC_NACC = 3;         // tensor memory: up to three accumulators of
 constexpr int TC_TMEM_COLS = 512;
 constexpr int TC_SPLIT = 4;        // read-back warps per quarter of tensor memory (each takes 1 / TC_SPLIT of a tile's columns)
 constexpr int TC_EPI = 128 * TC_SPLIT;                 // read-back threads
-constexpr int TC_THREADS = 96 + TC_EPI;                // warp 0: TMA producer; warp 1: tensor memory + MMA issue; warp 2: row norms; then the read-back warps
+constexpr int TC_THREADS = 96 + TC_EPI;                // warp 0: TMA producer; warp 1: tensor memory + MMA issue; warp 2: row norms; then the read-back warps (tc_threads: one more)
 constexpr int TC_EXTRA = 8;        // candidates kept beyond k: TC_EXTRA + k (the wider the margin, the rarer the exact fall-back)
 constexpr int TC_H_TMEM = 256;     // hidden layers up to this width sit in tensor memory beside two accumulators; wider ones are
                                    // streamed through shared memory with the tiles (WIDE)
@@ -52,6 +52,9 @@ constexpr int TC_BT = 8;           // tiles whose biases are in shared memory or
 constexpr int TC_BAHEAD = 6;       // tiles ahead that they are asked for: a tile takes less than a read from HBM under load
 // Neurons of a tile: 256 where the activations do not stand beside the accumulators in tensor memory and two blocks share a tile
 __host__ __device__ constexpr int tc_cols(bool wide, bool pair) { return wide && pair ? 2 * TC_N : TC_N; }
+
+// Pairs whose second block learns from the first of the rows that it sums have a warp for that
+__host__ __device__ constexpr int tc_threads(bool wide, bool pair) { return TC_THREADS + (pair && !wide ? 32 : 0); }
 
 struct TcParams {
   const RowHdr* hdr2;
@@ -190,11 +193,12 @@ __device__ __forceinline__ bool tc_better(float za, int ia, float zb, int ib) { 
 // latency per tile), and in WIDE the one warp that sums the rows' squares, element by element (26,000 cycles per tile at 512 units,
 // with packed pairs of four rows side by side 16,000).
 // The rows' norms in pairs: the second block reads its half of a tile once the first block, which counts the copies, has passed
-// that on; at cluster scope this takes 1,000 cycles, little beside a tile but more than a slab has (512 samples x 100,003
-// neurons x 512 units 229 us).  WIDE pairs take the norms from global memory, where L2 has the rows (135 us): the read-back
-// warps, before they wait for the tile's scores.
+// that on; at cluster scope this takes 1,000 cycles, which a warp of its own spends (by the norm warp itself 1,024 samples x
+// 253,855 neurons x 200 units took 262 us, so 256).  A slab has not that much time (512 samples x 100,003 neurons x 512 units 229 us):
+// WIDE pairs take the norms from global memory, where L2 has the rows (135 us; at 200 units it would be 283): the read-back warps,
+// before they wait for the tile's scores.
 template <bool DUMP, bool WIDE, bool PAIR>      // DUMP: write every score out (threshold pass); else append the scores that reach the sample's threshold
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __launch_bounds__(tc_threads(WIDE, PAIR), 1)
 k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH, const TcParams p) {
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -359,8 +363,8 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       const int nrr = RL / nshare;                     // rows of this block: nrr per lane
       // the bytes of a pair are counted in its first block, which tells the second
       auto arrived = [&](int st, int stround) {
-        tc_bar_wait<PAIR, PAIR>(PAIR && rank == 1 ? bar_landed + st : bar_full + st, stround & 1, abort_flag);
-        if (PAIR && rank == 0 && lane == 0) tc_bar_pass_on(tc_at_rank(bar_landed + st, 1u));
+        if (PAIR && rank == 1) tc_bar_wait<PAIR, true>(bar_landed + st, stround & 1, abort_flag);
+        else tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag);
       };
       for (int i = 0; i < my_tiles; ++i) {
         if (WIDE) {
@@ -416,6 +420,16 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
 #pragma unroll
       for (int d = 16; d > 0; d >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, d));
       if (lane == 0) atomicMax(p.norm2max, __float_as_uint(best));
+    }
+  } else if (PAIR && !WIDE && warp == TC_THREADS / 32) {
+    // ---------------- first block of a pair: what has landed is passed on to the second block's row norms ----------------
+    if (norms && rank == 0 && lane == 0) {
+      int st = 0, stround = 0;
+      for (int i = 0; i < my_tiles; ++i) {
+        if (!tc_bar_wait<PAIR, true>(bar_full + st, stround & 1, abort_flag)) break;
+        tc_bar_pass_on(tc_at_rank(bar_landed + st, 1u));
+        if (++st == nst) { st = 0; ++stround; }
+      }
     }
   } else {
     // ---------------- read-back: thread = (sample, share of a tile's columns) ----------------
@@ -1045,10 +1059,10 @@ static cudaError_t launch_exact_scan(Ctx* c, int batch, int k, int32_t* out_ids,
 }
 
 // As launch_dependent; the two blocks of a pair are a cluster.
-static cudaError_t launch_tc(void (*kernel)(const CUtensorMap, const CUtensorMap, const TcParams), bool pair, int slices, int groups, size_t smem,
+static cudaError_t launch_tc(void (*kernel)(const CUtensorMap, const CUtensorMap, const TcParams), bool wide, bool pair, int slices, int groups, size_t smem,
                              cudaStream_t stream, const CUtensorMap& tmW, const CUtensorMap& tmH, const TcParams& p) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((pair ? 2 : 1) * slices, groups); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cfg.gridDim = dim3((pair ? 2 : 1) * slices, groups); cfg.blockDim = dim3(tc_threads(wide, pair)); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1060,10 +1074,10 @@ static cudaError_t launch_tc(void (*kernel)(const CUtensorMap, const CUtensorMap
 
 // Whether two multiprocessors share a tile of W2 and 256 samples.  The tile then crosses from L2 once instead of twice, and a
 // stage takes half the shared memory; the multiplications take as long as in two blocks (63 to 68 cycles for 256 samples x
-// 128 neurons x 8 units, as for 128 x 128 x 8 in a block; of the 2,840 cycles of a tile of 200 units they are 1,650).  It pays where a block has room for one tile only
-// (more than 192 units), or streams the activations with the tiles (more than 256): us for a call of 1,024 samples x
-// 253,855 neurons x 200 units 371 by single blocks and 258 by pairs, 512 x 4,000,000 x 256 2,600 and 1,850, 512 x 100,003 x
-// 512 206 and 135; not at 160 units (300 x 100,003: 69 and 80) or 128 (147.9 and 148.8 for 670,091).  And where the tiles
+// 128 neurons x 8 units, as for 128 x 128 x 8 in a block; of the 2,840 cycles of a tile of 200 units they are 1,650).  It pays
+// where a block has room for one tile only (more than 192 units), or streams the activations with the tiles (more than 256):
+// us for a call of 1,024 samples x 253,855 neurons x 200 units 371 by single blocks and 256 by pairs, 512 x 4,000,000 x 256
+// 2,600 and 1,980, 512 x 100,003 x 512 206 and 135; not at 160 units (300 x 100,003: 69 and 80) or 128 (147.9 and 148.8 for 670,091).  And where the tiles
 // keep the pairs busy: a round of tiles takes a pair 0.7 of a block's time, at more than 256 units 1.2 for twice the tile.
 static bool use_pairs(const Ctx* c, int batch) {
   if (batch <= TC_M || c->H <= TC_H_SINGLE) return false;
@@ -1153,11 +1167,11 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
     p.nslices = nslices_sub; p.ntiles = nsub; p.tile_stride = stride; p.stages = stages_sub;
     // each kernel of the call may be placed while the kernel before it drains (they wait for it before they read or
     // write anything); the first follows the hidden-layer kernel in the same way
-    if ((e = launch_tc(k_sub, pair, nslices_sub, groups, smem_of(stages_sub), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
+    if ((e = launch_tc(k_sub, wide, pair, nslices_sub, groups, smem_of(stages_sub), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_tau, dim3(Bpad), dim3(TAU_THREADS), 0, c->stream, (const float*)dump, dump_cols, rank, tau)) != cudaSuccess)
       return e;
     p.nslices = nslices; p.ntiles = ntiles; p.tile_stride = 1; p.stages = stages;
-    if ((e = launch_tc(k_all, pair, nslices, groups, smem_of(stages), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
+    if ((e = launch_tc(k_all, wide, pair, nslices, groups, smem_of(stages), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
     if ((e = launch_dependent(k_tc_refine, dim3(batch), dim3(RF_THREADS), 0, c->stream, (const float*)c->W2, (const RowHdr*)c->hdr2,
                               (const float*)c->h, (const int2*)cand, (const int*)cand_cnt, gbuf, (const float*)tau, Bpad,
                               (const unsigned int*)norm2, batch, c->H, c->N, cap, nvs, k, out_ids, out_scores, (const int*)need_fix, n_fix, fix_list)) !=
