@@ -1022,16 +1022,17 @@ cudaError_t launch_update(Ctx* c, int batch, const int32_t* row_ptr, const int32
   const int smem = UPD_WARPS * 32 * 4;
   const int width = c->H <= 128 ? 0 : c->H <= 128 * LONG_P ? 1 : 2;
   // The last rows go out one by one, so that small batches keep every warp busy and a warp with one row waits for one chain
-  // of loads (a step of 1 sample 37 -> 33 us at 256 units, 89 -> 78 at 1,024, of 16 samples 108 -> 98 at 1,024); beyond 512
-  // units and 32 samples four at a time, with the next row asked into L2 meanwhile (64 samples, 768 units: 90 us, one by one 98).
-  const bool by_one = c->H <= 512 || batch <= 32;
+  // of loads (a step of 1 sample 37 -> 33 us at 256 units, 89 -> 78 at 1,024, of 16 samples 108 -> 98 at 1,024); four at a time,
+  // with the next row asked into L2 meanwhile, in large batches of up to 256 units (367 samples, 200 units: 150 us, one by one 152)
+  // and beyond 512 units and 32 samples (64 samples, 768 units: 90 us, one by one 98).
+  const bool by_one = width == 1 ? batch <= 256 : c->H <= 512 || batch <= 32;
   if (c->L1 > 0) {        // sampled hidden layer: rows of W1 are updated under their unit masks
     if (width == 0) return launch_k_update<0, 2, true>(c, p, smem);
-    if (width == 1) return launch_k_update<1, 1, true>(c, p, smem);
+    if (width == 1) return by_one ? launch_k_update<1, 1, true>(c, p, smem) : launch_k_update<1, UPD_TROWS, true>(c, p, smem);
     return by_one ? launch_k_update<2, 1, true>(c, p, smem) : launch_k_update<2, UPD_TROWS, true>(c, p, smem);
   }
   if (width == 0) return launch_k_update<0, 2, false>(c, p, smem);
-  if (width == 1) return launch_k_update<1, 1, false>(c, p, smem);
+  if (width == 1) return by_one ? launch_k_update<1, 1, false>(c, p, smem) : launch_k_update<1, UPD_TROWS, false>(c, p, smem);
   return by_one ? launch_k_update<2, 1, false>(c, p, smem) : launch_k_update<2, UPD_TROWS, false>(c, p, smem);
 }
 
