@@ -49,12 +49,11 @@ constexpr int TC_SUB_BYTES = TC_M * 128;               // one 32-unit slab of 12
 constexpr float TC_ERR = 2.2e-3f;  // |approximate - exact| <= TC_ERR * |h| * |w|: two operands cut to 10 mantissa bits, fp32 sums
 
 constexpr int TC_BT = 8;           // tiles whose biases are in shared memory or on their way there
-constexpr int TC_BAHEAD = 6;       // tiles ahead that they are asked for: a tile takes less than a read from HBM under load
 // Neurons of a tile: 256 where the activations do not stand beside the accumulators in tensor memory and two blocks share a tile
 __host__ __device__ constexpr int tc_cols(bool wide, bool pair) { return wide && pair ? 2 * TC_N : TC_N; }
 
-// Pairs whose second block learns from the first of the rows that it sums have a warp for that
-__host__ __device__ constexpr int tc_threads(bool wide, bool pair) { return TC_THREADS + (pair && !wide ? 32 : 0); }
+// A warp for the biases; pairs whose second block learns from the first of the rows that it sums have a warp for that too
+__host__ __device__ constexpr int tc_threads(bool wide, bool pair) { return TC_THREADS + 32 + (pair && !wide ? 32 : 0); }
 
 struct TcParams {
   const RowHdr* hdr2;
@@ -177,6 +176,16 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 
 __device__ __forceinline__ bool tc_better(float za, int ia, float zb, int ib) { return za > zb || (za == zb && ia < ib); }
 
+// One lane of a converged warp, the same at every call: the copies, multiplications and commits are its own, while the whole warp
+// walks the tiles and waits, so that their operands are the warp's.  Issued by one lane of a diverged warp an instruction took 84 to 134
+// cycles where the tensor pipe takes 64, which bounded the filter at every width (512 samples x 4,000,000 neurons x 256 units
+// 1,890 us, so 1,500; 1,024 x 253,855 x 200 246 and 218).
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t one;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+  return one != 0u;
+}
+
 // Grid: (slices of the neurons, groups of 128 samples).  Dynamic shared memory (1024-byte aligned):
 // TC_STAGES tiles of W2 as [ceil(H/32)][128 rows][128 B], then
 // the tiles' biases, the barriers.  (The samples' candidate buffers are in global memory.)
@@ -221,11 +230,13 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   uint64_t* bar_accempty = bars + 1 + 2 * NST + TC_NACC;   // [TC_NACC] accumulator read back
   uint64_t* bar_landed = bars + 1 + 2 * NST + 2 * TC_NACC; // [NST] second block of a pair: the stage has arrived (the pair's bytes are counted in the first)
   uint64_t* bar_drain = bars + 1 + 3 * NST + 2 * TC_NACC;  // after a wait has run out: the multiplications issued before have completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_drain + 1);
+  uint64_t* bar_bfull = bar_drain + 1;         // [TC_BT] the biases of a tile have arrived
+  uint64_t* bar_bempty = bar_bfull + TC_BT;    // [TC_BT] and have been read
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_bempty + TC_BT);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   unsigned* best_slot = tmem_slot + 2;         // OWN_ROWS: the block's largest squared norm, as bits
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const uint32_t rank = PAIR ? blockIdx.x & 1u : 0u;       // in the pair: the first block counts arrivals and issues the multiplications
   const int slice = PAIR ? blockIdx.x >> 1 : blockIdx.x, s0 = PAIR ? (2 * (int)blockIdx.y + (int)rank) * TC_M : (int)blockIdx.y * TC_M;
   // tiles of this slice: slice, slice + nslices, ... (both sample groups walk the same tiles at the same time: the
@@ -244,7 +255,8 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     tc_bar_init(bar_a, PAIR ? 8 : 4);            // a warp each
     tc_bar_init(bar_drain, 1);
     for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_landed + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
-    for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, PAIR ? 2 * TC_EPI / 32 : TC_EPI); }
+    for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, (PAIR ? 2 : 1) * TC_EPI / 32); }
+    for (int i = 0; i < TC_BT; ++i) { tc_bar_init(bar_bfull + i, 32); tc_bar_init(bar_bempty + i, TC_EPI / 32); }
     *abort_flag = 0;
     *best_slot = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -270,15 +282,15 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   int fills = 0;                     // stages that this block has asked for
   if (warp == 0) {
     // ---------------- producer: one thread feeds the TMA ----------------
-    if (lane == 0) {
-      int st = 0, stround = 0;
-      bool on = true;
-      for (int i = 0; on && i < my_tiles; ++i) {
-        const int row0 = (slice + i * p.nslices) * p.tile_stride * NT + (int)rank * ROWS;
-        if (WIDE) {
-          for (int ks = 0; ks < ksub; ++ks, ++fills) {
-            if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
-            unsigned char* to = smB + (size_t)st * tile_bytes;
+    int st = 0, stround = 0;
+    bool on = true;
+    for (int i = 0; on && i < my_tiles; ++i) {
+      const int row0 = (slice + i * p.nslices) * p.tile_stride * NT + (int)rank * ROWS;
+      if (WIDE) {
+        for (int ks = 0; ks < ksub; ++ks, ++fills) {
+          if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
+          unsigned char* to = smB + (size_t)st * tile_bytes;
+          if (tc_elect()) {
             if (PAIR) {
               if (rank == 0) tc_bar_expect(bar_full + st, 2u * tile_bytes);
               const uint32_t full = tc_at_rank(bar_full + st, 0u);
@@ -289,11 +301,14 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
               tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
               tc_tma_2d(to + SLAB, &tmH, ks * TC_KB, s0, bar_full + st);
             }
-            if (++st == nst) { st = 0; ++stround; }
           }
-          continue;
+          __syncwarp();
+          if (++st == nst) { st = 0; ++stround; }
         }
-        if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
+        continue;
+      }
+      if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
+      if (tc_elect()) {
         if (rank == 0) tc_bar_expect(bar_full + st, (PAIR ? 2u : 1u) * tile_bytes);
         const uint32_t full = PAIR ? tc_at_rank(bar_full + st, 0u) : 0u;
         for (int ks = 0; ks < ksub; ++ks) {
@@ -301,15 +316,16 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           if (PAIR) tc_tma_2d_pair(to, &tmW, ks * TC_KB, row0, full);
           else tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
         }
-        ++fills;
-        if (++st == nst) { st = 0; ++stround; }
       }
-      // the last fill of every stage has been consumed: no copy and no arrival at this block's barriers is on its way any more
-      for (int f = max(0, fills - nst); on && f < fills; ++f) on = tc_bar_wait<PAIR>(bar_empty + f % nst, (f / nst) & 1, abort_flag);
+      __syncwarp();
+      ++fills;
+      if (++st == nst) { st = 0; ++stround; }
     }
+    // the last fill of every stage has been consumed: no copy and no arrival at this block's barriers is on its way any more
+    for (int f = max(0, fills - nst); on && f < fills; ++f) on = tc_bar_wait<PAIR>(bar_empty + f % nst, (f / nst) & 1, abort_flag);
   } else if (warp == 1) {
     // ---------------- MMA issue: one thread (of a pair's first block) ----------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       const uint32_t idesc = tc_idesc(PAIR ? 2 * TC_M : TC_M, NT);
       bool on = WIDE || tc_bar_wait<PAIR>(bar_a, 0, abort_flag);
       const uint64_t b_base = tc_desc(tc_smem(smB));      // a descriptor's address field counts 16-byte units
@@ -323,33 +339,40 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           for (int ks = 0; ks < ksub; ++ks) {
             if (!(on = tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t b = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
-            const uint64_t a = b + (uint64_t)(SLAB >> 4);
-            const int kn = ks == ksub - 1 ? klast : TC_KB / 8;
-            for (int kk = 0; kk < kn; ++kk)
-              tc_mma_ss<PAIR>(d, a + (uint64_t)(kk * 2), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
-            tc_commit<PAIR>(bar_empty + st);
+            if (tc_elect()) {
+              const uint64_t b = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
+              const uint64_t a = b + (uint64_t)(SLAB >> 4);
+              const int kn = ks == ksub - 1 ? klast : TC_KB / 8;
+              for (int kk = 0; kk < kn; ++kk)
+                tc_mma_ss<PAIR>(d, a + (uint64_t)(kk * 2), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
+              tc_commit<PAIR>(bar_empty + st);
+            }
+            __syncwarp();
             if (++st == nst) { st = 0; ++stround; }
           }
           if (!on) break;
-          tc_commit<PAIR>(bar_accfull + acc);
+          if (tc_elect()) tc_commit<PAIR>(bar_accfull + acc);
+          __syncwarp();
           if (++acc == nacc) { acc = 0; ++accround; }
           continue;
         }
-        const uint64_t b_tile = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
-        for (int ks = 0; ks < kfull; ++ks) {
-          const uint32_t a = tmem_base + acol + (uint32_t)(ks * TC_KB);      // lanes = samples, columns = hidden units
-          const uint64_t b = b_tile + (uint64_t)((ks * SLAB) >> 4);
+        if (tc_elect()) {
+          const uint64_t b_tile = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
+          for (int ks = 0; ks < kfull; ++ks) {
+            const uint32_t a = tmem_base + acol + (uint32_t)(ks * TC_KB);      // lanes = samples, columns = hidden units
+            const uint64_t b = b_tile + (uint64_t)((ks * SLAB) >> 4);
 #pragma unroll
-          for (int kk = 0; kk < TC_KB / 8; ++kk)              // eight tf32 = 32 bytes per instruction
-            tc_mma<PAIR>(d, a + (uint32_t)(kk * 8), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
+            for (int kk = 0; kk < TC_KB / 8; ++kk)              // eight tf32 = 32 bytes per instruction
+              tc_mma<PAIR>(d, a + (uint32_t)(kk * 8), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
+          }
+          if (kfull < ksub)                                     // a last slab of fewer units
+            for (int kk = 0; kk < klast; ++kk)
+              tc_mma<PAIR>(d, tmem_base + acol + (uint32_t)(kfull * TC_KB + kk * 8), b_tile + (uint64_t)((kfull * SLAB) >> 4) + (uint64_t)(kk * 2),
+                     idesc, (kfull | kk) != 0 ? 1u : 0u);
+          tc_commit<PAIR>(bar_empty + st);          // the tile's shared memory is free once these instructions have read it
+          tc_commit<PAIR>(bar_accfull + acc);       // and the accumulator is complete
         }
-        if (kfull < ksub)                                     // a last slab of fewer units
-          for (int kk = 0; kk < klast; ++kk)
-            tc_mma<PAIR>(d, tmem_base + acol + (uint32_t)(kfull * TC_KB + kk * 8), b_tile + (uint64_t)((kfull * SLAB) >> 4) + (uint64_t)(kk * 2),
-                   idesc, (kfull | kk) != 0 ? 1u : 0u);
-        tc_commit<PAIR>(bar_empty + st);          // the tile's shared memory is free once these instructions have read it
-        tc_commit<PAIR>(bar_accfull + acc);       // and the accumulator is complete
+        __syncwarp();
         if (++st == nst) { st = 0; ++stround; }
         if (++acc == nacc) { acc = 0; ++accround; }
       }
@@ -421,7 +444,23 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       for (int d = 16; d > 0; d >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, d));
       if (lane == 0) atomicMax(p.norm2max, __float_as_uint(best));
     }
-  } else if (PAIR && !WIDE && warp == TC_THREADS / 32) {
+  } else if (warp == TC_THREADS / 32) {
+    // ---------------- biases: a tile's, TC_BT tiles ahead of the read-back (zero past the last neuron) ----------------
+    bool on = true;
+    for (int i = 0; on && i < my_tiles; ++i) {
+      const int slot = i & (TC_BT - 1), round = i / TC_BT;
+      if (round > 0 && !(on = tc_bar_wait<PAIR>(bar_bempty + slot, (round - 1) & 1, abort_flag))) break;
+      const int j0 = (slice + i * p.nslices) * p.tile_stride * NT + lane;
+#pragma unroll
+      for (int c = 0; c < NT; c += 32) {
+        const int j = j0 + c;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                     ::"r"(tc_smem(sb + slot * NT + c + lane)), "l"(&p.hdr2[j < p.N ? j : 0].b), "r"(j < p.N ? 4 : 0) : "memory");
+      }
+      asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tc_smem(bar_bfull + slot)) : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");      // nothing is on its way into shared memory when the block ends
+  } else if (PAIR && !WIDE && warp == TC_THREADS / 32 + 1) {
     // ---------------- first block of a pair: what has landed is passed on to the second block's row norms ----------------
     if (norms && rank == 0 && lane == 0) {
       int st = 0, stround = 0;
@@ -438,7 +477,6 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     const int q = warp & 3;                 // a warp reaches the 32 lanes of tensor memory of its number modulo four
     const int half = (warp - 3) >> 2;       // which share of a tile's columns
     const int row = 32 * q + lane;          // sample inside the block
-    const int et = tid - 96;                // the first NT read-back threads (whole warps) fetch the tile's biases
     const int vslice = slice * TC_SPLIT + half;    // buffers are kept per (slice, share of the columns)
     int2* mybuf = p.cand + ((size_t)vslice * p.Bpad + s0 + row) * p.gbuf;
     const float tau = DUMP ? 0.f : (s0 + row < p.B ? p.tau[s0 + row] : INFINITY);      // rows past the batch keep nothing
@@ -469,25 +507,11 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         else tc_bar_arrive(bar_a);
       }
     }
-    // a tile's biases are asked for TC_BAHEAD tiles ahead (a group of copies per tile, empty past the last one)
-    auto ask_bias = [&](int i) {
-      const int j = (slice + i * p.nslices) * p.tile_stride * NT + et;
-      if (i < my_tiles)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
-                     ::"r"(tc_smem(sb + (i & (TC_BT - 1)) * NT + et)), "l"(&p.hdr2[j < p.N ? j : 0].b), "r"(j < p.N ? 4 : 0) : "memory");
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    if (et < NT)
-      for (int i = 0; i < TC_BAHEAD; ++i) ask_bias(i);
     float best = 0.f;                              // OWN_ROWS: the largest squared norm of the thread's rows
     int acc = 0, accround = 0;
     for (int i = 0; i < my_tiles; ++i) {
       const int tile = slice + i * p.nslices;
       const int j0 = tile * p.tile_stride * NT;
-      if (et < NT) {
-        ask_bias(i + TC_BAHEAD);                   // where the biases of tile i - 2 were: every warp has left that tile
-        asm volatile("cp.async.wait_group %0;" ::"n"(TC_BAHEAD) : "memory");      // tile i's are there
-      }
       const float* tb = sb + (i & (TC_BT - 1)) * NT;
       if (OWN_ROWS && !DUMP) {
         // up to four groups share the tile's rows, and so do their blocks and a block's warps: 4, 8 or 16 lanes to a row
@@ -510,28 +534,32 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           best = fmaxf(best, n);
         }
       }
-      if (warp == 3) tc_bar_wait<PAIR>(bar_accfull + acc, accround & 1, abort_flag);      // one warp polls, the others sleep in the barrier
-      asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory");          // the accumulator is complete, the tile's biases are in place
+      // A warp waits for itself, takes its columns into registers and gives the accumulator back before it looks at them: the
+      // next tiles are multiplied meanwhile, and a warp with candidates to append holds up no other (300 samples x 600,011 neurons x
+      // 64 units 138 us, so 122).
+      tc_bar_wait<PAIR>(bar_bfull + (i & (TC_BT - 1)), (i / TC_BT) & 1, abort_flag);
+      tc_bar_wait<PAIR>(bar_accfull + acc, accround & 1, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
       for (int c0 = (NT / TC_SPLIT) * half; c0 < (NT / TC_SPLIT) * (half + 1); c0 += 32) {
         uint32_t r[32];
         tc_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * NT + c0), r);
+        if (c0 + 32 == (NT / TC_SPLIT) * (half + 1)) {      // the warp's last columns
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            if (PAIR) tc_bar_arrive_at(tc_at_rank(bar_accempty + acc, 0u));
+            else tc_bar_arrive(bar_accempty + acc);
+          }
+        }
         const int jb = j0 + c0;
         const float4* sb4 = reinterpret_cast<const float4*>(tb + c0);
-        unsigned hm = 0u;
+        float z[32];
 #pragma unroll
         for (int c4 = 0; c4 < 8; ++c4) {
           const float4 bq = sb4[c4];
-          const float z0 = __uint_as_float(r[4 * c4]) + bq.x, z1 = __uint_as_float(r[4 * c4 + 1]) + bq.y;
-          const float z2 = __uint_as_float(r[4 * c4 + 2]) + bq.z, z3 = __uint_as_float(r[4 * c4 + 3]) + bq.w;
-          r[4 * c4] = __float_as_uint(z0); r[4 * c4 + 1] = __float_as_uint(z1);
-          r[4 * c4 + 2] = __float_as_uint(z2); r[4 * c4 + 3] = __float_as_uint(z3);
-          if (!DUMP) {
-            if (z0 >= tau) hm |= 1u << (4 * c4);
-            if (z1 >= tau) hm |= 2u << (4 * c4);
-            if (z2 >= tau) hm |= 4u << (4 * c4);
-            if (z3 >= tau) hm |= 8u << (4 * c4);
-          }
+          z[4 * c4] = __uint_as_float(r[4 * c4]) + bq.x; z[4 * c4 + 1] = __uint_as_float(r[4 * c4 + 1]) + bq.y;
+          z[4 * c4 + 2] = __uint_as_float(r[4 * c4 + 2]) + bq.z; z[4 * c4 + 3] = __uint_as_float(r[4 * c4 + 3]) + bq.w;
         }
         if (DUMP) {
           // neurons past the end score -infinity; a thread's 32 scores are 128 contiguous bytes
@@ -539,36 +567,47 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
 #pragma unroll
           for (int c4 = 0; c4 < 8; ++c4) {
             float4 v;
-            v.x = jb + 4 * c4 < p.N ? __uint_as_float(r[4 * c4]) : -INFINITY;
-            v.y = jb + 4 * c4 + 1 < p.N ? __uint_as_float(r[4 * c4 + 1]) : -INFINITY;
-            v.z = jb + 4 * c4 + 2 < p.N ? __uint_as_float(r[4 * c4 + 2]) : -INFINITY;
-            v.w = jb + 4 * c4 + 3 < p.N ? __uint_as_float(r[4 * c4 + 3]) : -INFINITY;
+            v.x = jb + 4 * c4 < p.N ? z[4 * c4] : -INFINITY;
+            v.y = jb + 4 * c4 + 1 < p.N ? z[4 * c4 + 1] : -INFINITY;
+            v.z = jb + 4 * c4 + 2 < p.N ? z[4 * c4 + 2] : -INFINITY;
+            v.w = jb + 4 * c4 + 3 < p.N ? z[4 * c4 + 3] : -INFINITY;
             __stcg(out + c4, v);
           }
         } else {
-          if (p.N - jb < 32) hm &= p.N > jb ? (1u << (p.N - jb)) - 1u : 0u;      // neurons past the end (last tile only)
-          // the columns that some sample of the warp keeps (few): one more read of that column, same sum as above
-          unsigned any = __reduce_or_sync(0xffffffffu, hm);
-          while (any) {
-            const int c = __ffs(any) - 1;
-            any &= any - 1;
-            uint32_t raw;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;"
-                         : "=r"(raw) : "r"(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * NT + c0 + c)) : "memory");
-            if ((hm >> c) & 1u) {
-              const float z = __uint_as_float(raw) + tb[c0 + c];
-              if (cnt < p.gbuf) __stcg(mybuf + cnt, make_int2(__float_as_int(z), jb + c));
-              ++cnt;
+          float most = -INFINITY;            // a score that is not a number is none of them
+#pragma unroll
+          for (int c = 0; c < 32; c += 2) most = fmaxf(fmaxf(most, z[c]), z[c + 1]);
+          if (__any_sync(0xffffffffu, most >= tau)) {
+            unsigned hm = 0u;
+#pragma unroll
+            for (int c = 0; c < 32; ++c)
+              if (z[c] >= tau) hm |= 1u << c;
+            if (p.N - jb < 32) hm &= p.N > jb ? (1u << (p.N - jb)) - 1u : 0u;      // neurons past the end (last tile only)
+            // the columns that some sample of the warp keeps (few): halving picks a column's scores from the registers
+            unsigned any = __reduce_or_sync(0xffffffffu, hm);
+            while (any) {
+              const int c = __ffs(any) - 1;
+              any &= any - 1;
+              float w[16];
+#pragma unroll
+              for (int e = 0; e < 16; ++e) w[e] = (c & 16) ? z[e + 16] : z[e];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) w[e] = (c & 8) ? w[e + 8] : w[e];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) w[e] = (c & 4) ? w[e + 4] : w[e];
+#pragma unroll
+              for (int e = 0; e < 2; ++e) w[e] = (c & 2) ? w[e + 2] : w[e];
+              const float zc = (c & 1) ? w[1] : w[0];
+              if ((hm >> c) & 1u) {
+                if (cnt < p.gbuf) __stcg(mybuf + cnt, make_int2(__float_as_int(zc), jb + c));
+                ++cnt;
+              }
             }
           }
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      if (PAIR) {
-        __syncwarp();
-        if (lane == 0) tc_bar_arrive_at(tc_at_rank(bar_accempty + acc, 0u));
-      }
-      else tc_bar_arrive(bar_accempty + acc);      // every thread: up to 1 % faster than a lane for its warp
+      __syncwarp();
+      if (lane == 0) tc_bar_arrive(bar_bempty + (i & (TC_BT - 1)));
       if (++acc == nacc) { acc = 0; ++accround; }
     }
     if (OWN_ROWS && !DUMP) {
@@ -1149,7 +1188,7 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   p.hdr2 = c->hdr2; p.h = c->h; p.W2 = c->W2; p.cand = cand; p.cand_cnt = cand_cnt; p.dump = dump; p.tau = tau; p.need_fix = need_fix; p.norm2max = norm2; p.n_fix = n_fix; p.st = c->dstate;
   p.B = batch; p.Bpad = Bpad; p.H = c->H; p.N = c->N; p.dump_cols = dump_cols; p.gbuf = gbuf;
   const size_t tile_bytes = wide ? (size_t)rows * 128 + TC_SUB_BYTES : (size_t)((c->H + TC_KB - 1) / TC_KB) * rows * 128;
-  auto smem_of = [&](int st) { return 1024 + tile_bytes * st + (size_t)TC_BT * NT * 4 + (2 + 3 * TC_STAGES + 2 * TC_NACC) * 8 + 64; };
+  auto smem_of = [&](int st) { return 1024 + tile_bytes * st + (size_t)TC_BT * NT * 4 + (2 + 3 * TC_STAGES + 2 * TC_NACC + 2 * TC_BT) * 8 + 64; };
   // Tiles in flight: six of a narrow model, but beyond three only what 144 KB hold (300 samples x 600,011 neurons x 64 units: 143 us
   // with three or six, 139 with four), and in the threshold pass no more than a block has tiles, mostly one: its blocks and those of
   // the kernels that follow then find room side by side (1 x 5,003 x 64: 28.3 us, with six stages 29.6; 1 x 5,003 x 128 29.1 and 30.4).
