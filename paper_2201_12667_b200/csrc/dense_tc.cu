@@ -10,10 +10,10 @@
 //
 // TF32 rounds both operands to 10 mantissa bits, far from the 1e-4 the scores must meet.  The tensor pass is
 // therefore a FILTER, in two launches of the same kernel.  The first scores every TC_SUBSET-th tile of neurons and
-// writes the scores out; k_tc_tau takes, per sample, about the cap-th best of them (cap = 2k + TC_EXTRA) as the
-// sample's threshold -- about cap * TC_SUBSET neurons reach it over all N.  The second launch scores all tiles and a
+// writes the scores (or the largest of neighbours) out; k_tc_tau takes, per sample, about the (k + TC_RANK_OVER)-th best of them as the
+// sample's threshold -- about TC_TARGET times as many neurons reach it over all N.  The second launch scores all tiles and a
 // thread appends the few scores of its sample that reach the threshold to the sample's candidate buffer.
-// k_tc_refine recomputes the cap or so best candidates exactly in fp32 and orders them (logit descending, id
+// k_tc_refine recomputes the cap = 2k + TC_EXTRA or so best candidates exactly in fp32 and orders them (logit descending, id
 // ascending).  The filter is exact when the k-th exact score clears every discarded neuron's approximate score by
 // more than the approximation's error bound, 2^-9 |h| |w|_max (plus accumulation); a sample for which that cannot
 // be shown (or whose buffers ran over) is listed, and k_scan_all scores all N neurons for the listed samples in fp32.
@@ -34,16 +34,16 @@ constexpr int TC_TMEM_COLS = 512;
 constexpr int TC_SPLIT = 4;        // read-back warps per quarter of tensor memory (each takes 1 / TC_SPLIT of a tile's columns)
 constexpr int TC_EPI = 128 * TC_SPLIT;                 // read-back threads
 constexpr int TC_THREADS = 96 + TC_EPI;                // warp 0: TMA producer; warp 1: tensor memory + MMA issue; warp 2: row norms; then the read-back warps (tc_threads: one more)
-constexpr int TC_EXTRA = 8;        // candidates kept beyond k: TC_EXTRA + k (the wider the margin, the rarer the exact fall-back)
+constexpr int TC_EXTRA = 16;       // candidates kept beyond 2k (the wider the margin, the rarer the exact fall-back)
 constexpr int TC_H_TMEM = 256;     // hidden layers up to this width sit in tensor memory beside two accumulators; wider ones are
                                    // streamed through shared memory with the tiles (WIDE)
 constexpr int TC_H_SINGLE = 192;   // up to this width two tiles fit a block's shared memory
 constexpr int TC_WIDE_STAGES = TC_STAGES;      // WIDE: pairs of slabs (32 units of the samples, 32 units of the neurons) in flight
-constexpr int TC_RANK_CAP = 24;    // the threshold's rank in the subset grows with k up to this
+constexpr int TC_RANK_MIN = 8, TC_RANK_OVER = 5, TC_RANK_CAP = 24;      // the threshold's rank in the subset: k + TC_RANK_OVER, within these
 constexpr int TC_GBUF_MIN = 2;     // candidate slots per (buffer, sample) at least, in neighbouring neurons that the buffer takes of a tile (32, or 64 of
                                    // a wide pair's): many times the expected fill, but a trained model may favour neighbours together, and a buffer
                                    // that runs over sends the sample to the exact scan (512 x 100,003 neurons x 512 units all undecided: 3,300 us for 137)
-constexpr int TC_TARGET = 64;      // candidates aimed at per sample: TC_TARGET x min(cap, TC_RANK_CAP)
+constexpr int TC_TARGET = 64;      // candidates aimed at per sample: so many times that rank
 constexpr int TC_SUBSET = 64;      // the threshold pass scores every TC_SUBSET-th tile
 constexpr int TC_SUB_BYTES = TC_M * 128;               // one 32-unit slab of 128 rows
 constexpr float TC_ERR = 2.2e-3f;  // |approximate - exact| <= TC_ERR * |h| * |w|: two operands cut to 10 mantissa bits, fp32 sums
@@ -70,7 +70,7 @@ struct TcParams {
   int B, Bpad, H, N, nslices, ntiles;          // ntiles: tiles this launch walks
   int tile_stride;                 // tile i of the launch is tile i * tile_stride of W2
   int stages;                      // tiles of W2 in flight, 1 .. TC_STAGES
-  int dump_cols;
+  int dump_cols, dump_max;         // scores (or, dump_max, largest of 32 neighbours' scores) per sample
   int gbuf;                        // slots per candidate buffer
 };
 
@@ -562,16 +562,19 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           z[4 * c4 + 2] = __uint_as_float(r[4 * c4 + 2]) + bq.z; z[4 * c4 + 3] = __uint_as_float(r[4 * c4 + 3]) + bq.w;
         }
         if (DUMP) {
-          // neurons past the end score -infinity; a thread's 32 scores are 128 contiguous bytes
-          float4* out = reinterpret_cast<float4*>(p.dump + (size_t)(s0 + row) * p.dump_cols + (size_t)tile * NT + c0);
+          // neurons past the end score -infinity
 #pragma unroll
-          for (int c4 = 0; c4 < 8; ++c4) {
-            float4 v;
-            v.x = jb + 4 * c4 < p.N ? z[4 * c4] : -INFINITY;
-            v.y = jb + 4 * c4 + 1 < p.N ? z[4 * c4 + 1] : -INFINITY;
-            v.z = jb + 4 * c4 + 2 < p.N ? z[4 * c4 + 2] : -INFINITY;
-            v.w = jb + 4 * c4 + 3 < p.N ? z[4 * c4 + 3] : -INFINITY;
-            __stcg(out + c4, v);
+          for (int c = 0; c < 32; ++c)
+            if (jb + c >= p.N) z[c] = -INFINITY;
+          if (p.dump_max) {                  // the largest of the thread's 32 (none of them a number: minus infinity)
+            float most = -INFINITY;
+#pragma unroll
+            for (int c = 0; c < 32; c += 2) most = fmaxf(fmaxf(most, z[c]), z[c + 1]);
+            __stcg(p.dump + (size_t)(s0 + row) * p.dump_cols + (tile * NT + c0) / 32, most);
+          } else {                           // all of them: 128 contiguous bytes
+            float4* out = reinterpret_cast<float4*>(p.dump + (size_t)(s0 + row) * p.dump_cols + (size_t)tile * NT + c0);
+#pragma unroll
+            for (int c4 = 0; c4 < 8; ++c4) __stcg(out + c4, make_float4(z[4 * c4], z[4 * c4 + 1], z[4 * c4 + 2], z[4 * c4 + 3]));
           }
         } else {
           float most = -INFINITY;            // a score that is not a number is none of them
@@ -583,11 +586,9 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
             for (int c = 0; c < 32; ++c)
               if (z[c] >= tau) hm |= 1u << c;
             if (p.N - jb < 32) hm &= p.N > jb ? (1u << (p.N - jb)) - 1u : 0u;      // neurons past the end (last tile only)
-            // the columns that some sample of the warp keeps (few): halving picks a column's scores from the registers
-            unsigned any = __reduce_or_sync(0xffffffffu, hm);
-            while (any) {
-              const int c = __ffs(any) - 1;
-              any &= any - 1;
+            // every sample of the warp appends its next one; halving picks its score from the registers
+            while (__any_sync(0xffffffffu, hm != 0u)) {
+              const int c = (__ffs(hm) - 1) & 31;
               float w[16];
 #pragma unroll
               for (int e = 0; e < 16; ++e) w[e] = (c & 16) ? z[e + 16] : z[e];
@@ -598,10 +599,11 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
 #pragma unroll
               for (int e = 0; e < 2; ++e) w[e] = (c & 2) ? w[e + 2] : w[e];
               const float zc = (c & 1) ? w[1] : w[0];
-              if ((hm >> c) & 1u) {
+              if (hm != 0u) {
                 if (cnt < p.gbuf) __stcg(mybuf + cnt, make_int2(__float_as_int(zc), jb + c));
                 ++cnt;
               }
+              hm &= hm - 1u;
             }
           }
         }
@@ -664,22 +666,35 @@ __device__ __forceinline__ uint32_t tc_select(uint32_t mine, int cap) {
   return K;
 }
 
-// One block per sample.  Each thread takes the largest of its share of the sample's scores of the subset; the cap-th
-// largest of these maxima is the sample's threshold.  At least cap neurons of the subset reach it (exactly cap when
-// the cap best fell to different threads); -infinity when the subset is smaller than that.  Any threshold gives the
-// same results: it only decides how many candidates the filter pass hands on.
-constexpr int TAU_THREADS = 256;
-__global__ void __launch_bounds__(TAU_THREADS) k_tc_tau(const float* dump, int cols, int rank, float* tau) {
-  const int s = blockIdx.x, tid = threadIdx.x;
+// A warp per sample.  The sample's scores of the subset (or the largest of 32 neighbours each) are shared out to 512 places
+// of the warp's registers, each keeping the largest; the rank-th largest of these maxima, cut to 20 bits, is the sample's
+// threshold.  At least rank neurons of the subset reach it (about as many where the best fell to different places); -infinity when
+// the subset is smaller than that.  Any threshold gives the same results: it only decides how many candidates the filter pass hands on.
+constexpr int TAU_WARPS = 4, TAU_V = 16;
+__global__ void __launch_bounds__(32 * TAU_WARPS) k_tc_tau(const float* dump, int cols, int rank, float* tau) {
+  const int s = blockIdx.x * TAU_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   griddep_launch_dependents();
   griddep_wait();                    // the threshold pass has completed
-  uint32_t mine = 0u;
-  for (int e = tid; e < cols; e += TAU_THREADS) {
-    const uint32_t key = tc_key(__ldcg(dump + (size_t)s * cols + e));
-    mine = key > mine ? key : mine;
+  uint32_t v[TAU_V];
+#pragma unroll
+  for (int i = 0; i < TAU_V; ++i) v[i] = 0u;
+  const float* mine = dump + (size_t)s * cols;
+  for (int e0 = lane; e0 < cols; e0 += 32 * TAU_V) {
+    float z[TAU_V];
+#pragma unroll
+    for (int i = 0; i < TAU_V; ++i) z[i] = e0 + 32 * i < cols ? __ldcg(mine + e0 + 32 * i) : 0.f;
+#pragma unroll
+    for (int i = 0; i < TAU_V; ++i) v[i] = e0 + 32 * i < cols ? max(v[i], tc_key(z[i])) : v[i];
   }
-  const uint32_t K = tc_select(mine, rank);
-  if (tid == 0) {
+  uint32_t K = 0u;
+  for (int bit = 31; bit >= 12; --bit) {
+    const uint32_t trial = K | (1u << bit);
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < TAU_V; ++i) n += v[i] >= trial ? 1 : 0;
+    if (__reduce_add_sync(0xffffffffu, n) >= rank) K = trial;
+  }
+  if (lane == 0) {
     float t = tc_unkey(K);
     if (K == 0u || !(t == t)) t = -INFINITY;      // everything passes
     tau[s] = t;
@@ -1147,7 +1162,6 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   int stride = TC_SUBSET;
   if ((ntiles + stride - 1) / stride > TAU_MAX_TILES) stride = (ntiles + TAU_MAX_TILES - 1) / TAU_MAX_TILES;
   const int nsub = (ntiles + stride - 1) / stride;
-  const int dump_cols = nsub * NT;
   int nslices_sub = nslices < nsub ? nslices : nsub;
   // work space: the norm bound, the flags, the thresholds, the candidate buffers of every slice and their fill, the
   // threshold pass's scores
@@ -1157,12 +1171,17 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   const size_t off_part = WS_HEAD, off_fix = off_part + up(scan_part_bytes(c, k)), off_list = off_fix + up((size_t)Bpad * 4);
   const size_t off_tau = off_list + up((size_t)Bpad * 4), off_cnt = off_tau + up((size_t)Bpad * 4);
   const size_t off_cand = off_cnt + up((size_t)nvs * Bpad * 4);
-  // The threshold is the rank-th best of the subset's maxima, the rank chosen so that about TC_TARGET x cap neurons
-  // reach it over all N whatever the subset's share; a buffer has room for four times its expected fill.
-  const int want = cap < TC_RANK_CAP ? cap : TC_RANK_CAP;
+  // The threshold is the rank-th best of the subset's maxima, the rank chosen so that about TC_TARGET times as many neurons
+  // reach it over all N whatever the subset's share; a buffer has room for four times its expected fill.  A rank of TC_RANK_MIN
+  // leaves fewer than the cap of k = 5 once in 10^8 samples (such a sample is still decided by its threshold, mostly), and one
+  // above k keeps that so where the best neighbours are all in the subset.
+  const int want = min(TC_RANK_CAP, max(TC_RANK_MIN, k + TC_RANK_OVER));
   int rank = (want * TC_TARGET + stride - 1) / stride;
   if (rank > want) rank = want;
-  if (rank < 4) rank = 4;
+  if (rank < 5) rank = 5;
+  // Where the subset has enough groups of 32 neighbours, their largest scores stand for it.
+  const int dump_max = nsub * NT / 32 >= 8 * rank ? 1 : 0;
+  const int dump_cols = dump_max ? nsub * NT / 32 : nsub * NT;
   int gbuf = TC_GBUF_MIN * NT / TC_SPLIT;
   while (gbuf * nvs < 4 * rank * stride) gbuf <<= 1;
   const size_t off_dump = off_cand + up((size_t)nvs * Bpad * gbuf * sizeof(int2));
@@ -1186,7 +1205,7 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
 
   TcParams p;
   p.hdr2 = c->hdr2; p.h = c->h; p.W2 = c->W2; p.cand = cand; p.cand_cnt = cand_cnt; p.dump = dump; p.tau = tau; p.need_fix = need_fix; p.norm2max = norm2; p.n_fix = n_fix; p.st = c->dstate;
-  p.B = batch; p.Bpad = Bpad; p.H = c->H; p.N = c->N; p.dump_cols = dump_cols; p.gbuf = gbuf;
+  p.B = batch; p.Bpad = Bpad; p.H = c->H; p.N = c->N; p.dump_cols = dump_cols; p.dump_max = dump_max; p.gbuf = gbuf;
   const size_t tile_bytes = wide ? (size_t)rows * 128 + TC_SUB_BYTES : (size_t)((c->H + TC_KB - 1) / TC_KB) * rows * 128;
   auto smem_of = [&](int st) { return 1024 + tile_bytes * st + (size_t)TC_BT * NT * 4 + (2 + 3 * TC_STAGES + 2 * TC_NACC + 2 * TC_BT) * 8 + 64; };
   // Tiles in flight: six of a narrow model, but beyond three only what 144 KB hold (300 samples x 600,011 neurons x 64 units: 143 us
@@ -1207,7 +1226,7 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
     // each kernel of the call may be placed while the kernel before it drains (they wait for it before they read or
     // write anything); the first follows the hidden-layer kernel in the same way
     if ((e = launch_tc(k_sub, wide, pair, nslices_sub, groups, smem_of(stages_sub), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
-    if ((e = launch_dependent(k_tc_tau, dim3(Bpad), dim3(TAU_THREADS), 0, c->stream, (const float*)dump, dump_cols, rank, tau)) != cudaSuccess)
+    if ((e = launch_dependent(k_tc_tau, dim3(Bpad / TAU_WARPS), dim3(32 * TAU_WARPS), 0, c->stream, (const float*)dump, dump_cols, rank, tau)) != cudaSuccess)
       return e;
     p.nslices = nslices; p.ntiles = ntiles; p.tile_stride = 1; p.stages = stages;
     if ((e = launch_tc(k_all, wide, pair, nslices, groups, smem_of(stages), c->stream, tmW, tmH, p)) != cudaSuccess) return e;
