@@ -5,7 +5,7 @@
 // arrive in shared memory by TMA (cp.async.bulk.tensor, 128-byte swizzle), the 128 samples' hidden activations of a
 // block sit in tensor memory beside the accumulators, a single thread of one or two blocks issues tcgen05.mma (kind::tf32), and the
 // read-back warps fetch the accumulators (tcgen05.ld) and keep, per sample, the candidates of the block's slice of
-// neurons; one more warp takes the largest row norm of W2 from the tiles while they are in shared memory.  W2 is
+// neurons; four more warps take the largest row norm of W2 from the tiles while they are in shared memory.  W2 is
 // streamed once per 128 samples (the groups of samples walk the same tiles together, so HBM sees it once per call).
 //
 // TF32 rounds both operands to 10 mantissa bits, far from the 1e-4 the scores must meet.  The tensor pass is
@@ -33,7 +33,9 @@ constexpr int TC_NACC = 3;         // tensor memory: up to three accumulators of
 constexpr int TC_TMEM_COLS = 512;
 constexpr int TC_SPLIT = 4;        // read-back warps per quarter of tensor memory (each takes 1 / TC_SPLIT of a tile's columns)
 constexpr int TC_EPI = 128 * TC_SPLIT;                 // read-back threads
-constexpr int TC_THREADS = 96 + TC_EPI;                // warp 0: TMA producer; warp 1: tensor memory + MMA issue; warp 2: row norms; then the read-back warps (tc_threads: one more)
+constexpr int TC_THREADS = 64 + TC_EPI;                // warp 0: TMA producer; warp 1: tensor memory + MMA issue; then the read-back warps (tc_threads: further ones)
+constexpr int TC_NORM_WARPS = 4;   // that take the row norms.  One held a tile's stage for 2,050 cycles of 2,280 (128 units, two groups of samples); us for one,
+                                   // two and four: 256 x 670,091 x 128 139, 134, 129; 512 x 600,011 x 32 to 96 no more than one; 100 x 100,003 x 512 95, 88, 83
 constexpr int TC_EXTRA = 16;       // candidates kept beyond 2k (the wider the margin, the rarer the exact fall-back)
 constexpr int TC_H_TMEM = 256;     // hidden layers up to this width sit in tensor memory beside two accumulators; wider ones are
                                    // streamed through shared memory with the tiles (WIDE)
@@ -52,8 +54,9 @@ constexpr int TC_BT = 8;           // tiles whose biases are in shared memory or
 // Neurons of a tile: 256 where the activations do not stand beside the accumulators in tensor memory and two blocks share a tile
 __host__ __device__ constexpr int tc_cols(bool wide, bool pair) { return wide && pair ? 2 * TC_N : TC_N; }
 
-// A warp for the biases; pairs whose second block learns from the first of the rows that it sums have a warp for that too
-__host__ __device__ constexpr int tc_threads(bool wide, bool pair) { return TC_THREADS + 32 + (pair && !wide ? 32 : 0); }
+// Warps after the read-back's: one for the biases, those for the row norms, and, in pairs whose second block learns from the first of
+// the rows that it sums, one for that
+__host__ __device__ constexpr int tc_threads(bool wide, bool pair) { return TC_THREADS + 32 * (1 + (wide && pair ? 0 : TC_NORM_WARPS) + (pair && !wide ? 1 : 0)); }
 
 struct TcParams {
   const RowHdr* hdr2;
@@ -174,8 +177,34 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// (z0, z1) = (a0, a1) + the two floats of b
+__device__ __forceinline__ void tc_add2(float& z0, float& z1, uint32_t a0, uint32_t a1, unsigned long long b) {
+  asm("{\n\t.reg .b64 a;\n\tmov.b64 a, {%2, %3};\n\tadd.rn.f32x2 a, a, %4;\n\tmov.b64 {%0, %1}, a;\n\t}" : "=f"(z0), "=f"(z1) : "r"(a0), "r"(a1), "l"(b));
+}
+__device__ __forceinline__ float tc_max32(const float (&z)[32]) {
+  float m[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    m[i] = fmaxf(z[8 * i], z[8 * i + 1]);
+#pragma unroll
+    for (int c = 2; c < 8; c += 2) m[i] = fmaxf(fmaxf(m[i], z[8 * i + c]), z[8 * i + c + 1]);
+  }
+  return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
 __device__ __forceinline__ bool tc_better(float za, int ia, float zb, int ib) { return za > zb || (za == zb && ia < ib); }
 
+// Adds the squares of C of the eight 16-byte pieces of a 128-byte swizzled row, from piece c0 on
+template <int C>
+__device__ __forceinline__ void tc_squares(const unsigned char* row, int c0, int key, unsigned long long (&n)[2]) {
+  ulonglong2 w[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c) w[c] = *reinterpret_cast<const ulonglong2*>(row + (size_t)(((c0 + c) ^ key) * 16));
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(n[0]) : "l"(w[c].x));
+    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(n[1]) : "l"(w[c].y));
+  }
+}
 // One lane of a converged warp, the same at every call: the copies, multiplications and commits are its own, while the whole warp
 // walks the tiles and waits, so that their operands are the warp's.  Issued by one lane of a diverged warp an instruction took 84 to 134
 // cycles where the tensor pipe takes 64, which bounded the filter at every width (512 samples x 4,000,000 neurons x 256 units
@@ -198,12 +227,13 @@ __device__ __forceinline__ bool tc_elect() {
 // PAIR: two multiprocessors (a cluster of two blocks) share a tile, half of its rows in the shared memory of each, and take
 // 128 samples each; the first block issues instructions of 256 samples for both (use_pairs says when).  WIDE tiles are
 // then 256 neurons, so that the samples' slabs serve twice as many.
-// What a tile took besides the multiplications, 2,000 cycles at 128 units: its biases asked for only one tile ahead (an HBM
-// latency per tile), and in WIDE the one warp that sums the rows' squares, element by element (26,000 cycles per tile at 512 units,
-// with packed pairs of four rows side by side 16,000).
+// What a tile took besides the multiplications, 1,000 to 2,000 cycles: the issue of the multiplications (tc_elect), read-back warps that
+// waited for one another, the row norms (TC_NORM_WARPS).  Now 2,080 cycles at 256 units in pairs, of which the multiplications are
+// 2,050; 1,850 and 1,650 at 200 units in pairs; 1,740 and 1,060 at 128 units, where shared memory bounds it (the copies 64 KB,
+// the multiplications 64, the norms 32 to 64 per tile, at 128 bytes per cycle).
 // The rows' norms in pairs: the second block reads its half of a tile once the first block, which counts the copies, has passed
-// that on; at cluster scope this takes 1,000 cycles, which a warp of its own spends (by the norm warp itself 1,024 samples x
-// 253,855 neurons x 200 units took 262 us, so 256).  A slab has not that much time (512 samples x 100,003 neurons x 512 units 229 us):
+// that on; at cluster scope this takes 1,000 cycles, which a warp of its own spends (by the norm warps themselves 1,024 samples x
+// 253,855 neurons x 200 units took 262 us where a warp of its own took 256).  That warp's pace is the least time of a tile, 1,500 cycles.  A slab has not that much time (512 samples x 100,003 neurons x 512 units 229 us):
 // WIDE pairs take the norms from global memory, where L2 has the rows (135 us; at 200 units it would be 283): the read-back warps,
 // before they wait for the tile's scores.
 template <bool DUMP, bool WIDE, bool PAIR>      // DUMP: write every score out (threshold pass); else append the scores that reach the sample's threshold
@@ -244,8 +274,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   const int my_tiles = slice < p.ntiles ? (p.ntiles - slice + p.nslices - 1) / p.nslices : 0;
   // The filter launch also takes the largest squared row norm of W2 (the error bound needs it) from the tiles as
   // they pass through shared memory; up to four sample groups share a tile's rows (they all see the same tiles).
-  constexpr int RL = ROWS / 32;                                    // rows per lane, shared by the blocks that hold the same rows
-  const int nshare = (int)gridDim.y >= 4 && RL >= 4 ? 4 : ((int)gridDim.y >= 2 ? 2 : 1);
+  const int nshare = (int)gridDim.y >= 4 ? 4 : ((int)gridDim.y >= 2 ? 2 : 1);
   constexpr bool OWN_ROWS = WIDE && PAIR;                          // norms by the read-back warps
   const bool norms = !DUMP && !OWN_ROWS && (int)blockIdx.y < nshare;
   const int nacc = WIDE ? (PAIR ? 2 : TC_NACC) : (p.H <= TC_N ? TC_NACC : 2);      // accumulators in use; the activations follow them
@@ -254,7 +283,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   if (tid == 0) {
     tc_bar_init(bar_a, PAIR ? 8 : 4);            // a warp each
     tc_bar_init(bar_drain, 1);
-    for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_landed + i, 1); tc_bar_init(bar_empty + i, norms ? 2 : 1); }
+    for (int i = 0; i < NST; ++i) { tc_bar_init(bar_full + i, 1); tc_bar_init(bar_landed + i, 1); tc_bar_init(bar_empty + i, norms ? 1 + TC_NORM_WARPS : 1); }
     for (int i = 0; i < TC_NACC; ++i) { tc_bar_init(bar_accfull + i, 1); tc_bar_init(bar_accempty + i, (PAIR ? 2 : 1) * TC_EPI / 32); }
     for (int i = 0; i < TC_BT; ++i) { tc_bar_init(bar_bfull + i, 32); tc_bar_init(bar_bempty + i, TC_EPI / 32); }
     *abort_flag = 0;
@@ -377,73 +406,6 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         if (++acc == nacc) { acc = 0; ++accround; }
       }
     }
-  } else if (warp == 2) {
-    // ---------------- row norms: lane = row modulo 32; sums of squares do not care about the swizzle, but the
-    // lanes of a quarter-warp read different 16-byte pieces so that all banks are busy ----------------
-    if (norms) {
-      float best = 0.f;
-      int st = 0, stround = 0;
-      const int nrr = RL / nshare;                     // rows of this block: nrr per lane
-      // the bytes of a pair are counted in its first block, which tells the second
-      auto arrived = [&](int st, int stround) {
-        if (PAIR && rank == 1) tc_bar_wait<PAIR, true>(bar_landed + st, stround & 1, abort_flag);
-        else tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag);
-      };
-      for (int i = 0; i < my_tiles; ++i) {
-        if (WIDE) {
-          unsigned long long part[RL][2];              // the sums of the lane's rows over the slabs, in pairs
-#pragma unroll
-          for (int rr = 0; rr < RL; ++rr) part[rr][0] = part[rr][1] = 0ull;
-          for (int ks = 0; ks < ksub; ++ks) {
-            arrived(st, stround);
-            const unsigned char* tile = smB + (size_t)st * tile_bytes;
-#pragma unroll
-            for (int rr = 0; rr < RL; ++rr)
-              if (rr < nrr) {
-                const unsigned char* rowp = tile + (size_t)(32 * (nrr * (int)blockIdx.y + rr) + lane) * 128;
-                ulonglong2 w[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) w[c] = *reinterpret_cast<const ulonglong2*>(rowp + (size_t)((c ^ (lane & 7)) * 16));
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                  asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(part[rr][0]) : "l"(w[c].x));
-                  asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(part[rr][1]) : "l"(w[c].y));
-                }
-              }
-            __syncwarp();
-            if (lane == 0) tc_bar_arrive(bar_empty + st);
-            if (++st == nst) { st = 0; ++stround; }
-          }
-#pragma unroll
-          for (int rr = 0; rr < RL; ++rr)
-            best = fmaxf(best, (__uint_as_float((unsigned)part[rr][0]) + __uint_as_float((unsigned)(part[rr][0] >> 32))) +
-                                   (__uint_as_float((unsigned)part[rr][1]) + __uint_as_float((unsigned)(part[rr][1] >> 32))));
-          continue;
-        }
-        arrived(st, stround);
-        const unsigned char* tile = smB + (size_t)st * tile_bytes;
-        for (int rr = 0; rr < nrr; ++rr) {
-          const unsigned char* rowp = tile + (size_t)(32 * (nrr * (int)blockIdx.y + rr) + lane) * 128;
-          unsigned long long s0 = 0ull, s1 = 0ull;    // two pairs of partial sums (packed fp32 fused multiply-adds)
-          for (int ks = 0; ks < ksub; ++ks)
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(rowp + (size_t)ks * SLAB + (size_t)((c ^ (lane & 7)) * 16));
-              asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(s0) : "l"(w.x));
-              asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(s1) : "l"(w.y));
-            }
-          const float ssum = (__uint_as_float((unsigned)s0) + __uint_as_float((unsigned)(s0 >> 32))) +
-                             (__uint_as_float((unsigned)s1) + __uint_as_float((unsigned)(s1 >> 32)));
-          best = fmaxf(best, ssum);
-        }
-        __syncwarp();
-        if (lane == 0) tc_bar_arrive(bar_empty + st);
-        if (++st == nst) { st = 0; ++stround; }
-      }
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, d));
-      if (lane == 0) atomicMax(p.norm2max, __float_as_uint(best));
-    }
   } else if (warp == TC_THREADS / 32) {
     // ---------------- biases: a tile's, TC_BT tiles ahead of the read-back (zero past the last neuron) ----------------
     bool on = true;
@@ -460,7 +422,54 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tc_smem(bar_bfull + slot)) : "memory");
     }
     asm volatile("cp.async.wait_all;" ::: "memory");      // nothing is on its way into shared memory when the block ends
-  } else if (PAIR && !WIDE && warp == TC_THREADS / 32 + 1) {
+  } else if (!OWN_ROWS && warp > TC_THREADS / 32 && warp <= TC_THREADS / 32 + TC_NORM_WARPS) {
+    // ---------------- row norms: the lanes of the warps share the block's rows, one or more rows to a lane or 2 or 4 lanes to a
+    // row.  Sums of squares do not care about the swizzle, but the lanes of a quarter-warp read different 16-byte pieces so
+    // that all banks are busy ----------------
+    if (norms) {
+      constexpr int LANES = 32 * TC_NORM_WARPS, RMAX = ROWS / LANES > 1 ? ROWS / LANES : 1;
+      const int nrows = ROWS / nshare;                 // rows of this block
+      const int lpr = nrows < LANES ? LANES / nrows : 1, nrr = nrows < LANES ? 1 : nrows / LANES;
+      const int idx = (warp - TC_THREADS / 32 - 1) * 32 + lane, cn = 8 / lpr, c0 = idx % lpr * cn;
+      const int row0 = nrows * (int)blockIdx.y + idx / lpr;      // the lane's first row; the others LANES apart (multiples of eight)
+      float best = 0.f;
+      int st = 0, stround = 0;
+      for (int i = 0; i < my_tiles; ++i) {
+        unsigned long long n[RMAX][2];                 // sums of a row's squares, in pairs
+#pragma unroll
+        for (int rr = 0; rr < RMAX; ++rr) n[rr][0] = n[rr][1] = 0ull;
+        for (int k0 = 0; k0 < ksub; k0 += WIDE ? 1 : ksub) {      // the slabs of a stage
+          // the bytes of a pair are counted in its first block, which tells the second
+          if (PAIR && rank == 1) tc_bar_wait<PAIR, true>(bar_landed + st, stround & 1, abort_flag);
+          else tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag);
+          const unsigned char* tile = smB + (size_t)st * tile_bytes + (size_t)row0 * 128;
+#pragma unroll
+          for (int rr = 0; rr < RMAX; ++rr)
+            if (rr < nrr)
+              for (int ks = 0; ks < (WIDE ? 1 : ksub); ++ks) {
+                const unsigned char* rowp = tile + (size_t)ks * SLAB + (size_t)rr * LANES * 128;
+                if (cn == 8) tc_squares<8>(rowp, c0, row0 & 7, n[rr]);
+                else if (cn == 4) tc_squares<4>(rowp, c0, row0 & 7, n[rr]);
+                else tc_squares<2>(rowp, c0, row0 & 7, n[rr]);
+              }
+          __syncwarp();
+          if (lane == 0) tc_bar_arrive(bar_empty + st);
+          if (++st == nst) { st = 0; ++stround; }
+        }
+#pragma unroll
+        for (int rr = 0; rr < RMAX; ++rr) {
+          float sq = (__uint_as_float((unsigned)n[rr][0]) + __uint_as_float((unsigned)(n[rr][0] >> 32))) +
+                     (__uint_as_float((unsigned)n[rr][1]) + __uint_as_float((unsigned)(n[rr][1] >> 32)));
+          if (lpr >= 2) sq += __shfl_xor_sync(0xffffffffu, sq, 1);
+          if (lpr == 4) sq += __shfl_xor_sync(0xffffffffu, sq, 2);
+          best = fmaxf(best, sq);
+        }
+      }
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, d));
+      if (lane == 0) atomicMax(p.norm2max, __float_as_uint(best));
+    }
+  } else if (PAIR && !WIDE && warp == TC_THREADS / 32 + 1 + TC_NORM_WARPS) {
     // ---------------- first block of a pair: what has landed is passed on to the second block's row norms ----------------
     if (norms && rank == 0 && lane == 0) {
       int st = 0, stround = 0;
@@ -475,7 +484,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     // Per 32 columns the bias is added; then, threshold pass: the scores are written out; filter pass: which of them
     // reach the sample's threshold (32 independent comparisons, a bit each), then the appends of those that do.
     const int q = warp & 3;                 // a warp reaches the 32 lanes of tensor memory of its number modulo four
-    const int half = (warp - 3) >> 2;       // which share of a tile's columns
+    const int half = (warp - 2) >> 2;       // which share of a tile's columns
     const int row = 32 * q + lane;          // sample inside the block
     const int vslice = slice * TC_SPLIT + half;    // buffers are kept per (slice, share of the columns)
     int2* mybuf = p.cand + ((size_t)vslice * p.Bpad + s0 + row) * p.gbuf;
@@ -483,7 +492,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     int cnt = 0;
     if (DUMP && slice == 0 && half == 0) {      // the threshold pass also clears what the filter pass accumulates into
       if (s0 + row < p.B) p.need_fix[s0 + row] = 0;
-      if (tid == 96 && blockIdx.y == 0) { *p.norm2max = 0u; *p.n_fix = 0; }
+      if (tid == 64 && blockIdx.y == 0) { *p.norm2max = 0u; *p.n_fix = 0; }
     }
     if (!WIDE && half == 0) {
       // the block's activations -> tensor memory: lane = sample, column = hidden unit (samples past the batch: zeros)
@@ -516,7 +525,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       if (OWN_ROWS && !DUMP) {
         // up to four groups share the tile's rows, and so do their blocks and a block's warps: 4, 8 or 16 lanes to a row
         const int shares = (int)gridDim.y >= 4 ? 8 : ((int)gridDim.y >= 2 ? 4 : 2), share = 2 * (int)blockIdx.y + (int)rank;
-        const int lanes = 2 * shares, j = j0 + share * (NT / shares) + (warp - 3) * (32 / lanes) + lane / lanes;
+        const int lanes = 2 * shares, j = j0 + share * (NT / shares) + (warp - 2) * (32 / lanes) + lane / lanes;
         if (share < shares) {
           unsigned long long n0 = 0ull, n1 = 0ull;
           if (j < p.N) {
@@ -553,13 +562,12 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           }
         }
         const int jb = j0 + c0;
-        const float4* sb4 = reinterpret_cast<const float4*>(tb + c0);
         float z[32];
 #pragma unroll
-        for (int c4 = 0; c4 < 8; ++c4) {
-          const float4 bq = sb4[c4];
-          z[4 * c4] = __uint_as_float(r[4 * c4]) + bq.x; z[4 * c4 + 1] = __uint_as_float(r[4 * c4 + 1]) + bq.y;
-          z[4 * c4 + 2] = __uint_as_float(r[4 * c4 + 2]) + bq.z; z[4 * c4 + 3] = __uint_as_float(r[4 * c4 + 3]) + bq.w;
+        for (int c = 0; c < 32; c += 4) {    // two sums in one instruction
+          const ulonglong2 bq = *reinterpret_cast<const ulonglong2*>(tb + c0 + c);
+          tc_add2(z[c], z[c + 1], r[c], r[c + 1], bq.x);
+          tc_add2(z[c + 2], z[c + 3], r[c + 2], r[c + 3], bq.y);
         }
         if (DUMP) {
           // neurons past the end score -infinity
@@ -567,19 +575,14 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           for (int c = 0; c < 32; ++c)
             if (jb + c >= p.N) z[c] = -INFINITY;
           if (p.dump_max) {                  // the largest of the thread's 32 (none of them a number: minus infinity)
-            float most = -INFINITY;
-#pragma unroll
-            for (int c = 0; c < 32; c += 2) most = fmaxf(fmaxf(most, z[c]), z[c + 1]);
-            __stcg(p.dump + (size_t)(s0 + row) * p.dump_cols + (tile * NT + c0) / 32, most);
+            __stcg(p.dump + (size_t)(s0 + row) * p.dump_cols + (tile * NT + c0) / 32, tc_max32(z));
           } else {                           // all of them: 128 contiguous bytes
             float4* out = reinterpret_cast<float4*>(p.dump + (size_t)(s0 + row) * p.dump_cols + (size_t)tile * NT + c0);
 #pragma unroll
             for (int c4 = 0; c4 < 8; ++c4) __stcg(out + c4, make_float4(z[4 * c4], z[4 * c4 + 1], z[4 * c4 + 2], z[4 * c4 + 3]));
           }
         } else {
-          float most = -INFINITY;            // a score that is not a number is none of them
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) most = fmaxf(fmaxf(most, z[c]), z[c + 1]);
+          const float most = tc_max32(z);    // a score that is not a number is none of them
           if (__any_sync(0xffffffffu, most >= tau)) {
             unsigned hm = 0u;
 #pragma unroll
