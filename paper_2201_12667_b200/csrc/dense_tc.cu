@@ -73,7 +73,7 @@ struct TcParams {
   int B, Bpad, H, N, nslices, ntiles;          // ntiles: tiles this launch walks
   int tile_stride;                 // tile i of the launch is tile i * tile_stride of W2
   int stages;                      // tiles of W2 in flight, 1 .. TC_STAGES
-  int dump_cols, dump_max;         // scores (or, dump_max, largest of 32 neighbours' scores) per sample
+  int dump_cols, dump_max;         // per sample: largest scores of dump_max neighbours each
   int gbuf;                        // slots per candidate buffer
 };
 
@@ -574,8 +574,14 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
 #pragma unroll
           for (int c = 0; c < 32; ++c)
             if (jb + c >= p.N) z[c] = -INFINITY;
-          if (p.dump_max) {                  // the largest of the thread's 32 (none of them a number: minus infinity)
+          if (p.dump_max == 32) {            // the largest of the thread's 32 (none of them a number: minus infinity)
             __stcg(p.dump + (size_t)(s0 + row) * p.dump_cols + (tile * NT + c0) / 32, tc_max32(z));
+          } else if (p.dump_max == 4) {
+            float4* out = reinterpret_cast<float4*>(p.dump + (size_t)(s0 + row) * p.dump_cols + (tile * NT + c0) / 4);
+#pragma unroll
+            for (int c = 0; c < 32; c += 16)
+              __stcg(out + c / 16, make_float4(fmaxf(fmaxf(z[c], z[c + 1]), fmaxf(z[c + 2], z[c + 3])), fmaxf(fmaxf(z[c + 4], z[c + 5]), fmaxf(z[c + 6], z[c + 7])),
+                                               fmaxf(fmaxf(z[c + 8], z[c + 9]), fmaxf(z[c + 10], z[c + 11])), fmaxf(fmaxf(z[c + 12], z[c + 13]), fmaxf(z[c + 14], z[c + 15]))));
           } else {                           // all of them: 128 contiguous bytes
             float4* out = reinterpret_cast<float4*>(p.dump + (size_t)(s0 + row) * p.dump_cols + (size_t)tile * NT + c0);
 #pragma unroll
@@ -658,13 +664,17 @@ __device__ __forceinline__ uint32_t tc_key(float z) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 __device__ __forceinline__ float tc_unkey(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k); }
-// The cap-th largest of the block's per-thread keys, found bit by bit (a block-wide count per bit); 0 when fewer than
-// cap threads hold a key.
-__device__ __forceinline__ uint32_t tc_select(uint32_t mine, int cap) {
+// The rank-th largest of the keys in the warp's registers, V per lane, found bit by bit down to bit `last` (lower bits zero); 0
+// when fewer than rank of them are set.
+template <int V>
+__device__ __forceinline__ uint32_t tc_select(const uint32_t (&v)[V], int rank, int last) {
   uint32_t K = 0u;
-  for (int bit = 31; bit >= 0; --bit) {
+  for (int bit = 31; bit >= last; --bit) {
     const uint32_t trial = K | (1u << bit);
-    if (__syncthreads_count(mine >= trial) >= cap) K = trial;
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < V; ++i) n += v[i] >= trial ? 1 : 0;
+    if (__reduce_add_sync(0xffffffffu, n) >= rank) K = trial;
   }
   return K;
 }
@@ -689,14 +699,7 @@ __global__ void __launch_bounds__(32 * TAU_WARPS) k_tc_tau(const float* dump, in
 #pragma unroll
     for (int i = 0; i < TAU_V; ++i) v[i] = e0 + 32 * i < cols ? max(v[i], tc_key(z[i])) : v[i];
   }
-  uint32_t K = 0u;
-  for (int bit = 31; bit >= 12; --bit) {
-    const uint32_t trial = K | (1u << bit);
-    int n = 0;
-#pragma unroll
-    for (int i = 0; i < TAU_V; ++i) n += v[i] >= trial ? 1 : 0;
-    if (__reduce_add_sync(0xffffffffu, n) >= rank) K = trial;
-  }
+  const uint32_t K = tc_select(v, rank, 12);
   if (lane == 0) {
     float t = tc_unkey(K);
     if (K == 0u || !(t == t)) t = -INFINITY;      // everything passes
@@ -707,100 +710,125 @@ __global__ void __launch_bounds__(32 * TAU_WARPS) k_tc_tau(const float* dump, in
 // One block per sample: the slices' candidates -> those whose approximate score reaches the cap-th largest of the
 // threads' maxima (cap of them, or a few more) -> their exact fp32 logits -> the k best by (logit descending, id
 // ascending).  A sample for which the filter cannot be shown to be exact is listed for k_scan_all.
-constexpr int RF_THREADS = 256;
+// A chain of memory rounds, each of which asks for all it can: a thread reads the fill of its buffers and their first entries
+// together (most hold no more), a warp the rows of four candidates.  With the buffers' fills summed up, a search for every
+// entry, a count over the block for every bit of the cut and a row at a time it took 18.9 us for 256 samples x 670,091 neurons x
+// 128 units, now 12.4 (1,024 samples: 35 and 20).
+constexpr int RF_THREADS = 256, RF_WARPS = RF_THREADS / 32;
 constexpr int RF_MAXV = 512;       // buffers per sample at most
 constexpr int RF_SLOTS = 384;      // candidates scored exactly at most (k = 64: about 190 reach the cut)
-__global__ void __launch_bounds__(RF_THREADS)
+static_assert(RF_MAXV == 2 * RF_THREADS, "two places to a thread");
+constexpr int RF_ROWS = 4;         // candidates of a warp side by side
+__global__ void __launch_bounds__(RF_THREADS, 4)      // 512 samples in one wave
 k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* cand, const int* cand_cnt, int gbuf, const float* tau, int Bpad,
             const unsigned int* norm2max, int B, int H, int N, int cap, int nvs, int k, int32_t* out_ids, float* out_scores,
             const int* need_fix, int* n_fix, int* fix_list) {
-  __shared__ int offs[RF_MAXV + 1];
+  __shared__ uint32_t most[RF_THREADS];          // the threads' largest keys
+  __shared__ uint32_t sh_K;
   __shared__ float ez[RF_SLOTS], sz[RF_SLOTS];
   __shared__ int ei[RF_SLOTS], si[RF_SLOTS];
-  __shared__ float red[RF_THREADS / 32];
-  __shared__ int wsum[RF_THREADS / 32];
-  __shared__ int sh_n, sh_fix;
+  __shared__ float red[RF_WARPS];
+  __shared__ int sh_n, sh_fix, sh_total;
   const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) { sh_n = 0; sh_total = 0; }
   griddep_launch_dependents();
   griddep_wait();                                // the filter pass has completed
-  // fill of the sample's buffers -> their places in one list (exclusive scan; each thread owns RF_MAXV / RF_THREADS buffers)
-  {
-    constexpr int PER = RF_MAXV / RF_THREADS;
-    int c[PER], mine = 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) { const int v = tid * PER + i; c[i] = v < nvs ? __ldcg(cand_cnt + (size_t)v * Bpad + s) : 0; mine += c[i]; }
-    int inc = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) { const int o = __shfl_up_sync(0xffffffffu, inc, d); if (lane >= d) inc += o; }
-    if (lane == 31) wsum[warp] = inc;
-    if (tid == 0) { sh_n = 0; sh_fix = need_fix[s]; }      // a buffer of the sample ran over in the filter pass
-    __syncthreads();
-    int base = 0;
-    for (int w = 0; w < warp; ++w) base += wsum[w];
-    int run = base + inc - mine;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) { offs[tid * PER + i] = run; run += c[i]; }
-    if (tid == RF_THREADS - 1) offs[RF_MAXV] = run;
-    __syncthreads();
-  }
-  const int total = offs[RF_MAXV];
-  int nc = 0;
-  uint32_t K = 0u;
-  bool fix = false;
-  {
-  // Entry e of the sample's list lies in the buffer v with offs[v] <= e < offs[v + 1].  First walk: a thread keeps the
-  // largest key of its entries.  The candidates that reach the cap-th largest of these maxima go on (all of them when
-  // there are no more than cap): a second walk over the same entries (they are in L2) collects them.
-  auto entry = [&](int e) {
-    int lo = 0, hi = RF_MAXV;                     // invariant: offs[lo] <= e < offs[hi]
-    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (offs[mid] <= e) lo = mid; else hi = mid; }
-    return __ldcg(cand + ((size_t)lo * Bpad + s) * gbuf + (e - offs[lo]));
-  };
-  constexpr int KEEP = 8;                         // entries per thread that stay in registers between the walks
-  int2 keep[KEEP];
-  uint32_t mine = 0u;
-#pragma unroll
-  for (int i = 0; i < KEEP; ++i) {
-    const int e = tid + i * RF_THREADS;
-    keep[i] = e < total ? entry(e) : make_int2(0, 0);
-    const uint32_t key = e < total ? tc_key(__int_as_float(keep[i].x)) : 0u;
-    mine = key > mine ? key : mine;
-  }
-  for (int e = tid + KEEP * RF_THREADS; e < total; e += RF_THREADS) {
-    const uint32_t key = tc_key(__int_as_float(entry(e).x));
-    mine = key > mine ? key : mine;
-  }
-  K = total > cap ? tc_select(mine, cap) : 0u;
-#pragma unroll
-  for (int i = 0; i < KEEP; ++i)
-    if (tid + i * RF_THREADS < total && tc_key(__int_as_float(keep[i].x)) >= K) {
-      const int slot = atomicAdd(&sh_n, 1);
-      if (slot < RF_SLOTS) ei[slot] = keep[i].y;
-    }
-  for (int e = tid + KEEP * RF_THREADS; e < total; e += RF_THREADS) {
-    const int2 x = entry(e);
-    if (tc_key(__int_as_float(x.x)) >= K) { const int slot = atomicAdd(&sh_n, 1); if (slot < RF_SLOTS) ei[slot] = x.y; }
-  }
-  __syncthreads();
-  nc = sh_n;
-  fix = nc > RF_SLOTS;                            // many equal scores at the cut: the sample is scored exactly
-  }
-  if (!fix) {
-  // exact logits of the kept candidates: a warp per candidate, four partial sums per lane as in the exact path
+  if (tid == 0) sh_fix = need_fix[s];            // a buffer of the sample ran over in the filter pass
   const float4* h4 = reinterpret_cast<const float4*>(h + (size_t)s * H);
   const int H4 = H >> 2;
-  for (int e = warp; e < nc; e += RF_THREADS / 32) {
-    const int j = ei[e];
-    const float4* r = reinterpret_cast<const float4*>(W2 + (size_t)j * H);
-    float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
-    for (int c = lane; c < H4; c += 32) {
-      const float4 w = r[c], x = h4[c];
-      d0 = fmaf(w.x, x.x, d0); d1 = fmaf(w.y, x.y, d1); d2 = fmaf(w.z, x.z, d2); d3 = fmaf(w.w, x.w, d3);
-    }
-    float d = (d0 + d1) + (d2 + d3);
+  // A buffer's entries are shared out to 2^lg places, which makes more places than threads: a thread has two at most, and nearly
+  // every thread has a largest key to go by (with 64 results the cut is at the 144th).
+  const int lg = 31 - __clz(RF_MAXV / nvs), g = 1 << lg;
+  const int p1 = tid + RF_THREADS, s0 = tid & (g - 1), s1 = p1 & (g - 1);
+  const bool two = (p1 >> lg) < nvs;
+  const int c0 = (tid >> lg) < nvs ? __ldcg(cand_cnt + (size_t)(tid >> lg) * Bpad + s) : 0;
+  const int c1 = two ? __ldcg(cand_cnt + (size_t)(p1 >> lg) * Bpad + s) : 0;
+  const int2* buf0 = cand + ((size_t)(tid >> lg) * Bpad + s) * gbuf;
+  const int2* buf1 = cand + ((size_t)(p1 >> lg) * Bpad + s) * gbuf;
+  int2 first[4];                                 // two entries of each place
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-    if (lane == 0) ez[e] = hdr2[j].b + d;
+  for (int u = 0; u < 4; ++u) {
+    const int e = (u < 2 ? s0 : s1) + (u & 1) * g;
+    first[u] = e < (u < 2 ? c0 : c1) ? __ldcg((u < 2 ? buf0 : buf1) + e) : make_int2(0, 0);
+  }
+  // the thread's entries: f(score bits, id)
+  auto entries = [&](auto f) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if ((u < 2 ? s0 : s1) + (u & 1) * g < (u < 2 ? c0 : c1)) f(first[u].x, first[u].y);
+#pragma unroll 1
+    for (int i = 0; i < 2; ++i) {
+      const int2* buf = i ? buf1 : buf0;
+      const int c = i ? c1 : c0;
+#pragma unroll 1
+      for (int e0 = (i ? s1 : s0) + 2 * g; e0 < c; e0 += 4 * g) {
+        int2 x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = e0 + e * g < c ? __ldcg(buf + e0 + e * g) : make_int2(0, 0);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (e0 + e * g < c) f(x[e].x, x[e].y);
+      }
+    }
+  };
+  int total = 0;
+  uint32_t mine = 0u;
+  entries([&](int z, int) { const uint32_t key = tc_key(__int_as_float(z)); mine = key > mine ? key : mine; });
+  total = __reduce_add_sync(0xffffffffu, (s0 == 0 ? c0 : 0) + (s1 == 0 ? c1 : 0));
+  most[tid] = mine;
+  if (lane == 0) atomicAdd(&sh_total, total);
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t v[RF_WARPS];
+#pragma unroll
+    for (int i = 0; i < RF_WARPS; ++i) v[i] = most[32 * i + lane];
+    const uint32_t cut = tc_select(v, cap, 12);
+    if (lane == 0) sh_K = cut;
+  }
+  __syncthreads();
+  total = sh_total;
+  // The candidates that reach the cap-th largest of the threads' maxima, cut to 20 bits, go on, all of them when there are no more than cap
+  const uint32_t K = total <= cap ? 0u : sh_K;
+  entries([&](int z, int id) {
+    if (tc_key(__int_as_float(z)) >= K) { const int slot = atomicAdd(&sh_n, 1); if (slot < RF_SLOTS) ei[slot] = id; }
+  });
+  __syncthreads();
+  const int nc = sh_n;
+  const bool fix = nc > RF_SLOTS;                // many equal scores at the cut: the sample is scored exactly
+  if (!fix) {
+  // exact logits of the kept candidates, RF_ROWS of a warp side by side
+  for (int e0 = warp; e0 < nc; e0 += RF_ROWS * RF_WARPS) {
+    int j[RF_ROWS];
+    float4 q[RF_ROWS];                           // four partial sums per lane as in the exact path
+#pragma unroll
+    for (int u = 0; u < RF_ROWS; ++u) {
+      j[u] = ei[e0 + u * RF_WARPS < nc ? e0 + u * RF_WARPS : e0];
+      q[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const int mine = e0 + (lane < RF_ROWS ? lane : 0) * RF_WARPS;
+    const float bias = hdr2[ei[mine < nc ? mine : e0]].b;
+#pragma unroll 1
+    for (int i = lane; i < H4; i += 32) {
+      const float4 x = h4[i];
+      float4 a[RF_ROWS];
+#pragma unroll
+      for (int u = 0; u < RF_ROWS; ++u) a[u] = reinterpret_cast<const float4*>(W2 + (size_t)j[u] * H)[i];
+#pragma unroll
+      for (int u = 0; u < RF_ROWS; ++u) {
+        q[u].x = fmaf(a[u].x, x.x, q[u].x); q[u].y = fmaf(a[u].y, x.y, q[u].y);
+        q[u].z = fmaf(a[u].z, x.z, q[u].z); q[u].w = fmaf(a[u].w, x.w, q[u].w);
+      }
+    }
+    float d[RF_ROWS];
+#pragma unroll
+    for (int u = 0; u < RF_ROWS; ++u) d[u] = (q[u].x + q[u].y) + (q[u].z + q[u].w);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < RF_ROWS; ++u) d[u] += __shfl_xor_sync(0xffffffffu, d[u], o);
+#pragma unroll
+    for (int u = 0; u < RF_ROWS; ++u)
+      if (lane == u && mine < nc) ez[mine] = bias + d[u];
   }
   // |h|^2 of the sample
   float hs = 0.f;
@@ -823,7 +851,7 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
   }
   if (tid == 0) {
     float hn = 0.f;
-    for (int w = 0; w < RF_THREADS / 32; ++w) hn += red[w];
+    for (int w = 0; w < RF_WARPS; ++w) hn += red[w];
     // Every neuron that did not go on to the exact pass has an approximate score below T: the cut when candidates
     // were dropped here, else the sample's threshold (a neuron below it was never a candidate).  Its exact score is
     // at most T plus the error bound; the k best are certain when the k-th exact score lies above.
@@ -1182,9 +1210,9 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   int rank = (want * TC_TARGET + stride - 1) / stride;
   if (rank > want) rank = want;
   if (rank < 5) rank = 5;
-  // Where the subset has enough groups of 32 neighbours, their largest scores stand for it.
-  const int dump_max = nsub * NT / 32 >= 8 * rank ? 1 : 0;
-  const int dump_cols = dump_max ? nsub * NT / 32 : nsub * NT;
+  // Where the subset has enough groups of 32 or 4 neighbours, their largest scores stand for it.
+  const int dump_max = nsub * NT / 32 >= 8 * rank ? 32 : (nsub * NT / 4 >= 8 * rank ? 4 : 1);
+  const int dump_cols = nsub * NT / dump_max;
   int gbuf = TC_GBUF_MIN * NT / TC_SPLIT;
   while (gbuf * nvs < 4 * rank * stride) gbuf <<= 1;
   const size_t off_dump = off_cand + up((size_t)nvs * Bpad * gbuf * sizeof(int2));

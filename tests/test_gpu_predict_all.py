@@ -14,6 +14,7 @@ SHAPES = [            # H, N, batch, k
     (4, 3001, 3, 1), (36, 129, 5, 10), (36, 128, 1, 64), (36, 100, 2, 5), (36, 40, 3, 64), (200, 20011, 130, 5),
     (252, 9000, 33, 64), (256, 5000, 129, 9), (260, 5000, 40, 5), (516, 3000, 131, 17), (1024, 2049, 260, 3), (1020, 700, 1, 64),
     (132, 9000, 200, 3),
+    (32, 170003, 3, 5), (32, 170003, 130, 64), (64, 600, 1, 5), (32, 900, 2048, 2),      # the largest of 32 neighbours in the threshold pass; many and few buffers to a sample
 ]
 PAIRS = [             # two multiprocessors to a tile: more than 192 units, more than 128 samples, tiles that keep them busy
     (196, 19001, 256, 5), (200, 38017, 257, 9), (256, 18945, 256, 64), (224, 30011, 130, 3), (260, 38145, 140, 5), (292, 19001, 300, 5),
