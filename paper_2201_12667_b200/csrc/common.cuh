@@ -106,6 +106,17 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// two fused multiply-adds in one instruction: a += b * c on pairs of floats
+__device__ __forceinline__ void fma2(unsigned long long& a, unsigned long long b, unsigned long long c) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(b), "l"(c));
+}
+__device__ __forceinline__ unsigned long long pair2(float lo, float hi) {
+  return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
+__device__ __forceinline__ void mul2(unsigned long long& a, unsigned long long b) { asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b)); }
+
 struct Ctx;
 
 // Kernel ids for the per-kernel timing (must match the DSLIDE_K_* enum of the C ABI).

@@ -22,7 +22,6 @@ namespace dslide {
 
 constexpr int FWD_THREADS = 256;
 constexpr int FWD_WARPS = FWD_THREADS / 32;
-constexpr int MAX_KPT = 4;        // hidden units per thread: H <= 4 * 256
 constexpr int ACT_SM = 1024;      // active ids and logits are mirrored in shared memory when the set is this small
 constexpr int HID_MIN_BYTES = 64 * 1024;   // staging space for the hidden layer's rows of W1
 constexpr int RANK_MAX = 1024;    // candidate sets up to this size are put in order by counting, larger ones by a bitonic sort
@@ -90,9 +89,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
@@ -231,8 +230,104 @@ __device__ __forceinline__ float block_sum(float v, float* sh) {
   return r;
 }
 
-__device__ __forceinline__ bool topk_better(float za, int ia, float zb, int ib) {
-  return za > zb || (za == zb && ia < ib);
+// Floats as keys that order like them (unsigned), those that are no numbers last; no number has key 0.
+__device__ __forceinline__ uint32_t score_key(float z) {
+  const uint32_t b = __float_as_uint(z);
+  return z != z ? 1u : (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+// A score and its position as a word: the larger is the better, of equal scores the earlier
+__device__ __forceinline__ unsigned long long place_of(float z, int a) { return ((unsigned long long)score_key(z) << 32) | (uint32_t)~a; }
+// Inference: the k best of the scores zp[0 .. na) by (score descending, id ascending); ids ascend with the position (ids
+// null: they are the positions).  The scores that reach the k-th largest of the threads' maxima (about k of them) are counted
+// against one another: a score's place is the number of better ones.  Where too many are equal there, the best is taken k times.
+// Lists of k per warp, fed one score at a time by lane 0, took 11,000 to 14,600 of the 35,000 to 45,000 cycles of a block (154 to
+// 238 scores, 1 and 5 results), and their merge 1,400 to 5,700: 256 samples x 670,091 neurons, 5 results, 29.4 us, now 20.0;
+// 64 samples with 6,000 scores of 128 units, 64 results, 620 us, now 108.
+// mine: the best of the thread's own scores (any sharing out; place_of: zero when it has none).  work: [512].  Called by the whole
+// block.  With k = 1 the scores are not read again (zp need not hold them).
+constexpr int BEST_N = 384;
+__device__ __noinline__ void best_of(int32_t* out_i, float* out_z, int k, const int* ids, const float* zp, int na, unsigned long long mine,
+                                     unsigned long long* work, int* sh_n) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto most = [&](unsigned long long best) {         // over the block
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(FULLM, best, d);
+      best = o > best ? o : best;
+    }
+    if (lane == 0) work[warp] = best;
+    __syncthreads();
+    for (int w = 0; w < FWD_WARPS; ++w) best = work[w] > best ? work[w] : best;
+    return best;
+  };
+  if (k == 1) {
+    const unsigned long long best = most(mine);
+    if (tid == 0) {
+      const uint32_t key = (uint32_t)(best >> 32);
+      const int a = (int)~(uint32_t)best;
+      out_i[0] = na == 0 ? -1 : ids ? ids[a] : a;
+      out_z[0] = na == 0 ? -INFINITY : key == 1u ? NAN : __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
+    }
+    return;
+  }
+  uint32_t* sh_max = reinterpret_cast<uint32_t*>(work + BEST_N);      // [FWD_THREADS]
+  sh_max[tid] = (uint32_t)(mine >> 32);
+  if (tid == 0) *sh_n = 0;
+  __syncthreads();                     // the scores are visible to the block, too
+  // every warp finds the cut by itself, bit by bit; the last bits are left out: a few more scores reach it
+  uint32_t v[FWD_WARPS], K = 0u;
+#pragma unroll
+  for (int i = 0; i < FWD_WARPS; ++i) v[i] = sh_max[32 * i + lane];
+  for (int bit = 31; bit >= 12; --bit) {
+    const uint32_t trial = K | (1u << bit);
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < FWD_WARPS; ++i) c += v[i] >= trial ? 1 : 0;
+    if (__reduce_add_sync(FULLM, c) >= k) K = trial;
+  }
+  constexpr int U = 8;
+  for (int a0 = tid; a0 < na; a0 += U * FWD_THREADS) {
+    uint32_t key[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) key[u] = a0 + u * FWD_THREADS < na ? score_key(zp[a0 + u * FWD_THREADS]) : 0u;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (a0 + u * FWD_THREADS < na && key[u] >= K) {
+        const int at = atomicAdd(sh_n, 1);
+        if (at < BEST_N) work[at] = ((unsigned long long)key[u] << 32) | (uint32_t)~(a0 + u * FWD_THREADS);
+      }
+  }
+  __syncthreads();
+  const int n = *sh_n;
+  auto put = [&](int place, unsigned long long x) {
+    const int a = (int)~(uint32_t)x;
+    out_i[place] = ids ? ids[a] : a;
+    out_z[place] = zp[a];
+  };
+  for (int q = na + tid; q < k; q += FWD_THREADS) { out_i[q] = -1; out_z[q] = -INFINITY; }      // fewer scores than results
+  if (n <= BEST_N) {
+    for (int e = tid; e < n; e += FWD_THREADS) {
+      const unsigned long long x = work[e];
+      int place = 0;
+#pragma unroll 4
+      for (int u = 0; u < n; ++u) place += work[u] > x ? 1 : 0;
+      if (place < k) put(place, x);
+    }
+    return;
+  }
+  __syncthreads();
+  unsigned long long last = ~0ull;     // (na > BEST_N >= k)
+  for (int q = 0; q < k; ++q) {
+    unsigned long long best = 0ull;
+    for (int a = tid; a < na; a += FWD_THREADS) {
+      const unsigned long long x = place_of(zp[a], a);
+      if (x < last && x > best) best = x;
+    }
+    best = most(best);
+    __syncthreads();
+    last = best;
+    if (tid == 0) put(q, best);
+  }
 }
 
 // Puts n <= PER * FWD_THREADS values in ascending order by counting: the place of a value is the number of values
@@ -487,11 +582,18 @@ __device__ __forceinline__ void skip_sample(const FwdParams& p, int s, int code)
   if (tid == 0) set_status(p.st, code);
 }
 
+// Rows of a group in the pass over the active rows: eight 16-byte pieces of them in a lane's registers, four rows at most (a reduction,
+// an exponential and a look at the maximum for all of them)
+template <int NP> struct RowPass { static constexpr int ROWS = NP <= 2 ? 4 : 8 / NP; };
+constexpr int RING_DEPTH = 8;      // groups of a warp's ring at most
+constexpr int RING_HEAD = FWD_WARPS * RING_DEPTH * 8 + 16;      // the rings' barriers, and 16 bytes of zeros
+
 // MODE 0 = training step, 1 = predict top-k, 2 = the part of a training step up to the active sets (tiles.cu goes on from
-// there: sets of many neurons that the batch's samples share); KPT = hidden units per thread (H <= KPT * FWD_THREADS); BULK: active sets of
-// many chunks are expected (the host's estimate from the tables' shape) and their rows come by bulk copies
-template <int MODE, int KPT, bool BULK = false>
+// there: sets of many neurons that the batch's samples share); NP = 16-byte pieces of a row that a lane holds (H <= 128 * NP);
+// BULK, of NP = 1: active sets of many chunks are expected (the host's estimate from the tables' shape) and their rows come by bulk copies
+template <int MODE, int NP, bool BULK = false>
 __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
+  constexpr int KPT = NP <= 2 ? 1 : NP / 2;      // hidden units per thread
   extern __shared__ __align__(128) unsigned char smem[];
   float* sh_h = reinterpret_cast<float*>(smem);
   float* sh_dh = reinterpret_cast<float*>(smem + p.off_dh);          // [FWD_WARPS][H]
@@ -500,7 +602,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   int* sh_misc = reinterpret_cast<int*>(smem + p.off_misc);          // 32 ints
   float* sh_red = reinterpret_cast<float*>(sh_misc + 16);
   uint64_t* sh_bar = reinterpret_cast<uint64_t*>(sh_misc + 26);      // 8-byte aligned: off_misc is 16-byte aligned
-  uint64_t* sh_bar2 = reinterpret_cast<uint64_t*>(sh_misc + 28);     // completion of the hash functions' mirror
+  uint64_t* sh_bar2 = reinterpret_cast<uint64_t*>(sh_misc + 28);     // completion of the hash functions' mirror 
   int* sh_lab = reinterpret_cast<int*>(smem + p.off_lab);            // [max_labels]
   int* sh_tbase = reinterpret_cast<int*>(smem + p.off_tbase);        // [L + 1]
   int* sh_tbeg = reinterpret_cast<int*>(smem + p.off_tbeg);          // [L]
@@ -1074,19 +1176,27 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     if (tid == 0) {
       int ny = 0;
       for (int i = 0; i < nlab; ++i) ny += sh_lab[i] >= 0 ? 1 : 0;
-      sh_misc[0] = ny;
+      sh_misc[8] = ny;
     }
   }
 
+  float* z = p.act_z + (size_t)s * p.act_stride;
+  unsigned long long mine = 0ull;                  // predict: the thread's best score
+  const bool keep_z = MODE == 0 || (!small && p.topk > 1);
+  // hand-off to the update kernel: the touch counters of the sample's rows of W1 (one per thread) and of HO_PER of its active
+  // rows per thread (act0: which) are asked while the first rows of W2 are on their way, the list places after the
+  // first logits, and everything is written at the end -- no warp waits for an answer
+  constexpr int HO_PER = 2;
+  int jj0[HO_PER], act0[HO_PER], ho_rows = HO_PER * FWD_THREADS;
+  unsigned nth1 = 0u, nth0[HO_PER], base1 = 0u, base0[HO_PER];
+#pragma unroll
+  for (int u = 0; u < HO_PER; ++u) { jj0[u] = 0; act0[u] = -1; nth0[u] = 0u; base0[u] = 0u; }
+  if constexpr (NP == 1) {
   // ---- logits over the active set.  The active rows of W2 are copied into shared memory, as many as fit at a
   //      time.  When the whole set fits, the rows stay there for the back-propagation below.  When it does not, the
   //      back-propagated error is accumulated in the same pass, chunk by chunk, with a running maximum M and sums
   //      rescaled whenever M grows: S = sum_a exp(z_a - M) W2[j_a,:], E = sum_a exp(z_a - M), and T = the sum of the
   //      label rows; then dh = (S / E - T / |Y|) / B, and every row is fetched once. ----
-  float* z = p.act_z + (size_t)s * p.act_stride;
-  float* tk_z = reinterpret_cast<float*>(smem + p.off_topk);          // predict: [FWD_WARPS][topk]
-  int* tk_id = reinterpret_cast<int*>(tk_z + FWD_WARPS * p.topk);
-  int tk_cnt = 0;                                                     // used by lane 0
   const float4* sh_h4 = reinterpret_cast<const float4*>(sh_h);
   const int ldr = H + 4;                           // staged rows are padded by 16 bytes: a thread per row reads without bank conflicts
   const int stage_rows = p.stage_bytes / (ldr * 4 + 4);      // a row and one float of the chunk's exp(z - M)
@@ -1098,17 +1208,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   for (int u = 0; u < KPT; ++u) { accS[u] = 0.f; accT[u] = 0.f; }
   const int ngrp = H >= FWD_THREADS ? 1 : min(FWD_WARPS, FWD_THREADS / H);   // groups of H threads (sh_dh holds FWD_WARPS)
   const int grp = H >= FWD_THREADS ? 0 : tid / H;
-  // hand-off to the update kernel: the touch counters of the sample's rows of W1 (one per thread) and of its first
-  // HO_PER * FWD_THREADS active rows are asked while the first rows of W2 are on their way, the list places after the
-  // first logits, and everything is written at the end -- no warp waits for an answer
-  constexpr int HO_PER = 2;
-  int jj0[HO_PER];
-  unsigned nth1 = 0u, nth0[HO_PER], base1 = 0u, base0[HO_PER];
   // a thread's place in the copy pattern of the padded rows: H4 + 1 pieces per row
   const int rp_dr = FWD_THREADS / (H4 + 1), rp_dc = FWD_THREADS - rp_dr * (H4 + 1);
   const int rp_r0 = tid / (H4 + 1), rp_c0 = tid - rp_r0 * (H4 + 1);
-#pragma unroll
-  for (int u = 0; u < HO_PER; ++u) { jj0[u] = 0; nth0[u] = 0u; base0[u] = 0u; }
   uint32_t w2phase = 0u;
   bool timed_out = false;                          // block-uniform
   const bool bulk = BULK && streaming && na >= 4 * stage_rows;      // many chunks: the batch's samples share most rows (see below)
@@ -1155,6 +1257,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
           const int a = tid + u * FWD_THREADS;
           if (a < na) {
             jj0[u] = idp[a];
+            act0[u] = a;
             nth0[u] = atomicAdd(&p.hdr2[jj0[u]].cnt, 1u) & CNT_MASK;
           }
         }
@@ -1186,35 +1289,12 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
         }
         dot = (d0 + d1) + (d2 + d3);
       }
-      if (MODE == 0) {
-        if (live) {
-          const float zv = stage[(size_t)a * ldr + H + 1] + dot;      // the bias came with the row
-          if (small) sh_z[c0 + a] = zv;
-          z[c0 + a] = zv;
-          if (streaming) sh_ce[a] = zv;
-        }
-      } else {
-        // predict: lane 0 of each warp keeps the warp's best k so far, fed one lane's logit at a time
-        int j = -1;
-        float zv = 0.f;
-        if (live) { j = dense ? c0 + a : idp[c0 + a]; zv = stage[(size_t)a * ldr + H + 1] + dot; }
-        float* lz = tk_z + warp * p.topk;
-        int* li = tk_id + warp * p.topk;
-        // a lane offers its logit only when the list is not full yet or the logit beats the list's last entry
-        const int n = __shfl_sync(FULLM, tk_cnt, 0);
-        unsigned m = __ballot_sync(FULLM, j >= 0 && (n < p.topk || topk_better(zv, j, lz[p.topk - 1], li[p.topk - 1])));
-        while (m) {
-          const int l = __ffs(m) - 1;
-          m &= m - 1;
-          const int jl = __shfl_sync(FULLM, j, l);
-          const float zl = __shfl_sync(FULLM, zv, l);
-          if (lane == 0 && (tk_cnt < p.topk || topk_better(zl, jl, lz[tk_cnt - 1], li[tk_cnt - 1]))) {
-            int q = tk_cnt < p.topk ? tk_cnt++ : p.topk - 1;
-            while (q > 0 && topk_better(zl, jl, lz[q - 1], li[q - 1])) { lz[q] = lz[q - 1]; li[q] = li[q - 1]; --q; }
-            lz[q] = zl; li[q] = jl;
-          }
-          __syncwarp();
-        }
+      if (live) {
+        const float zv = stage[(size_t)a * ldr + H + 1] + dot;      // the bias came with the row
+        if (small) sh_z[c0 + a] = zv;
+        if (keep_z) z[c0 + a] = zv;
+        if (streaming) sh_ce[a] = zv;
+        if (MODE == 1) mine = max(mine, place_of(zv, c0 + a));
       }
     }
     if (MODE == 0 && c0 == 0) {
@@ -1277,29 +1357,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     if (tid == 0) set_status(p.st, DSLIDE_ERR_TIMEOUT);
   }
   if (MODE == 1) {
-    // ---- merge the per-warp lists: k rounds over the list heads ----
-    if (lane == 0) sh_misc[warp] = tk_cnt;
-    __syncthreads();
-    if (tid == 0) {
-      int head[FWD_WARPS];
-      for (int w = 0; w < FWD_WARPS; ++w) head[w] = 0;
-      for (int q = 0; q < p.topk; ++q) {
-        int bw = -1;
-        for (int w = 0; w < FWD_WARPS; ++w) {
-          if (head[w] >= sh_misc[w]) continue;
-          if (bw < 0 || topk_better(tk_z[w * p.topk + head[w]], tk_id[w * p.topk + head[w]],
-                                    tk_z[bw * p.topk + head[bw]], tk_id[bw * p.topk + head[bw]])) bw = w;
-        }
-        if (bw >= 0) {
-          p.out_ids[(size_t)s * p.topk + q] = tk_id[bw * p.topk + head[bw]];
-          p.out_scores[(size_t)s * p.topk + q] = tk_z[bw * p.topk + head[bw]];
-          head[bw]++;
-        } else {
-          p.out_ids[(size_t)s * p.topk + q] = -1;
-          p.out_scores[(size_t)s * p.topk + q] = -INFINITY;
-        }
-      }
-    }
+    unsigned long long* work = reinterpret_cast<unsigned long long*>(smem + p.off_topk);
+    best_of(p.out_ids + (size_t)s * p.topk, p.out_scores + (size_t)s * p.topk, p.topk, dense ? nullptr : idp, zp, na, mine, work,
+            sh_misc);
     return;
   }
   __syncthreads();           // logits visible to the block
@@ -1328,7 +1388,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     }
   }
   const float fB = (float)p.B;
-  const int ny = sh_misc[0];
+  const int ny = sh_misc[8];
   if (tid == FWD_THREADS - 1) {                    // the last thread has the fewest rows below
     float sum = 0.f;
     const float logE = logf(E);
@@ -1353,7 +1413,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   //      the staged rows w, w + 8, ...; a lane holds four consecutive hidden units of every 128; the warps' sums are
   //      then added in warp order.  When the rows were streamed the sums exist already (per group of threads). ----
   {
-    constexpr int NCH = KPT == 1 ? 2 : 2 * MAX_KPT;        // 16-byte pieces of a row per lane: H <= 128 * NCH
+    constexpr int NCH = 2;                                 // 16-byte pieces of a row per lane: H <= 128 * NCH
     int nparts = ngrp;
     if (!streaming) {
       nparts = FWD_WARPS;
@@ -1393,6 +1453,268 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       p.dh[(size_t)s * H + k] = sh_h[k] > 0.f && !(BULK && timed_out) ? v : 0.f;
     }
   }
+  } else {
+  // ---- one pass over the active rows of W2: logits and, with a running maximum M, the sums S = sum_a exp(z_a - M) W2[j_a,:]
+  //      and E = sum_a exp(z_a - M); then dh = (S / E - T / |Y|) / B with T the sum of the label rows.  Warp w takes the groups
+  //      w, w + 8, ... of ROWS rows through its own ring in shared memory: a bulk copy per row, completion on an mbarrier per
+  //      group; the groups ahead are in flight while a group is read, once, for both sums.  No warp waits for another, and
+  //      whatever the set's size the rings are full until its end.  Bound by the instructions of a warp (about 400 a group at
+  //      four cycles), by what a multiprocessor keeps in flight (2 x 90 KB) for few rows.  In chunks of the whole space, with
+  //      barriers around each and a thread per staged row, logits and copies took 57,000 cycles of a block's 96,000 at 512 units and
+  //      160 rows.  At up to 128 units that is the better way still: a thread per row takes a fortieth of the instructions
+  //      for a logit, and most sets are one chunk (256 x 670,091 x 128: a step 64.1 us, by rings 64.9; 32 x 2,000 x 32: 31.1 and 39.8) ----
+  float M = -INFINITY, E = 0.f;
+  float accT[KPT];
+#pragma unroll
+  for (int u = 0; u < KPT; ++u) accT[u] = 0.f;
+  {
+    constexpr int R = RowPass<NP>::ROWS, Q = 32 / R;         // rows of a group; lanes that end with the same row's sum
+    const int row_b = H * 4, nw = min(FWD_WARPS, (p.stage_bytes - RING_HEAD) / (R * row_b));      // warps that have a ring (all but in tight layouts)
+    const int depth = min(RING_DEPTH, (p.stage_bytes - RING_HEAD) / nw / (R * row_b));            // groups of a ring
+    uint64_t* bars = reinterpret_cast<uint64_t*>(stage) + warp * RING_DEPTH;
+    float* zeros = stage + RING_HEAD / 4 - 4;
+    float* ring = stage + RING_HEAD / 4 + (size_t)warp * depth * R * H;
+    const int ngroups = (na + R - 1) / R, mygroups = warp < nw && warp < ngroups ? (ngroups - warp + nw - 1) / nw : 0;
+    fence_proxy_async();
+    __syncthreads();                               // the readers of the space before this are done
+    if (lane < RING_DEPTH) mbar_init(bars + lane, 1);
+    if (tid == 0) { zeros[0] = zeros[1] = zeros[2] = zeros[3] = 0.f; sh_misc[9] = 0; }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_proxy_async();
+    __syncthreads();
+    // Rows of the warp, 32 at a time: lane l has row l % R of group l / R -- its id, its bias and, of the first two rounds, the
+    // touch counter's answer
+    auto row_of = [&](int l) { const int a = (warp + (l / R) * nw) * R + l % R; return l / R < mygroups && a < na ? a : -1; };
+    auto id_of = [&](int a) { return a < 0 ? 0 : (dense ? a : idp[a]); };
+    int ac = row_of(lane), idc = id_of(ac), an = row_of(32 + lane), idn = id_of(an);
+    float bc = ac < 0 ? 0.f : p.hdr2[idc].b, bn = 0.f;      // of the batch that is summed; of the one that is asked for
+    int gi = 0, gslot = 0;                                   // group to ask for, and its place in the ring
+    static_assert(HO_PER == 2, "the counters of a warp's first 64 rows");
+    auto count_in = [&](int u) {                             // training: the touch counters of the rows
+      if (MODE != 0 || dense || u >= HO_PER) return;
+      const unsigned nth = ac >= 0 ? atomicAdd(&p.hdr2[idc].cnt, 1u) & CNT_MASK : 0u;
+      if (u == 0) { act0[0] = ac; jj0[0] = idc; nth0[0] = nth; }
+      else { act0[1] = ac; jj0[1] = idc; nth0[1] = nth; }
+    };
+    auto ask = [&]() {
+      if (gi < mygroups) {
+        const int l0 = (gi * R) & 31, l = lane - l0, m = min(R, na - (warp + gi * nw) * R);
+        if (l0 == 0 && gi > 0) {                             // the next 32 rows
+          ac = an; idc = idn;
+          bn = ac < 0 ? 0.f : p.hdr2[idc].b;
+          count_in(gi * R / 32);
+          an = row_of(gi * R + 32 + lane);
+          idn = id_of(an);
+        }
+        if (lane == 0) mbar_expect_tx(bars + gslot, (uint32_t)(m * row_b));
+        __syncwarp();
+        if (l >= 0 && l < m) bulk_g2s(ring + (gslot * R + l) * H, p.W2 + (size_t)idc * H, (uint32_t)row_b, bars + gslot);
+        ++gi;
+        gslot = gslot + 1 == depth ? 0 : gslot + 1;
+      }
+    };
+    for (int i = 0; i < depth - 1; ++i) ask();
+    if (MODE == 0) {
+      // the touch counter of this thread's nonzero of the sample
+      if (tid < nnz) {
+        if (tid >= p.hid_rows) {                     // beyond the first chunk: not kept in registers above
+          c1 = __ldg(p.col_idx + rbeg + tid);
+          x1 = __ldg(p.vals + rbeg + tid);
+          line1 = __ldcg(p.hotmap1 + c1);
+        }
+        nth1 = atomicAdd(&p.hdr1[c1].cnt, 1u) & CNT_MASK;
+        if (line1 >= 0) p.hotcoef1[(size_t)line1 * p.bstride + s] = x1;
+      }
+      count_in(0);
+      ho_rows = HO_PER * 32 * nw;
+    }
+    constexpr bool HREG = NP <= 4;                 // the sample's activations in registers, else read again for every row
+    constexpr int SURE = NP / 2;                   // pieces that every lane has; past the row's end it reads zeros (not a piece of the
+    ulonglong2 hx[HREG ? NP : 1], S[NP];           // row: a weight of minus infinity times an activation of zero is no number)
+    const ulonglong2* sh_h2 = reinterpret_cast<const ulonglong2*>(sh_h);
+    const float* base[NP - SURE];
+    int mul[NP - SURE];
+#pragma unroll
+    for (int u = 0; u < NP; ++u) {
+      const bool in = lane + 32 * u < H4;
+      if (HREG) hx[HREG ? u : 0] = in ? sh_h2[lane + 32 * u] : make_ulonglong2(0ull, 0ull);
+      S[u] = make_ulonglong2(0ull, 0ull);            // pairs of floats: two multiply-adds per instruction
+      if (u >= SURE) {
+        base[u < SURE ? 0 : u - SURE] = in ? ring + 4 * (lane + 32 * u) : zeros;
+        mul[u < SURE ? 0 : u - SURE] = in ? H : 0;
+      }
+    }
+    int slot = 0;
+    uint32_t phase = 0u;
+#pragma unroll 1
+    for (int i = 0; i < mygroups; ++i) {
+      ask();
+      if (!bar_wait_limited(bars + slot, phase)) {
+        if (lane == 0) sh_misc[9] = 1;
+        for (int q = i; q < gi; ++q) {             // what is still in flight gets one more bounded wait
+          bar_wait_limited(bars + slot, phase);
+          if (++slot == depth) { slot = 0; phase ^= 1u; }
+        }
+        break;
+      }
+      const int a0 = (warp + i * nw) * R, m = min(R, na - a0), at0 = slot * R, l0 = (i * R) & 31;
+      if (++slot == depth) { slot = 0; phase ^= 1u; }
+      if (l0 == 0 && i > 0) bc = bn;
+      ulonglong2 x[R][NP];
+      float d[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        unsigned long long d0 = 0ull, d1 = 0ull;
+        if (r < m) {
+#pragma unroll
+          for (int u = 0; u < NP; ++u) {
+            x[r][u] = *reinterpret_cast<const ulonglong2*>(u < SURE ? ring + (at0 + r) * H + 4 * (lane + 32 * u)
+                                                                    : base[u < SURE ? 0 : u - SURE] + (at0 + r) * mul[u < SURE ? 0 : u - SURE]);
+            const ulonglong2 hv = HREG ? hx[HREG ? u : 0] : *(u < SURE || lane + 32 * u < H4 ? sh_h2 + lane + 32 * u : reinterpret_cast<const ulonglong2*>(zeros));
+            fma2(d0, x[r][u].x, hv.x);
+            fma2(d1, x[r][u].y, hv.y);
+          }
+        }
+        d[r] = (lo2(d0) + hi2(d0)) + (lo2(d1) + hi2(d1));
+      }
+      // every exchange halves the rows a lane has part of
+#pragma unroll
+      for (int n2 = R / 2, o = 16; n2 > 0; n2 >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int r = 0; r < n2; ++r) d[r] = (up ? d[r + n2] : d[r]) + __shfl_xor_sync(FULLM, up ? d[r] : d[r + n2], o);
+      }
+      float y = d[0];
+#pragma unroll
+      for (int o = Q / 2; o > 0; o >>= 1) y += __shfl_xor_sync(FULLM, y, o);
+      const int q = lane / Q, at = a0 + q;         // the row whose sum this lane has
+      const float bias = __shfl_sync(FULLM, bc, l0 + q);
+      const float zv = q < m ? bias + y : -INFINITY;
+      if (q < m && (lane & (Q - 1)) == (i & (Q - 1))) {      // a lane of the row's, in turn (predict: the threads' maxima)
+        if (small) sh_z[at] = zv;
+        if (keep_z) z[at] = zv;
+        if (MODE == 1) mine = max(mine, place_of(zv, at));
+      }
+      if (MODE == 0) {
+        if (__any_sync(FULLM, zv > M)) {
+          float zm = fmaxf(zv, M);
+#pragma unroll
+          for (int o = Q; o < 32; o <<= 1) zm = fmaxf(zm, __shfl_xor_sync(FULLM, zm, o));
+          const float scale = expf(M - zm);
+          const unsigned long long sc = pair2(scale, scale);
+          M = zm;
+          E *= scale;
+#pragma unroll
+          for (int u = 0; u < NP; ++u) {
+            mul2(S[u].x, sc);
+            mul2(S[u].y, sc);
+          }
+        }
+        // a masked neuron (bias of minus infinity) weighs nothing, also while nothing else has been met and M is minus infinity
+        const float e = zv != -INFINITY ? expf(zv - M) : 0.f;
+        E += e;                                    // this lane's rows only, until the end
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const float g = __shfl_sync(FULLM, e, Q * r);
+          const unsigned long long gg = pair2(g, g);
+          if (r < m) {
+#pragma unroll
+            for (int u = 0; u < NP; ++u) {
+              fma2(S[u].x, gg, x[r][u].x);
+              fma2(S[u].y, gg, x[r][u].y);
+            }
+          }
+        }
+      }
+      __syncwarp();                                // the rows have been read: their places may be filled again
+    }
+    if (MODE == 0) {
+#pragma unroll
+      for (int o = Q; o < 32; o <<= 1) E += __shfl_xor_sync(FULLM, E, o);      // lanes hold different rows
+#pragma unroll
+      for (int u = 0; u < NP; ++u)
+        if (lane + 32 * u < H4) reinterpret_cast<ulonglong2*>(sh_dh + (size_t)warp * H)[lane + 32 * u] = S[u];
+      if (lane == 0) { sh_misc[warp] = __float_as_int(M); sh_red[warp] = E; }
+    }
+  }
+  if (MODE == 1) {
+    __syncthreads();
+    if (sh_misc[9] != 0) {                         // a copy did not complete in time
+      skip_sample<MODE>(p, s, DSLIDE_ERR_TIMEOUT);
+      return;
+    }
+    unsigned long long* work = reinterpret_cast<unsigned long long*>(smem + p.off_topk);
+    best_of(p.out_ids + (size_t)s * p.topk, p.out_scores + (size_t)s * p.topk, p.topk, dense ? nullptr : idp, zp, na, mine, work,
+            sh_misc);
+    return;
+  }
+  // the label rows (they are in L2 by now)
+  for (int i = 0; i < nlab; ++i)
+    if (sh_lab[i] >= 0) {
+      const float* row = p.W2 + (size_t)p.labels[lbeg + i] * H;
+#pragma unroll
+      for (int u = 0; u < KPT; ++u)
+        if (tid + u * FWD_THREADS < H) accT[u] += row[tid + u * FWD_THREADS];
+    }
+  // the touch counters have answered by now.  W1 side: slot / mask entries (the coefficient is the input value);
+  // both sides: places in the lists of distinct rows asked for, used at the end of the kernel
+  touch_mark<false>(p, tid < nnz, p.hdr1 + c1, p.mask1 + (size_t)c1 * p.Wd, p.ovf1 + (size_t)c1 * PAIR_T, ~c1, nth1, s, x1);
+  base1 = own_reserve(tid < nnz && nth1 == 0u, &p.st->n_own[p.parity][1]);
+#pragma unroll
+  for (int u = 0; u < HO_PER; ++u) base0[u] = own_reserve(act0[u] >= 0 && nth0[u] == 0u, &p.st->n_own[p.parity][0]);
+  __syncthreads();           // logits and the warps' sums visible to the block
+  // A copy did not complete in time: the sample is given up.  Its touches are already counted, so the hand-off below still
+  // runs, with every coefficient zero.
+  const bool timed_out = sh_misc[9] != 0;
+  if (timed_out && tid == 0) set_status(p.st, DSLIDE_ERR_TIMEOUT);
+
+  // ---- the warps' maxima and sums put together; loss, errors, error at the hidden layer ----
+  float* pr = p.act_p + (size_t)s * p.act_stride;
+  float* g = p.act_g + (size_t)s * p.act_stride;
+  float fac[FWD_WARPS];
+  M = __int_as_float(sh_misc[0]);
+#pragma unroll
+  for (int w = 1; w < FWD_WARPS; ++w) M = fmaxf(M, __int_as_float(sh_misc[w]));
+  E = 0.f;
+#pragma unroll
+  for (int w = 0; w < FWD_WARPS; ++w) {
+    const float ew = sh_red[w];
+    fac[w] = ew == 0.f ? 0.f : expf(__int_as_float(sh_misc[w]) - M);
+    E = fmaf(ew, fac[w], E);
+  }
+  const float fB = (float)p.B;
+  const int ny = sh_misc[8];
+#pragma unroll
+  for (int u = 0; u < KPT; ++u) {
+    const int k = tid + u * FWD_THREADS;
+    if (k < H) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < FWD_WARPS; ++w) v = fmaf(fac[w], sh_dh[(size_t)w * H + k], v);
+      v = na > 0 ? (v / E - (ny > 0 ? accT[u] / (float)ny : 0.f)) / fB : 0.f;
+      p.dh[(size_t)s * H + k] = sh_h[k] > 0.f && !timed_out ? v : 0.f;
+    }
+  }
+  if (tid == FWD_THREADS - 1) {                    // the last thread has the fewest rows below
+    float sum = 0.f;
+    const float logE = logf(E);
+    for (int i = 0; i < nlab; ++i)
+      if (sh_lab[i] >= 0) sum += zp[sh_lab[i]] - M - logE;
+    p.loss[s] = ny > 0 && !timed_out ? -sum / (float)ny : 0.f;
+  }
+  // the errors of a small set go to shared memory as well (beside the logits: no barrier before they are written)
+  for (int a = tid; a < na; a += FWD_THREADS) {
+    const float pa = expf(zp[a] - M) / E;
+    pr[a] = pa;
+    float ga = pa / fB;
+    for (int i = 0; i < nlab; ++i)
+      if (sh_lab[i] == a) ga = (pa - 1.f / (float)ny) / fB;
+    if (timed_out) ga = 0.f;
+    g[a] = ga;
+    if (small) sh_g[a] = ga;
+  }
+  __syncthreads();
+  }
 
   // ---- the rest of the hand-off: slot / mask entries of the rows of W2 (their coefficient is the error), the
   //      entries of both lists of distinct rows, and whatever did not fit the registers above ----
@@ -1409,13 +1731,13 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
 #pragma unroll
     for (int u = 0; u < HO_PER; ++u)
       if (u * FWD_THREADS < na) {          // uniform over the block
-        const int a = tid + u * FWD_THREADS;
-        const bool live = a < na;
+        const int a = act0[u];
+        const bool live = a >= 0;
         touch_mark(p, live, p.hdr2 + jj0[u], p.mask2 + (size_t)jj0[u] * p.Wd, p.ovf2 + (size_t)jj0[u] * PAIR_T, jj0[u], nth0[u], s,
                    live ? gp[a] : 0.f);
         own_store(live && nth0[u] == 0u, base0[u], p.own2, jj0[u], s);
       }
-    for (int a0 = HO_PER * FWD_THREADS; a0 < na; a0 += FWD_THREADS) {
+    for (int a0 = ho_rows; a0 < na; a0 += FWD_THREADS) {
       const int a = a0 + tid;
       const bool live = a < na;
       int jj = 0;
@@ -1542,14 +1864,10 @@ cudaError_t setup_forward(Ctx* c) {
     }
   }
   c->fwd_smem = l.fixed_bytes + c->fwd_stage_bytes;
-  cudaError_t e = cudaFuncSetAttribute(k_forward<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<0, MAX_KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<0, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<0, MAX_KPT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<2, MAX_KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_forward<1, MAX_KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  cudaError_t e = cudaSuccess;
+  for (void (*k)(const FwdParams) : {k_forward<0, 1>, k_forward<0, 1, true>, k_forward<0, 2>, k_forward<0, 4>, k_forward<0, 8>, k_forward<1, 1>, k_forward<1, 2>, k_forward<1, 4>,
+                                     k_forward<1, 8>, k_forward<2, 2>, k_forward<2, 8>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   return e;
 }
 
@@ -1585,33 +1903,38 @@ static FwdParams make_params(Ctx* c, int batch, const int32_t* row_ptr, const in
   return p;
 }
 
+// Expected size of an active set from the tables' shape: L buckets of about N / 2^bits ids, cut at the cap (and at the sampling budget)
+static double expected_set(const Ctx* c) {
+  const double per_bucket = (double)c->N / (double)(1ll << c->bits);
+  double expect = c->cfg.force_dense ? (double)c->N : (double)c->L * (per_bucket < c->cfg.bucket_cap ? per_bucket : (double)c->cfg.bucket_cap);
+  if (c->cfg.sample_budget > 0 && expect > c->cfg.sample_budget) expect = c->cfg.sample_budget;
+  return expect;
+}
+// Whether the active rows go through the warps' rings (k_forward<., 2 ...>) or are staged in chunks of the block's space.  us, staged /
+// by rings: a step of 256 samples x 256 units x 200 rows 84.7 / 79.6, 16 x 200 units x 200 rows 36.7 / 34.8, one sample x 512 units
+// 54.9 / 36.9, 1,024 x 1,024 units 615 / 498; but 1,024 x 200 units x 100 rows, which are one chunk, 167 / 171, one sample x 136
+// units x 200 rows (a chunk and a quarter) 26.0 / 27.0.  (A DWTA bucket that is met holds a row more than the mean.)
+static bool by_rings(const Ctx* c) {
+  if (c->H <= 128 || c->H > 256) return c->H > 256;
+  return expected_set(c) + c->L > 1.25 * (double)(c->fwd_stage_bytes / ((c->H + 4) * 4 + 4));
+}
+
 cudaError_t launch_forward_train(Ctx* c, int batch, const int32_t* row_ptr, const int32_t* col_idx, const float* vals,
                                  const int32_t* label_ptr, const int32_t* labels, int inputs_ready) {
   FwdParams p = make_params(c, batch, row_ptr, col_idx, vals, label_ptr, labels);
   p.inputs_ready = inputs_ready;
   if (use_tiles(c, batch)) {
     LaunchScope ls(c, KID_FORWARD);
-    cudaError_t e = c->H <= FWD_THREADS
-                        ? launch_dependent(k_forward<2, 1>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p)
-                        : launch_dependent(k_forward<2, MAX_KPT>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
+    const cudaError_t e = launch_dependent(c->H <= FWD_THREADS ? k_forward<2, 2> : k_forward<2, 8>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
     return e != cudaSuccess ? e : launch_tiles_forward(c, batch, label_ptr, labels);
   }
   {
     LaunchScope ls(c, KID_FORWARD);
-    // hidden layers of up to FWD_THREADS units take the variant with one unit per thread (less code, fewer registers)
-    // Expected size of an active set from the tables' shape: L buckets of about N / 2^bits ids, cut at the cap (and at
-    // the sampling budget).  Sets of many chunks of the staging space take the variant that fetches rows by bulk copies.
-    const double per_bucket = (double)c->N / (double)(1ll << c->bits);
-    double expect = c->cfg.force_dense ? (double)c->N : (double)c->L * (per_bucket < c->cfg.bucket_cap ? per_bucket : (double)c->cfg.bucket_cap);
-    if (c->cfg.sample_budget > 0 && expect > c->cfg.sample_budget) expect = c->cfg.sample_budget;
+    // Sets of many chunks of the staging space take the variant that fetches rows by bulk copies.
+    const double expect = expected_set(c);
     const bool bulk = expect >= 4.0 * (double)(p.stage_bytes / ((c->H + 4) * 4 + 4));
-    cudaError_t e;
-    if (c->H <= FWD_THREADS)
-      e = bulk ? launch_dependent(k_forward<0, 1, true>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p)
-               : launch_dependent(k_forward<0, 1>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
-    else
-      e = bulk ? launch_dependent(k_forward<0, MAX_KPT, true>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p)
-               : launch_dependent(k_forward<0, MAX_KPT>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
+    const cudaError_t e = launch_dependent(!by_rings(c) ? (bulk ? k_forward<0, 1, true> : k_forward<0, 1>) : c->H <= 256 ? k_forward<0, 2> : c->H <= 512 ? k_forward<0, 4> : k_forward<0, 8>,
+                                           dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
@@ -1627,8 +1950,8 @@ cudaError_t launch_predict(Ctx* c, int batch, const int32_t* row_ptr, const int3
   p.inputs_ready = 0;            // the batch may come from the kernel before this one in the stream: nothing is read before it has completed
   LaunchScope ls(c, KID_PREDICT);
   // placed while the kernel before it drains (the call before this one, in a serving loop)
-  cudaError_t e = c->H <= FWD_THREADS ? launch_dependent(k_forward<1, 1>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p)
-                                      : launch_dependent(k_forward<1, MAX_KPT>, dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
+  cudaError_t e = launch_dependent(!by_rings(c) ? k_forward<1, 1> : c->H <= 256 ? k_forward<1, 2> : c->H <= 512 ? k_forward<1, 4> : k_forward<1, 8>,
+                                   dim3(batch), dim3(FWD_THREADS), (size_t)c->fwd_smem, c->stream, p);
   if (e != cudaSuccess || !dense) return e;
   return launch_dense_tc(c, batch, k, out_ids, out_scores);      // over all neurons: the kernel above has left the hidden activations
 }

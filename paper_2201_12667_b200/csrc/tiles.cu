@@ -27,15 +27,6 @@ constexpr unsigned TFULL = 0xffffffffu;
 // x / step for 0 <= x <= TILE_N_MAX and step <= TILE_ROWS_MAX, by a multiplication with ceil(2^32 / step)
 __host__ __device__ __forceinline__ unsigned tile_magic(int step) { return (unsigned)(((1ull << 32) + (unsigned)step - 1) / (unsigned)step); }
 __device__ __forceinline__ int tile_of(int x, unsigned magic, int step) { return step == 1 ? x : (int)__umulhi((unsigned)x, magic); }
-// two fused multiply-adds in one instruction: a += b * c on pairs of floats
-__device__ __forceinline__ void fma2(unsigned long long& a, unsigned long long b, unsigned long long c) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(b), "l"(c));
-}
-__device__ __forceinline__ unsigned long long pair2(float lo, float hi) {
-  return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
-}
-__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
-__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
 constexpr int TS_THREADS = 1024;
 constexpr int TS_WORDS = 16;
 constexpr int TI_THREADS = 512;
@@ -348,11 +339,6 @@ __device__ __forceinline__ bool load_tile(const TileParams& p, int t, float* til
   if (threadIdx.x == 0) { p.tinfo[1] = 1; atomicCAS(&p.st->status, 0, (int)DSLIDE_ERR_TIMEOUT); }
   return false;
 }
-__device__ __forceinline__ void scale2(ulonglong2& v, unsigned long long f) {
-  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v.x) : "l"(f));
-  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v.y) : "l"(f));
-}
-
 // Grid (row chunks, groups of samples).  A group of G lanes takes a row: lane g of it holds the 16-byte pieces g, g + G,
 // ... (NP of them).  R rows per group at a time: their dot products with the sample's activations are reduced
 // together (lanes exchange the values they give up, so that Q lanes of the group end with each row's sum).  Rows of
@@ -519,7 +505,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) k_tile_forward(const TileParams
               E *= scale;
               E0 *= scale;
 #pragma unroll
-              for (int u = 0; u < NP; ++u) scale2(S[u], sc);
+              for (int u = 0; u < NP; ++u) { mul2(S[u].x, sc); mul2(S[u].y, sc); }
             }
             // a masked neuron (bias of minus infinity) weighs nothing, also while nothing else has been met and M is minus infinity
             const float e = z != -INFINITY ? expf(z - M) : 0.f;
