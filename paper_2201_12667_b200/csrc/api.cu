@@ -229,7 +229,7 @@ dslide_status dslide_init(const dslide_config* cfg, dslide_ctx** out) {
   A(b1, H, true); A(mb1, H, true); A(vb1, H, true);
   A(W2, N * H, false); A(mW2, N * H, true); A(vW2, N * H, true);
   A(hdr2, N, true);
-  A(hash_idx, (size_t)c->KL * fn_len, true); A(hash_sign, (size_t)c->KL * fn_len, true); A(hash_pk, (size_t)c->KL * fn_len, true);
+  A(hash_idx, (size_t)c->KL * fn_len, true); A(hash_sign, (size_t)c->KL * fn_len, true); A(hash_pk, ((size_t)c->KL * fn_len + 7) & ~(size_t)7, true);
   A(h, B * H, true); A(dh, B * H, true); A(loss, B, true); A(codes, B * c->L, true);
   A(act_cnt, B, true); A(act_z, B * S, true); A(act_p, B * S, true); A(act_g, B * S, true);
   A(hdr1, D, true); A(mask1, D * c->Wd, true); A(own1, D, true); A(ovf1, D * PAIR_T, false);

@@ -64,6 +64,7 @@ struct FwdParams {
   unsigned long long seed, rcount;   // for the probe sequence of the densification: the model's seed, rebuilds so far
   int hash_sm_off;     // where in the staging region the hash functions' index tables are mirrored (-1: read from global memory)
   int hash_sm_bytes;
+  int hash_sm_late;    // of which the first ones lie where the hidden layer's rows are staged
   int sort_small;      // candidate sets up to this size are deduplicated by sorting even when a bitmap is available
   // LSH-sampled hidden layer (L1 > 0): projections over the input coordinates, tables over the hidden neurons
   const int8_t* proj1;
@@ -538,32 +539,67 @@ __device__ __noinline__ int budget_select(int budget, int fill, int N, uint64_t 
   return total;
 }
 
-// One SimHash bit of the hidden activation: the projection's sum in stored order, its sign.  (In line: as a call it cost
-// 0.5 us of a step of 26 with 32 functions, and gave the DWTA shapes nothing: 65.6 us per step either way.)
-__device__ __forceinline__ unsigned char simhash_bit(const float* h, const int32_t* ix, const int32_t* sg, int n) {
-  float sum = 0.f;
-  for (int i = 0; i < n; ++i) {
-    const float x = h[ix[i]];
-    sum = __fadd_rn(sum, sg[i] > 0 ? x : -x);
+// SimHash sums of the hidden activation, carried on over n rows (coordinates) of the packed table: a warp reads 32 functions'
+// i-th coordinates (top bit = minus) side by side; their places in h are close together (a function's coordinates ascend), so
+// few of the reads conflict.  A thread has the functions f and f + FWD_THREADS: each a chain of additions in stored order.
+__device__ __forceinline__ void simhash_rows(const float* h, const uint16_t* pk, int f, int KL, int n, float& sum0, float& sum1) {
+  auto term = [&](unsigned e) { return __uint_as_float(__float_as_uint(h[e & 0x7fffu]) ^ (e & 0x8000u) << 16); };
+  const uint16_t* q = pk + f;
+  if (f + FWD_THREADS < KL) {
+#pragma unroll 4
+    for (int i = 0; i < n; ++i, q += KL) {
+      const unsigned e0 = q[0], e1 = q[FWD_THREADS];
+      sum0 = __fadd_rn(sum0, term(e0));
+      sum1 = __fadd_rn(sum1, term(e1));
+    }
+  } else if (f < KL) {
+#pragma unroll 4
+    for (int i = 0; i < n; ++i, q += KL) sum0 = __fadd_rn(sum0, term(q[0]));
   }
-  return sum >= 0.f ? 1 : 0;
 }
-// The same from the packed table, where a warp reads 32 functions' i-th coordinates (top bit = minus) side by side,
-// sixteen rounds of them in flight.
-__device__ __noinline__ unsigned char simhash_bit_packed(const float* h, const uint16_t* pk, int KL, int n) {
-  float sum = 0.f;
-  for (int i0 = 0; i0 < n; i0 += 16) {
-    unsigned e[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) e[i] = i0 + i < n ? (unsigned)__ldg(pk + (size_t)(i0 + i) * KL) : 0u;
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if (i0 + i < n) {
-        const float x = h[e[i] & 0x7fffu];
-        sum = __fadd_rn(sum, (e[i] & 0x8000u) ? -x : x);
-      }
+// A packed table larger than the staging space passes through its two halves, a piece on its way while the other is read (700
+// functions of 171 coordinates: 20,500 cycles of a block, 55,000 from global memory; a step of 16 samples x 512 units 147 us, now
+// 79).  Up to SIM_SUMS functions per thread.  The number of pieces (bar0 has completed half of them, rounded up, bar1 the others);
+// 0 when one did not come in time, with nothing left in flight.  Called by the whole block; out of line, so that the other
+// families' blocks stay short (in line a step of 256 samples of the 670,091-neuron shape took 65.0 us for 64.3).
+constexpr int SIM_SUMS = 4;
+__device__ __noinline__ int simhash_in_pieces(const float* h, const uint16_t* table, int KL, int n_all, unsigned char* space, int space_bytes, uint64_t* bar0,
+                                              uint64_t* bar1, unsigned char* bits) {
+  const int tid = threadIdx.x;
+  const int half = (space_bytes / 2) & ~127, per = max(8, (half / (2 * KL)) & ~7), pieces = (n_all + per - 1) / per;
+  float sum[SIM_SUMS] = {0.f, 0.f, 0.f, 0.f};
+  auto fetch = [&](int c) {
+    const uint32_t bytes = (uint32_t)((min(per, n_all - c * per) * KL * 2 + 15) & ~15);
+    uint64_t* bar = (c & 1) ? bar1 : bar0;
+    mbar_expect_tx(bar, bytes);
+    bulk_g2s(space + (c & 1) * half, table + (size_t)c * per * KL, bytes, bar);
+  };
+  fence_proxy_async();
+  __syncthreads();
+  if (tid == 0) {
+    fetch(0);
+    if (pieces > 1) fetch(1);
   }
-  return sum >= 0.f ? 1 : 0;
+  for (int c = 0; c < pieces; ++c) {
+    const bool ok = bar_wait_limited((c & 1) ? bar1 : bar0, (uint32_t)(c >> 1) & 1u);
+    if (__syncthreads_or(ok ? 0 : 1)) {
+      bar_wait_limited((c & 1) ? bar1 : bar0, (uint32_t)(c >> 1) & 1u);
+      if (c + 1 < pieces) bar_wait_limited((c & 1) ? bar0 : bar1, (uint32_t)((c + 1) >> 1) & 1u);
+      __syncthreads();
+      return 0;
+    }
+    const uint16_t* pk = reinterpret_cast<const uint16_t*>(space + (c & 1) * half);
+    const int n = min(per, n_all - c * per);
+    simhash_rows(h, pk, tid, KL, n, sum[0], sum[1]);
+    simhash_rows(h, pk, tid + 2 * FWD_THREADS, KL, n, sum[2], sum[3]);
+    fence_proxy_async();
+    __syncthreads();
+    if (tid == 0 && c + 2 < pieces) fetch(c + 2);
+  }
+#pragma unroll
+  for (int u = 0; u < SIM_SUMS; ++u)
+    if (tid + u * FWD_THREADS < KL) bits[tid + u * FWD_THREADS] = sum[u] >= 0.f ? 1 : 0;
+  return pieces;
 }
 
 // The sample is skipped: no loss, no gradient, nothing touched (predict: no candidates).
@@ -633,18 +669,18 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   if (MODE != 1) { lbeg = p.label_ptr[s]; nlab = p.label_ptr[s + 1] - lbeg; }
 
   griddep_launch_dependents();       // the update kernel may be placed as blocks of this one leave
+  const void* hash_tab = p.family == DSLIDE_SIMHASH ? static_cast<const void*>(p.hash_pk) : static_cast<const void*>(p.hash_idx);
   if (tid == 0) {
     sh_misc[24] = 0;                 // bucket entries fetched by this sample
     mbar_init(sh_bar, 1);
-    mbar_init(sh_bar2, 1);
+    mbar_init(sh_bar2, p.hash_sm_late > 0 ? 2 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // the hash functions' tables (constant between rebuilds) come into the upper part of the staging region, which
-    // is free until the candidates are collected
+    // is free until the candidates are collected; what reaches down into the rows of W1 comes after the hidden layer
     if (p.hash_sm_off >= 0 && !p.dense) {
-      mbar_expect_tx(sh_bar2, (uint32_t)p.hash_sm_bytes);
-      const int half = p.family == DSLIDE_SIMHASH ? p.hash_sm_bytes / 2 : p.hash_sm_bytes;
-      bulk_g2s(smem + p.off_dedup + p.hash_sm_off, p.hash_idx, (uint32_t)half, sh_bar2);
-      if (p.family == DSLIDE_SIMHASH) bulk_g2s(smem + p.off_dedup + p.hash_sm_off + half, p.hash_sign, (uint32_t)half, sh_bar2);
+      const int now = p.hash_sm_bytes - p.hash_sm_late;
+      mbar_expect_tx(sh_bar2, (uint32_t)now);
+      if (now > 0) bulk_g2s(smem + p.off_dedup + p.hash_sm_off + p.hash_sm_late, static_cast<const unsigned char*>(hash_tab) + p.hash_sm_late, (uint32_t)now, sh_bar2);
     }
   }
 
@@ -742,7 +778,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     }
   }
   if (bad || too_many_labels) {
-    if (p.hash_sm_off >= 0 && !p.dense) bar_wait_limited(sh_bar2, 0u);     // no copy into this block may be left in flight
+    if (p.hash_sm_off >= 0 && !p.dense) {          // no copy into this block may be left in flight
+      if (p.hash_sm_late > 0 && tid == 0) mbar_expect_tx(sh_bar2, 0u);
+      bar_wait_limited(sh_bar2, 0u);
+    }
     skip_sample<MODE>(p, s, (!bad && too_many_labels) ? DSLIDE_ERR_OVERFLOW : DSLIDE_ERR_BAD_INDEX);
     return;
   }
@@ -783,16 +822,22 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     }
   }
   if (MODE == 1 && p.dense) return;        // inference over all neurons: the logits are taken by the kernels of dense_tc.cu
+  if (p.hash_sm_late > 0) fence_proxy_async();
   __syncthreads();
+  if (p.hash_sm_late > 0 && !p.dense && tid == 0) {
+    mbar_expect_tx(sh_bar2, (uint32_t)p.hash_sm_late);
+    bulk_g2s(smem + p.off_dedup + p.hash_sm_off, hash_tab, (uint32_t)p.hash_sm_late, sh_bar2);
+  }
 
   const bool dense = p.dense != 0;
+  uint32_t w2phase = 0u;             // of sh_bar
   int na = N;
   int32_t* ids = p.act_ids + (size_t)s * p.act_stride;
 
   if (!dense) {
     // ---- bucket codes of the hidden activation ----
     const int32_t* hidx = p.hash_idx;
-    const int32_t* hsgn = p.hash_sign;
+    const uint16_t* hpk = p.hash_pk;
     if (p.hash_sm_off >= 0) {
       const bool ok = bar_wait_limited(sh_bar2, 0u);
       if (__syncthreads_or(ok ? 0 : 1)) {          // the mirror did not arrive in time: the sample is given up
@@ -802,14 +847,28 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
         return;
       }
       hidx = reinterpret_cast<const int32_t*>(smem + p.off_dedup + p.hash_sm_off);
-      hsgn = reinterpret_cast<const int32_t*>(smem + p.off_dedup + p.hash_sm_off + p.hash_sm_bytes / 2);
+      hpk = reinterpret_cast<const uint16_t*>(hidx);
     }
+    if (p.family == DSLIDE_SIMHASH) {
+      if (p.hash_sm_off >= 0 || p.KL > SIM_SUMS * FWD_THREADS) {      // mirrored, or from global memory: thousands of functions
+        for (int f = tid; f < p.KL; f += 2 * FWD_THREADS) {
+          float sum0 = 0.f, sum1 = 0.f;
+          simhash_rows(sh_h, hpk, f, p.KL, p.fn_len, sum0, sum1);
+          sh_part[f] = sum0 >= 0.f ? 1 : 0;
+          if (f + FWD_THREADS < p.KL) sh_part[f + FWD_THREADS] = sum1 >= 0.f ? 1 : 0;
+        }
+      } else {
+        const int pieces = simhash_in_pieces(sh_h, p.hash_pk, p.KL, p.fn_len, smem + p.off_dedup, p.stage_bytes, sh_bar2, sh_bar, sh_part);
+        if (pieces == 0) {                           // not in time: the sample is given up
+          skip_sample<MODE>(p, s, DSLIDE_ERR_TIMEOUT);
+          return;
+        }
+        w2phase = (uint32_t)(pieces >> 1) & 1u;      // of sh_bar
+      }
+    } else
     for (int f = tid; f < p.KL; f += FWD_THREADS) {
       const int32_t* ix = hidx + (size_t)f * p.fn_len;
-      if (p.family == DSLIDE_SIMHASH) {
-        sh_part[f] = p.hash_sm_off < 0 ? simhash_bit_packed(sh_h, p.hash_pk + f, p.KL, p.fn_len)
-                                       : simhash_bit(sh_h, ix, hsgn + (size_t)f * p.fn_len, p.fn_len);
-      } else if (p.fn_len == 8 && (reinterpret_cast<uintptr_t>(hidx) & 15) == 0) {
+      if (p.fn_len == 8 && (reinterpret_cast<uintptr_t>(hidx) & 15) == 0) {
         // bins of eight: both halves of the index list in one load each, the eight values fetched side by side
         const int4 ia = reinterpret_cast<const int4*>(ix)[0], ib = reinterpret_cast<const int4*>(ix)[1];
         const float v0 = sh_h[ia.x], v1 = sh_h[ia.y], v2 = sh_h[ia.z], v3 = sh_h[ia.w];
@@ -1211,7 +1270,6 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   // a thread's place in the copy pattern of the padded rows: H4 + 1 pieces per row
   const int rp_dr = FWD_THREADS / (H4 + 1), rp_dc = FWD_THREADS - rp_dr * (H4 + 1);
   const int rp_r0 = tid / (H4 + 1), rp_c0 = tid - rp_r0 * (H4 + 1);
-  uint32_t w2phase = 0u;
   bool timed_out = false;                          // block-uniform
   const bool bulk = BULK && streaming && na >= 4 * stage_rows;      // many chunks: the batch's samples share most rows (see below)
   // (a training sample with nothing active still goes through once: its rows of W1 are counted in here)
@@ -1373,9 +1431,11 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   if (!streaming) {
     if (small) {
       float m = -INFINITY;
+#pragma unroll 4
       for (int a = lane; a < na; a += 32) m = fmaxf(m, sh_z[a]);
       M = warp_max(m);
       float e = 0.f;
+#pragma unroll 4
       for (int a = lane; a < na; a += 32) e += expf(sh_z[a] - M);
       E = warp_sum(e);
     } else {
@@ -1420,6 +1480,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       float4 av[NCH];
 #pragma unroll
       for (int q = 0; q < NCH; ++q) av[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
       for (int a = warp; a < na; a += FWD_WARPS) {
         const float ga = gp[a];
         const float4* row = reinterpret_cast<const float4*>(stage + (size_t)a * ldr);
@@ -1840,15 +1901,19 @@ cudaError_t setup_forward(Ctx* c) {
     const int most = c->N <= BITMAP_CHEAP ? SORT_FEW : SORT_SMALL;
     c->fwd_sort_small = cap_small < most ? cap_small : most;
   }
-  // the hash functions' tables are mirrored above the hidden layer's chunk when they fit there
+  // the hash functions' tables are mirrored at the end of the staging space: SimHash's packed ones wherever they fit (from global
+  // memory the 450 functions of 67 coordinates of a block took 20,000 to 29,000 cycles, from the mirror 5,000 to 6,800), DWTA's above the hidden layer's chunk
   {
     const long long one = (long long)c->KL * c->fn_len * 4;
-    const long long hb = c->cfg.hash_family == DSLIDE_SIMHASH ? 2 * one : one;
+    const bool sim = c->cfg.hash_family == DSLIDE_SIMHASH;
+    const long long hb = sim ? (one / 2 + 15) & ~15ll : one;
     c->fwd_hash_sm_off = -1;
-    c->fwd_hash_sm_bytes = 0;
-    if (!c->dense && one % 16 == 0 && hb <= 32 * 1024 && stage_min + hb <= (long long)c->fwd_stage_bytes) {
+    c->fwd_hash_sm_bytes = c->fwd_hash_sm_late = 0;
+    if (!c->dense && (sim ? hb <= (long long)c->fwd_stage_bytes : one % 16 == 0 && hb <= 32 * 1024 && stage_min + hb <= (long long)c->fwd_stage_bytes)) {
       c->fwd_hash_sm_bytes = (int)hb;
       c->fwd_hash_sm_off = (c->fwd_stage_bytes - (int)hb) & ~15;
+      c->fwd_hash_sm_late = c->fwd_hash_sm_off < stage_min ? (stage_min - c->fwd_hash_sm_off + 15) & ~15 : 0;
+      if (c->fwd_hash_sm_late > c->fwd_hash_sm_bytes) c->fwd_hash_sm_late = c->fwd_hash_sm_bytes;
     }
   }
   if (c->cfg.sample_budget > 0 && !c->dense) {
@@ -1892,7 +1957,7 @@ static FwdParams make_params(Ctx* c, int batch, const int32_t* row_ptr, const in
   p.stage_bytes = c->fwd_stage_bytes; p.hid_rows = l.hid_rows; p.sort_small = c->fwd_sort_small;
   p.densify = c->cfg.dwta_densify; p.seed = c->cfg.seed; p.rcount = (unsigned long long)c->r_host;
   p.budget = c->cfg.sample_budget; p.budget_fill = c->cfg.budget_fill; p.tcount = (unsigned long long)c->t_host;
-  p.hash_sm_off = c->fwd_hash_sm_off; p.hash_sm_bytes = c->fwd_hash_sm_bytes; p.inputs_ready = 1;
+  p.hash_sm_off = c->fwd_hash_sm_off; p.hash_sm_bytes = c->fwd_hash_sm_bytes; p.hash_sm_late = c->fwd_hash_sm_late; p.inputs_ready = 1;
   p.off_dh = l.off_dh; p.off_code = l.off_code; p.off_part = l.off_part; p.off_misc = l.off_misc;
   p.off_lab = l.off_lab; p.off_tbase = l.off_tbase; p.off_tbeg = l.off_tbeg; p.off_topk = l.off_topk;
   p.off_ids = l.off_ids; p.off_z = l.off_z; p.off_col = l.off_col; p.off_val = l.off_val; p.off_dedup = l.off_dedup;

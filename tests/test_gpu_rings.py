@@ -43,3 +43,15 @@ def test_equal_scores_go_by_id(H, k):
         check_predict(pr, wl.batch(0), 0, k, b2=np.where(np.arange(4001) % 701 == 5, 0.5, 0.25).astype(np.float32), same_ids=True)
     finally:
         pr.close()
+
+
+@pytest.mark.parametrize("H,K,L", [(64, 4, 8), (200, 9, 50), (260, 5, 51), (512, 14, 50), (1024, 13, 40), (1020, 21, 50)])
+def test_simhash_bits_of_queries(H, K, L):
+    """The packed table of the hash functions mirrored whole, partly after the hidden layer, in two pieces and more (an odd number of
+    functions: pieces that end inside a 16-byte word), and read from global memory (more than 1,024 functions)."""
+    pr = Pair(D=501, H=H, N=1501, family=SIMHASH, K=K, L=L, bucket_cap=8, max_batch=6, max_labels=3, lr=1e-3, seed=H + K)
+    try:
+        wl = workloads.Workload(dict(workloads.config("tiny"), D=501, N=1501, batch=6), seed=5)
+        one_and_two_steps(pr, [wl.batch(0), wl.batch(1)])
+    finally:
+        pr.close()
