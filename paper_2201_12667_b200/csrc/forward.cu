@@ -831,6 +831,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
 
   const bool dense = p.dense != 0;
   uint32_t w2phase = 0u;             // of sh_bar
+  bool marked = false;               // MODE 2: the rows' bits have been set from the sample's bitmap
   int na = N;
   int32_t* ids = p.act_ids + (size_t)s * p.act_stride;
 
@@ -999,26 +1000,34 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       for (int w = tid; w < n4; w += FWD_THREADS) dd4[w] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
     }
-    constexpr int CU = MODE == 0 ? 1 : 4;      // thousands of candidates: several per thread and round, their loads in flight together
-    for (int c0 = tid; c0 < ncand; c0 += CU * FWD_THREADS) {
-      int j[CU];
+    if (bitmap && ncand >= 16 * p.L) {
+      // long slices: a warp takes two tables at a time, their entries side by side and four rounds in flight (a thread per
+      // candidate searched for its table first: 27,000 cycles for 50 slices of 128, so 7,000)
+      for (int t = warp; t < p.L; t += 2 * FWD_WARPS) {
+        const int t1 = t + FWD_WARPS < p.L ? t + FWD_WARPS : t;
+        const int n0 = sh_tbase[t + 1] - sh_tbase[t], n1 = t1 != t ? sh_tbase[t1 + 1] - sh_tbase[t1] : 0;
+        const int32_t *s0 = p.bucket_ids + (size_t)t * N + sh_tbeg[t], *s1 = p.bucket_ids + (size_t)t1 * N + sh_tbeg[t1];
+        for (int i0 = lane; i0 - lane < max(n0, n1); i0 += 128) {
+          int j0[4], j1[4];
 #pragma unroll
-      for (int u = 0; u < CU; ++u) {
-        const int c = c0 + u * FWD_THREADS;
-        j[u] = 0;
-        if (c < ncand) {
-          int lo = 0, hi = p.L - 1;        // last table whose candidates start at or before c
-          while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (sh_tbase[mid] <= c) lo = mid; else hi = mid - 1; }
-          j[u] = __ldg(p.bucket_ids + (size_t)lo * N + sh_tbeg[lo] + (c - sh_tbase[lo]));
+          for (int u = 0; u < 4; ++u) {
+            j0[u] = i0 + 32 * u < n0 ? __ldg(s0 + i0 + 32 * u) : -1;
+            j1[u] = i0 + 32 * u < n1 ? __ldg(s1 + i0 + 32 * u) : -1;
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (j0[u] >= 0) atomicOr(&sh_dd[j0[u] >> 5], 1u << (j0[u] & 31));
+            if (j1[u] >= 0) atomicOr(&sh_dd[j1[u] >> 5], 1u << (j1[u] & 31));
+          }
         }
       }
-#pragma unroll
-      for (int u = 0; u < CU; ++u) {
-        const int c = c0 + u * FWD_THREADS;
-        if (c < ncand) {
-          if (bitmap) atomicOr(&sh_dd[j[u] >> 5], 1u << (j[u] & 31));
-          else sh_dd[c] = packed ? ((uint32_t)j[u] << RANK_BITS) | (uint32_t)c : (uint32_t)j[u];
-        }
+    } else {
+      for (int c = tid; c < ncand; c += FWD_THREADS) {
+        int lo = 0, hi = p.L - 1;          // last table whose candidates start at or before c
+        while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (sh_tbase[mid] <= c) lo = mid; else hi = mid - 1; }
+        const int j = __ldg(p.bucket_ids + (size_t)lo * N + sh_tbeg[lo] + (c - sh_tbase[lo]));
+        if (bitmap) atomicOr(&sh_dd[j >> 5], 1u << (j & 31));
+        else sh_dd[c] = packed ? ((uint32_t)j << RANK_BITS) | (uint32_t)c : (uint32_t)j;
       }
     }
     if (MODE != 1)
@@ -1029,14 +1038,16 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       }
     if (bitmap) {
       __syncthreads();
-      // every warp takes a contiguous share of the words, 32 at a time; a lane writes out the ids of its word
+      // every warp takes a contiguous share of the words, WU times 32 at a time; a lane writes out the ids of its words, one of
+      // each in turn (one word at a time 31,000 cycles for 6,000 ids of 253,855, so 20,000)
+      constexpr int WU = 4;
       const int nwords = (N + 31) >> 5;
       const int share = ((nwords + FWD_WARPS - 1) / FWD_WARPS + 31) & ~31;
       const int wbeg = min(nwords, warp * share), wend = min(nwords, wbeg + share);
       int cnt = 0;
+#pragma unroll 4
       for (int w = wbeg + lane; w < wend; w += 32) cnt += __popc(sh_dd[w]);
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) cnt += __shfl_xor_sync(FULLM, cnt, d);
+      cnt = __reduce_add_sync(FULLM, cnt);
       if (lane == 0) sh_misc[warp] = cnt;
       __syncthreads();
       int pos = 0;
@@ -1045,26 +1056,84 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
         if (q < warp) pos += cq;
         total += cq;
       }
-      if (total <= p.act_stride && cnt > 0)
-        for (int w0 = wbeg; w0 < wend; w0 += 32) {
-          uint32_t bits = w0 + lane < wend ? sh_dd[w0 + lane] : 0u;
-          const int mine = __popc(bits);
-          int incl = mine;
+      if (total <= p.act_stride && cnt > 0 && share == 32) {       // few words: all of the warp's at once
+        const uint32_t mine = wbeg + lane < wend ? sh_dd[wbeg + lane] : 0u;
+        int at = __popc(mine);
 #pragma unroll
-          for (int d = 1; d < 32; d <<= 1) {
-            const int n = __shfl_up_sync(FULLM, incl, d);
-            if (lane >= d) incl += n;
-          }
-          int at = pos + incl - mine;
-          while (bits) {
-            const int j = ((w0 + lane) << 5) + __ffs(bits) - 1;
-            ids[at] = j;
-            if (at < ACT_SM) sh_ids[at] = j;
-            ++at;
-            bits &= bits - 1;
-          }
-          pos += __shfl_sync(FULLM, incl, 31);
+        for (int d = 1; d < 32; d <<= 1) {
+          const int n = __shfl_up_sync(FULLM, at, d);
+          if (lane >= d) at += n;
         }
+        at += pos - __popc(mine);
+        for (uint32_t bits = mine; bits; bits &= bits - 1) {
+          const int j = ((wbeg + lane) << 5) + __ffs(bits) - 1;
+          ids[at] = j;
+          if (MODE != 2 && at < ACT_SM) sh_ids[at] = j;
+          ++at;
+        }
+      } else if (total <= p.act_stride && cnt > 0)
+#pragma unroll 1
+        for (int w0 = wbeg; w0 < wend; w0 += 32 * WU) {
+          uint32_t bits[WU];
+          int at[WU];
+#pragma unroll
+          for (int u = 0; u < WU; ++u) {
+            bits[u] = w0 + 32 * u + lane < wend ? sh_dd[w0 + 32 * u + lane] : 0u;
+            at[u] = __popc(bits[u]);
+          }
+#pragma unroll
+          for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+            for (int u = 0; u < WU; ++u) {
+              const int n = __shfl_up_sync(FULLM, at[u], d);
+              if (lane >= d) at[u] += n;
+            }
+#pragma unroll
+          for (int u = 0; u < WU; ++u) {
+            const int all = __shfl_sync(FULLM, at[u], 31);
+            at[u] += pos - __popc(bits[u]);
+            pos += all;
+          }
+          while (bits[0] | bits[1] | bits[2] | bits[3]) {
+#pragma unroll
+            for (int u = 0; u < WU; ++u)
+              if (bits[u]) {
+                const int j = ((w0 + 32 * u + lane) << 5) + __ffs(bits[u]) - 1;
+                ids[at[u]] = j;
+                if (MODE != 2 && at[u] < ACT_SM) sh_ids[at[u]] = j;
+                ++at[u];
+                bits[u] &= bits[u] - 1;
+              }
+          }
+        }
+      if (MODE == 2 && p.budget > 0) {                       // the budget reads the mirror
+        __syncthreads();
+        for (int a = tid; a < min(total, ACT_SM) && total <= p.act_stride; a += FWD_THREADS) sh_ids[a] = ids[a];
+      }
+      if (MODE == 2 && total <= p.act_stride && p.budget == 0) {
+        // The rows of W2 that the batch touches, as a bit per row: the words of the sample's own bitmap, those already marked passed
+        // over; blocks begin at different words, so that most of their bits have been marked by others when they come to them
+        // (bit by bit from the list of ids it took 30,000 cycles in the first wave of blocks; a step of 256 samples x 325,056 neurons
+        // 365 us, by long slices, this and the words above 339).
+        marked = true;
+        const int nw = (N + 31) >> 5, rounds = (nw + FWD_THREADS - 1) / FWD_THREADS;
+        int r = (int)(blockIdx.x % (unsigned)rounds);
+        constexpr int TU = 4;
+        for (int i = 0; i < rounds; i += TU) {
+          uint32_t have[TU], bits[TU];
+          int w[TU];
+#pragma unroll
+          for (int u = 0; u < TU; ++u) {
+            w[u] = r * FWD_THREADS + tid;
+            bits[u] = i + u < rounds && w[u] < nw ? sh_dd[w[u]] : 0u;
+            have[u] = bits[u] ? __ldcg(p.touch2 + w[u]) : 0u;
+            if (++r == rounds) r = 0;
+          }
+#pragma unroll
+          for (int u = 0; u < TU; ++u)
+            if (bits[u] & ~have[u]) atomicOr(p.touch2 + w[u], bits[u]);
+        }
+      }
     } else if (ncand + nlab <= RANK_MAX) {
       const int n = ncand + nlab;
       if (packed && tid < 4 && n + tid < ((n + 3) & ~3)) sh_dd[n + tid] = 0xffffffffu;
@@ -1183,10 +1252,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   }
   if (MODE != 1 && tid == 0) p.act_cnt[s] = na;
   if (MODE == 2) {
-    // ---- the rows of W2 that the batch touches, as a bit per row (most are marked already: a read is enough), and the
-    //      hand-off of the sample's rows of W1 ----
+    // ---- the rows of W2 that the batch touches (most are marked already: a read is enough), unless the bitmap has told, and
+    //      the hand-off of the sample's rows of W1 ----
     constexpr int TU = 4;
-    for (int a0 = tid; a0 < na; a0 += TU * FWD_THREADS) {
+    for (int a0 = tid; a0 < na && !marked; a0 += TU * FWD_THREADS) {
       int j[TU];
       uint32_t have[TU];
 #pragma unroll
