@@ -89,7 +89,8 @@ static int call_step(const Ctx* c, int batch) {
   if (want < TILE_STEP_MIN) want = TILE_STEP_MIN;
   return want < c->tile_step ? (int)want : c->tile_step;
 }
-static int call_tiles(const Ctx* c, int batch) { return c->N / call_step(c, batch) + 2; }      // tiles at most
+// Tiles at most (k_tile_scan makes them smaller, so that the row chunks get the same number: up to one more each)
+static int call_tiles(const Ctx* c, int batch) { return c->N / call_step(c, batch) + 2 + c->num_sms; }
 
 // Row chunks (blocks that walk the tiles side by side) and groups of samples of k_tile_forward.
 static void tile_grid(const Ctx* c, int batch, int* chunks, int* groups) {
@@ -102,7 +103,8 @@ static void tile_grid(const Ctx* c, int batch, int* chunks, int* groups) {
   if (q < 1) q = 1;
   int p = c->num_sms / q;
   if (p < 1) p = 1;
-  if (p > call_tiles(c, batch)) p = call_tiles(c, batch);
+  const int tiles = c->N / call_step(c, batch) + 2;
+  if (p > tiles) p = tiles;
   *chunks = p;
   *groups = q;
 }
@@ -132,7 +134,7 @@ cudaError_t setup_tiles(Ctx* c) {
   const size_t nw = ((size_t)c->N + 31) / 32;
   struct Part { void** p; size_t bytes; };
   const Part parts[] = {{(void**)&c->touch2, nw * 4}, {(void**)&c->wpre, (nw + 1) * 4}, {(void**)&c->trows, (size_t)c->N * 4},
-                        {(void**)&c->tstart, tiles * 4}, {(void**)&c->tinfo, 16}, {(void**)&c->act_loc, B * (size_t)c->act_stride * 2},
+                        {(void**)&c->tstart, tiles * 4}, {(void**)&c->tinfo, 32}, {(void**)&c->act_loc, B * (size_t)c->act_stride * 2},
                         {(void**)&c->seg, runs * 4}, {(void**)&c->tpart, most * 4}, {(void**)&c->rinfo, (size_t)c->N * 8},
                         {(void**)&c->tlist, B * (size_t)c->act_stride * 8}, {(void**)&c->tlab, B * (size_t)c->cfg.max_labels * 4}};
   // The context works without (every step sample by sample), so the work space never stands in its way: it takes at most
@@ -158,9 +160,11 @@ cudaError_t setup_tiles(Ctx* c) {
 }
 
 // One block: touched rows before every word (exclusive running sum of the words' bit counts), and the first row of
-// every tile: word w belongs to tile wpre[w] / step.
+// every tile: word w belongs to tile wpre[w] / step.  The step is `most`, or, where the row chunks would take two to four rounds of
+// tiles, so much less that the last round is a whole one (a step of 256 samples x 325,056 neurons x 128 units 340 us, so 333; 512
+// x 200,003 x 64 471 and 459; not tiles of few words of the bitmap, whose sizes jump: 512 x 50,021 x 128, 32 rows, 259 and 272).
 __global__ void __launch_bounds__(TS_THREADS)
-k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int* tinfo, unsigned int* n_touched) {
+k_tile_scan(const uint32_t* touch, int nw, int most, int chunks, int* wpre, int* tstart, int* tinfo, unsigned int* n_touched) {
   __shared__ int sh[TS_THREADS / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   griddep_launch_dependents();
@@ -195,6 +199,10 @@ k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int
   __syncthreads();
   const int total = sh[TS_THREADS / 32 - 1];
   int run = incl - mine + (warp > 0 ? sh[warp - 1] : 0);
+  // (a tile starts at a word, so up to one more tile than rows / step)
+  const int rounds = (total / most + chunks) / chunks;
+  const int even = (total + rounds * chunks - 1) / (rounds * chunks);
+  const int step = rounds < 2 || rounds > 4 || even < 96 ? most : min(most, even);
   // the tile of the word before this thread's first one: its start, or that of a tile further back, covers `run`
   const unsigned magic = tile_magic(step);
   int tile = -1;
@@ -218,6 +226,8 @@ k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int
     tinfo[0] = tile + 1;
     tinfo[1] = 0;
     tinfo[2] = 0;
+    tinfo[3] = step;
+    tinfo[4] = (int)magic;
     *n_touched = (unsigned)total;
   }
 }
@@ -225,7 +235,7 @@ k_tile_scan(const uint32_t* touch, int nw, int step, int* wpre, int* tstart, int
 // Blocks [0, B): a sample's entries -- place in the tile, and where the runs of the tiles start (a tile without
 // entries has an empty run).  The blocks after them write the list of touched rows.
 __global__ void __launch_bounds__(TI_THREADS + 32)
-k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const int* tinfo, int nw, int step, int B, int bstride,
+k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const int* tinfo, int nw, int B, int bstride,
              const int* act_cnt, const int32_t* act_ids, int act_stride, const int32_t* label_ptr, const int32_t* labels,
              int max_labels, uint16_t* act_loc, int* seg, int* trows, int* tlab) {
   const int tid = threadIdx.x;
@@ -265,7 +275,8 @@ k_tile_index(const uint32_t* touch, const int* wpre, const int* tstart, const in
     return;
   }
   constexpr int U = 4;                       // entries per thread and round: their chains of loads run side by side
-  const unsigned magic = tile_magic(step);
+  const int step = __ldcg(tinfo + 3);
+  const unsigned magic = (unsigned)__ldcg(tinfo + 4);
   for (int a0 = 0; a0 < na; a0 += U * TI_THREADS) {
     int j[U], pre[U], prev[U], ts[U];
     uint32_t bits[U];
@@ -795,12 +806,12 @@ cudaError_t launch_tiles_forward(Ctx* c, int batch, const int32_t* label_ptr, co
   tile_grid(c, batch, &chunks, &groups);
   const int step = call_step(c, batch);
   c->launches += 5;          // with the kernel before them they make one entry of the profile
-  cudaError_t e = launch_dependent(k_tile_scan, dim3(1), dim3(TS_THREADS), 0, c->stream, (const uint32_t*)c->touch2, nw, step,
+  cudaError_t e = launch_dependent(k_tile_scan, dim3(1), dim3(TS_THREADS), 0, c->stream, (const uint32_t*)c->touch2, nw, step, chunks,
                                    c->wpre, c->tstart, c->tinfo, &c->dstate->n_own[c->t_host & 1][0]);
   if (e != cudaSuccess) return e;
   const int extra = (nw + 4 * TI_THREADS - 1) / (4 * TI_THREADS);
   e = launch_dependent(k_tile_index, dim3(batch + extra), dim3(TI_THREADS + 32), 0, c->stream, (const uint32_t*)c->touch2, (const int*)c->wpre,
-                       (const int*)c->tstart, (const int*)c->tinfo, nw, step, batch, batch, (const int*)c->act_cnt,
+                       (const int*)c->tstart, (const int*)c->tinfo, nw, batch, batch, (const int*)c->act_cnt,
                        (const int32_t*)c->act_ids, c->act_stride, label_ptr, labels, c->cfg.max_labels, c->act_loc, c->seg, c->trows, c->tlab);
   if (e != cudaSuccess) return e;
   TileParams p;
