@@ -91,6 +91,20 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Until at most n of the thread's groups of copies are in flight, n <= 7
+__device__ __forceinline__ void cp_async_wait_pending(int n) {
+  switch (n) {
+    case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+    case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+    case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+    case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+    case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+    case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
+    case 6: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 7;" ::: "memory");
+  }
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -709,7 +723,71 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   // a thread's place in the copy pattern: 16-byte piece c4 of row r, advancing FWD_THREADS pieces per round
   const int cp_dr = FWD_THREADS / H4, cp_dc = FWD_THREADS - cp_dr * H4;
   const int cp_r0 = tid / H4, cp_c0 = tid - cp_r0 * H4;
-  for (int c0 = 0; c0 < nnz; c0 += R) {
+  bool pieced = false;
+  if constexpr (NP == 8) {
+  if (p.L1 == 0 && nnz > R && nnz <= ACT_SM) {
+    // More rows than a chunk (more than 512 units): a thread owns a 16-byte piece of every row, copies it and adds it up, HID_G rows to a
+    // group of copies, as many groups ahead as fit -- no barriers.  (In chunks, a barrier before and after each, 76 rows of 1,024
+    // units took 33,000 cycles of a block: a step of 1,024 samples 498 us, so 472; of one sample 48.6 and 43.7.  Of up to 512 units,
+    // half of the threads or fewer, it is the slower: 64 x 512 units 72.0 and 73.2.)
+    pieced = true;
+    constexpr int HID_G = 4;
+    for (int i = tid; i < nnz; i += FWD_THREADS) {
+      const int c = __ldg(p.col_idx + rbeg + i);
+      const int prev = i > 0 ? __ldg(p.col_idx + rbeg + i - 1) : -1;
+      const bool okc = c >= 0 && c < p.D && prev < c;
+      if (!okc) bad = DSLIDE_ERR_BAD_INDEX;
+      const float xv = __ldg(p.vals + rbeg + i);
+      sh_ids[i] = okc ? c : 0;
+      sh_z[i] = xv;
+      if (i == tid) { c1 = okc ? c : 0; x1 = xv; }
+    }
+    bad = __syncthreads_or(bad);
+    if (!bad) {
+      if (!waited) {
+        griddep_wait();
+        waited = true;
+      }
+      if (MODE == 0 && tid < R) line1 = __ldcg(p.hotmap1 + c1);      // (nnz > R)
+      if (tid < H4) {
+        float4 a = reinterpret_cast<const float4*>(p.b1)[tid];
+        const int depth = min(8, R / HID_G), ngroups = (nnz + HID_G - 1) / HID_G;
+        int asked = 0, to = 0, from = 0;
+        auto ask = [&]() {
+#pragma unroll
+          for (int q = 0; q < HID_G; ++q) {
+            const int i = asked * HID_G + q;
+            if (i < nnz) cp_async16(stage + (size_t)(to * HID_G + q) * H + 4 * tid, p.W1 + (size_t)sh_ids[i] * H + 4 * tid);
+          }
+          cp_async_commit();
+          ++asked;
+          to = to + 1 == depth ? 0 : to + 1;
+        };
+        for (int g = 0; g < depth - 1; ++g) ask();
+#pragma unroll 1
+        for (int g = 0; g < ngroups; ++g) {
+          ask();
+          cp_async_wait_pending(depth - 1);
+#pragma unroll
+          for (int q = 0; q < HID_G; ++q) {
+            const int i = g * HID_G + q;
+            if (i < nnz) {
+              const float4 w = *reinterpret_cast<const float4*>(stage + (size_t)(from * HID_G + q) * H + 4 * tid);
+              const float xv = sh_z[i];
+              a.x = __fmaf_rn(xv, w.x, a.x); a.y = __fmaf_rn(xv, w.y, a.y); a.z = __fmaf_rn(xv, w.z, a.z); a.w = __fmaf_rn(xv, w.w, a.w);
+            }
+          }
+          from = from + 1 == depth ? 0 : from + 1;
+        }
+        reinterpret_cast<float4*>(sh_h)[tid] = a;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) acc[u] = tid + u * FWD_THREADS < H ? sh_h[tid + u * FWD_THREADS] : 0.f;
+  }
+  }
+  for (int c0 = 0; c0 < nnz && !pieced; c0 += R) {
     const int nr = min(R, nnz - c0);
     for (int i = tid; i < nr; i += FWD_THREADS) {
       const int c = __ldg(p.col_idx + rbeg + c0 + i);
