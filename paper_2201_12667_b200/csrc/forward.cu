@@ -9,12 +9,13 @@
 // The same kernel in predict mode stops after the logits and selects the top k.
 //
 // Every phase is a short chain of memory rounds, so each round puts as much in flight as it can:
-// the rows of W1 of a chunk of nonzeros arrive by one bulk copy each (cp.async.bulk, completion on an
-// mbarrier) and are then summed in the stored order; the L bucket offsets are fetched in one round and
-// all bucket entries in a second; the active rows of W2 are copied the same way into the shared memory
-// the dedup work space no longer needs, and serve both the logits and the back-propagated error (in
-// one pass when the set is larger than that space).  Optional steps of the selection: densification
+// the rows of W1 of a chunk of nonzeros arrive together by 16-byte asynchronous copies and are summed in the stored order
+// (beyond 512 units a thread copies and adds its own piece of every row); the L bucket offsets are fetched in one round and
+// all bucket entries in a second; the active rows of W2 are staged in the shared memory the dedup work space no longer needs and
+// serve logits, sums and the back-propagated error, or, in wide layers and sets larger than that space, pass through a ring of
+// every warp, which takes all of these in one pass.  Optional steps of the selection: densification
 // of all-zero DWTA bins of the query (Section 4.1) and the sampling budget of Section 3.7.
+// A block's eight warps issue an instruction every four cycles or so: code that is run once costs more than the loads it waits for.
 #include "common.cuh"
 #include "waits.cuh"
 
