@@ -1410,11 +1410,31 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   float* sh_ce = stage + (size_t)stage_rows * ldr;           // [stage_rows]
   const bool streaming = MODE == 0 && na > stage_rows;
   float Mrun = -INFINITY, Erun = 0.f;
-  float accS[KPT], accT[KPT];
+  // The sums of a warp's rows of a chunk, or of all that is staged: a lane holds four consecutive units of every 128, and of up to 64
+  // units 8 or 16 lanes have a row each.  (A thread per unit, with rows shared out to groups of threads, read four times as
+  // often: 64 samples of SimHash sets of 400 rows x 128 units, a step 68.8 us, so 67.5; the 670,091-neuron shape, whose sets are
+  // one chunk or a little more, 64.5 and 63.1.)
+  constexpr int NCH = 2;                           // H <= 128 * NCH
+  float4 av[NCH];
 #pragma unroll
-  for (int u = 0; u < KPT; ++u) { accS[u] = 0.f; accT[u] = 0.f; }
-  const int ngrp = H >= FWD_THREADS ? 1 : min(FWD_WARPS, FWD_THREADS / H);   // groups of H threads (sh_dh holds FWD_WARPS)
-  const int grp = H >= FWD_THREADS ? 0 : tid / H;
+  for (int q = 0; q < NCH; ++q) av[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int rl = H4 <= 8 ? 8 : H4 <= 16 ? 16 : 32, lg_rl = H4 <= 8 ? 3 : H4 <= 16 ? 4 : 5;      // lanes of a row
+  auto add_rows = [&](const float* coef, int n) {
+#pragma unroll 4
+    for (int a = (tid >> lg_rl); a < n; a += FWD_THREADS >> lg_rl) {
+      const float ga = coef[a];
+      const float4* row = reinterpret_cast<const float4*>(stage + (size_t)a * ldr);
+#pragma unroll
+      for (int q = 0; q < NCH; ++q) {
+        const int c = (lane & (rl - 1)) + 32 * q;
+        if (c < H4) {
+          const float4 w = row[c];
+          av[q].x = fmaf(ga, w.x, av[q].x); av[q].y = fmaf(ga, w.y, av[q].y);
+          av[q].z = fmaf(ga, w.z, av[q].z); av[q].w = fmaf(ga, w.w, av[q].w);
+        }
+      }
+    }
+  };
   // a thread's place in the copy pattern of the padded rows: H4 + 1 pieces per row
   const int rp_dr = FWD_THREADS / (H4 + 1), rp_dc = FWD_THREADS - rp_dr * (H4 + 1);
   const int rp_r0 = tid / (H4 + 1), rp_c0 = tid - rp_r0 * (H4 + 1);
@@ -1530,29 +1550,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
       }
       Erun = Erun * scale + block_sum(es, sh_red);      // its barriers make the chunk's exp values visible
       Mrun = Mnew;
-      if (grp < ngrp) {
 #pragma unroll
-        for (int u = 0; u < KPT; ++u) {
-          const int k = (H >= FWD_THREADS ? tid : tid - grp * H) + u * FWD_THREADS;
-          if (k < H && (u == 0 || H > FWD_THREADS)) {
-            float v0 = accS[u] * scale, v1 = 0.f, v2 = 0.f, v3 = 0.f;
-            int a = grp;
-            for (; a + 3 * ngrp < nr; a += 4 * ngrp) {
-              v0 = fmaf(sh_ce[a], stage[(size_t)a * ldr + k], v0);
-              v1 = fmaf(sh_ce[a + ngrp], stage[(size_t)(a + ngrp) * ldr + k], v1);
-              v2 = fmaf(sh_ce[a + 2 * ngrp], stage[(size_t)(a + 2 * ngrp) * ldr + k], v2);
-              v3 = fmaf(sh_ce[a + 3 * ngrp], stage[(size_t)(a + 3 * ngrp) * ldr + k], v3);
-            }
-            for (; a < nr; a += ngrp) v0 = fmaf(sh_ce[a], stage[(size_t)a * ldr + k], v0);
-            accS[u] = (v0 + v1) + (v2 + v3);
-            if (grp == 0)                               // the label rows of this chunk, once
-              for (int i = 0; i < nlab; ++i) {
-                const int pos = sh_lab[i] - c0;
-                if (sh_lab[i] >= 0 && pos >= 0 && pos < nr) accT[u] += stage[(size_t)pos * ldr + k];
-              }
-          }
-        }
-      }
+      for (int q = 0; q < NCH; ++q) { av[q].x *= scale; av[q].y *= scale; av[q].z *= scale; av[q].w *= scale; }
+      add_rows(sh_ce, nr);
     }
   }
   if (BULK && timed_out) {
@@ -1617,48 +1617,31 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   }
   __syncthreads();
 
-  // ---- error at the hidden layer: dh = [h > 0] * sum_a g_a W2[j_a, :] (weights before the update).  Warp w takes
-  //      the staged rows w, w + 8, ...; a lane holds four consecutive hidden units of every 128; the warps' sums are
-  //      then added in warp order.  When the rows were streamed the sums exist already (per group of threads). ----
+  // ---- error at the hidden layer: dh = [h > 0] * sum_a g_a W2[j_a, :] (weights before the update).  Every warp has
+  //      its staged rows; the warps' sums are then added in warp order.  When the rows were streamed the sums
+  //      exist already ----
   {
-    constexpr int NCH = 2;                                 // 16-byte pieces of a row per lane: H <= 128 * NCH
-    int nparts = ngrp;
-    if (!streaming) {
-      nparts = FWD_WARPS;
-      float4 av[NCH];
+    if (!streaming) add_rows(gp, na);
+    for (int o = rl; o < 32; o <<= 1) {            // the rows side by side
+      av[0].x += __shfl_xor_sync(FULLM, av[0].x, o); av[0].y += __shfl_xor_sync(FULLM, av[0].y, o);
+      av[0].z += __shfl_xor_sync(FULLM, av[0].z, o); av[0].w += __shfl_xor_sync(FULLM, av[0].w, o);
+    }
 #pragma unroll
-      for (int q = 0; q < NCH; ++q) av[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-      for (int a = warp; a < na; a += FWD_WARPS) {
-        const float ga = gp[a];
-        const float4* row = reinterpret_cast<const float4*>(stage + (size_t)a * ldr);
-#pragma unroll
-        for (int q = 0; q < NCH; ++q) {
-          const int c = lane + 32 * q;
-          if (c < H4) {
-            const float4 w = row[c];
-            av[q].x = fmaf(ga, w.x, av[q].x); av[q].y = fmaf(ga, w.y, av[q].y);
-            av[q].z = fmaf(ga, w.z, av[q].z); av[q].w = fmaf(ga, w.w, av[q].w);
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < NCH; ++q) {
-        const int c = lane + 32 * q;
-        if (c < H4) reinterpret_cast<float4*>(sh_dh + (size_t)warp * H)[c] = av[q];
-      }
-    } else if (grp < ngrp) {
-#pragma unroll
-      for (int u = 0; u < KPT; ++u) {
-        const int k = (H >= FWD_THREADS ? tid : tid - grp * H) + u * FWD_THREADS;
-        if (k < H && (u == 0 || H > FWD_THREADS))
-          sh_dh[(size_t)grp * H + k] = (accS[u] / E - (ny > 0 ? accT[u] / (float)ny : 0.f)) / fB;
-      }
+    for (int q = 0; q < NCH; ++q) {
+      const int c = lane + 32 * q;
+      if (c < H4) reinterpret_cast<float4*>(sh_dh + (size_t)warp * H)[c] = av[q];
     }
     __syncthreads();
     for (int k = tid; k < H; k += FWD_THREADS) {
       float v = 0.f;
-      for (int w = 0; w < nparts; ++w) v += sh_dh[(size_t)w * H + k];
+#pragma unroll
+      for (int w = 0; w < FWD_WARPS; ++w) v += sh_dh[(size_t)w * H + k];
+      if (streaming) {                             // (the label rows are in L2)
+        float T = 0.f;
+        for (int i = 0; i < nlab; ++i)
+          if (sh_lab[i] >= 0) T += p.W2[(size_t)(dense ? sh_lab[i] : idp[sh_lab[i]]) * H + k];
+        v = (v / E - (ny > 0 ? T / (float)ny : 0.f)) / fB;
+      }
       p.dh[(size_t)s * H + k] = sh_h[k] > 0.f && !(BULK && timed_out) ? v : 0.f;
     }
   }
