@@ -1633,9 +1633,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
     }
     __syncthreads();
     for (int k = tid; k < H; k += FWD_THREADS) {
-      float v = 0.f;
+      float y[FWD_WARPS];
 #pragma unroll
-      for (int w = 0; w < FWD_WARPS; ++w) v += sh_dh[(size_t)w * H + k];
+      for (int w = 0; w < FWD_WARPS; ++w) y[w] = sh_dh[(size_t)w * H + k];
+      float v = ((y[0] + y[1]) + (y[2] + y[3])) + ((y[4] + y[5]) + (y[6] + y[7]));      // in pairs, so that no sum is long
       if (streaming) {                             // (the label rows are in L2)
         float T = 0.f;
         for (int i = 0; i < nlab; ++i)
@@ -1867,22 +1868,23 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   M = __int_as_float(sh_misc[0]);
 #pragma unroll
   for (int w = 1; w < FWD_WARPS; ++w) M = fmaxf(M, __int_as_float(sh_misc[w]));
-  E = 0.f;
 #pragma unroll
-  for (int w = 0; w < FWD_WARPS; ++w) {
-    const float ew = sh_red[w];
-    fac[w] = ew == 0.f ? 0.f : expf(__int_as_float(sh_misc[w]) - M);
-    E = fmaf(ew, fac[w], E);
-  }
+  for (int w = 0; w < FWD_WARPS; ++w) fac[w] = sh_red[w] == 0.f ? 0.f : expf(__int_as_float(sh_misc[w]) - M);
+  // (in pairs, so that no sum is long)
+  auto of_warps = [&](const float* x, int stride) {
+    float y[FWD_WARPS / 2];
+#pragma unroll
+    for (int w = 0; w < FWD_WARPS / 2; ++w) y[w] = fmaf(fac[2 * w], x[(size_t)(2 * w) * stride], fac[2 * w + 1] * x[(size_t)(2 * w + 1) * stride]);
+    return (y[0] + y[1]) + (y[2] + y[3]);
+  };
+  E = of_warps(sh_red, 1);
   const float fB = (float)p.B;
   const int ny = sh_misc[8];
 #pragma unroll
   for (int u = 0; u < KPT; ++u) {
     const int k = tid + u * FWD_THREADS;
     if (k < H) {
-      float v = 0.f;
-#pragma unroll
-      for (int w = 0; w < FWD_WARPS; ++w) v = fmaf(fac[w], sh_dh[(size_t)w * H + k], v);
+      float v = of_warps(sh_dh + k, H);
       v = na > 0 ? (v / E - (ny > 0 ? accT[u] / (float)ny : 0.f)) / fB : 0.f;
       p.dh[(size_t)s * H + k] = sh_h[k] > 0.f && !timed_out ? v : 0.f;
     }
