@@ -736,8 +736,8 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
   if (tid == 0) sh_fix = need_fix[s];            // a buffer of the sample ran over in the filter pass
   const float4* h4 = reinterpret_cast<const float4*>(h + (size_t)s * H);
   const int H4 = H >> 2;
-  // A buffer's entries are shared out to 2^lg places, which makes more places than threads: a thread has two at most, and nearly
-  // every thread has a largest key to go by (with 64 results the cut is at the 144th).
+  // A buffer's entries are shared out to 2^lg places, which makes more places than threads: a thread has two at most.  (Where
+  // candidates are many in most buffers nearly every thread has a largest key to go by; with 64 results the cut is at the 144th.)
   const int lg = 31 - __clz(RF_MAXV / nvs), g = 1 << lg;
   const int p1 = tid + RF_THREADS, s0 = tid & (g - 1), s1 = p1 & (g - 1);
   const bool two = (p1 >> lg) < nvs;
@@ -787,7 +787,8 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
   }
   __syncthreads();
   total = sh_total;
-  // The candidates that reach the cap-th largest of the threads' maxima, cut to 20 bits, go on, all of them when there are no more than cap
+  // The candidates that reach the cap-th largest of the threads' maxima, cut to 20 bits, go on; all of them when there are no more than
+  // cap, or when fewer threads than that have any (the cut is 0 then)
   const uint32_t K = total <= cap ? 0u : sh_K;
   entries([&](int z, int id) {
     if (tc_key(__int_as_float(z)) >= K) { const int slot = atomicAdd(&sh_n, 1); if (slot < RF_SLOTS) ei[slot] = id; }
@@ -852,10 +853,10 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
   if (tid == 0) {
     float hn = 0.f;
     for (int w = 0; w < RF_WARPS; ++w) hn += red[w];
-    // Every neuron that did not go on to the exact pass has an approximate score below T: the cut when candidates
-    // were dropped here, else the sample's threshold (a neuron below it was never a candidate).  Its exact score is
-    // at most T plus the error bound; the k best are certain when the k-th exact score lies above.
-    const float T = total > cap ? tc_unkey(K) : tau[s];
+    // Every neuron that did not go on to the exact pass has an approximate score below T: the cut when there was one
+    // here, else the sample's threshold (a neuron below it was never a candidate; the cut is no lower, both are cut to 20 bits).
+    // Its exact score is at most T plus the error bound; the k best are certain when the k-th exact score lies above.
+    const float T = K != 0u ? tc_unkey(K) : tau[s];
     if (nc < k && nc < N) sh_fix = 1;            // scores that are not numbers never become candidates
     if (T > -INFINITY) {
       const float bound = T + TC_ERR * sqrtf(hn) * sqrtf(__uint_as_float(*norm2max)) + 1e-30f;

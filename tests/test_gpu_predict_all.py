@@ -227,3 +227,40 @@ def test_neighbours_that_are_favoured_together_fit_their_buffer():
         assert best < 1.0, best
     finally:
         ds.dslide_destroy(ctx)
+
+
+def predict_all(ctx, batch, k):
+    import torch
+    from paper_2201_12667_b200 import binding as ds
+    B = len(batch[0]) - 1
+    ids, sc = torch.empty(B, k, dtype=torch.int32, device="cuda"), torch.empty(B, k, device="cuda")
+    ds.dslide_predict_topk(ctx, B, *batch, k, 1, ids, sc)
+    ds.dslide_sync(ctx)
+    return ids.cpu().numpy(), sc.cpu().numpy()
+
+
+@pytest.mark.parametrize("H,N,k", [(64, 384, 1), (64, 384, 5), (128, 512, 10), (300, 512, 5), (64, 600, 5), (64, 1024, 64), (128, 1024, 64)])
+def test_near_ties_of_few_neurons(H, N, k):
+    """Rows that resemble one another: their scores differ by less than the filter's error, so that no sample can be decided by
+    it, however its candidates are shared out to the threads that look for the cut."""
+    from paper_2201_12667_b200 import binding as ds
+    from tests.gpu_harness import to_dev
+    B, spread = 1000, 1e-5
+    r = np.random.default_rng(H + N + k)
+    ctx = ds.dslide_init(ds.make_config(input_dim=B, hidden_dim=H, output_dim=N, hash_family=workloads.SIMHASH, K=4, L=2, bucket_cap=16, max_batch=B))
+    try:
+        W1 = r.standard_normal((B, H)).astype(np.float32)
+        W2 = (0.05 + spread * r.standard_normal((N, H))).astype(np.float32)
+        ds.dslide_set_tensor(ctx, "W1", W1)
+        ds.dslide_set_tensor(ctx, "W2", W2)
+        ids, sc = predict_all(ctx, to_dev([np.arange(B + 1, dtype=np.int32), np.arange(B, dtype=np.int32), np.ones(B, np.float32)]), k)
+        h = np.maximum(0, W1).astype(np.float64)
+        z = h @ W2.T.astype(np.float64)
+        # at most H / 32 + 9 additions after one another make a score in 32 bits
+        tol = (H / 32 + 9) * 2.0 ** -24 * (h @ np.abs(W2.T.astype(np.float64))).max(axis=1, keepdims=True)
+        kth = np.sort(z, axis=1)[:, ::-1][:, k - 1:k]
+        assert (np.diff(np.sort(ids, axis=1), axis=1) > 0).all() and (ids >= 0).all()
+        assert (np.abs(np.take_along_axis(z, ids, 1) - sc) <= tol).all()
+        assert (np.take_along_axis(z, ids, 1) >= kth - 2 * tol).all()
+    finally:
+        ds.dslide_destroy(ctx)
