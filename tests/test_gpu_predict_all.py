@@ -264,3 +264,50 @@ def test_near_ties_of_few_neurons(H, N, k):
         assert (np.take_along_axis(z, ids, 1) >= kth - 2 * tol).all()
     finally:
         ds.dslide_destroy(ctx)
+
+
+@pytest.mark.parametrize("H,N,B", [s for s in NORMS if s[2] < 1100] + [
+    (200, 38017, 700), (200, 20011, 769), (196, 20011, 1024), (256, 20011, 1100), (256, 38017, 1300)])      # three to six groups of samples in pairs
+def test_the_bound_takes_the_whole_norm(H, N, B):
+    """The best scores stand 0.25 above a plateau that the cut falls on.  A row whose norm makes the error bound 0.9 of that leaves
+    every sample decided, one that makes it 1.1 none: the scores then come from the scan, which adds up in another order.  The row's
+    weight lies in all of its 16-byte pieces, or in one of them."""
+    from paper_2201_12667_b200 import binding as ds
+    from tests.gpu_harness import to_dev
+    k, err = 16, 2.2e-3                                         # the filter's error for |h| = |w| = 1
+    r = np.random.default_rng(H + B)
+    ctx = ds.dslide_init(ds.make_config(input_dim=4, hidden_dim=H, output_dim=N, hash_family=workloads.SIMHASH, K=4, L=2, bucket_cap=16, max_batch=B))
+    try:
+        ds.dslide_set_tensor(ctx, "W1", np.zeros((4, H), np.float32))
+        ds.dslide_set_tensor(ctx, "b1", np.ones(H, np.float32))               # |h|^2 = H
+        W2, b2 = np.zeros((N, H), np.float32), (-1 - r.random(N)).astype(np.float32)
+        some = r.permutation(N)[:k + 120]
+        W2[some[:k]] = 0.05 * r.standard_normal((k, H))
+        b2[some[:k]] = 1.25 + 0.05 * np.arange(k) - W2[some[:k]].astype(np.float64).sum(axis=1)
+        b2[some[k:]] = 1                                        # the plateau: more rows than the cut is at, fewer than are scored exactly
+        ds.dslide_set_tensor(ctx, "b2", b2)
+        batch = to_dev([np.arange(B + 1, dtype=np.int32), np.zeros(B, np.int32), np.ones(B, np.float32)])
+
+        def scores(row=None, units=None, share=1.0):
+            keep = W2[row].copy() if row is not None else None
+            if row is not None:                                 # the row's score: 0 and its bias, for its weights cancel
+                W2[row] = 0
+                W2[row, units] = share * 0.25 / (err * np.sqrt(H * len(units))) * (-1.0) ** np.arange(len(units))
+            ds.dslide_set_tensor(ctx, "W2", W2)
+            if row is not None:
+                W2[row] = keep
+            return predict_all(ctx, batch, k)[1]
+
+        free = np.setdiff1d(np.arange(N), some)
+        filtered, scanned = scores(), scores(int(free[0]), np.arange(2), 1e6)
+        assert np.allclose(filtered, 2 - 0.05 * np.arange(k), rtol=1e-5) and np.allclose(scanned, filtered, rtol=1e-5)
+        assert (filtered != scanned).any(axis=1).all()
+        slab = 32 * r.integers(0, H // 32)
+        pieces = [np.arange(H)] + [slab + 4 * p + np.arange(4) for p in range(8)]
+        at = [0, 31, 63, 64, 100, 127, 128, 161, 255]           # of a tile: in either block of a pair, in any group's share
+        for i, units in enumerate(pieces):
+            row = int(free[min(np.searchsorted(free, 256 * (N // 512) + at[(i + B) % 9]), len(free) - 1)])
+            assert (scores(row, units, 0.9) == filtered).all(), (i, row)
+            assert (scores(row, units, 1.1) == scanned).all(), (i, row)
+    finally:
+        ds.dslide_destroy(ctx)
