@@ -1924,7 +1924,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   if (!dense) {
 #pragma unroll
     for (int u = 0; u < HO_PER; ++u)
-      if (u * FWD_THREADS < na) {          // uniform over the block
+      if (u * (ho_rows / HO_PER) < na) {   // uniform over the block; the rows counted in above, of fewer rings than warps not one per thread
         const int a = act0[u];
         const bool live = a >= 0;
         touch_mark(p, live, p.hdr2 + jj0[u], p.mask2 + (size_t)jj0[u] * p.Wd, p.ovf2 + (size_t)jj0[u] * PAIR_T, jj0[u], nth0[u], s,

@@ -11,7 +11,7 @@ if torch.cuda.is_available():
     from paper_2201_12667_b200 import workloads
     from tests.gpu_harness import Pair
     from tests.test_gpu_parity import check_predict
-    from tests.test_gpu_shapes import one_and_two_steps
+    from tests.test_gpu_shapes import dense_features_batch, one_and_two_steps
 
 SIMHASH, DWTA = 0, 1
 
@@ -53,5 +53,24 @@ def test_simhash_bits_of_queries(H, K, L):
     try:
         wl = workloads.Workload(dict(workloads.config("tiny"), D=501, N=1501, batch=6), seed=5)
         one_and_two_steps(pr, [wl.batch(0), wl.batch(1)])
+    finally:
+        pr.close()
+
+
+@pytest.mark.parametrize("H,K,max_labels,nlab,budget,least", [
+    (512, 16, 4096, 190, 0, 160),      # five rings: a warp's first 32 rows are the set's first 160
+    (1024, 10, 16, 3, 250, 224),       # seven rings, one group deep
+    (1020, 10, 16, 3, 231, 224),
+])
+def test_fewer_rings_than_warps(H, K, max_labels, nlab, budget, least):
+    """1,024 tables and many labels leave staging space for fewer rings than the block has warps.  Sets between the rows that the
+    rings' warps count first and 256: all of them are handed to the update kernel, in steps after one another."""
+    N = 1500
+    pr = Pair(D=501, H=H, N=N, family=SIMHASH, K=K, L=1024, srp_nnz=8, bucket_cap=1, max_batch=6, max_labels=max_labels, budget=budget, lr=1e-3, seed=H)
+    try:
+        r = np.random.default_rng(H)
+        one_and_two_steps(pr, [dense_features_batch(r, 6, 501, N, 20, nlab) for _ in range(2)])
+        cnt = pr.gpu_active_sets(6)[1]
+        assert cnt.min() > least and cnt.max() <= 256, cnt
     finally:
         pr.close()
