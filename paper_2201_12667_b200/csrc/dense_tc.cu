@@ -428,7 +428,8 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     // that all banks are busy ----------------
     if (norms) {
       constexpr int LANES = 32 * TC_NORM_WARPS, RMAX = ROWS / LANES > 1 ? ROWS / LANES : 1;
-      static_assert(LANES / (ROWS / 4) <= 8 && (ROWS % LANES == 0 || LANES % ROWS == 0), "no more lanes to a row than it has pieces");
+      constexpr int LPR_MAX = LANES / (ROWS / 4);      // lanes of a row at most
+      static_assert(LPR_MAX <= 8 && (ROWS % LANES == 0 || LANES % ROWS == 0), "no more lanes to a row than it has pieces");
       const int nrows = ROWS / nshare;                 // rows of this block
       const int lpr = nrows < LANES ? LANES / nrows : 1, nrr = nrows < LANES ? 1 : nrows / LANES;
       const int idx = (warp - TC_THREADS / 32 - 1) * 32 + lane, cn = 8 / lpr, c0 = idx % lpr * cn;
@@ -451,7 +452,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
                 const unsigned char* rowp = tile + (size_t)ks * SLAB + (size_t)rr * LANES * 128;
                 if (cn == 8) tc_squares<8>(rowp, c0, row0 & 7, n[rr]);
                 else if (cn == 4) tc_squares<4>(rowp, c0, row0 & 7, n[rr]);
-                else if (cn == 2) tc_squares<2>(rowp, c0, row0 & 7, n[rr]);
+                else if (LPR_MAX < 8 || cn == 2) tc_squares<2>(rowp, c0, row0 & 7, n[rr]);
                 else tc_squares<1>(rowp, c0, row0 & 7, n[rr]);
               }
           __syncwarp();
@@ -462,7 +463,9 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         for (int rr = 0; rr < RMAX; ++rr) {
           float sq = (__uint_as_float((unsigned)n[rr][0]) + __uint_as_float((unsigned)(n[rr][0] >> 32))) +
                      (__uint_as_float((unsigned)n[rr][1]) + __uint_as_float((unsigned)(n[rr][1] >> 32)));
-          for (int o = 1; o < lpr; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+          if (lpr >= 2) sq += __shfl_xor_sync(0xffffffffu, sq, 1);
+          if (lpr >= 4) sq += __shfl_xor_sync(0xffffffffu, sq, 2);
+          if (LPR_MAX == 8 && lpr == 8) sq += __shfl_xor_sync(0xffffffffu, sq, 4);
           best = fmaxf(best, sq);
         }
       }
