@@ -206,7 +206,7 @@ __device__ __forceinline__ void tc_squares(const unsigned char* row, int c0, int
   }
 }
 // One lane of a converged warp, the same at every call: the copies, multiplications and commits are its own, while the whole warp
-// walks the tiles and waits, so that their operands are the warp's.  Issued by one lane of a diverged warp an instruction took 84 to 134
+// walks the tiles, waits and agrees on what a wait has answered, so that their operands are the warp's.  Issued by one lane of a diverged warp an instruction took 84 to 134
 // cycles where the tensor pipe takes 64, which bounded the filter at every width (512 samples x 4,000,000 neurons x 256 units
 // 1,890 us, so 1,500; 1,024 x 253,855 x 200 246 and 218).
 __device__ __forceinline__ bool tc_elect() {
@@ -317,7 +317,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       const int row0 = (slice + i * p.nslices) * p.tile_stride * NT + (int)rank * ROWS;
       if (WIDE) {
         for (int ks = 0; ks < ksub; ++ks, ++fills) {
-          if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
+          if (stround > 0 && !(on = tc_bar_wait_warp<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
           unsigned char* to = smB + (size_t)st * tile_bytes;
           if (tc_elect()) {
             if (PAIR) {
@@ -336,7 +336,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
         }
         continue;
       }
-      if (stround > 0 && !(on = tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
+      if (stround > 0 && !(on = tc_bar_wait_warp<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
       if (tc_elect()) {
         if (rank == 0) tc_bar_expect(bar_full + st, (PAIR ? 2u : 1u) * tile_bytes);
         const uint32_t full = PAIR ? tc_at_rank(bar_full + st, 0u) : 0u;
@@ -351,22 +351,22 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       if (++st == nst) { st = 0; ++stround; }
     }
     // the last fill of every stage has been consumed: no copy and no arrival at this block's barriers is on its way any more
-    for (int f = max(0, fills - nst); on && f < fills; ++f) on = tc_bar_wait<PAIR>(bar_empty + f % nst, (f / nst) & 1, abort_flag);
+    for (int f = max(0, fills - nst); on && f < fills; ++f) on = tc_bar_wait_warp<PAIR>(bar_empty + f % nst, (f / nst) & 1, abort_flag);
   } else if (warp == 1) {
     // ---------------- MMA issue: one thread (of a pair's first block) ----------------
     if (rank == 0) {
       const uint32_t idesc = tc_idesc(PAIR ? 2 * TC_M : TC_M, NT);
-      bool on = WIDE || tc_bar_wait<PAIR>(bar_a, 0, abort_flag);
+      bool on = WIDE || tc_bar_wait_warp<PAIR>(bar_a, 0, abort_flag);
       const uint64_t b_base = tc_desc(tc_smem(smB));      // a descriptor's address field counts 16-byte units
       int st = 0, stround = 0, acc = 0, accround = 0;
       for (int i = 0; on && i < my_tiles; ++i) {
-        if (!WIDE && !tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag)) break;
-        if (accround > 0 && !tc_bar_wait<PAIR>(bar_accempty + acc, (accround - 1) & 1, abort_flag)) break;
+        if (!WIDE && !tc_bar_wait_warp<PAIR>(bar_full + st, stround & 1, abort_flag)) break;
+        if (accround > 0 && !tc_bar_wait_warp<PAIR>(bar_accempty + acc, (accround - 1) & 1, abort_flag)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem_base + (uint32_t)(acc * NT);
         if (WIDE) {
           for (int ks = 0; ks < ksub; ++ks) {
-            if (!(on = tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag))) break;
+            if (!(on = tc_bar_wait_warp<PAIR>(bar_full + st, stround & 1, abort_flag))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (tc_elect()) {
               const uint64_t b = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
@@ -552,6 +552,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       // 64 units 138 us, so 122).
       tc_bar_wait<PAIR>(bar_bfull + (i & (TC_BT - 1)), (i / TC_BT) & 1, abort_flag);
       tc_bar_wait<PAIR>(bar_accfull + acc, accround & 1, abort_flag);
+      __syncwarp();                          // lanes may leave a wait one by one; tensor memory is read by whole warps
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
       for (int c0 = (NT / TC_SPLIT) * half; c0 < (NT / TC_SPLIT) * (half + 1); c0 += 32) {
@@ -646,8 +647,10 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       else
         while (clock64() < until) __nanosleep(1000);      // its copies are counted in the first block, which may not have asked for the same stages
     }
-    if (tid == 32 && rank == 0) {
-      tc_commit<PAIR>(bar_drain, 1);
+    if (warp == 1 && rank == 0) {
+      __syncwarp();
+      if (tc_elect()) tc_commit<PAIR>(bar_drain, 1);      // of the lane that has issued them
+      __syncwarp();
       tc_bar_drain(bar_drain, 0, until);
     }
     if (PAIR) tc_cluster_sync();

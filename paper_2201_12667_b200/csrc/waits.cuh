@@ -52,7 +52,16 @@ __device__ __forceinline__ bool tc_bar_wait(uint64_t* bar, uint32_t parity, vola
   }
   return true;
 }
-// The same, for a block that has given up: it waits until the time `until`, whatever the flag says.
+// The same by a whole warp: true where all of its lanes have seen the phase complete, and the same answer for all.  A lane that has
+// seen the flag, or that a wait has kept longer, is with the others again for what follows: an election, or an instruction that
+// takes the whole warp.
+template <bool PAIR, bool CLUSTER = false>
+__device__ __forceinline__ bool tc_bar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  const bool ok = tc_bar_wait<PAIR, CLUSTER>(bar, parity, abort);
+  __syncwarp();
+  return __all_sync(0xffffffffu, ok) != 0;
+}
+// For a block that has given up: it waits until the time `until`, whatever the flag says.
 __device__ __forceinline__ void tc_bar_drain(uint64_t* bar, uint32_t parity, long long until) {
   while (!tc_bar_try(tc_smem(bar), parity) && clock64() < until) {}
 }

@@ -35,3 +35,11 @@ def test_a_pair_gives_up_together(probe):
     assert probe.run_waits(1, out, cycles) == 0
     assert list(out) == [0, 1, 1, 0]
     assert cycles[0] < 0.5e9 and 2.0e7 <= cycles[1] < 5.0e8, list(cycles)
+
+
+def test_a_warp_gets_one_answer(probe):
+    """Lanes whose own waits would end differently once the block has given up: none goes on while others leave."""
+    out, cycles = (ctypes.c_int * 4)(), (ctypes.c_longlong * 2)()
+    assert probe.run_waits(2, out, cycles) == 0
+    assert list(out) == [0, 1, 32, 1]
+    assert cycles[1] < 0.5e9, list(cycles)

@@ -52,13 +52,38 @@ __global__ void __cluster_dims__(2, 1, 1) k_pair(int* out, long long* cycles) {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-extern "C" int run_waits(int pair, int* out, long long* cycles) {      // host arrays of 4 and 2
+// A warp whose block has given up waits, half of its lanes for a phase that has completed and half for one that nobody completes: all
+// lanes get the same answer, and one of them is elected after it.  Then all for the completed one, with the flag set.
+// out: [0] lanes told that the mixed phase has completed, [1] lanes elected after it, [2] and [3] the same of the second wait
+__global__ void k_warp(int* out, long long* cycles) {
+  __shared__ __align__(8) uint64_t never, done;
+  __shared__ int flag;
+  if (threadIdx.x == 0) {
+    flag = 1;
+    init_bar(&never);
+    init_bar(&done);
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc_smem(&done)) : "memory");
+  }
+  __syncthreads();
+  const long long t0 = clock64();
+  for (int i = 0; i < 2; ++i) {
+    const bool ok = tc_bar_wait_warp<false>(i == 0 && (threadIdx.x & 1) ? &never : &done, 0, &flag);
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    const int told = __popc(__ballot_sync(0xffffffffu, ok)), elected = __popc(__ballot_sync(0xffffffffu, one != 0u));
+    if (threadIdx.x == 0) { out[2 * i] = told; out[2 * i + 1] = elected; }
+    if (threadIdx.x == 0) cycles[i] = clock64() - t0;
+  }
+}
+
+extern "C" int run_waits(int which, int* out, long long* cycles) {      // host arrays of 4 and 2
   int* d = nullptr;
   long long* c = nullptr;
   cudaError_t e = cudaMalloc(&d, 16);
   if (e == cudaSuccess) e = cudaMalloc(&c, 16);
   if (e == cudaSuccess) {
-    if (pair) k_pair<<<2, 32>>>(d, c);
+    if (which == 2) k_warp<<<1, 32>>>(d, c);
+    else if (which == 1) k_pair<<<2, 32>>>(d, c);
     else k_waits<<<1, 32>>>(d, c);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpy(out, d, 16, cudaMemcpyDeviceToHost);
