@@ -784,23 +784,46 @@ k_tc_refine(const float* W2, const RowHdr* hdr2, const float* h, const int2* can
   total = __reduce_add_sync(0xffffffffu, (s0 == 0 ? c0 : 0) + (s1 == 0 ? c1 : 0));
   most[tid] = mine;
   if (lane == 0) atomicAdd(&sh_total, total);
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t v[RF_WARPS];
+  auto find_cut = [&]() {                        // the cap-th of the maxima
+    __syncthreads();
+    if (warp == 0) {
+      uint32_t v[RF_WARPS];
 #pragma unroll
-    for (int i = 0; i < RF_WARPS; ++i) v[i] = most[32 * i + lane];
-    const uint32_t cut = tc_select(v, cap, 12);
-    if (lane == 0) sh_K = cut;
-  }
-  __syncthreads();
+      for (int i = 0; i < RF_WARPS; ++i) v[i] = most[32 * i + lane];
+      const uint32_t cut = tc_select(v, cap, 12);
+      if (lane == 0) sh_K = cut;
+    }
+    __syncthreads();
+  };
+  find_cut();
   total = sh_total;
   // The candidates that reach the cap-th largest of the threads' maxima, cut to 20 bits, go on; all of them when there are no more than
   // cap, or when fewer threads than that have any (the cut is 0 then)
-  const uint32_t K = total <= cap ? 0u : sh_K;
-  entries([&](int z, int id) {
-    if (tc_key(__int_as_float(z)) >= K) { const int slot = atomicAdd(&sh_n, 1); if (slot < RF_SLOTS) ei[slot] = id; }
-  });
+  uint32_t K = total <= cap ? 0u : sh_K;
+  auto collect = [&]() {
+    entries([&](int z, int id) {
+      if (tc_key(__int_as_float(z)) >= K) { const int slot = atomicAdd(&sh_n, 1); if (slot < RF_SLOTS) ei[slot] = id; }
+    });
+  };
+  collect();
   __syncthreads();
+  if (sh_n > RF_SLOTS) {
+    // More than are scored exactly: the best are neighbours, in few buffers and so with few threads, and a cut that the other
+    // threads' maxima make up for lets all of them pass.  Shared out anew, by their ids, neighbours have a maximum each
+    // (512 of them favoured by 256 samples of 670,091 neurons x 128 units: 162 us, by k_scan_all 2,954; of one sample of 100,003 neurons 62 and 96).
+    __syncthreads();
+    most[tid] = 0u;
+    if (tid == 0) sh_n = 0;
+    __syncthreads();
+    entries([&](int z, int id) {
+      const uint32_t key = tc_key(__int_as_float(z));
+      if (key >= K) atomicMax(&most[((unsigned)id * 2654435761u) >> 24], key);
+    });
+    find_cut();
+    if (sh_K > K) K = sh_K;
+    collect();
+    __syncthreads();
+  }
   const int nc = sh_n;
   const bool fix = nc > RF_SLOTS;                // many equal scores at the cut: the sample is scored exactly
   if (!fix) {

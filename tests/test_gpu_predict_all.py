@@ -311,3 +311,35 @@ def test_the_bound_takes_the_whole_norm(H, N, B):
             assert (scores(row, units, 1.1) == scanned).all(), (i, row)
     finally:
         ds.dslide_destroy(ctx)
+
+
+@pytest.mark.parametrize("B", [1, 200])
+def test_many_neighbours_that_are_favoured_together(B):
+    """512 neighbouring neurons that all samples prefer fill a few buffers, and the other buffers hold candidates as well: the cut by
+    the threads' maxima lets all of the neighbours pass, which are more than are scored exactly.  It is then taken among all
+    candidates, and no sample is scored over all neurons."""
+    from paper_2201_12667_b200 import binding as ds
+    from tests.gpu_harness import to_dev
+    N, H, k = 100003, 128, 16
+    r = np.random.default_rng(2)
+    ctx = ds.dslide_init(ds.make_config(input_dim=50, hidden_dim=H, output_dim=N, hash_family=workloads.SIMHASH, K=4, L=2, bucket_cap=16, max_batch=B))
+    try:
+        W1 = r.standard_normal((50, H)).astype(np.float32)
+        W2 = (r.standard_normal((N, H)) * (0.5 / np.sqrt(H))).astype(np.float32)
+        b2 = np.full(N, -2, np.float32)
+        first = 128 * 65                                        # every 64th tile gives the threshold
+        b2[first:first + 512] = 0
+        for name, x in (("W1", W1), ("W2", W2), ("b2", b2)):
+            ds.dslide_set_tensor(ctx, name, x)
+        cols, vals = r.integers(0, 50, B).astype(np.int32), r.uniform(0.5, 1, B).astype(np.float32)
+        batch = to_dev([np.arange(B + 1, dtype=np.int32), cols, vals])
+        ids, sc = predict_all(ctx, batch, k)
+        z = np.maximum(0, W1[cols].astype(np.float64) * vals[:, None]) @ W2.T.astype(np.float64) + b2
+        assert np.allclose(sc, np.sort(z, axis=1)[:, ::-1][:, :k], rtol=1e-5)
+        W2[0, 0] = -1e8                                         # now no sample can be decided: the scan adds up in another order
+        ds.dslide_set_tensor(ctx, "W2", W2)
+        ids_s, sc_s = predict_all(ctx, batch, k)
+        assert np.allclose(sc_s, sc, rtol=1e-5)
+        assert (sc_s != sc).any(axis=1).mean() > 0.9
+    finally:
+        ds.dslide_destroy(ctx)
