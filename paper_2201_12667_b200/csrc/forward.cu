@@ -246,9 +246,9 @@ __device__ __forceinline__ float block_sum(float v, float* sh) {
   return r;
 }
 
-// Floats as keys that order like them (unsigned), those that are no numbers last; no number has key 0.
+// Floats as keys that order like them (unsigned; both zeros are one), those that are no numbers last; no number has key 0.
 __device__ __forceinline__ uint32_t score_key(float z) {
-  const uint32_t b = __float_as_uint(z);
+  const uint32_t b = __float_as_uint(z + 0.f);      // minus zero plus zero is zero
   return z != z ? 1u : (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 // A score and its position as a word: the larger is the better, of equal scores the earlier

@@ -74,3 +74,21 @@ def test_fewer_rings_than_warps(H, K, max_labels, nlab, budget, least):
         assert cnt.min() > least and cnt.max() <= 256, cnt
     finally:
         pr.close()
+
+
+@pytest.mark.parametrize("H,k", [(64, 1), (64, 20), (260, 20)])
+def test_zeros_of_both_signs_are_equal(H, k):
+    """Scores of minus zero (a bias of minus zero, products too small for a number) and of zero go by id, too."""
+    N = 901
+    pr = Pair(D=501, H=H, N=N, family=SIMHASH, K=1, L=8, bucket_cap=N, max_batch=4, max_labels=3, seed=3)
+    try:
+        W2 = np.zeros((N, H), dtype=np.float32)
+        W2[::2] = -1e-30
+        pr.o.set("W2", W2.ravel())
+        pr.o.set("W1", np.zeros(501 * H, dtype=np.float32))
+        pr.o.set("b1", np.full(H, 1e-30, dtype=np.float32))
+        pr.o.build_tables()
+        wl = workloads.Workload(dict(workloads.config("tiny"), D=501, N=N, batch=4), seed=5)
+        check_predict(pr, wl.batch(0), 0, k, b2=np.full(N, -0.0, dtype=np.float32), same_ids=True)
+    finally:
+        pr.close()
