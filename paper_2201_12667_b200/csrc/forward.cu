@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   int* sh_tbeg = reinterpret_cast<int*>(smem + p.off_tbeg);          // [L]
   int* sh_ids = reinterpret_cast<int*>(smem + p.off_ids);            // [ACT_SM]
   float* sh_z = reinterpret_cast<float*>(smem + p.off_z);            // [ACT_SM]
-  float* sh_g = reinterpret_cast<float*>(smem + p.off_topk);         // [ACT_SM] training: errors of a small set (predict: its best-k lists)
+  float* sh_g = reinterpret_cast<float*>(smem + p.off_topk);         // [ACT_SM] training: errors of a small set (predict: work space of best_of)
   int* sh_col = reinterpret_cast<int*>(smem + p.off_col);            // [hid_rows]
   float* sh_val = reinterpret_cast<float*>(smem + p.off_val);        // [hid_rows]
   unsigned char* sh_b1 = smem + p.off_h1;                            // [256] bits of the hidden layer's projections
@@ -726,11 +726,12 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
   const int cp_r0 = tid / H4, cp_c0 = tid - cp_r0 * H4;
   bool pieced = false;
   if constexpr (NP == 8) {
-  if (p.L1 == 0 && nnz > R && nnz <= ACT_SM) {
+  if (p.L1 == 0 && H > 512 && nnz > R && nnz <= ACT_SM) {
     // More rows than a chunk (more than 512 units): a thread owns a 16-byte piece of every row, copies it and adds it up, HID_G rows to a
     // group of copies, as many groups ahead as fit -- no barriers.  (In chunks, a barrier before and after each, 76 rows of 1,024
     // units took 33,000 cycles of a block: a step of 1,024 samples 498 us, so 472; of one sample 48.6 and 43.7.  Of up to 512 units,
-    // half of the threads or fewer, it is the slower: 64 x 512 units 72.0 and 73.2.)
+    // half of the threads or fewer, it is the slower: 64 x 512 units 72.0 and 73.2; steps by tiles, which take this instance from 257 units
+    // on, of 64 samples x 200 nonzeros x 260 units 197.9 and 206.3, 256 x 76 x 384 340.9 and 344.0.)
     pieced = true;
     constexpr int HID_G = 4;
     for (int i = tid; i < nnz; i += FWD_THREADS) {
