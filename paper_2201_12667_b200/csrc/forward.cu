@@ -1743,7 +1743,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) k_forward(const FwdParams p) {
 #pragma unroll 1
     for (int i = 0; i < mygroups; ++i) {
       ask();
-      if (!bar_wait_limited(bars + slot, phase)) {
+      if (!bar_wait_limited_warp(bars + slot, phase)) {
         if (lane == 0) sh_misc[9] = 1;
         for (int q = i; q < gi; ++q) {             // what is still in flight gets one more bounded wait
           bar_wait_limited(bars + slot, phase);

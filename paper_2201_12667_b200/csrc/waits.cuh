@@ -31,6 +31,12 @@ __device__ __forceinline__ bool bar_wait_limited(uint64_t* bar, uint32_t parity)
     if (clock64() - t0 > WAIT_CYCLES) return false;
   return true;
 }
+// The same by a whole warp: one answer for all lanes, true where all have seen the phase complete.  (Each lane looks at the clock for
+// itself; one that gives up must not leave the others to exchange values without it.)
+__device__ __forceinline__ bool bar_wait_limited_warp(uint64_t* bar, uint32_t parity) {
+  const bool ok = bar_wait_limited(bar, parity);
+  return __all_sync(0xffffffffu, ok) != 0;
+}
 // Sets the flag of this block and, in a pair (PAIR: a cluster of two blocks), of the other one.
 template <bool PAIR>
 __device__ __forceinline__ void tc_give_up(volatile int* abort) {
@@ -52,7 +58,7 @@ __device__ __forceinline__ bool tc_bar_wait(uint64_t* bar, uint32_t parity, vola
   }
   return true;
 }
-// The same by a whole warp: true where all of its lanes have seen the phase complete, and the same answer for all.  A lane that has
+// The same by a whole warp, one answer for all lanes: true where all of them have seen the phase complete.  A lane that has
 // seen the flag, or that a wait has kept longer, is with the others again for what follows: an election, or an instruction that
 // takes the whole warp.
 template <bool PAIR, bool CLUSTER = false>

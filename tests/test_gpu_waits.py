@@ -43,3 +43,11 @@ def test_a_warp_gets_one_answer(probe):
     assert probe.run_waits(2, out, cycles) == 0
     assert list(out) == [0, 1, 32, 1]
     assert cycles[1] < 0.5e9, list(cycles)
+
+
+def test_a_warp_gives_up_together(probe):
+    """Half of the lanes' waits run out, the others' do not: all lanes are told so, after the limit of one wait."""
+    out, cycles = (ctypes.c_int * 4)(), (ctypes.c_longlong * 2)()
+    assert probe.run_waits(3, out, cycles) == 0
+    assert list(out)[:2] == [0, 32]
+    assert 2.0e9 < cycles[0] < 2.5e9, list(cycles)

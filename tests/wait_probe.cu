@@ -76,13 +76,32 @@ __global__ void k_warp(int* out, long long* cycles) {
   }
 }
 
+// The same of a wait without a flag, whose lanes give up by the clock.  out: [0] lanes told that the mixed phase has completed, [1] that
+// the completed one has; cycles: of the first
+__global__ void k_warp_limited(int* out, long long* cycles) {
+  __shared__ __align__(8) uint64_t never, done;
+  if (threadIdx.x == 0) {
+    init_bar(&never);
+    init_bar(&done);
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc_smem(&done)) : "memory");
+  }
+  __syncthreads();
+  const long long t0 = clock64();
+  for (int i = 0; i < 2; ++i) {
+    const bool ok = bar_wait_limited_warp(i == 0 && (threadIdx.x & 1) ? &never : &done, 0);
+    const int told = __popc(__ballot_sync(0xffffffffu, ok));
+    if (threadIdx.x == 0) { out[i] = told; cycles[i] = clock64() - t0; }
+  }
+}
+
 extern "C" int run_waits(int which, int* out, long long* cycles) {      // host arrays of 4 and 2
   int* d = nullptr;
   long long* c = nullptr;
   cudaError_t e = cudaMalloc(&d, 16);
   if (e == cudaSuccess) e = cudaMalloc(&c, 16);
   if (e == cudaSuccess) {
-    if (which == 2) k_warp<<<1, 32>>>(d, c);
+    if (which == 3) k_warp_limited<<<1, 32>>>(d, c);
+    else if (which == 2) k_warp<<<1, 32>>>(d, c);
     else if (which == 1) k_pair<<<2, 32>>>(d, c);
     else k_waits<<<1, 32>>>(d, c);
     e = cudaGetLastError();
