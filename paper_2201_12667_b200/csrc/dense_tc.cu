@@ -206,7 +206,7 @@ __device__ __forceinline__ void tc_squares(const unsigned char* row, int c0, int
   }
 }
 // One lane of a converged warp, the same at every call: the copies, multiplications and commits are its own, while the whole warp
-// walks the tiles, waits and agrees on what a wait has answered, so that their operands are the warp's.  Issued by one lane of a diverged warp an instruction took 84 to 134
+// walks the tiles and waits, so that their operands are the warp's.  Issued by one lane of a diverged warp an instruction took 84 to 134
 // cycles where the tensor pipe takes 64, which bounded the filter at every width (512 samples x 4,000,000 neurons x 256 units
 // 1,890 us, so 1,500; 1,024 x 253,855 x 200 246 and 218).
 __device__ __forceinline__ bool tc_elect() {
@@ -307,8 +307,12 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
   griddep_launch_dependents();       // the next kernel of the call may be placed as blocks of this one leave
   griddep_wait();                    // the filter launch reads the thresholds of the kernel before it
 
-  // Copies, multiplications and commits stop where a wait has run out; the other roles run through to their ends.
-  int fills = 0;                     // stages that this block has asked for
+  // Copies, multiplications and commits stop where a wait has run out; the other roles run through to their ends.  Each lane of the
+  // warps that issue them has a wait of its own.  All take part in the election whatever it has answered, the elected one issues by
+  // its own answer, and then they agree whether to go on, while what has been issued is under way.  (us for a call of 256 samples x
+  // 1,024 neurons x 1,024 units: 54.1 so, 54.8 with the vote before the election, 53.0 with none.)
+  auto agreed = [](bool ok) { return __all_sync(0xffffffffu, ok) != 0; };
+  int fills = 0;                     // stages that this block has asked for, or would have when a wait ran out
   if (warp == 0) {
     // ---------------- producer: one thread feeds the TMA ----------------
     int st = 0, stround = 0;
@@ -316,10 +320,10 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
     for (int i = 0; on && i < my_tiles; ++i) {
       const int row0 = (slice + i * p.nslices) * p.tile_stride * NT + (int)rank * ROWS;
       if (WIDE) {
-        for (int ks = 0; ks < ksub; ++ks, ++fills) {
-          if (stround > 0 && !(on = tc_bar_wait_warp<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
+        for (int ks = 0; on && ks < ksub; ++ks, ++fills) {
+          const bool ok = stround == 0 || tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag);
           unsigned char* to = smB + (size_t)st * tile_bytes;
-          if (tc_elect()) {
+          if (tc_elect() && ok) {
             if (PAIR) {
               if (rank == 0) tc_bar_expect(bar_full + st, 2u * tile_bytes);
               const uint32_t full = tc_at_rank(bar_full + st, 0u);
@@ -331,13 +335,13 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
               tc_tma_2d(to + SLAB, &tmH, ks * TC_KB, s0, bar_full + st);
             }
           }
-          __syncwarp();
+          on = agreed(ok);
           if (++st == nst) { st = 0; ++stround; }
         }
         continue;
       }
-      if (stround > 0 && !(on = tc_bar_wait_warp<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag))) break;
-      if (tc_elect()) {
+      const bool ok = stround == 0 || tc_bar_wait<PAIR>(bar_empty + st, (stround - 1) & 1, abort_flag);
+      if (tc_elect() && ok) {
         if (rank == 0) tc_bar_expect(bar_full + st, (PAIR ? 2u : 1u) * tile_bytes);
         const uint32_t full = PAIR ? tc_at_rank(bar_full + st, 0u) : 0u;
         for (int ks = 0; ks < ksub; ++ks) {
@@ -346,7 +350,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           else tc_tma_2d(to, &tmW, ks * TC_KB, row0, bar_full + st);
         }
       }
-      __syncwarp();
+      on = agreed(ok);
       ++fills;
       if (++st == nst) { st = 0; ++stround; }
     }
@@ -360,15 +364,15 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
       const uint64_t b_base = tc_desc(tc_smem(smB));      // a descriptor's address field counts 16-byte units
       int st = 0, stround = 0, acc = 0, accround = 0;
       for (int i = 0; on && i < my_tiles; ++i) {
-        if (!WIDE && !tc_bar_wait_warp<PAIR>(bar_full + st, stround & 1, abort_flag)) break;
-        if (accround > 0 && !tc_bar_wait_warp<PAIR>(bar_accempty + acc, (accround - 1) & 1, abort_flag)) break;
+        bool ok = WIDE || tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag);
+        ok = (accround == 0 || tc_bar_wait<PAIR>(bar_accempty + acc, (accround - 1) & 1, abort_flag)) && ok;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem_base + (uint32_t)(acc * NT);
         if (WIDE) {
-          for (int ks = 0; ks < ksub; ++ks) {
-            if (!(on = tc_bar_wait_warp<PAIR>(bar_full + st, stround & 1, abort_flag))) break;
+          for (int ks = 0; on && ks < ksub; ++ks) {
+            ok = tc_bar_wait<PAIR>(bar_full + st, stround & 1, abort_flag) && ok;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (tc_elect()) {
+            if (tc_elect() && ok) {
               const uint64_t b = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
               const uint64_t a = b + (uint64_t)(SLAB >> 4);
               const int kn = ks == ksub - 1 ? klast : TC_KB / 8;
@@ -376,7 +380,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
                 tc_mma_ss<PAIR>(d, a + (uint64_t)(kk * 2), b + (uint64_t)(kk * 2), idesc, (ks | kk) != 0 ? 1u : 0u);
               tc_commit<PAIR>(bar_empty + st);
             }
-            __syncwarp();
+            on = agreed(ok);
             if (++st == nst) { st = 0; ++stround; }
           }
           if (!on) break;
@@ -385,7 +389,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           if (++acc == nacc) { acc = 0; ++accround; }
           continue;
         }
-        if (tc_elect()) {
+        if (tc_elect() && ok) {
           const uint64_t b_tile = b_base + (uint64_t)(((uint32_t)st * tile_bytes) >> 4);
           for (int ks = 0; ks < kfull; ++ks) {
             const uint32_t a = tmem_base + acol + (uint32_t)(ks * TC_KB);      // lanes = samples, columns = hidden units
@@ -401,7 +405,7 @@ k_dense_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUte
           tc_commit<PAIR>(bar_empty + st);          // the tile's shared memory is free once these instructions have read it
           tc_commit<PAIR>(bar_accfull + acc);       // and the accumulator is complete
         }
-        __syncwarp();
+        on = agreed(ok);
         if (++st == nst) { st = 0; ++stround; }
         if (++acc == nacc) { acc = 0; ++accround; }
       }
