@@ -207,8 +207,8 @@ __device__ __forceinline__ void tc_squares(const unsigned char* row, int c0, int
 }
 // One lane of a converged warp, the same at every call: the copies, multiplications and commits are its own, while the whole warp
 // walks the tiles and waits, so that their operands are the warp's.  Issued by one lane of a diverged warp an instruction took 84 to 134
-// cycles where the tensor pipe takes 64, which bounded the filter at every width (512 samples x 4,000,000 neurons x 256 units
-// 1,890 us, so 1,500; 1,024 x 253,855 x 200 246 and 218).
+// cycles where the tensor pipe takes 64, which bounded the filter at every width (a tile of 256 units in pairs 2,970 cycles, so 2,080;
+// 1,024 samples x 253,855 neurons x 200 units 246 us, so 218).
 __device__ __forceinline__ bool tc_elect() {
   uint32_t one;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
@@ -1238,9 +1238,11 @@ cudaError_t launch_dense_tc(Ctx* c, int batch, int k, int32_t* out_ids, float* o
   const size_t off_tau = off_list + up((size_t)Bpad * 4), off_cnt = off_tau + up((size_t)Bpad * 4);
   const size_t off_cand = off_cnt + up((size_t)nvs * Bpad * 4);
   // The threshold is the rank-th best of the subset's maxima, the rank chosen so that about TC_TARGET times as many neurons
-  // reach it over all N whatever the subset's share; a buffer has room for four times its expected fill.  A rank of TC_RANK_MIN
-  // leaves fewer than the cap of k = 5 once in 10^8 samples (such a sample is still decided by its threshold, mostly), and one
-  // above k keeps that so where the best neighbours are all in the subset.
+  // reach it over all N whatever the subset's share; a buffer has room for four times its expected fill.  A rank of TC_RANK_MIN,
+  // for k up to 3, leaves fewer candidates than the cap once in 10^9 samples or less, that of k = 5, 10, once in 10^11 (such a sample
+  // is still decided by its threshold, mostly), and one above k keeps that so where the best neighbours are all in the subset.  With a
+  // few tiles the subset is one of them: of 129 neurons x 1,024 units 1 in 80 samples is undecided with k = 5, and with k = 64 all of 129
+  // neurons and up to 80 % of 384 are, for fewer than k reach rank 24 of 128.
   const int want = min(TC_RANK_CAP, max(TC_RANK_MIN, k + TC_RANK_OVER));
   int rank = (want * TC_TARGET + stride - 1) / stride;
   if (rank > want) rank = want;

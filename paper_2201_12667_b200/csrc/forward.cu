@@ -2112,7 +2112,11 @@ static double expected_set(const Ctx* c) {
 // Whether the active rows go through the warps' rings (k_forward<., 2 ...>) or are staged in chunks of the block's space.  us, staged /
 // by rings: a step of 256 samples x 256 units x 200 rows 84.7 / 79.6, 16 x 200 units x 200 rows 36.7 / 34.8, one sample x 512 units
 // 54.9 / 36.9, 1,024 x 1,024 units 615 / 498; but 1,024 x 200 units x 100 rows, which are one chunk, 167 / 171, one sample x 136
-// units x 200 rows (a chunk and a quarter) 26.0 / 27.0.  (A DWTA bucket that is met holds a row more than the mean.)
+// units x 200 rows (a chunk and a quarter) 26.0 / 27.0.  Both ways over 136, 200 and 256 units, 1 to 1,024 samples and sets of 48 to 694
+// rows, 168 shapes, by the set's size in chunks: steps staged / by rings 0.94 to 1.04 below one chunk, 0.97 to 1.05 from 1.25 to 1.6,
+// 0.99 to 1.19 above; inference 0.90 to 1.03, 0.89 to 1.03 and 0.89 to 1.14.  What loses by the rule: inference at 136 units, where
+// two lanes of 32 have a second piece (up to 12 %), and steps of 256 units at 1.15 chunks, which are staged (up to 11 %).
+// (A DWTA bucket that is met holds a row more than the mean.)
 static bool by_rings(const Ctx* c) {
   if (c->H <= 128 || c->H > 256) return c->H > 256;
   return expected_set(c) + c->L > 1.25 * (double)(c->fwd_stage_bytes / ((c->H + 4) * 4 + 4));

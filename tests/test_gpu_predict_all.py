@@ -73,7 +73,8 @@ FLAGGED = [           # H, N, batch, k, samples whose filter cannot decide (of t
 @pytest.mark.parametrize("H,N,B,k,flagged", FLAGGED)
 def test_samples_that_are_scored_over_all_neurons(H, N, B, k, flagged):
     """One row of W2 with a huge norm widens the error bound of the filter, so that every sample with a hidden activation
-    is scored over all neurons; the others (hidden activation zero, scores the biases alone) are not."""
+    is scored over all neurons; the others (hidden activation zero, scores the biases alone) need not be.  Results are right for
+    both, call after call; which samples are scored so is asked by test_the_bound_takes_the_whole_norm."""
     import torch
     from paper_2201_12667_b200 import binding as ds
     from tests.gpu_harness import to_dev

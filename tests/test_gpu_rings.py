@@ -1,6 +1,6 @@
 """The pass over the active rows by the warps' rings (hidden layers wider than 128 units, sets of more than a chunk; always beyond 256
 units) and the selection of the k best scores, against the oracle: widths at the edges of a lane's pieces, sets of a few rows and of
-thousands, groups of rows that end in the middle, equal scores."""
+thousands, groups of rows that end in the middle, fewer rings than warps, equal scores and zeros of both signs."""
 import numpy as np
 import pytest
 import torch
